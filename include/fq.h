@@ -118,7 +118,8 @@ typedef struct fq_layout {
     uint32_t max_bucket_packets; /* longest packet list (depth + tail) of one bucket in one tile */
     uint32_t max_tail_packets; /* longest tail; 0 = every packet is column-slotted */
     uint32_t tilecoo_encoded;  /* 1 = the three maxima above describe the arrays in use (set by
-                                  fq_encode_tilecoo); 0 = unknown: the kernels assume the worst */
+                                  fq_encode_tilecoo); 2 = likewise, and some position holds more than one outlier (their
+                                  sum counts); 0 = unknown: the kernels assume the worst */
     uint32_t kernel_hint;      /* 0 = the library chooses the kernel of a launch from its rows and the layer's
                                   shape; 1 = never the short-job kernel (one CTA per strip of 32 columns), so
                                   that tests reach the streaming kernels on small layers too */
@@ -229,12 +230,11 @@ fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes);
  *     CTA per strip, whose warps split K among themselves and read the weights
  *     straight into registers; every other layer streams (tile, k-step) units
  *     through a bulk-copy/mbarrier ring on persistent CTAs;
- *   - 17 to 32 rows (a larger M is cut into such launches), groups of 128: a
- *     kernel built on tcgen05.mma with 8-bit integer operands.  Its
- *     activations are block fixed point, 22 bits plus sign relative to the
- *     largest |x| of each row and group, so activations more than 2^14 below
- *     that maximum are rounded (to 2^-22 of it).  Groups of 64 stay with
- *     launches of 16 rows.
+ *   - 17 to 128 rows: one launch of a kernel built on tcgen05.mma with BF16
+ *     operands (the exact integers q - z, and the outliers as a second matrix
+ *     that is zero elsewhere).  If the encoding names a position twice, or was
+ *     not made by fq_encode_tilecoo (L->tilecoo_encoded), M is cut into
+ *     launches of 16 rows instead.
  * L->kernel_hint = 1 keeps the one-CTA-per-strip kernel out (for tests).
  * X: device, M x K BF16.  M in [1, FQ_MAX_M].  Y: device, M x N BF16,
  * overwritten.  All other arrays: device copies of the host packer/encoder

@@ -271,6 +271,7 @@ struct Encoded {
     uint32_t max_tile_packets = 0;
     uint32_t max_bucket_packets = 0;
     uint32_t max_tail_packets = 0;
+    bool repeated = false;          // some position appears more than once
 };
 
 // Bucket of a tile column: the four columns {g, g + 8, g + 16, g + 24} of a 32-column block share
@@ -349,7 +350,7 @@ fq_status_t encode_impl(const fq_layout_t* L, const uint32_t* k, const uint32_t*
     E.indptr.assign(ntile + 1, 0);
     E.info.assign(ntile * NB, 0);
     std::vector<std::vector<uint32_t>> tile_words(ntile);
-    int bad = 0;
+    int bad = 0, repeated = 0;
 #pragma omp parallel for schedule(dynamic, 16)
     for (int64_t t = 0; t < (int64_t)ntile; ++t) {
         std::vector<std::vector<Entry>> per(NB * 4);      // by (bucket, number in bucket)
@@ -364,6 +365,11 @@ fq_status_t encode_impl(const fq_layout_t* L, const uint32_t* k, const uint32_t*
                 std::vector<Entry>& col = per[b * 4 + j];
                 std::sort(col.begin(), col.end(), [](const Entry& x, const Entry& y) { return x.k < y.k; });
                 longest = std::max(longest, col.size());
+                for (size_t e = 1; e < col.size(); ++e)
+                    if (col[e].k == col[e - 1].k) {
+#pragma omp atomic write
+                        repeated = 1;
+                    }
             }
             depths[b] = longest > kSlottedMax ? kSlottedWithTail : (uint32_t)longest;
         }
@@ -467,6 +473,7 @@ fq_status_t encode_impl(const fq_layout_t* L, const uint32_t* k, const uint32_t*
         E.indptr[t + 1] = off;
     }
     if (bad) return fq::fail(FQ_ERR_UNSUPPORTED_SHAPE, "a bucket exceeds the packet offset/count range of its descriptor");
+    E.repeated = repeated != 0;
     for (size_t i = 0; i < E.info.size(); ++i) {
         const uint32_t depth = (E.info[i] >> 16) & 0xffu, tail = E.info[i] >> 24;
         E.max_bucket_packets = std::max(E.max_bucket_packets, depth + tail);
@@ -524,7 +531,7 @@ fq_status_t fq_encode_tilecoo(fq_layout_t* L, const uint32_t* k, const uint32_t*
     L->max_tile_packets = E.max_tile_packets;
     L->max_bucket_packets = E.max_bucket_packets;
     L->max_tail_packets = E.max_tail_packets;
-    L->tilecoo_encoded = 1;
+    L->tilecoo_encoded = E.repeated ? 2 : 1;
     return FQ_OK;
 }
 

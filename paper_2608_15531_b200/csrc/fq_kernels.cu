@@ -1,14 +1,12 @@
 // CUDA side of the library (sm_100a): the fused W4A16 + Tile-COO outlier decode matmul
 // (Eq. 1; Sections 3.1, 4.1, 4.2), its two unfused baselines and the launchers behind the C ABI.
 //
-// The fused operator is one persistent, warp-specialised kernel (one CTA per SM), fq_tc_kernel in
-// fq_tc_kernel.cuh: (tile, k-step) units of 128 rows x BN columns stream through a ring of shared-memory
-// stages (bulk copies + mbarrier expect_tx); the codes are unpacked to the exact integers q - z in BF16
-// and written to tensor memory as the A operand of tcgen05.mma, the activations are the B operand, and
-// the scale is applied once per group in FP32:
+// Three kernels serve the fused operator, chosen per launch from its rows and the layer's shape (launch_gemm): a
+// streaming kernel and a short-job kernel with warp-level MMAs for up to 16 rows (fq_mma_kernel.cuh,
+// fq_direct_kernel.cuh) and a tcgen05 kernel for 17 to 128 (fq_tc_kernel.cuh).  The streaming kernels are
+// persistent and warp-specialised: (tile, k-step) units of 128 rows stream through a ring of shared-memory stages
+// (bulk copies + mbarrier expect_tx).  All feed the tensor cores exact integers and apply the scale once per group in FP32:
 //     acc[m] += s * sum_k x (q - z)                                     (Eq. 3 inside Eq. 1)
-// The unit's Tile-COO outliers are added in the registers of the epilogue threads, one thread per
-// output column.
 //
 // Units are split over CTAs as contiguous ranges (stream-K) or, for layers with few column tiles, as
 // tile-aligned parts.  A tile whose k-range is shared by several CTAs is finished by the last to
@@ -16,6 +14,7 @@
 // is bounded: on expiry the CTA raises the scratch status word, drains and leaves through the common
 // exit that frees its tensor memory.
 #include <cooperative_groups.h>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -33,28 +32,6 @@ constexpr int kSmemBudget = 232448;    // 227 KB per CTA on sm_100
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 constexpr uint32_t kTmemCols = 512;
 
-
-struct Params {
-    const uint8_t* wq;
-    const uint16_t* scale;
-    const uint16_t* zero;
-    const uint32_t* indptr;
-    const uint32_t* info;
-    const uint4* packed;
-    uint16_t* Y;
-    uint32_t* status;
-    uint32_t* counters;
-    float* partials;
-    const uint8_t* xblob; // per k-step: the activation block fq_prep_x_kernel wrote (limbs, scales and sums, FP32 copy)
-    uint32_t M, K, N, KT, NT;
-    uint32_t NB, coo_cap, stages;
-    uint32_t split;   // 0 = units dealt out as one contiguous range per CTA (stream-K);
-                      // c > 0 = every column tile belongs to c CTAs, CTA b takes part b mod c of tile b / c
-    // shared-memory offsets (bytes); all but the last are relative to a stage
-    uint32_t stage_bytes, off_sz, off_xcan, off_xmeta, off_xt, off_info, off_coo;
-    uint32_t off_xch;     // hand-over of the second epilogue set's sums (BN x RR floats), if there are two sets
-    uint32_t off_bar;
-};
 
 // ----------------------------------------------------------------------------- PTX helpers
 
@@ -79,14 +56,15 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// The time hint lets a waiting thread sleep in hardware (up to about 20 us per attempt) instead of
-// spinning on the issue slots that the working warps of the CTA need.
+// A waiting thread sleeps in hardware for a while instead of spinning on the issue slots that the working warps of the
+// CTA need.  No suspend-time hint: with one of 20 us the waits of the tcgen05 kernel returned later (8192 x 28672 at
+// 32 rows 80.4 us, without it 78.0; spinning on test_wait instead 83.1).
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(20000u)
+        : "r"(bar), "r"(parity)
         : "memory");
     return ok;
 }
@@ -173,28 +151,6 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// D[128 x N] (+)= A[128 x 16] (TMEM) * B[16 x N] (shared-memory descriptor), BF16 in, FP32 out
-// Called by the whole (converged) warp with warp-uniform operands; one elected lane issues.
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile(
-        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar)
-        : "memory");
-}
-// K-major, no swizzle: 8 rows x 16 B core matrices; LBO = step between the two K halves of one MMA,
-// SBO = step between 8-row groups.
-__device__ __forceinline__ uint64_t make_b_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    return (uint64_t)((saddr & 0x3ffffu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
-           (1ull << 46);
-}
-
 // Which CTA owns unit u when U units are dealt out as contiguous ranges, the first r CTAs one longer.
 __device__ __forceinline__ uint32_t cta_of_unit(uint32_t u, uint32_t q, uint32_t r) {
     const uint32_t big = r * (q + 1);
@@ -374,12 +330,6 @@ __global__ void __launch_bounds__(kSpmmThreads, 2) fq_spmm_kernel(const uint16_t
 
 // ----------------------------------------------------------------------------- launch plumbing
 
-struct Plan {
-    Params p;
-    uint32_t threads, smem, grid;
-    bool general;    // the layer needs the general form of the outlier step
-};
-
 static inline uint32_t round_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
 static int sm_count_cached() {
@@ -396,67 +346,78 @@ static int sm_count_cached() {
     return cached[dev];
 }
 
-// Rows kept per epilogue thread of the tcgen05 kernel, and the MMA's batch columns, for a launch of M rows.
-static inline uint32_t rr_of(uint32_t m) { return m <= 1 ? 1u : (m <= 4 ? 4u : (m <= 8 ? 8u : (m <= 16 ? 16u : 32u))); }
-static inline uint32_t nmma_of(uint32_t m) { return (uint32_t)nmma_rows((int)rr_of(m)); }      // limb rows of the MMA operand
+// The tcgen05 kernel's variant for a launch: the batch rows its tensor memory and drain warps are laid out for.
+static inline uint32_t tc_rows(uint32_t m) { return m <= 32 ? 32u : (m <= 64 ? 64u : 128u); }
 
-// Plan of a launch of up to 32 rows (16 with groups of 64: the accumulators of both groups must fit in tensor memory).
-static fq_status_t make_plan(const fq_layout_t* L, uint32_t M, bool sparse, Plan& pl) {
-    const uint32_t BN = L->BN, NB = L->buckets_per_tile, GPS = kBK / L->group;
-    const uint32_t NMMA = nmma_of(M), RR = rr_of(M);
-    Params& p = pl.p;
+struct TcPlan {
+    TcParams p;
+    uint32_t threads, smem, grid, nr;
+};
+
+static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
+    TcParams& p = pl.p;
     std::memset(&p, 0, sizeof(p));
-    p.M = M; p.K = L->K; p.N = L->N; p.KT = L->K / kBK; p.NT = L->N / BN; p.NB = NB;
+    pl.nr = tc_rows(M);
+    const uint32_t GPS = kBK / L->group;
     const int sms = sm_count_cached();
     if (sms <= 0) return fail(FQ_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
+    p.M = M; p.K = L->K; p.N = L->N; p.KT = L->K / kBK; p.NT = L->N / 128;
+    p.halves = L->BN / 128;
+    p.nmma = round_up(M, 16);
+    p.parts = L->value_type == FQ_VALUE_FP16 ? 2 : 1;
     const uint32_t NT = p.NT, KT = p.KT;
     uint32_t grid = std::min<uint32_t>({(uint32_t)sms, kMaxCtas, NT * KT});
-    uint32_t units_per_cta = (NT * KT + grid - 1) / grid;
+    const uint32_t units_per_cta = (NT * KT + grid - 1) / grid;
     // Tile-aligned split instead of one contiguous range per CTA when it costs at most one more unit
     // per CTA: then no CTA has to settle two split tiles in a row.
-    uint32_t split = 0;
     if (NT <= grid) {
         const uint32_t c = std::min<uint32_t>(grid / NT, KT);
         if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) {
-            split = c;
+            p.split = c;
             grid = NT * c;
-            units_per_cta = (KT + c - 1) / c;
         }
     }
-    p.split = split;
-    const uint32_t w_bytes = 16 * BN * 4, sz_bytes = 2 * GPS * BN * 2;
-    const uint32_t xt_bytes = sparse ? kBK * RR * 4 : 0;                 // FP32 k-major copy [k][RR]
-    uint32_t cap = 0;
-    if (sparse) {
-        cap = L->tilecoo_encoded ? std::max<uint32_t>(8, round_up(L->max_tile_packets, 8)) : 256;
-        cap = std::min<uint32_t>(cap, 1024);
-    }
-    const uint32_t xch_bytes = epilogue_sets((int)RR) == 2 ? BN * RR * 4 : 0;
-    uint32_t stage = 0, S = 0;
+    const uint32_t fixed = 1024 /* alignment */ + 1024 /* barriers */ + tc_outlier_tiles(pl.nr) * kWoTile;
+    uint32_t cap = std::min<uint32_t>(1024, std::max<uint32_t>(8, round_up(L->max_tile_packets, 8))), stage = 0, S = 0;
     for (;;) {
-        p.off_sz = w_bytes;
-        p.off_xcan = p.off_sz + round_up(sz_bytes, 128);
-        // the k-step's activation block lands here as one copy: limbs (NMMA rows x 128 k, one byte each),
-        // scales and sums, FP32 copy (kernels with outliers only)
-        p.off_xmeta = p.off_xcan + blob_meta_off((int)RR);
-        p.off_xt = p.off_xcan + blob_xt_off((int)RR, (int)GPS);
-        p.off_info = p.off_xt + xt_bytes;
-        p.off_coo = p.off_info + (sparse ? round_up(NB * 4, 128) : 0);
-        stage = round_up(p.off_coo + cap * 16, 128);
-        S = std::min<uint32_t>(8, (kSmemBudget - 1024 - xch_bytes) / stage);
-        if (S >= 4 || cap <= 64) break;
-        cap = std::max<uint32_t>(64, cap / 2);  // oversized tiles read their tail from global memory
+        p.off_w = 256 * p.nmma;
+        p.off_sz = p.off_w + 8192;
+        p.off_info = p.off_sz + 2 * GPS * 256;
+        p.off_coo = p.off_info + 128;
+        stage = round_up(p.off_coo + cap * 16, 1024);
+        S = std::min<uint32_t>(8, (kSmemBudget - fixed) / stage);
+        if (S >= 3 || cap <= 64) break;
+        cap = std::max<uint32_t>(64, cap / 2);                 // the rest of an oversized tile is read from global memory
     }
     if (S < 2) return fail(FQ_ERR_UNSUPPORTED_SHAPE, "shared-memory stages do not fit");
     p.coo_cap = cap; p.stages = S; p.stage_bytes = stage;
-    // hot columns, tiles larger than the staged part, or an encoding whose sizes were not recorded
-    pl.general = sparse && (L->max_tail_packets > 0 || L->max_tile_packets > cap || !L->tilecoo_encoded);
-    p.off_xch = S * stage;
-    p.off_bar = p.off_xch + xch_bytes;
-    pl.smem = p.off_bar + 1024;
-    pl.threads = 32 * (kTcFirstUnpack + (1 + epilogue_sets((int)RR)) * (BN / 32));
+    p.general = L->max_tile_packets > cap;
+    p.off_wo = S * stage;
+    p.off_bar = p.off_wo + tc_outlier_tiles(pl.nr) * kWoTile;
+    pl.smem = p.off_bar + 2048;
+    const uint32_t drain = 4 * (pl.nr / 32);
+    pl.threads = 32 * (12 + drain + (12 + drain + 8 <= 32 ? 8 : 4));            // as TcShape::WARPS
     pl.grid = grid;
     return FQ_OK;
+}
+
+// The tiled tensor map of a launch's activations: boxes of 64 K values by the MMA's batch rows, 128-byte swizzle;
+// rows beyond M read as zero.
+static fq_status_t encode_x_map(const fq_layout_t* L, const uint16_t* X, uint32_t M, uint32_t nmma, CUtensorMap* map) {
+    typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                 const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const EncodeFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult qr;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &qr) != cudaSuccess || qr != cudaDriverEntryPointSuccess) f = nullptr;
+        return (EncodeFn)f;
+    }();
+    if (!fn) return fail(FQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
+    const cuuint64_t dims[2] = {L->K, M}, strides[1] = {(cuuint64_t)L->K * 2};
+    const cuuint32_t box[2] = {64, nmma}, ones[2] = {1, 1};
+    const CUresult e = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)X, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return e == CUDA_SUCCESS ? FQ_OK : fail(FQ_ERR_CUDA, "cuTensorMapEncodeTiled: %d", (int)e);
 }
 
 // Short jobs go to fq_direct_kernel: launches of up to 16 rows on layers with so few strips of 32 columns and
@@ -492,30 +453,25 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
     return warps == 32 ? pick_direct_rows<32>(rows, g, sparse) : pick_direct_rows<16>(rows, g, sparse);
 }
 
-// Scratch layout: status word and header, tile-arrival counters, FP32 partial slots, then the activation
-// blocks fq_prep_x_kernel writes for the launch in flight (one per k-step).
+// Which kernel serves a launch: up to 16 rows the warp-level MMA kernels, more rows the tcgen05 kernel, whose cost
+// grows slowly with them.  The latter writes outliers into a tile instead of adding them, so an encoding that names a
+// position twice (or whose origin is unknown) stays with launches of 16 rows.
+static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) { return rows > 16 && sparse && L->tilecoo_encoded == 1; }
+static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
+
+// Scratch layout: status word and header, tile-arrival counters, FP32 partial slots (two per CTA).
 struct Scratch {
-    size_t off_partials, off_xb, total;
+    size_t off_partials, total;
 };
-// Which kernel serves a launch is decided by its rows alone: up to 16 rows the warp-level MMA kernel, 17 to 32
-// rows the tcgen05 kernel (its MMAs cost the same for any number of batch rows up to 42; with groups of 64 its
-// two accumulators per unit fit in tensor memory only up to 16 rows, so such layers stay with the first).
-static inline bool tc_serves(const fq_layout_t* L, uint32_t rows) { return rows > 16 && L->group == 128; }
-static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left) { return tc_serves(L, rows_left) ? std::min<uint32_t>(rows_left, 32u) : std::min<uint32_t>(rows_left, 16u); }
-static Scratch scratch_layout(const fq_layout_t* L, uint32_t rows) {
-    const bool tc = tc_serves(L, rows);
-    const size_t prow = tc ? 32 : 16;                     // batch rows of an FP32 partial slot
+static Scratch scratch_layout(uint32_t BN, uint32_t rows) {
     Scratch sc;
     sc.off_partials = kWsHeaderBytes + kWsCounterBytes;
-    sc.off_xb = sc.off_partials + (size_t)kMaxCtas * 2 * L->BN * prow * 4;
-    sc.total = sc.off_xb + (tc ? (size_t)(L->K / kBK) * blob_bytes(32, (int)(kBK / L->group)) : 0);
+    // a slot: the columns of a stored tile by 16 rows, or the tcgen05 kernel's 128 columns by its rows (not less than the
+    // stored tile by 32: FQ_STATIC_SCRATCH_MAX_M states what the built-in scratch holds)
+    const size_t slot = rows <= 16 ? (size_t)BN * 16 : std::max<size_t>(128 * (size_t)tc_rows(rows), (size_t)BN * 32);
+    sc.total = sc.off_partials + (size_t)kMaxCtas * 2 * slot * 4;
     return sc;
 }
-
-typedef void (*PrepFn)(const uint16_t*, uint32_t, uint32_t, uint8_t*);
-static PrepFn pick_prep() { return fq_prep_x_kernel<32, 128>; }      // 17 to 32 rows, groups of 128: one variant
-
-typedef void (*KernelFn)(const Params);
 
 struct MmaPlan {
     MmaParams p;
@@ -624,13 +580,11 @@ static MmaKernelFn pick_mma_kernel(uint32_t bn, uint32_t M, uint32_t g, bool spa
     return mo == 1 ? pick_mma_group<256, 1>(g, sparse, ms, ngrp, hot) : pick_mma_group<256, 2>(g, sparse, ms, ngrp, hot);
 }
 
-template <int BN, int RR, int G>
-static KernelFn pick_tc_sparse(bool sparse, bool hot) {
-    if (!sparse) return (KernelFn)fq_tc_kernel<BN, RR, G, false, false>;
-    return hot ? (KernelFn)fq_tc_kernel<BN, RR, G, true, true> : (KernelFn)fq_tc_kernel<BN, RR, G, true, false>;
-}
-static KernelFn pick_kernel(uint32_t bn, bool sparse, bool hot) {      // 17 to 32 rows, groups of 128: one variant per tile width
-    return bn == 128 ? pick_tc_sparse<128, 32, 128>(sparse, hot) : pick_tc_sparse<256, 32, 128>(sparse, hot);
+typedef void (*TcKernelFn)(const CUtensorMap, const TcParams);
+template <int NR>
+static TcKernelFn pick_tc_group(uint32_t g) { return g == 64 ? (TcKernelFn)fq_tc_kernel<NR, 64> : (TcKernelFn)fq_tc_kernel<NR, 128>; }
+static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g) {
+    return nr == 128 ? pick_tc_group<128>(g) : (nr == 64 ? pick_tc_group<64>(g) : pick_tc_group<32>(g));
 }
 
 // cudaFuncSetAttribute costs several microseconds: do it once per (kernel, device).
@@ -672,9 +626,8 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
                                void* workspace, size_t workspace_bytes, void* stream, bool sparse) {
     fq_status_t st = check_gemm_args(L, X, M, wq, scale, zero, indptr, info, packed, Y, workspace, sparse);
     if (st != FQ_OK) return st;
-    const size_t need = scratch_layout(L, M).total;
-    if (workspace_bytes < need) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, need);
-    const Scratch sc = scratch_layout(L, M);
+    const Scratch sc = scratch_layout(L->BN, M);
+    if (workspace_bytes < sc.total) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, sc.total);
     cudaLaunchAttribute attr[1];
     std::memset(attr, 0, sizeof(attr));
     // Programmatic dependent launch: a grid may become resident while the kernel before it in the stream
@@ -684,7 +637,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     for (uint32_t m0 = 0; m0 < M;) {
-        const uint32_t mb = rows_per_launch(L, M - m0);
+        const uint32_t mb = rows_per_launch(L, M - m0, sparse);
         const uint16_t* Xm = (const uint16_t*)X + (size_t)m0 * L->K;
         uint16_t* Ym = (uint16_t*)Y + (size_t)m0 * L->N;
         cudaLaunchConfig_t cfg;
@@ -693,34 +646,27 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaError_t e;
-        if (tc_serves(L, mb)) {
-            Plan pl;
-            st = make_plan(L, mb, sparse, pl);
+        if (tc_serves(L, mb, sparse)) {
+            TcPlan pl;
+            st = make_plan_tc(L, mb, pl);
             if (st != FQ_OK) return st;
-            Params& p = pl.p;
-            const uint32_t rr = rr_of(mb);
-            uint8_t* xb = (uint8_t*)workspace + sc.off_xb;
+            TcParams& p = pl.p;
             p.Y = Ym;
             p.wq = (const uint8_t*)wq; p.scale = (const uint16_t*)scale; p.zero = (const uint16_t*)zero;
             p.indptr = (const uint32_t*)indptr; p.info = (const uint32_t*)info; p.packed = (const uint4*)packed;
             p.status = (uint32_t*)workspace;
             p.counters = (uint32_t*)((uint8_t*)workspace + kWsHeaderBytes);
             p.partials = (float*)((uint8_t*)workspace + sc.off_partials);
-            p.xblob = xb;
-            KernelFn fn = pick_kernel(L->BN, sparse, pl.general);
+            CUtensorMap xmap;
+            st = encode_x_map(L, Xm, mb, p.nmma, &xmap);
+            if (st != FQ_OK) return st;
+            TcKernelFn fn = pick_tc_kernel(pl.nr, L->group);
             e = ensure_smem_attr((const void*)fn, (int)kSmemBudget);
             if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-            // the activation blocks of these rows, then the fused kernel
-            const uint32_t warps = rr * (L->K / kBK);
-            cfg.gridDim = dim3((warps + 3) / 4);
-            cfg.blockDim = dim3(128);
-            cfg.dynamicSmemBytes = 0;
-            e = cudaLaunchKernelEx(&cfg, pick_prep(), Xm, mb, L->K, xb);
-            if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "activation preparation launch: %s", cudaGetErrorString(e));
             cfg.gridDim = dim3(pl.grid);
             cfg.blockDim = dim3(pl.threads);
             cfg.dynamicSmemBytes = pl.smem;
-            e = cudaLaunchKernelEx(&cfg, fn, p);
+            e = cudaLaunchKernelEx(&cfg, fn, xmap, p);
         } else if (direct_warps(L, mb)) {
             DirectParams p;
             std::memset(&p, 0, sizeof(p));
@@ -795,7 +741,7 @@ extern "C" {
 fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes) {
     if (!layout_ok(L) || !bytes) return fail(FQ_ERR_INVALID_ARG, "bad layout or null output");
     if (M < 1 || M > FQ_MAX_M) return fail(FQ_ERR_INVALID_ARG, "M = %u outside [1, %u]", M, FQ_MAX_M);
-    *bytes = scratch_layout(L, M).total;
+    *bytes = scratch_layout(L->BN, M).total;
     return FQ_OK;
 }
 
@@ -840,7 +786,7 @@ fq_status_t fq_fused_w4a16_outlier_gemm_noalloc(const fq_layout_t* L, const void
     // every argument error is reported before anything is put on the stream (the scratch pointer stands in for itself)
     fq_status_t st = check_gemm_args(L, X, M, wq, scale, zero, tile_indptr, bucket_info, packed_outliers, Y, (void*)256, true);
     if (st != FQ_OK) return st;
-    const size_t need = scratch_layout(L, M).total;
+    const size_t need = scratch_layout(L->BN, M).total;
     if (need > (size_t)FQ_STATIC_SCRATCH_BYTES)
         return fail(FQ_ERR_BUFFER_TOO_SMALL,
                     "this call needs %zu bytes of scratch but the built-in scratch holds %zu (M <= %u always fits); "

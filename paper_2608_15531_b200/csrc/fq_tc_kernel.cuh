@@ -1,298 +1,204 @@
-// The fused operator on the fifth-generation tensor cores (tcgen05.mma kind::i8, operands in tensor memory).
-// Included by fq_kernels.cu inside namespace fq, after the PTX helpers.
+// The fused operator on the fifth-generation tensor cores (tcgen05.mma kind::f16, FP32 accumulation), for launches of
+// more rows than a warp-level MMA is made for.  Included by fq_kernels.cu inside namespace fq, after the PTX helpers.
 //
-// Arithmetic.  The tensor core multiplies 8-bit integers exactly: the INT4 codes q go in as they are, and the
-// BF16 activations go in as block fixed point.  For every batch row and quantisation group (64 or 128 k) a
-// small kernel (fq_prep_x_kernel) writes x as an integer x_int = round(x * 2^(21-E)) (E = exponent of the
-// group's largest |x|, so |x_int| < 2^22: exact for every element within 2^14 of the largest, rounded to 2^-22
-// of the largest below that), split into three signed 8-bit limbs x_int = l0 + 2^8 l1 + 2^16 l2, together with
-// 2^(E-21), sum_k x_int and a k-major FP32 copy of x for the outlier step.  Then
-//     sum_k x (q - z)  =  2^(E-21) * ( sum_j 2^(8j) sum_k q l_j  -  z sum_k x_int )            (Eq. 3 inside Eq. 1)
-// with the inner sums exact INT32 results of the MMA, and the scale s applied once per group in FP32.
+// Arithmetic.  The A operand is the exact integers q - z as BF16 (weights on the M side, thread = output column), the
+// B operand the BF16 activations as they are (batch rows on the N side).  Once per quantisation group the FP32 sums
+// leave tensor memory and the scale is applied in FP32:
+//     acc[m] += s * sum_k x (q - z)                                     (Eq. 3 inside Eq. 1)
+// The outliers need no scale.  They are written, as they are, into a dense BF16 tile in shared memory that is zero
+// elsewhere (Section 4.2's scatter, with the weights instead of the products as what is scattered), and a second MMA
+// with the same activations adds X W_O into an accumulator of its own that stays in tensor memory over all of K.  A
+// tile of zeros costs MMA time whatever the density, but none of the gathers, multiply-adds and registers of a step that
+// adds each outlier for every batch row: with 32 rows and more, the tensor pipe does it in less time than the shared
+// memory could deliver the activations to such a step.  An FP16 outlier (ten fraction bits) goes in two parts, each a
+// BF16 number, one tile after the other.
 //
-// A unit is one (column tile, 128-row k-step): 128 x BN INT4 codes with their scales, zero-points and
-// Tile-COO slice.  One persistent CTA per SM walks a range of units through a ring of shared-memory
-// stages (bulk copies + mbarrier expect_tx, Section 4.1).  Thread = output column throughout: tensor
-// memory lane c of a 128-column half holds row c of the A operand (the column's 128 codes) and row c of
-// the accumulator D (the column's batch rows, one column of D per limb and row).
+// A unit is one k-step of 128 rows by 128 columns (a stored tile of 256 columns is two column tiles here).  One
+// persistent CTA per SM walks a range of units through a ring of shared-memory stages (bulk copies + mbarrier
+// expect_tx, Section 4.1).
 //
-//   warps 0, 2      producers (cp.async.bulk): warp 0 copies a unit's codes, scales and zero-points, warp 2
-//                   its bucket descriptors, its outlier packets and the k-step's activation block, which the
-//                   preparation kernel wrote in the stage's own layout (limbs as the K-major MMA operand of
-//                   8-row x 16-byte core matrices, then scales and sums, then the FP32 copy).  Issuing a bulk
-//                   copy occupies its warp for about 120 ns, whichever lane issues it: one warp with all six
-//                   to eight copies of a unit bounded the kernel
-//   warp 1          tensor: per unit 4 x BN/128 tcgen05.mma (M = 128 columns, N = NMMA limb rows, K = 32;
-//                   A from tensor memory, B from shared memory, D = INT32 in tensor memory), tcgen05.commit
-//                   to mbarriers.  An MMA occupies the tensor pipe for 55-66 cycles whatever N <= 128 and
-//                   the operand type are, which is why the 8-bit type (K = 32 per instruction instead of
-//                   16) matters: with BF16 operands the tensor pipe, not HBM, bounds the kernel
-//   unpack warps    BN/32: per 32 rows one 128-bit load of 32 codes, two masks and a shift per 8 codes,
-//                   tcgen05.st into the A operand
-//   epilogue warps  BN/32: tcgen05.ld of the limb sums, the FP32 combination above, then the unit's outliers
-//                   of the thread's own column straight into the same registers (Section 4.2 without the
-//                   shared-memory scatter: no atomics, no read-modify-write), and at the end of a piece the
-//                   split-tile settlement and the BF16 store of Y
+//   warps 0, 2      producers: warp 0 copies a unit's codes, scales and zero-points, warp 2 its X block (tiled tensor
+//                   copies, 128-byte swizzle: the K-major MMA operand), bucket descriptors and packets
+//   warps 1, 3      tensor: per unit 8 MMAs of K = 16 with A from tensor memory (warp 1, dense) and 8 with A from shared
+//                   memory (warp 3, outliers).  Two warps, because a warp's wait on a barrier costs it about 100 clocks
+//                   even when the barrier is ready, and the MMAs of the other fill them
+//   8 unpack warps  per 32 rows one 128-bit load of a column's 32 codes, seven logic operations and four BF16 pair
+//                   subtractions per eight codes, tcgen05.st into a ring of A operands
+//   drain warps     thread = column, 32 batch rows (4 warps for each 32 rows): tcgen05.ld of the group's sums, one FMA per
+//                   batch row; at the end of a piece the outlier accumulator, the split-tile settlement and the BF16
+//                   store of Y
+//   4-8 scatter w.  thread = column: take the previous outliers out of the tile and put the unit's in
 //
-// Lane l of an epilogue warp owns column 32 * strip + l = 8 t + g with g = l % 8, t = l / 8: bucket g of
-// the strip, column number t of that bucket, so it takes slot t of every column-slotted packet of the
-// bucket.  The k-major FP32 copy xt[k][RR] is stored with its 16-byte chunks XOR-swizzled by k
-// (Section 3.2.2's concern, shared-memory bank conflicts of the sparse step, met on the activation side:
-// the rows a warp's lanes pick are random, and the swizzle spreads them over all eight 16-byte bank groups).
+// What bounds it, per unit in SM clocks (MMAs issued back to back from one warp, two commits each): 8 dense + 8
+// outlier MMAs take 430 clocks at N = 16, 490 at 32, 650 at 64, 1030 at 128 (an outlier MMA is bound by reading its 4 KB
+// of A from shared memory up to N = 64); HBM at the measured copy rate would need 425.  The kernel takes 1450 at 32 rows and
+// 2320 at 128 on an 8192 x 28672 layer (78 and 125 us): the chain copy - unpack - MMA - drain of a stage through its
+// barriers times the stages that fit, and the scatter (its walk costs 10 to 20 % of the time: 124 us at 3 % of outliers).
+// It replaces a kernel on the 8-bit integer tensor path whose activations took three limbs and which applied the
+// outliers row by row: 65.6 us on 8192 x 10240 at 32 rows against 30.
 
-constexpr int kLimbs = 3;
-
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
-                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}" : "=r"(e));
+    return e != 0;
 }
 
-// N consecutive 32-bit cells of this thread's tensor-memory lane (N = 1, 4, 8, 16 or 32)
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+        "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+// 16 or 32 consecutive 32-bit cells of this thread's tensor-memory lane
 template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[N]) {
-    if constexpr (N == 1) {
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(taddr) : "memory");
-    } else if constexpr (N == 4) {
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-    } else if constexpr (N == 8) {
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(taddr) : "memory");
-    } else if constexpr (N == 16) {
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&r)[N]) {
+    if constexpr (N == 16) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]),
+              "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
             : "r"(taddr) : "memory");
     } else {
         static_assert(N == 32, "unsupported tcgen05.ld width");
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
             "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-              "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-              "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+            : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]),
+              "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]), "=f"(r[16]),
+              "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]), "=f"(r[24]),
+              "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]), "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
             : "r"(taddr) : "memory");
     }
 }
 
-// (float)v for |v| < 2^22 without a conversion instruction (those issue at a quarter of the ALU rate, and an
-// epilogue thread needs three per batch row and group): v + 1.5 * 2^23 as an integer bit pattern is the float
-// 1.5 * 2^23 + v exactly.
-__device__ __forceinline__ float small_int_to_float(uint32_t v) { return __uint_as_float(v + 0x4B400000u) - 12582912.0f; }
-
-// XOR applied to the 16-byte chunk index of row k of the k-major FP32 copy (RR floats per row): with C
-// chunks per row, 8 / C consecutive rows share a 128-byte line, and the swizzle makes the chunk a lane
-// reads in one load instruction depend on k, so that lanes with random k cover all eight bank groups.
-template <int RR>
-__device__ __forceinline__ uint32_t xt_swizzle(uint32_t k) {
-    constexpr uint32_t C = RR / 4;
-    if constexpr (C <= 1) return 0u;
-    else return ((k * C) >> 3) & (C - 1);
+// D[128 x N] (+)= A[128 x 16] * B[16 x N], BF16 in, FP32 out; A in tensor memory or behind a shared-memory descriptor.
+// Issued by one thread.  Descriptors come as their two words, of which only the lower (the address) changes.
+__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 y;\n setp.ne.b32 p, %5, 0;\n mov.b64 y, {%2, %3};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], y, %4, p;\n}"
+                 ::"r"(d), "r"(a), "r"(b), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_ss(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 x, y;\n setp.ne.b32 p, %6, 0;\n mov.b64 x, {%1, %2};\n mov.b64 y, {%3, %4};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, p;\n}"
+                 ::"r"(d), "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// K-major operands.  No swizzle (the outlier tile): core matrices of 8 rows x 16 bytes, `lbo` bytes from one 16-byte
+// column of K to the next, 128 bytes from one group of eight rows to the next.
+__device__ __forceinline__ uint64_t desc_plain(uint32_t saddr, uint32_t lbo) {
+    return (uint64_t)((saddr & 0x3ffffu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+// 128-byte swizzle (the activations): rows of 64 K values, 1024 bytes from one group of eight rows to the next.
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t x, uint32_t y, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
 }
 
-// acc[0..RR) += v * x[0..RR)[k] for NP outliers of the thread's column, each a slot word (BF16 value in the
-// upper half, row k of the unit in bits 5-11; a padding slot has value 0 and adds 0).  The activation rows
-// of all NP are requested before the first multiply-add, so that their shared-memory latencies overlap.
-template <int RR, int NP>
-__device__ __forceinline__ void add_outliers(float (&acc)[RR], const uint32_t (&wd)[NP], const char* xtb) {
-    if constexpr (RR == 1) {
-        float x[NP];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) x[j] = *reinterpret_cast<const float*>(xtb + ((wd[j] >> 3) & 0x1fcu));
-#pragma unroll
-        for (int j = 0; j < NP; ++j) acc[0] = fmaf(__uint_as_float(wd[j] & kSlotValueMask), x[j], acc[0]);
-    } else {
-        float4 x[NP][RR / 4];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const uint32_t k = (wd[j] >> 5) & 127u;
-            const char* row = xtb + k * (4 * RR);
-            const uint32_t sw = xt_swizzle<RR>(k) << 4;
-#pragma unroll
-            for (int c = 0; c < RR / 4; ++c) x[j][c] = *reinterpret_cast<const float4*>(row + (((uint32_t)c << 4) ^ sw));
-        }
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-            const float v = __uint_as_float(wd[j] & kSlotValueMask);
-#pragma unroll
-            for (int c = 0; c < RR / 4; ++c) {
-                acc[4 * c + 0] = fmaf(v, x[j][c].x, acc[4 * c + 0]);
-                acc[4 * c + 1] = fmaf(v, x[j][c].y, acc[4 * c + 1]);
-                acc[4 * c + 2] = fmaf(v, x[j][c].z, acc[4 * c + 2]);
-                acc[4 * c + 3] = fmaf(v, x[j][c].w, acc[4 * c + 3]);
-            }
-        }
-    }
+// Bounded wait of a whole warp: every lane polls (the instructions after it want the warp converged), and the lanes give
+// up together.
+__device__ __forceinline__ bool wait_converged(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
+    const bool ok = mbar_wait(bar, parity, abort_flag, status);
+    return __all_sync(0xffffffffu, ok);
 }
 
-// D[128 x N] (+)= A[128 x 32] (tensor memory) * B[32 x N] (shared-memory descriptor), signed 8-bit in, INT32 out.
-// Called by the whole (converged) warp with warp-uniform operands; one elected lane issues.
-__device__ __forceinline__ void umma_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-        " @e tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
+struct TcParams {
+    const uint8_t* wq;
+    const uint16_t* scale;
+    const uint16_t* zero;
+    const uint32_t* indptr;
+    const uint32_t* info;
+    const uint4* packed;
+    uint16_t* Y;
+    uint32_t* status;
+    uint32_t* counters;
+    float* partials;
+    uint32_t M, K, N, KT, NT;       // NT: column tiles of 128 H columns
+    uint32_t halves;                // such tiles to a stored tile of BN columns (1, or 2: BN = 256 and H = 1)
+    uint32_t coo_cap, general, stages;
+    uint32_t split;                 // as in the streaming kernel
+    uint32_t nmma;                  // batch rows of the MMAs: M rounded up to 16
+    uint32_t parts;                 // BF16 parts of an outlier: 1, or 2 (FP16 values)
+    // shared-memory offsets (bytes); the first four are relative to a stage, whose X block is at 0
+    uint32_t off_w, off_sz, off_info, off_coo, stage_bytes, off_wo, off_bar;
+};
 
-// Rows of the activation arrays kept per unit for RR batch rows (at least four, so that every copy is a
-// multiple of 16 bytes).
-__host__ __device__ constexpr int meta_rows(int rr) { return rr < 4 ? 4 : rr; }
+constexpr int kWoTile = 128 * 128 * 2;      // bytes of the outlier tile of a half-step
+// outlier tiles in flight: four where a stage is small enough to leave the room
+__host__ __device__ constexpr int tc_outlier_tiles(int nr) { return nr <= 32 ? 4 : 2; }
+constexpr int kScatterKeep = 8;             // outliers of a column and half-step that are taken out one by one
 
-// ----------------------------------------------------------------------------- activation preparation
+// The variant's tensor-memory columns (NAB A operands of 64 columns, NDB sets of dense accumulators, one per group, and
+// the outlier accumulators), outlier tiles (NWO) and warps: a drain warp keeps 32 batch rows of its 32
+// columns in registers; SG groups of four scatter warps take the units in turn.
+template <int NR, int GROUP>
+struct TcShape {
+    static constexpr int GPS = kBK / GROUP, SETS = NR / 32;
+    static constexpr int NDB = 2 * 64 + 2 * GPS * NR + NR <= 512 ? 2 : 1;
+    static constexpr int NAB = 4 * 64 + NDB * GPS * NR + NR <= 512 ? 4 : 2;
+    static constexpr int D_BASE = NAB * 64, O_BASE = D_BASE + NDB * GPS * NR;
+    static_assert(O_BASE + NR <= 512, "tensor memory");
+    static constexpr int SG = 12 + 4 * SETS + 8 <= 32 ? 2 : 1;
+    static constexpr int NWO = tc_outlier_tiles(NR);
+    static constexpr int WARPS = 12 + 4 * SETS + 4 * SG;
+    static_assert(WARPS <= 32 && NWO % SG == 0, "warps");
+};
 
-// Bytes of the activation block of one k-step for RR batch rows: the limb operand (NMMA rows x 128 k, one byte
-// each), scales and sums (padded to 128 bytes), the FP32 copy.
-__host__ __device__ constexpr int nmma_rows(int rr) { return (kLimbs * rr + 15) / 16 * 16; }
-__host__ __device__ constexpr int blob_meta_off(int rr) { return nmma_rows(rr) * 128; }
-__host__ __device__ constexpr int blob_xt_off(int rr, int gps) { return blob_meta_off(rr) + (gps * 2 * meta_rows(rr) * 4 + 127) / 128 * 128; }
-__host__ __device__ constexpr int blob_bytes(int rr, int gps) { return blob_xt_off(rr, gps) + kBK * rr * 4; }
+template <int NR, int GROUP>
+__global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
+fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
+    using S_ = TcShape<NR, GROUP>;
+    constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, SG = S_::SG;
+    constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256, INFO_BYTES = 128;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
 
-// One warp per (batch row m < RR, k-step kt): the row's 128 activations of the k-step -> limbs, scale,
-// integer sum and FP32 copy, per quantisation group (GROUP = 64: lanes 0-15 and 16-31; 128: the warp), into
-// the k-step's block xb + kt * blob_bytes, laid out as a stage of the fused kernel holds it:
-//   limbs  [16-k block c = 0..7][row n = j * RR + m][16 bytes]: limb j of batch row m, the K-major MMA operand
-//          (8-row x 16-byte core matrices); rows n >= 3 RR are zero
-//   meta   [128 / GROUP][2][meta_rows(RR)] floats: 2^(E-21), then sum_k x_int (as a float)
-//   xt     [128][RR] floats, 16-byte chunks XOR-swizzled by k (xt_swizzle)
-// Rows m >= M are written as zeros.  A group with a non-finite activation gets the scale NaN.
-template <int RR, int GROUP>
-__global__ void __launch_bounds__(128) fq_prep_x_kernel(const uint16_t* __restrict__ X, uint32_t M, uint32_t K, uint8_t* __restrict__ xb) {
-    constexpr int GPS = kBK / GROUP, RM = meta_rows(RR), NMMA = nmma_rows(RR);
-    // the grid after this one (the fused kernel) may start streaming weights; this one reads X and writes
-    // scratch that the grid before it may still be using
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint32_t lane = threadIdx.x & 31, wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t KT = K / kBK;
-    if (wg >= RR * KT) return;
-    const uint32_t m = wg / KT, kt = wg - m * KT, k0 = kt * kBK + 4 * lane;
-    uint8_t* blob = xb + (size_t)kt * blob_bytes(RR, GPS);
-    uint2 raw = make_uint2(0, 0);
-    if (m < M) raw = __ldg(reinterpret_cast<const uint2*>(X + (size_t)m * K + k0));
-    const uint32_t bits[4] = {raw.x & 0xffffu, raw.x >> 16, raw.y & 0xffffu, raw.y >> 16};
-    float x[4];
-    uint32_t amax = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { x[i] = __uint_as_float(bits[i] << 16); amax = max(amax, bits[i] & 0x7fffu); }
-#pragma unroll
-    for (int d = 1; d < 32 / GPS; d <<= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-    const uint32_t ef_raw = amax >> 7;                        // biased exponent of the group's largest |x|
-    const uint32_t ef = max(ef_raw, 22u);                     // keeps 2^(E-21) a normal number; tinier groups lose nothing that matters
-    const float up = __uint_as_float((275u - ef) << 23);      // 2^(21-E)
-    int xi[4], sum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { xi[i] = __float2int_rn(x[i] * up); sum += xi[i]; }
-#pragma unroll
-    for (int d = 1; d < 32 / GPS; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-    // signed limbs: x_int = l0 + 256 l1 + 65536 l2
-    uint32_t w[kLimbs] = {0, 0, 0};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int l0 = (xi[i] << 24) >> 24;
-        const int r1 = (xi[i] - l0) >> 8;
-        const int l1 = (r1 << 24) >> 24;
-        const int l2 = (r1 - l1) >> 8;
-        w[0] |= (uint32_t)(l0 & 0xff) << (8 * i);
-        w[1] |= (uint32_t)(l1 & 0xff) << (8 * i);
-        w[2] |= (uint32_t)(l2 & 0xff) << (8 * i);
-    }
-    // Byte position of k inside its 16-k block: the unpack's two masks put row r of an 8-row word at position
-    // 2 (r % 4) + r / 4 of the word's eight (rows 0, 4, 1, 5, 2, 6, 3, 7), and the MMA pairs operand bytes by
-    // position.  This lane's four k are rows 4 (lane % 2) .. of 8-row word lane / 2.
-    uint8_t* lrow = blob + (lane >> 2) * (NMMA * 16) + ((lane >> 1) & 1) * 8 + (lane & 1);
-#pragma unroll
-    for (int j = 0; j < kLimbs; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) lrow[(j * RR + m) * 16 + 2 * i] = (uint8_t)(w[j] >> (8 * i));
-    if (m == 0) {
-#pragma unroll
-        for (int n = kLimbs * RR; n < NMMA; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) lrow[n * 16 + 2 * i] = 0;          // padding rows of the operand
-    }
-    if ((lane & (32 / GPS - 1)) == 0) {
-        const uint32_t gi = lane / (32 / GPS);
-        float* mt = reinterpret_cast<float*>(blob + blob_meta_off(RR)) + gi * 2 * RM;
-        mt[m] = ef_raw == 0xffu ? __uint_as_float(0x7fc00000u) : __uint_as_float((ef - 21u) << 23);     // 2^(E-21)
-        mt[RM + m] = (float)sum;
-    }
-    uint8_t* xtu = blob + blob_xt_off(RR, GPS);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t k = 4 * lane + i;
-        *reinterpret_cast<float*>(xtu + k * (4 * RR) + ((((m >> 2) ^ xt_swizzle<RR>(k)) << 4) | ((m & 3) << 2))) = x[i];
-    }
-}
-
-// ----------------------------------------------------------------------------- the fused kernel
-
-// Sets of epilogue warps; with two, the sets take alternate units (set e the units in D buffer e) and set 1
-// hands its sums to set 0 through shared memory at the end of a piece.  An epilogue thread's work on a unit is
-// a chain of latencies (barrier, tensor-memory load, packet, activation row, multiply-add) of 0.6-1.2 us;
-// two warps per strip keep two such chains in flight.
-__host__ __device__ constexpr int epilogue_sets(int rr) { return rr <= 16 ? 2 : 1; }
-
-constexpr int kTcFirstUnpack = 4;  // a warp reaches the tensor-memory lanes 32 * (warp % 4) ..., so strips start at a multiple of 4
-
-// BN: tile columns (128 or 256).  RR: batch rows kept per epilogue thread (1, 4, 8, 16, 32; M <= RR).  The
-// MMA's N is NMMA = kLimbs * RR rounded up to 16.  HOT: general form of the outlier step (buckets with a tail,
-// tiles with more packets than a stage holds).
-template <int BN, int RR, int GROUP, bool SPARSE, bool HOT>
-__global__ void __launch_bounds__(32 * (kTcFirstUnpack + (1 + epilogue_sets(RR)) * (BN / 32)), 1) fq_tc_kernel(const Params p) {
-    constexpr int NDW = BN / 32;              // unpack warps = epilogue warps = 32-column strips
-    constexpr int NT128 = BN / 128;           // 128-column halves per unit
-    constexpr int UW0 = kTcFirstUnpack, EW0 = UW0 + NDW;
-    constexpr int NEPI = epilogue_sets(RR);
-    constexpr int GPS = kBK / GROUP;          // groups per k-step
-    constexpr int NMMA = nmma_rows(RR);
-    constexpr int RM = meta_rows(RR);
-    constexpr int DCOLS = GPS * NMMA;         // accumulator columns per half and buffer
-    // A buffers (one unit's codes each): four if tensor memory has room beside the two D buffers, so that the
-    // unpack warps run up to three units ahead of the MMAs; else two
-    constexpr int NAB = (4 * NT128 * 32 + 2 * NT128 * DCOLS <= 512) ? 4 : 2;
-    constexpr uint32_t D_BASE = NAB * NT128 * 32;
-    constexpr int W_BYTES = 16 * BN * 4;
-    constexpr int SZ_ROW = BN * 2;
-    // what a stage takes of the k-step's activation block: without outliers, not the FP32 copy at its end
-    constexpr int XB_BYTES = SPARSE ? blob_bytes(RR, GPS) : blob_xt_off(RR, GPS);
-    constexpr uint32_t IDESC = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NMMA >> 3) << 17) | (8u << 24);
-    static_assert(D_BASE + 2 * NT128 * DCOLS <= 512, "tensor memory: the A buffers and two D buffers must fit");
-    static_assert(RR == 1 || RR % 4 == 0, "rows per thread");
-    extern __shared__ __align__(128) uint8_t smem[];
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const uint32_t S = p.stages;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * S;
-    const uint32_t bar_a_full = bar_empty + 8 * S;       // [4] A buffer written (unpack warps)
-    const uint32_t bar_a_empty = bar_a_full + 32;        // [4] the MMAs that read the A buffer are complete
-    const uint32_t bar_d_free = bar_a_empty + 32;        // [2] D buffer read (epilogue warps)
-    const uint32_t bar_d_ready = bar_d_free + 16;        // [2] MMAs of a unit complete: D written
-    const uint32_t bar_final = bar_d_ready + 16;
-    const uint32_t bar_xfull = bar_final + 8, bar_xempty = bar_xfull + 8 * NDW;   // [NDW] each: hand-over of set 1's sums, per strip
-    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 13 + 2 * NDW);
+    const uint32_t bar_a_full = bar_empty + 8 * S;        // [4] A operand written (unpack warps)
+    const uint32_t bar_a_empty = bar_a_full + 32;         // [4] the MMAs that read it are complete
+    const uint32_t bar_d_full = bar_a_empty + 32;         // [2] a half-step's dense MMAs are complete
+    const uint32_t bar_d_free = bar_d_full + 16;          // [2] its sums are read (drain warps)
+    const uint32_t bar_wo_full = bar_d_free + 16;         // [4] outlier tile written (scatter warps)
+    const uint32_t bar_wo_empty = bar_wo_full + 32;       // [4] the MMAs that read it are complete
+    const uint32_t bar_o_full = bar_wo_empty + 32;        // the piece's outlier sums are complete
+    const uint32_t bar_o_free = bar_o_full + 8;           // and read
+    const uint32_t bar_final = bar_o_free + 8;
+    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 23);
     volatile uint32_t* tmem_slot = abort_flag + 1;
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
-            mbar_init(bar_full + 8 * s, 2);                    // the two producers' expect_tx arrivals
-            mbar_init(bar_empty + 8 * s, 2 * NDW + 1);         // unpack warps, epilogue warps, the MMAs' commit
+            mbar_init(bar_full + 8 * s, 2);                                  // the two producers' expect_tx arrivals
+            mbar_init(bar_empty + 8 * s, 4 * (1 + SETS) + 4 + 2);   // unpack, drain, scatter warps, the MMAs' commits
         }
-        for (uint32_t b = 0; b < 2; ++b) {
-            mbar_init(bar_d_free + 8 * b, NDW);                // the epilogue warps of the unit two before
-            mbar_init(bar_d_ready + 8 * b, 1);
+        for (uint32_t i = 0; i < 4; ++i) {
+            mbar_init(bar_a_full + 8 * i, 4);
+            mbar_init(bar_a_empty + 8 * i, 1);
+            mbar_init(bar_wo_full + 8 * i, 4);
+            mbar_init(bar_wo_empty + 8 * i, 1);
         }
-        for (uint32_t a = 0; a < 4; ++a) {
-            mbar_init(bar_a_full + 8 * a, NDW);
-            mbar_init(bar_a_empty + 8 * a, 1);
+        for (uint32_t i = 0; i < 2; ++i) {
+            mbar_init(bar_d_full + 8 * i, 1);
+            mbar_init(bar_d_free + 8 * i, 4 * SETS);
         }
-        mbar_init(bar_final, 1);
-        for (uint32_t i = 0; i < 2 * NDW; ++i) mbar_init(bar_xfull + 8 * i, 1);
+        mbar_init(bar_o_full, 1);
+        mbar_init(bar_o_free, 4 * SETS);
+        mbar_init(bar_final, 2);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -305,12 +211,10 @@ __global__ void __launch_bounds__(32 * (kTcFirstUnpack + (1 + epilogue_sets(RR))
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // The grid after this one in the stream may start now (it takes SMs as this grid's CTAs leave).  The
-    // warps that write Y or touch the scratch wait for the grids before this one, and so does the producer
-    // before its first copy of the activation arrays; the weight arrays are read before: no kernel writes
-    // them while calls are in flight.
+    // The grid after this one in the stream may start now (it takes SMs as this grid's CTAs leave).  The weight arrays
+    // are read at once (no kernel writes them while calls are in flight); whoever reads X or writes Y or the scratch
+    // waits for the grids before this one.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (warp >= EW0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const uint32_t KT = p.KT;
     const uint32_t U = p.NT * KT, P = gridDim.x, q = U / P, r = U % P;
@@ -323,396 +227,434 @@ __global__ void __launch_bounds__(32 * (kTcFirstUnpack + (1 + epilogue_sets(RR))
         u_begin = unit_begin_of(blockIdx.x, q, r);
         u_end = u_begin + q + (blockIdx.x < r ? 1u : 0u);
     }
+    // stored tile of a unit (Tile-COO and codes) and the unit's half of it
+    auto chunk_of = [&](uint32_t tn, uint32_t kt) { return (p.halves == 2 ? tn >> 1 : tn) * KT + kt; };
 
-    if (warp == 0) {
-        // ------------------------------------------------------------------ producer of the dense arrays
-        // codes, scales and zero-points of every unit: weights, which no kernel writes while calls are in
-        // flight, so this warp never waits for the grids before this one
-        uint32_t issued = 0;
-        bool ok = true;
-        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-            const uint32_t s = w.s, full = bar_full + 8 * s;
-            if (!warp_wait(bar_empty + 8 * s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-            const uint32_t st = smem_u32(smem) + s * p.stage_bytes;
-            if (lane == 0) {
-                mbar_arrive_expect_tx(full, W_BYTES + 2 * GPS * SZ_ROW);
-                bulk_g2s(st, p.wq + (size_t)w.u * W_BYTES, W_BYTES, full);
+    if (warp < 4) {
+        if (warp == 0) {
+            // ---------------------------------------------------------------- producer of the dense arrays
+            uint32_t issued = 0;
+            bool ok = true;
+            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+                const uint32_t full = bar_full + 8 * w.s;
+                if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+                const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, W_BYTES + 2 * GPS * SZ_ROW);
+                    if (p.halves == 2) {
+                        const uint8_t* src = p.wq + (size_t)chunk_of(w.tn, w.kt) * 16384 + (w.tn & 1) * 2048;
 #pragma unroll
-                for (int gi = 0; gi < GPS; ++gi) {
-                    const size_t row = (size_t)(w.kt * GPS + gi) * p.N + (size_t)w.tn * BN;
-                    bulk_g2s(st + p.off_sz + gi * SZ_ROW, p.scale + row, SZ_ROW, full);
-                    bulk_g2s(st + p.off_sz + (GPS + gi) * SZ_ROW, p.zero + row, SZ_ROW, full);
+                        for (int j = 0; j < 4; ++j) bulk_g2s(st + p.off_w + j * 2048, src + j * 4096, 2048, full);
+                    } else {
+                        bulk_g2s(st + p.off_w, p.wq + (size_t)w.u * W_BYTES, W_BYTES, full);
+                    }
+#pragma unroll
+                    for (int gi = 0; gi < GPS; ++gi) {
+                        const size_t row = (size_t)(w.kt * GPS + gi) * p.N + (size_t)w.tn * 128;
+                        bulk_g2s(st + p.off_sz + gi * SZ_ROW, p.scale + row, SZ_ROW, full);
+                        bulk_g2s(st + p.off_sz + (GPS + gi) * SZ_ROW, p.zero + row, SZ_ROW, full);
+                    }
                 }
+                __syncwarp();
+                issued = w.it + 1;
             }
-            issued = w.it + 1;
-        }
-        if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
-            for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
-                for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
-        }
-    } else if (warp == 2) {
-        // ------------------------------------------------------------------ producer of the outlier arrays and the activations
-        uint32_t ip_a = 0, ip_b = 0;                                   // packet ranges of the next 32 units, read 32 at a time
-        uint32_t last_bar = 0, last_ph = 0;
-        bool ok = true;
-        auto outliers = [&](const UnitIter& w, uint32_t extra) {       // arrival with the byte count of this warp's copies
-            const uint32_t s = w.s, full = bar_full + 8 * s;
-            const uint32_t st = smem_u32(smem) + s * p.stage_bytes;
-            if (SPARSE && (w.it & 31) == 0) {
-                const uint32_t i = w.u + lane;
-                ip_a = (i <= U) ? __ldg(p.indptr + i) : 0;
-                ip_b = (i + 1 <= U) ? __ldg(p.indptr + i + 1) : 0;
+            if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
+                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
+                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
             }
-            uint32_t pk0 = 0, npk = 0;
-            if (SPARSE) {
+        } else if (warp == 2) {
+            // ---------------------------------------------------------------- producer of X and the outlier arrays
+            uint32_t ip_a = 0, ip_b = 0;                                   // packet ranges of the next 32 units, read 32 at a time
+            uint32_t last_bar = 0, last_ph = 0;
+            bool ok = true;
+            const uint32_t x_half = p.nmma * 128;                          // bytes of 64 K values of every batch row
+            auto outliers = [&](const UnitIter& w) {                       // arrival with the byte count of this warp's copies
+                const uint32_t full = bar_full + 8 * w.s, st = smem_u32(smem) + w.s * p.stage_bytes;
+                uint32_t pk0 = 0, npk = 0, chunk = 0;
+                if ((w.it & 31) == 0) {
+                    const uint32_t i = w.u + lane;
+                    if (i < U) {
+                        const uint32_t c = chunk_of(i / KT, i % KT);
+                        ip_a = __ldg(p.indptr + c), ip_b = __ldg(p.indptr + c + 1);
+                    }
+                }
+                chunk = chunk_of(w.tn, w.kt);
                 pk0 = __shfl_sync(0xffffffffu, ip_a, w.it & 31);
                 npk = min(__shfl_sync(0xffffffffu, ip_b, w.it & 31) - pk0, p.coo_cap);
-            }
-            if (lane == 0) {
-                mbar_arrive_expect_tx(full, extra + (SPARSE ? p.NB * 4 + npk * 16 : 0));
-                if (SPARSE) {
-                    bulk_g2s(st + p.off_info, p.info + (size_t)w.u * p.NB, p.NB * 4, full);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, 2 * x_half + INFO_BYTES + npk * 16);
+                    const uint32_t half = p.halves == 2 ? (w.tn & 1) : 0;
+                    bulk_g2s(st + p.off_info, p.info + ((size_t)chunk * p.halves + half) * 32, INFO_BYTES, full);
                     if (npk) bulk_g2s(st + p.off_coo, p.packed + pk0, npk * 16, full);
                 }
-            }
-            last_bar = full, last_ph = w.ph;
-        };
-        auto activations = [&](const UnitIter& w) {                    // the k-step's block, as the preparation kernel laid it out
-            if (lane == 0)
-                bulk_g2s(smem_u32(smem) + w.s * p.stage_bytes + p.off_xcan, p.xblob + (size_t)w.kt * blob_bytes(RR, GPS), XB_BYTES, bar_full + 8 * w.s);
-        };
-        // the first pass over the ring finds every stage empty: its outlier arrays (weights) are requested
-        // before the wait for the grids before this one, its activation blocks after
-        const uint32_t n_first = min(S, u_end - u_begin);
-        {
-            UnitIter w(u_begin, KT);
-            for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) outliers(w, XB_BYTES);
-        }
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        {
-            UnitIter w(u_begin, KT);
-            for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) activations(w);
-            for (; w.u < u_end; w.next(S, KT)) {
-                if (!warp_wait(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-                outliers(w, XB_BYTES);
-                activations(w);
-            }
-        }
-        if (!ok && last_bar)                // gave up: let this warp's last copies land before the CTA exits
-            for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(last_bar, last_ph); ++spin) {}
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ tensor warp
-        // One warp issues every MMA of the CTA (issued from two warps in turn, MMAs run several times slower).
-        // The first MMA of a CTA takes microseconds to start (the tensor pipe wakes up): issue a throw-away
-        // one now, while the first loads are in flight.  It reads whatever A buffer 0 and stage 0 hold and
-        // writes D buffer 1, which the first real MMA into that buffer overwrites.
-        umma_i8_ts(tmem_base + D_BASE + NT128 * DCOLS, tmem_base, make_b_desc(smem_u32(smem) + p.off_xcan, NMMA * 16, 128), IDESC, 0);
-        // The tensor pipe should never wait for this warp: the completion signals of a unit go out after the
-        // first MMA of the next one has been issued (they then fire one MMA, about 30 ns, later), and the next
-        // unit's barriers are tested while the last MMAs of this one run.
-        uint32_t ready = 0, pending = 0, pv_b = 0, pv_a = 0, pv_s = 0;
-        auto signal = [&]() {                                  // completion of the unit before: D written, A and stage read
-            if (pending) {
-                umma_commit(bar_d_ready + 8 * pv_b);
-                umma_commit(bar_a_empty + 8 * pv_a);
-                umma_commit(bar_empty + 8 * pv_s);
-                pending = 0;
-            }
-        };
-        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-            const uint32_t it = w.it, s = w.s, b = w.it & 1;    // D buffer b, A buffer it % NAB
-            if (!ready) {
-                // the stage's activation operand, the unit's A buffer, and the D buffer's last reader
-                signal();
-                if (!warp_wait(bar_full + 8 * s, w.ph, abort_flag, p.status)) break;
-                if (!warp_wait(bar_a_full + 8 * (it % NAB), (it / NAB) & 1, abort_flag, p.status)) break;
-                if (it >= 2 && !warp_wait(bar_d_free + 8 * b, ((it - 2) >> 1) & 1, abort_flag, p.status)) break;
-            }
-            tc_fence_after();
-            UnitIter nx = w;
-            nx.next(S, KT);
-            uint32_t seen = 0;
-            const uint64_t bd0 = make_b_desc(smem_u32(smem) + s * p.stage_bytes + p.off_xcan, NMMA * 16, 128);
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {             // 32 k per MMA: 16-k blocks 2 ks, 2 ks + 1 of the operand
-                const int gi = ks / (4 / GPS);
-#pragma unroll
-                for (int h = 0; h < NT128; ++h) {
-                    const uint32_t d = tmem_base + D_BASE + (b * NT128 + h) * DCOLS + gi * NMMA;
-                    const uint32_t a = tmem_base + ((it % NAB) * NT128 + h) * 32 + ks * 8;
-                    umma_i8_ts(d, a, bd0 + (uint64_t)((ks * 2 * NMMA * 16) >> 4), IDESC, (ks % (4 / GPS)) != 0);
-                    if (ks == 0 && h == 0) signal();
+                __syncwarp();
+                last_bar = full, last_ph = w.ph;
+            };
+            auto activations = [&](const UnitIter& w) {
+                if (elect_one()) {
+                    const uint32_t full = bar_full + 8 * w.s, st = smem_u32(smem) + w.s * p.stage_bytes;
+                    tma_load_2d(st, &xmap, w.kt * kBK, 0, full);
+                    tma_load_2d(st + x_half, &xmap, w.kt * kBK + 64, 0, full);
                 }
-                if (ks == 2 && nx.u < u_end && lane == 0)   // one lane, three tests whose latencies overlap
-                    seen = mbar_test_wait(bar_full + 8 * nx.s, nx.ph) & mbar_test_wait(bar_a_full + 8 * (nx.it % NAB), (nx.it / NAB) & 1) &
-                           (nx.it < 2 ? 1u : mbar_test_wait(bar_d_free + 8 * (nx.it & 1), ((nx.it - 2) >> 1) & 1));
+                __syncwarp();
+            };
+            // the first pass over the ring finds every stage empty: its outlier arrays (weights) are requested before
+            // the wait for the grids before this one, its activations after
+            const uint32_t n_first = min(S, u_end - u_begin);
+            {
+                UnitIter w(u_begin, KT);
+                for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) outliers(w);
             }
-            pending = 1, pv_b = b, pv_a = it % NAB, pv_s = s;
-            ready = __shfl_sync(0xffffffffu, seen, 0);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            {
+                UnitIter w(u_begin, KT);
+                for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) activations(w);
+                for (; w.u < u_end; w.next(S, KT)) {
+                    if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+                    outliers(w);
+                    activations(w);
+                }
+            }
+            if (!ok && last_bar)                // gave up: let this warp's last copies land before the CTA exits
+                for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(last_bar, last_ph); ++spin) {}
+        } else if (warp == 1) {
+            // ---------------------------------------------------------------- dense tensor warp
+            // (the unpack warps have waited for the unit's stage, its X block included)
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
+            const uint32_t x_half = (p.nmma * 128) >> 4;
+            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+                const uint32_t ab = w.it % NAB, db = w.it % NDB;
+                const uint64_t xd = desc_sw128(smem_u32(smem) + w.s * p.stage_bytes);
+                if (w.it >= NDB && !wait_converged(bar_d_free + 8 * db, (w.it / NDB - 1) & 1, abort_flag, p.status)) break;
+                if (!wait_converged(bar_a_full + 8 * ab, (w.it / NAB) & 1, abort_flag, p.status)) break;
+                tc_fence_after();
+                if (elect_one()) {
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_ts(tmem_base + S_::D_BASE + (db * GPS + ks * GPS / 8) * NR, tmem_base + ab * 64 + ks * 8,
+                                (uint32_t)xd + (ks >> 2) * x_half + (ks & 3) * 2, (uint32_t)(xd >> 32), idesc, (ks % (8 / GPS)) != 0);
+                    umma_commit(bar_d_full + 8 * db);
+                    umma_commit(bar_a_empty + 8 * ab);
+                    umma_commit(bar_empty + 8 * w.s);
+                }
+                __syncwarp();
+            }
+            if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
+            __syncwarp();
+        } else {
+            // ---------------------------------------------------------------- outlier tensor warp
+            // (the scatter warps have waited for the unit's stage)
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
+            const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048);
+            const uint32_t x_half = (p.nmma * 128) >> 4;
+            bool ok = true;
+            uint32_t piece = 0;
+            for (UnitIter w(u_begin, KT); w.u < u_end && ok; w.next(S, KT)) {
+                const bool first = w.it == 0 || w.kt == 0, last = w.u + 1 == u_end || w.kt + 1 == KT;
+                const uint32_t wb = w.it % NWO;
+                const uint64_t xd = desc_sw128(smem_u32(smem) + w.s * p.stage_bytes);
+                const uint32_t wo = (uint32_t)wo0 + wb * (kWoTile >> 4);
+                if (first && piece > 0 && !wait_converged(bar_o_free, (piece - 1) & 1, abort_flag, p.status)) break;
+                for (uint32_t part = 0; part < p.parts; ++part) {
+                    if (!wait_converged(bar_wo_full + 8 * wb, ((w.it / NWO) * p.parts + part) & 1, abort_flag, p.status)) { ok = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            umma_ss(tmem_base + S_::O_BASE, wo + ks * (4096 >> 4), (uint32_t)(wo0 >> 32), (uint32_t)xd + (ks >> 2) * x_half + (ks & 3) * 2,
+                                    (uint32_t)(xd >> 32), idesc, (ks > 0 || part > 0 || !first) ? 1u : 0u);
+                        umma_commit(bar_wo_empty + 8 * wb);
+                        if (part + 1 == p.parts) {
+                            if (last) umma_commit(bar_o_full);
+                            umma_commit(bar_empty + 8 * w.s);
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (last) ++piece;
+            }
+            if (elect_one()) umma_commit(bar_final);
+            __syncwarp();
         }
-        signal();
-        __syncwarp();
-        umma_commit(bar_final);                 // fires when every MMA this warp issued has retired
-    } else if (warp < UW0) {
-        // idle: keeps the strips' warps at a multiple of four
-    } else if (warp < EW0) {
-        // ------------------------------------------------------------------ unpack warps: thread = column
-        const int dw = warp - UW0;
-        const int col = dw * 32 + lane;
-        const uint32_t t_lane = ((uint32_t)((dw & 3) * 32)) << 16;
-        const uint32_t t_a = tmem_base + t_lane + (uint32_t)(dw >> 2) * 32;
+    } else if (warp < 12) {
+        // -------------------------------------------------------------------- unpack warps: thread = column
+        const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % 2 == ug
+        const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t col = (warp & 3) * 32 + lane;
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-            const uint32_t it = w.it, s = w.s, b = w.it & 1;
-            const uint8_t* st = smem + s * p.stage_bytes;
-            if (!warp_wait(bar_full + 8 * s, w.ph, abort_flag, p.status)) break;
-            // the column's 128 codes: four 16-byte loads (32 rows each), lanes contiguous
-            const uint4* wp = reinterpret_cast<const uint4*>(st) + col;
+            const uint32_t ab = w.it % NAB;
+            const uint8_t* st = smem + w.s * p.stage_bytes;
+            if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
+            // The groups take alternate units.  A group waits for the others' units too: a parity wait is only
+            // valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not advance
+            // past a unit that this group has yet to release.)
+            if ((w.it & 1) != ug) continue;
+            const uint4* wp = reinterpret_cast<const uint4*>(st + p.off_w) + col;
             uint4 w4[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w4[j] = wp[j * BN];
-            // this A buffer was last read by the MMAs of unit it - NAB
-            if (it >= NAB && !warp_wait(bar_a_empty + 8 * (it % NAB), ((it - NAB) / NAB) & 1, abort_flag, p.status)) break;
+            for (int j = 0; j < 4; ++j) w4[j] = wp[j * 128];
+            uint32_t nz[GPS];                                              // -(128 + z) twice
+#pragma unroll
+            for (int gi = 0; gi < GPS; ++gi) {
+                const uint32_t z = reinterpret_cast<const uint16_t*>(st + p.off_sz + (GPS + gi) * SZ_ROW)[col];
+                nz[gi] = 0x80008000u ^ add_bf16x2(z | (z << 16), 0x43004300u);
+            }
+            if (w.it >= NAB && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const uint32_t ww[4] = {w4[j].x, w4[j].y, w4[j].z, w4[j].w};
-                uint32_t a[8];
+                uint32_t a[16];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    // nibble i + 4h of a word is row 2i + h of its eight: the even nibbles are rows 0, 4, 1, 5 and the
-                    // odd ones rows 2, 6, 3, 7, two cells of four bytes; the limb operand is stored in the same k order
-                    a[2 * x + 0] = ww[x] & 0x0f0f0f0fu;
-                    a[2 * x + 1] = (ww[x] >> 4) & 0x0f0f0f0fu;
-                }
-                tmem_st8(t_a + (it % NAB) * (NT128 * 32) + j * 8, a);
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) a[4 * x + i] = add_bf16x2(codes_to_bf16x2(ww[x] >> (4 * i)), nz[j * GPS / 4]);
+                tmem_st16(t_a + ab * 64 + j * 16, a);
             }
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive_relaxed(bar_a_full + 8 * (it % NAB));
-                mbar_arrive_relaxed(bar_empty + 8 * s);
+                mbar_arrive_relaxed(bar_a_full + 8 * ab);
+                mbar_arrive_relaxed(bar_empty + 8 * w.s);
             }
         }
-    } else {
-        // ------------------------------------------------------------------ epilogue warps: thread = column
-        const int ew = warp - EW0, es = ew / NDW, dw = ew % NDW;     // set es (its units: it % NEPI == es), strip dw
+    } else if (warp < 12 + 4 * SETS) {
+        // -------------------------------------------------------------------- drain warps: thread = column, 32 batch rows
+        const int set = (warp - 12) >> 2, dw = warp & 3;                   // rows, strip of the unit
         const int col = dw * 32 + lane;
-        const uint32_t g = lane & 7, t = lane >> 3;          // bucket of the strip, column number in the bucket
-        const uint32_t t_lane = ((uint32_t)((dw & 3) * 32)) << 16;
-        const uint32_t t_d = tmem_base + t_lane + D_BASE + (uint32_t)(dw >> 2) * DCOLS;
-        float* xch = reinterpret_cast<float*>(smem + p.off_xch) + dw * (RR * 32) + lane;     // hand-over slot of this column
-        float accf[RR];
+        constexpr int RT = 32, CH = 16;                                   // rows of a thread, rows per tensor-memory load
+        const uint32_t r0 = set * RT;
+        const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        float acc[RT];
 #pragma unroll
-        for (int i = 0; i < RR; ++i) accf[i] = 0.0f;
+        for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
         bool ok = true;
-        // outer loop: the pieces of this CTA's range (a piece = its units of one column tile); inner loop: this
-        // set's units of the piece
         UnitIter w(u_begin, KT);
-        if (es == 1) w.next(S, KT);
         uint32_t tn = u_begin / KT, piece = 0;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        // outer loop: the pieces of this CTA's range (a piece = its units of one column tile)
         for (uint32_t piece_first = u_begin; piece_first < u_end && ok; ++tn, ++piece) {
-          const uint32_t piece_stop = min(u_end, (tn + 1) * KT);        // one past the piece's last unit
-          piece_first = piece_stop;
-          for (; w.u < piece_stop; w.next(S, KT), (NEPI == 2 ? w.next(S, KT) : (void)0)) {
-            const uint32_t u = w.u, it = w.it, s = w.s, b = w.it & 1;
-            const uint8_t* st = smem + s * p.stage_bytes;
-            if (!warp_wait(bar_full + 8 * s, w.ph, abort_flag, p.status)) { ok = false; break; }
-            // outliers: the bucket descriptor and this lane's slots of the first packets are requested now
-            uint32_t sp_off = 0, sp_cnt = 0, sp_tail = 0, cmax = 0;
-            constexpr int NP = RR <= 16 ? 2 : 1;                     // packet rounds in flight
-            uint32_t pk[NP];
-            const uint32_t* pk_s = reinterpret_cast<const uint32_t*>(st + p.off_coo);
-            const uint32_t* pk_g = nullptr;
-            const char* xtb = reinterpret_cast<const char*>(st + p.off_xt);
-            if (SPARSE) {
-                const uint32_t info = reinterpret_cast<const uint32_t*>(st + p.off_info)[dw * 8 + g];
-                sp_off = info & 0xffffu;
-                sp_cnt = (info >> 16) & 0xffu;
-                if (HOT) {
-                    sp_tail = info >> 24;
-                    if (__reduce_max_sync(0xffffffffu, sp_off + sp_cnt + sp_tail) > p.coo_cap)
-                        pk_g = reinterpret_cast<const uint32_t*>(p.packed + __ldg(p.indptr + u));   // packets beyond the staged part
-                } else if (__any_sync(0xffffffffu, sp_off + sp_cnt > p.coo_cap)) {
-                    // a descriptor that does not belong to the staged packets (layout struct and arrays
-                    // out of step): report it and skip the unit's outliers instead of reading past the stage
-                    if (lane == 0) atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
-                    sp_cnt = 0;
+            const uint32_t piece_stop = min(u_end, (tn + 1) * KT);        // one past the piece's last unit
+            piece_first = piece_stop;
+            for (; w.u < piece_stop; w.next(S, KT)) {
+                const uint32_t db = w.it % NDB;
+                const uint8_t* st = smem + w.s * p.stage_bytes;
+                if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) { ok = false; break; }
+                float sv[GPS];
+#pragma unroll
+                for (int gi = 0; gi < GPS; ++gi) sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz + gi * SZ_ROW)[col]);
+                if (!wait_converged(bar_d_full + 8 * db, (w.it / NDB) & 1, abort_flag, p.status)) { ok = false; break; }
+                tc_fence_after();
+#pragma unroll
+                for (int gi = 0; gi < GPS; ++gi)
+#pragma unroll
+                    for (int c0 = 0; c0 < RT; c0 += CH)
+                        if (r0 + c0 < p.nmma) {
+                            float d[CH];
+                            tmem_ld<CH>(t_lane + S_::D_BASE + (db * GPS + gi) * NR + r0 + c0, d);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < CH; ++i) acc[c0 + i] = fmaf(sv[gi], d[i], acc[c0 + i]);
+                        }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive_relaxed(bar_d_free + 8 * db);
+                    mbar_arrive_relaxed(bar_empty + 8 * w.s);
                 }
-                cmax = __reduce_max_sync(0xffffffffu, sp_cnt);
             }
-            auto slot_word = [&](uint32_t idx) -> uint32_t {           // word t of packet idx of the tile
-                if (!HOT || idx < p.coo_cap) return pk_s[idx * 4 + t];
-                return __ldg(pk_g + idx * 4 + t);
-            };
-#pragma unroll
-            for (int j = 0; j < NP; ++j) pk[j] = (SPARSE && (uint32_t)j < sp_cnt) ? slot_word(sp_off + j) : 0u;
-            float sv[GPS], zv[GPS];
-#pragma unroll
-            for (int gi = 0; gi < GPS; ++gi) {
-                sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz)[gi * BN + col]);
-                zv[gi] = -bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz)[(GPS + gi) * BN + col]);
-            }
-            const float* meta = reinterpret_cast<const float*>(st + p.off_xmeta);
-            // the unit's sums, once its MMAs are complete
-            if (!warp_wait(bar_d_ready + 8 * b, (it >> 1) & 1, abort_flag, p.status)) { ok = false; break; }
+            if (!ok) break;
+            // ---------------------------------------------------------------- end of a piece
+            if (!wait_converged(bar_o_full, piece & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
-            for (int gi = 0; gi < GPS; ++gi) {
-                // sum_k x (q - z) = 2^(E-21) * (D0 + 2^8 D1 + 2^16 D2 - z sum_k x_int), D_j = sum_k q l_j exact in INT32
-                if constexpr (RR == 1) {
-                    uint32_t c[4];                                  // one load of four cells covers the three limbs of the single row
-                    tmem_ld<4>(t_d + b * (NT128 * DCOLS) + gi * NMMA, c);
+            for (int c0 = 0; c0 < RT; c0 += CH)
+                if (r0 + c0 < p.nmma) {
+                    float d[CH];
+                    tmem_ld<CH>(t_lane + S_::O_BASE + r0 + c0, d);
                     tmem_wait_ld();
-                    const float f = fmaf(zv[gi], meta[gi * 2 * RM + RM],
-                                         fmaf(small_int_to_float(c[2]), 65536.0f, fmaf(small_int_to_float(c[1]), 256.0f, small_int_to_float(c[0]))));
-                    accf[0] = fmaf(sv[gi] * meta[gi * 2 * RM], f, accf[0]);
-                } else {
 #pragma unroll
-                    for (int i0 = 0; i0 < RR; i0 += 8 < RR ? 8 : RR) {     // eight rows at a time (four with RR = 4)
-                        constexpr int CH = 8 < RR ? 8 : RR;
-                        uint32_t c[kLimbs][CH];
-#pragma unroll
-                        for (int j = 0; j < kLimbs; ++j) tmem_ld<CH>(t_d + b * (NT128 * DCOLS) + gi * NMMA + j * RR + i0, c[j]);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < CH; ++i) {
-                            const float xs = meta[gi * 2 * RM + i0 + i], sx = meta[gi * 2 * RM + RM + i0 + i];
-                            const float f = fmaf(zv[gi], sx, fmaf(small_int_to_float(c[2][i]), 65536.0f, fmaf(small_int_to_float(c[1][i]), 256.0f, small_int_to_float(c[0][i]))));
-                            accf[i0 + i] = fmaf(sv[gi] * xs, f, accf[i0 + i]);
-                        }
-                    }
+                    for (int i = 0; i < CH; ++i) acc[c0 + i] += d[i];
                 }
-            }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar_d_free + 8 * b);     // the MMAs of unit it + 2 may overwrite this D buffer
-            if (SPARSE) {
-                // ---- the unit's outliers of this thread's column (padding slots have value 0: they add 0)
-                for (uint32_t i = 0; i < cmax; i += NP) {
-                    uint32_t nx[NP];                               // the next rounds' slots, requested before this round's math
+            if (lane == 0) mbar_arrive_relaxed(bar_o_free);
+            const uint32_t kt = piece_stop - 1 - tn * KT;                 // k-step of the piece's last unit
+            const uint32_t u_tile0 = tn * KT;
+            const uint32_t piece_k0 = max(u_tile0, u_begin) - u_tile0;
+            const bool full_piece = (piece_k0 == 0) && (kt == KT - 1);
+            bool write_y = full_piece;
+            if (!full_piece) {
+                // Split tile.  Every warp settles its own 32 columns and rows, without CTA-wide barriers: FP32 partial, four
+                // rows of a column to 16 bytes, then one arrival per (tile, strip, set of rows: a byte of the strip's
+                // counter each); the last warp to arrive adds the partials in CTA order (the same order in every run)
+                // and writes Y.
+                constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;      // float4 per slot
+                const uint32_t which = (p.split || u_begin / KT == tn) ? 0u : 1u;
+                float4* slots = reinterpret_cast<float4*>(p.partials) + (size_t)(r0 / 4) * COLS + col;
+                float4* slot = slots + ((size_t)blockIdx.x * 2 + which) * SLOT;
 #pragma unroll
-                    for (int j = 0; j < NP; ++j) nx[j] = (i + NP + j < sp_cnt) ? slot_word(sp_off + i + NP + j) : 0u;
-                    add_outliers<RR, NP>(accf, pk, xtb);
-#pragma unroll
-                    for (int j = 0; j < NP; ++j) pk[j] = nx[j];
+                for (int i = 0; i < RT / 4; ++i)
+                    if (r0 + 4 * i < p.M) __stcg(slot + i * COLS, make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]));
+                __syncwarp();
+                const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q, r);
+                const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q, r);
+                uint32_t* counter = p.counters + tn * 4 + dw;
+                uint32_t last = 0;
+                if (lane == 0) {
+                    // one arrival, release and acquire at GPU scope: the warp's stores (ordered before this lane by
+                    // the __syncwarp above) precede it, and the warp that finds itself last sees the stores of all
+                    // contributors that arrived before
+                    uint32_t old;
+                    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(counter), "r"(1u << (8 * set)) : "memory");
+                    last = (((old >> (8 * set)) & 0xffu) == c_last - c_first) ? 1u : 0u;
                 }
-                if (HOT) {
-                    // a bucket with a tail: its packets (slots name their column) are shared out over the eight
-                    // lane groups g, each adding into sums of its own that are added up over g afterwards
-                    for (uint32_t hot = __ballot_sync(0xffffffffu, sp_tail != 0); hot; ) {     // warp-uniform
-                        const uint32_t hot_lane = __ffs(hot) - 1;
-                        hot &= ~(0x01010101u << (hot_lane & 7u));
-                        const uint32_t hot_off = __shfl_sync(0xffffffffu, sp_off + sp_cnt, hot_lane);
-                        const uint32_t hot_cnt = __shfl_sync(0xffffffffu, sp_tail, hot_lane);
-                        float hacc[RR];
+                last = __shfl_sync(0xffffffffu, last, 0);
+                __syncwarp();
+                if (last) {
+                    write_y = true;
+                    // 16 rows at a time, ND contributors' loads in flight; the additions keep CTA order
+                    constexpr int ND = 2;
 #pragma unroll
-                        for (int ri = 0; ri < RR; ++ri) hacc[ri] = 0.0f;
-                        for (uint32_t i = g; i < hot_cnt; i += 8) {
-                            const uint32_t idx = hot_off + i;
-                            const uint4 pkt = (idx < p.coo_cap) ? reinterpret_cast<const uint4*>(pk_s)[idx]
-                                                                : __ldg(reinterpret_cast<const uint4*>(pk_g) + idx);
-                            const uint32_t wd[4] = {pkt.x, pkt.y, pkt.z, pkt.w};
+                    for (int i0 = 0; i0 < RT / 4; i0 += 4)
+                        if (r0 + 4 * i0 < p.M) {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                // a tail slot names its column: slots of other columns count as padding (value 0)
-                                const uint32_t mine[1] = {((wd[e] >> kSlotColShift) & 3u) == t ? wd[e] : (wd[e] & ~kSlotValueMask)};
-                                add_outliers<RR, 1>(hacc, mine, xtb);
+                            for (int i = 0; i < 16; ++i) acc[4 * i0 + i] = 0.0f;
+                            for (uint32_t c = c_first; c <= c_last; c += ND) {
+                                float4 v[ND][4];
+#pragma unroll
+                                for (int dd = 0; dd < ND; ++dd) {
+                                    const uint32_t cc = min(c + dd, c_last);
+                                    const uint32_t wch = (p.split || unit_begin_of(cc, q, r) / KT == tn) ? 0u : 1u;
+                                    const float4* sl = slots + ((size_t)cc * 2 + wch) * SLOT;
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) v[dd][i] = __ldcg(sl + (i0 + i) * COLS);
+                                }
+#pragma unroll
+                                for (int dd = 0; dd < ND; ++dd)
+                                    if (c + dd <= c_last) {
+#pragma unroll
+                                        for (int i = 0; i < 4; ++i) {
+                                            acc[4 * (i0 + i) + 0] += v[dd][i].x;
+                                            acc[4 * (i0 + i) + 1] += v[dd][i].y;
+                                            acc[4 * (i0 + i) + 2] += v[dd][i].z;
+                                            acc[4 * (i0 + i) + 3] += v[dd][i].w;
+                                        }
+                                    }
                             }
                         }
-#pragma unroll
-                        for (int ri = 0; ri < RR; ++ri) {
-                            float v = hacc[ri];
-                            v += __shfl_xor_sync(0xffffffffu, v, 1);
-                            v += __shfl_xor_sync(0xffffffffu, v, 2);
-                            v += __shfl_xor_sync(0xffffffffu, v, 4);
-                            if (g == (hot_lane & 7u)) accf[ri] += v;
-                        }
-                    }
+                    if (lane == 0) atomicSub(counter, (c_last - c_first + 1) << (8 * set));      // ready for the next call
                 }
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * s);
-          }
-          if (!ok) break;
-          {
-                // ---------------------------------------------------------- end of a piece
-                if (NEPI == 2) {
-                    if (es == 1) {
-                        // hand the sums over (after set 0 has taken the previous piece's) and start afresh
-                        if (piece > 0 && !warp_wait(bar_xempty + 8 * dw, (piece - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+            if (write_y) {
+                uint16_t* y = p.Y + (size_t)r0 * p.N + (size_t)tn * 128 + col;
 #pragma unroll
-                        for (int mm = 0; mm < RR; ++mm) { xch[mm * 32] = accf[mm]; accf[mm] = 0.0f; }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar_xfull + 8 * dw);
-                        continue;
-                    }
-                    if (!warp_wait(bar_xfull + 8 * dw, piece & 1, abort_flag, p.status)) { ok = false; break; }
+                for (int m = 0; m < RT; ++m)
+                    if (r0 + m < p.M) y[(size_t)m * p.N] = float_to_bf16_bits(acc[m]);
+            }
 #pragma unroll
-                    for (int mm = 0; mm < RR; ++mm) accf[mm] += xch[mm * 32];
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_xempty + 8 * dw);
+            for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
+        }
+    } else {
+        // -------------------------------------------------------------------- scatter warps: thread = column
+        // Column 32 strip + l of a half is column number t = l / 8 of bucket g = l % 8 of the strip: slot t of every
+        // column-slotted packet of the bucket.  The thread owns the column's row of the tile (2 bytes per k, eight k
+        // to 16 bytes, those 2048 bytes apart) and knows which places it has filled: a byte each in two registers, or
+        // the whole row where they are more than kScatterKeep or a tail was shared out over the warp.
+        const uint32_t sg = SG == 2 ? (uint32_t)(warp - (12 + 4 * SETS)) >> 2 : 0u;      // takes the units it with it % SG == sg
+        const uint32_t strip = warp & 3, g = lane & 7, t = lane >> 3;
+        uint8_t* row = smem + p.off_wo + (strip * 32 + lane) * 16;
+        for (int b = sg; b < NWO; b += SG)
+            for (int i = 0; i < 16; ++i) *reinterpret_cast<uint4*>(row + b * kWoTile + i * 2048) = make_uint4(0, 0, 0, 0);
+        auto place = [&](uint32_t k) { return (k >> 3) * 2048 + (k & 7) * 2; };
+        // what a part of an outlier is: its BF16 bits, or (second part) the fraction bits that BF16 cuts off
+        auto bits_of = [&](uint32_t wd, uint32_t part) -> uint16_t {
+            const uint32_t hi = wd & 0xffff0000u;
+            if (part == 0) return (uint16_t)(hi >> 16);
+            return (wd & 0x7f800000u) == 0x7f800000u ? (uint16_t)0 : float_to_bf16_bits(__uint_as_float(wd & kSlotValueMask) - __uint_as_float(hi));
+        };
+        // filled places of the tile in turn, and of the group's other tile
+        uint32_t k0 = 0, k1 = 0, cnt = 0, o_k0 = 0, o_k1 = 0, o_cnt = 0;
+        bool ok = true;
+        for (UnitIter w(u_begin, KT); w.u < u_end && ok; w.next(S, KT)) {
+            const uint8_t* st = smem + w.s * p.stage_bytes;
+            if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
+            if (SG == 2 && (w.it & 1) != sg) continue;           // waited for all the same, see the unpack warps
+            const uint32_t* pk = reinterpret_cast<const uint32_t*>(st + p.off_coo);
+            const uint32_t wb = w.it % NWO;
+            const uint32_t info = reinterpret_cast<const uint32_t*>(st + p.off_info)[strip * 8 + g];
+            const uint32_t off = info & 0xffffu;
+            uint32_t depth = (info >> 16) & 0xffu, tail = info >> 24;
+            const uint32_t* pg = nullptr;
+            if (__any_sync(0xffffffffu, off + depth + tail > p.coo_cap)) {
+                // packets beyond the staged part of a large tile come from global memory; a descriptor that
+                // reaches past its tile (or, for a layer whose tiles all fit, past the staged part: layout struct
+                // and arrays out of step) is reported and skipped
+                const uint32_t c = chunk_of(w.tn, w.kt), a = __ldg(p.indptr + c), npk = __ldg(p.indptr + c + 1) - a;
+                pg = reinterpret_cast<const uint32_t*>(p.packed + a);
+                if (off + depth + tail > (p.general ? npk : p.coo_cap)) {
+                    asm volatile("griddepcontrol.wait;" ::: "memory");     // before the scratch is written
+                    atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
+                    depth = 0, tail = 0;
                 }
-                const uint32_t kt = piece_stop - 1 - tn * KT;               // k-step of the piece's last unit
-                const uint32_t u_tile0 = tn * KT;
-                const uint32_t piece_k0 = max(u_tile0, u_begin) - u_tile0;
-                const bool full_piece = (piece_k0 == 0) && (kt == KT - 1);
-                bool write_y = full_piece;
-                if (!full_piece) {
-                    // Split tile.  Every warp settles its own 32-column strip, without CTA-wide barriers: FP32
-                    // partial [row][column], then one arrival per (tile, strip); the last warp to arrive adds
-                    // the partials in CTA order (the same order in every run) and writes Y.
-                    const uint32_t which = (p.split || u_begin / KT == tn) ? 0u : 1u;
-                    float* slot = p.partials + ((size_t)blockIdx.x * 2 + which) * (size_t)(BN * RR) + col;
+            }
+            auto slot = [&](uint32_t d) { return off + d < p.coo_cap ? pk[(off + d) * 4 + t] : __ldg(pg + (off + d) * 4 + t); };
+            uint32_t wd[4];                                    // the first slots, requested before the wait below
 #pragma unroll
-                    for (int mm = 0; mm < RR; ++mm) __stcg(slot + mm * BN, accf[mm]);
-                    __syncwarp();
-                    const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q, r);
-                    const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q, r);
-                    uint32_t last = 0;
-                    if (lane == 0) {
-                        // one arrival, release and acquire at GPU scope: the warp's stores (ordered before this
-                        // lane by the __syncwarp above) precede it, and the warp that finds itself last sees the
-                        // stores of all contributors that arrived before
-                        uint32_t old;
-                        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.counters + tn * NDW + dw) : "memory");
-                        last = (old == c_last - c_first) ? 1u : 0u;
-                    }
-                    last = __shfl_sync(0xffffffffu, last, 0);
-                    __syncwarp();
-                    if (last) {
-                        write_y = true;
+            for (uint32_t d = 0; d < 4; ++d) wd[d] = d < depth ? slot(d) : 0u;
+            for (uint32_t part = 0; part < p.parts; ++part) {
+                uint8_t* tile = row + wb * kWoTile;
+                // ---- take out what the tile held; the MMAs that read it are complete
+                const uint32_t n = (w.it / NWO) * p.parts + part;
+                if (n > 0 && !wait_converged(bar_wo_empty + 8 * wb, (n - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                if (cnt <= kScatterKeep) {
 #pragma unroll
-                        for (int mm = 0; mm < RR; ++mm) accf[mm] = 0.0f;
-                        constexpr int ND = RR <= 4 ? 8 : (RR <= 8 ? 4 : 2);       // contributors' loads in flight
-                        for (uint32_t c = c_first; c <= c_last; c += ND) {
-                            float v[ND][RR];
-#pragma unroll
-                            for (int dd = 0; dd < ND; ++dd) {
-                                const uint32_t cc = min(c + dd, c_last);
-                                const uint32_t wch = (p.split || unit_begin_of(cc, q, r) / KT == tn) ? 0u : 1u;
-                                const float* sl = p.partials + ((size_t)cc * 2 + wch) * (size_t)(BN * RR) + col;
-#pragma unroll
-                                for (int mm = 0; mm < RR; ++mm) v[dd][mm] = __ldcg(sl + mm * BN);
-                            }
-#pragma unroll
-                            for (int dd = 0; dd < ND; ++dd)
-                                if (c + dd <= c_last) {
-#pragma unroll
-                                    for (int mm = 0; mm < RR; ++mm) accf[mm] += v[dd][mm];
-                                }
-                        }
-                        if (lane == 0) p.counters[tn * NDW + dw] = 0;  // ready for the next call
-                    }
+                    for (uint32_t i = 0; i < 4; ++i)
+                        if (i < cnt) *reinterpret_cast<uint16_t*>(tile + place((k0 >> (8 * i)) & 127u)) = 0;
+                    for (uint32_t i = 4; i < cnt; ++i) *reinterpret_cast<uint16_t*>(tile + place((k1 >> (8 * (i - 4))) & 127u)) = 0;
+                } else {
+#pragma unroll 4
+                    for (int i = 0; i < 16; ++i) *reinterpret_cast<uint4*>(tile + i * 2048) = make_uint4(0, 0, 0, 0);
                 }
-                if (write_y) {
+                __syncwarp();
+                cnt = 0;
+                // ---- put this half-step's in
+                auto put = [&](uint32_t v) {
+                    if (v & kSlotValueMask) {                  // not padding
+                        const uint32_t k = (v >> 5) & 127u;
+                        *reinterpret_cast<uint16_t*>(tile + place(k)) = bits_of(v, part);
+                        k1 = (k1 << 8) | (k0 >> 24), k0 = (k0 << 8) | k;
+                        ++cnt;
+                    }
+                };
 #pragma unroll
-                    for (int mm = 0; mm < RR; ++mm)
-                        if ((uint32_t)mm < p.M) p.Y[(size_t)mm * p.N + (size_t)tn * BN + col] = float_to_bf16_bits(accf[mm]);
+                for (int d = 0; d < 4; ++d) put(wd[d]);
+                for (uint32_t d = 4; d < depth; ++d) put(slot(d));
+                for (uint32_t hot = __ballot_sync(0xffffffffu, tail != 0); hot;) {     // buckets with a tail: warp-uniform
+                    const uint32_t b = (__ffs(hot) - 1) & 7u;      // its four lanes b, b + 8, b + 16, b + 24 agree
+                    hot &= ~(0x01010101u << b);
+                    const uint32_t t_off = __shfl_sync(0xffffffffu, off + depth, b), t_cnt = __shfl_sync(0xffffffffu, tail, b);
+                    uint8_t* base = smem + p.off_wo + wb * kWoTile + (strip * 32 + b) * 16;
+                    for (uint32_t i = lane; i < 4 * t_cnt; i += 32) {
+                        const uint32_t v = t_off + i / 4 < p.coo_cap ? pk[t_off * 4 + i] : __ldg(pg + t_off * 4 + i);
+                        if (v & kSlotValueMask)                    // a tail slot names its column
+                            *reinterpret_cast<uint16_t*>(base + ((v >> kSlotColShift) & 3u) * 128 + place((v >> 5) & 127u)) = bits_of(v, part);
+                    }
+                    if (g == b) cnt = kScatterKeep + 1;
                 }
-#pragma unroll
-                for (int mm = 0; mm < RR; ++mm) accf[mm] = 0.0f;
-          }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_wo_full + 8 * wb);
+            }
+            if (!ok) break;
+            if (NWO / SG == 2) {
+                const uint32_t a = k0, b = k1, c = cnt;
+                k0 = o_k0, k1 = o_k1, cnt = o_cnt;
+                o_k0 = a, o_k1 = b, o_cnt = c;
+            }
+            if (!ok) break;
+            if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * w.s);
         }
     }
 

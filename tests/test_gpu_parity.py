@@ -543,3 +543,57 @@ def test_back_to_back_dependent_calls_keep_stream_order(M):
             H.check_tolerances(b.cpu().numpy().view(np.uint16), Yref, Yabs, K)
         for Y in Ys:
             Y.fill_(0x7fc0)
+
+
+# ------------------------------------------------------------------ more than 16 rows per launch
+
+@pytest.mark.parametrize("K,N,g,BN", [(128, 128, 128, 128), (1280, 384, 64, 128), (2944, 512, 128, 256), (8192, 256, 64, 256)])
+@pytest.mark.parametrize("M", [17, 33, 48, 65, 113, 128])
+def test_launches_of_more_than_16_rows(K, N, g, BN, M):
+    """One unit per CTA and many, an odd number of k-steps, both tile widths and group sizes; rows at the edges of the
+    kernel's variants (32, 64, 128) and of the MMA's steps of 16."""
+    lay = synth.layer(synth.tensor_seed(12, K // 128 + N // 128), K, N, density=0.02, layout="mixed")
+    P = H.pack_layer(lay, g, BN)
+    X = _x(lay.seed + M, M, K)
+    Yref, Yabs = H.oracle_result(P, X)
+    Y = H.run_fused(P, X)
+    H.check_tolerances(Y, Yref, Yabs, K)
+    assert np.array_equal(H.run_fused(P, X), Y)
+    assert not P.ws[: 256 + 32768].cpu().numpy().any()
+
+
+@pytest.mark.parametrize("M", [17, 64, 128])
+def test_more_than_16_rows_with_tails_oversized_tiles_and_dense_columns(M):
+    """Columns of 0 to 9 outliers in a tile (the kernel undoes up to 8 one by one), columns with a tail, and a tile whose
+    packets exceed a stage, next to tiles without any; each tile's places must be clear for the next."""
+    K, N, g, BN = 1536, 512, 128, 256
+    lay = synth.layer(synth.tensor_seed(12, 99), K, N, density=0.0)
+    rng = np.random.default_rng(7)
+    mask = np.zeros((K, N), dtype=np.uint8)
+    for col in range(N):
+        for kt in (0, 2, 3, 7, 9):
+            mask[kt * 128 + rng.choice(128, size=(col + kt) % 10, replace=False), col] = 1
+    mask[5 * 128:6 * 128, 0:256] = 1
+    mask[8 * 128:8 * 128 + 100, 300] = 1
+    kk, nn = np.nonzero(mask)
+    vb = ((rng.uniform(0.12, 0.4, size=kk.size) * rng.choice([-1, 1], size=kk.size)).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
+    lay.mask, lay.coo_k, lay.coo_n, lay.coo_v = mask, kk.astype(np.uint32), nn.astype(np.uint32), vb
+    lay.W[kk, nn] = synth.bf16_bits_to_f32(vb)
+    P = H.pack_layer(lay, g, BN)
+    assert P.L.max_tile_packets == 8192 and P.L.max_tail_packets > 0
+    X = _x(lay.seed, M, K)
+    Yref, Yabs = H.oracle_result(P, X)
+    H.check_tolerances(H.run_fused(P, X), Yref, Yabs, K)
+
+
+def test_more_than_16_rows_of_a_layer_that_names_a_position_twice():
+    """Several outliers at one position count with their sum in every kernel: the encoder says so in the layout, and such
+    a layer is not given to the kernel that writes outliers into a tile."""
+    K, N, g, M = 512, 256, 128, 40
+    lay = synth.layer(synth.tensor_seed(12, 98), K, N, density=0.01, layout="uniform")
+    lay.coo_k, lay.coo_n, lay.coo_v = (np.concatenate([a, a[:50]]) for a in (lay.coo_k, lay.coo_n, lay.coo_v))
+    P = H.pack_layer(lay, g)
+    assert P.L.tilecoo_encoded == 2
+    X = _x(3, M, K)
+    Yref, Yabs = H.oracle_result(P, X)
+    H.check_tolerances(H.run_fused(P, X), Yref, Yabs, K)
