@@ -157,13 +157,14 @@ def fq_encode_tilecoo_sizes(L: Layout, k, n, val):
 def fq_encode_tilecoo(L: Layout, k, n, val):
     """Returns (tile_indptr uint32, bucket_info uint32, packed uint8[n_packets, 16]); sets L.max_tile_packets."""
     k, n, val = _np(k, np.uint32), _np(n, np.uint32), _np(val, np.uint16)
-    n_ip, n_bi, n_pk, _ = fq_encode_tilecoo_sizes(L, k, n, val)
-    indptr = np.empty(n_ip, dtype=np.uint32)
-    info = np.empty(n_bi, dtype=np.uint32)
-    packed = np.zeros((max(n_pk, 1), 16), dtype=np.uint8)
+    tiles = (L.K // max(L.BK, 1)) * (L.N // max(L.BN, 1))
+    indptr = np.empty(tiles + 1, dtype=np.uint32)
+    info = np.empty(tiles * L.buckets_per_tile, dtype=np.uint32)
+    # every packet holds at least one outlier, so there are at most as many; pages that stay unwritten cost nothing
+    packed = np.empty((max(k.shape[0], 1), 16), dtype=np.uint8)
     _check(lib().fq_encode_tilecoo(ctypes.byref(L), _hp(k), _hp(n), _hp(val), ctypes.c_size_t(k.shape[0]),
-                                   _hp(indptr), _hp(info), _hp(packed), ctypes.c_size_t(n_pk)))
-    return indptr, info, packed[:n_pk]
+                                   _hp(indptr), _hp(info), _hp(packed), ctypes.c_size_t(k.shape[0])))
+    return indptr, info, packed[:int(indptr[-1])]
 
 
 def fq_decode_tilecoo(L: Layout, indptr, info, packed):

@@ -389,3 +389,19 @@ def test_validator_rejects_corrupted_arrays():
     # more column-slotted packets than the format allows
     bad = info.copy(); bad[0] = (bad[0] & 0xffff) | (33 << 16)
     expect_format_error(indptr, bad, packed)
+
+
+def test_tilecoo_arrays_do_not_depend_on_the_order_of_the_input():
+    """More entries than one thread's share of the encoder's counting sort, in two orders, zeros among them; columns short
+    and long (tails)."""
+    K, N = 1024, 768
+    lay = synth.layer(synth.tensor_seed(11, 3), K, N, density=0.03, layout="clustered")
+    k, n, v = lay.coo_k.copy(), lay.coo_n.copy(), lay.coo_v.copy()
+    v[::97] = 0x8000                                          # -0 is not an outlier
+    perm = np.random.default_rng(2).permutation(k.size)
+    La, Lb = fq.fq_get_layout(K, N, 128), fq.fq_get_layout(K, N, 128)
+    a = fq.fq_encode_tilecoo(La, k, n, v)
+    b = fq.fq_encode_tilecoo(Lb, k[perm], n[perm], v[perm])
+    assert La.max_tail_packets > 0 and k.size > 16384
+    assert all(np.array_equal(x, y) for x, y in zip(a, b)) and bytes(La) == bytes(Lb)
+    assert fq.fq_encode_tilecoo_sizes(La, k, n, v) == (a[0].size, a[1].size, a[2].shape[0], La.max_tile_packets)
