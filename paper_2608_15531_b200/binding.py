@@ -65,6 +65,20 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_call = None
+
+
+def _pycall():
+    """The CPython entry to the fused calls (``_fqcall.so``), which passes tensors on without ctypes."""
+    global _call
+    if _call is None:
+        lib()
+        import torch  # noqa: F401  (its libraries have to be there first)
+        from . import _fqcall
+        _call = _fqcall
+    return _call
+
+
 def _check(code: int) -> None:
     if code != FQ_OK:
         raise FqError(code, lib().fq_last_error().decode(errors="replace"))
@@ -88,6 +102,11 @@ def _dp(t):
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
     return ctypes.c_void_p(t.data_ptr())
+
+
+def _host(a) -> int:
+    """Address of a host tensor or numpy array."""
+    return a.data_ptr() if hasattr(a, "data_ptr") else a.ctypes.data
 
 
 def _stream(stream=None):
@@ -196,10 +215,9 @@ def fq_workspace_bytes(L: Layout, M: int) -> int:
 
 def fq_fused_w4a16_outlier_gemm(L: Layout, X, M: int, wq, scale, zero, tile_indptr, bucket_info, packed, Y,
                                 workspace, stream=None) -> None:
-    _check(lib().fq_fused_w4a16_outlier_gemm(ctypes.byref(L), _dp(X), ctypes.c_uint32(M), _dp(wq), _dp(scale),
-                                             _dp(zero), _dp(tile_indptr), _dp(bucket_info), _dp(packed), _dp(Y),
-                                             _dp(workspace), ctypes.c_size_t(workspace.numel() * workspace.element_size()),
-                                             _stream(stream)))
+    code = (_call or _pycall()).fused(L, X, M, wq, scale, zero, tile_indptr, bucket_info, packed, Y, workspace, stream)
+    if code != FQ_OK:
+        _check(code)
 
 
 def fq_fused_w4a16_outlier_gemm_noalloc(L: Layout, X, M: int, wq, scale, zero, tile_indptr, bucket_info, packed, Y,
@@ -227,23 +245,16 @@ def fq_unfused_spmm(L: Layout, X, M: int, tile_indptr, bucket_info, packed, Y, s
 def fq_fused_host_io(L: Layout, X_host, M: int, x_dev, wq, scale, zero, tile_indptr, bucket_info, packed, y_dev,
                      Y_host, workspace, stream=None) -> None:
     """X_host / Y_host: host tensors (pinned for speed) or numpy arrays; the call returns after Y_host is filled."""
-    xh = ctypes.c_void_p(X_host.data_ptr() if hasattr(X_host, "data_ptr") else X_host.ctypes.data)
-    yh = ctypes.c_void_p(Y_host.data_ptr() if hasattr(Y_host, "data_ptr") else Y_host.ctypes.data)
-    _check(lib().fq_fused_host_io(ctypes.byref(L), xh, ctypes.c_uint32(M), _dp(x_dev), _dp(wq), _dp(scale), _dp(zero),
-                                  _dp(tile_indptr), _dp(bucket_info), _dp(packed), _dp(y_dev), yh, _dp(workspace),
-                                  ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)))
+    _check((_call or _pycall()).host_io(L, _host(X_host), M, x_dev, wq, scale, zero, tile_indptr, bucket_info, packed, y_dev,
+                                        _host(Y_host), workspace, stream, True))
 
 
 def fq_fused_host_io_async(L: Layout, X_host, M: int, x_dev, wq, scale, zero, tile_indptr, bucket_info, packed, y_dev,
                            Y_host, workspace, stream=None) -> None:
     """As fq_fused_host_io, without the final wait: the caller synchronises the stream before reading Y_host
     (pinned host tensors)."""
-    xh = ctypes.c_void_p(X_host.data_ptr() if hasattr(X_host, "data_ptr") else X_host.ctypes.data)
-    yh = ctypes.c_void_p(Y_host.data_ptr() if hasattr(Y_host, "data_ptr") else Y_host.ctypes.data)
-    _check(lib().fq_fused_host_io_async(ctypes.byref(L), xh, ctypes.c_uint32(M), _dp(x_dev), _dp(wq), _dp(scale),
-                                        _dp(zero), _dp(tile_indptr), _dp(bucket_info), _dp(packed), _dp(y_dev), yh,
-                                        _dp(workspace),
-                                        ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)))
+    _check((_call or _pycall()).host_io(L, _host(X_host), M, x_dev, wq, scale, zero, tile_indptr, bucket_info, packed, y_dev,
+                                        _host(Y_host), workspace, stream, False))
 
 
 def fq_check_status(workspace, stream=None) -> None:

@@ -1,4 +1,5 @@
-"""Build the C-ABI library ``libfq.so`` (nvcc, sm_100a) and the generator's ``libfq_synth.so`` in-tree."""
+"""Build the C-ABI library ``libfq.so`` (nvcc, sm_100a), its CPython entry ``_fqcall.so`` and the generator's
+``libfq_synth.so`` in-tree."""
 from __future__ import annotations
 
 import os
@@ -20,11 +21,15 @@ NVCC_FLAGS = [
 ]
 
 
-def stale() -> bool:
-    if not os.path.exists(LIB):
+PYCALL = os.path.join(HERE, "_fqcall.so")
+PYCALL_SOURCE = os.path.join(CSRC, "fq_pycall.cpp")
+
+
+def stale(lib: str = LIB, sources=tuple(SOURCES + HEADERS)) -> bool:
+    if not os.path.exists(lib):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS)
+    t = os.path.getmtime(lib)
+    return any(os.path.getmtime(f) > t for f in sources)
 
 
 def build_lib(force: bool = False, verbose: bool = False) -> str:
@@ -35,8 +40,26 @@ def build_lib(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_pycall(force: bool = False) -> str:
+    """The CPython entry to the fused calls: links libfq.so (beside it) and the libraries of the torch that will be
+    imported with it."""
+    if force or stale(PYCALL, (PYCALL_SOURCE, HEADERS[-1])):
+        import sysconfig
+        import torch
+        t = os.path.join(os.path.dirname(torch.__file__))
+        cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(t, "include"),
+               "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
+               "-o", PYCALL, PYCALL_SOURCE, "-L", HERE, "-l:libfq.so", "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda",
+               "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{os.path.join(t, 'lib')}"]
+        subprocess.run(cmd, check=True)
+    return PYCALL
+
+
 def build_all(force: bool = False, verbose: bool = False) -> None:
     build_lib(force, verbose)
+    build_pycall(force)
     from . import synth
     synth.build(force)
 

@@ -835,6 +835,47 @@ fq_status_t fq_unfused_spmm(const fq_layout_t* L, const void* X, uint32_t M, con
     return FQ_OK;
 }
 
+// The copies of X and Y.  A copy engine's copy between two kernels of a stream costs about 12 us beyond its transfer
+// (the engine and the SMs wait for each other through the memory system, and no part of the next kernel is resident
+// meanwhile); a kernel that reads or writes the pinned host memory itself starts like any other of the chain.  So short
+// copies of pinned memory are copied by a kernel, and the engine keeps pageable memory, which only it can read,
+// and long copies.
+constexpr size_t kKernelCopyMax = 4u << 20;
+__global__ void __launch_bounds__(256) fq_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, uint32_t n) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t i0 = blockIdx.x * 1024 + threadIdx.x;
+    uint4 v[4];                                            // four loads in flight: a read of host memory takes over a microsecond
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (i0 + 256 * j < n) v[j] = src[i0 + 256 * j];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (i0 + 256 * j < n) dst[i0 + 256 * j] = v[j];
+}
+// `host`: the one of the two that is host memory.
+static cudaError_t enqueue_copy(void* dst, const void* src, const void* host, size_t bytes, cudaMemcpyKind kind, cudaStream_t s) {
+    if (bytes <= kKernelCopyMax && bytes % 16 == 0 && aligned(src, 16) && aligned(dst, 16)) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer) {
+            const uint32_t n = (uint32_t)(bytes / 16);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((n + 1023) / 1024);
+            cfg.blockDim = dim3(256);
+            cfg.stream = s;
+            cudaLaunchAttribute pdl[1];
+            std::memset(pdl, 0, sizeof(pdl));
+            pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            pdl[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = pdl, cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, fq_copy_kernel, (const uint4*)(src == host ? at.devicePointer : src),
+                                      (uint4*)(dst == host ? at.devicePointer : dst), n);
+        }
+        cudaGetLastError();                                // an unregistered pointer is not an error here
+    }
+    return cudaMemcpyAsync(dst, src, bytes, kind, s);
+}
+
 fq_status_t fq_fused_host_io_async(const fq_layout_t* L, const void* X_host, uint32_t M, void* x_dev, const void* wq,
                                    const void* scale, const void* zero, const void* tile_indptr,
                                    const void* bucket_info, const void* packed_outliers, void* y_dev, void* Y_host,
@@ -843,12 +884,12 @@ fq_status_t fq_fused_host_io_async(const fq_layout_t* L, const void* X_host, uin
     if (!X_host || !Y_host || !x_dev || !y_dev) return fail(FQ_ERR_INVALID_ARG, "null pointer");
     if (M < 1 || M > FQ_MAX_M) return fail(FQ_ERR_INVALID_ARG, "M = %u outside [1, %u]", M, FQ_MAX_M);
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaMemcpyAsync(x_dev, X_host, (size_t)M * L->K * 2, cudaMemcpyHostToDevice, s);
+    cudaError_t e = enqueue_copy(x_dev, X_host, X_host, (size_t)M * L->K * 2, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "copy of X: %s", cudaGetErrorString(e));
     fq_status_t st = fq_fused_w4a16_outlier_gemm(L, x_dev, M, wq, scale, zero, tile_indptr, bucket_info,
                                                  packed_outliers, y_dev, workspace, workspace_bytes, cuda_stream);
     if (st != FQ_OK) return st;
-    e = cudaMemcpyAsync(Y_host, y_dev, (size_t)M * L->N * 2, cudaMemcpyDeviceToHost, s);
+    e = enqueue_copy(Y_host, y_dev, Y_host, (size_t)M * L->N * 2, cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "copy of Y: %s", cudaGetErrorString(e));
     return FQ_OK;
 }

@@ -31,11 +31,11 @@
 //
 // What bounds it, per unit in SM clocks (MMAs issued back to back from one warp, two commits each): 8 dense + 8
 // outlier MMAs take 430 clocks at N = 16, 490 at 32, 650 at 64, 1030 at 128 (an outlier MMA is bound by reading its 4 KB
-// of A from shared memory up to N = 64); HBM at the measured copy rate would need 425.  The kernel takes 1450 at 32 rows and
-// 2320 at 128 on an 8192 x 28672 layer (78 and 125 us): the chain copy - unpack - MMA - drain of a stage through its
-// barriers times the stages that fit, and the scatter (its walk costs 10 to 20 % of the time: 124 us at 3 % of outliers).
-// It replaces a kernel on the 8-bit integer tensor path whose activations took three limbs and which applied the
-// outliers row by row: 65.6 us on 8192 x 10240 at 32 rows against 30.
+// of A from shared memory up to N = 64); HBM at the measured copy rate would need 425.  The kernel takes 1560 at 32 rows and
+// 2480 at 128 (8192 x 28672, 1 % of outliers: 77.2 and 122.5 us): the chain copy - unpack - MMA - drain of a stage through its
+// barriers times the stages that fit, and the scatter (68.6 us without outliers, 116 at 3 %).  It replaces a
+// kernel on the 8-bit integer tensor path whose activations took three limbs and which applied the outliers row by row,
+// 32 rows to a launch (8192 x 10240 at 32 rows 65.1 us, now 34.6; 4096 x 28672 at 128 rows 305, now 68.4).
 
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
