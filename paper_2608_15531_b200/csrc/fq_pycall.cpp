@@ -1,8 +1,8 @@
 // CPython entry to the fused calls: takes the torch tensors as they are and calls the C ABI.
 //
-// What bounds a short call is the host: marshalling thirteen arguments through ctypes, with a method call or two on every
-// tensor, took 7 us of the 10.4 us between two calls on a 4096 x 4096 layer whose kernel runs 5.7 us.  Here a
-// tensor costs a type check and a pointer read.
+// What bounds a short call is the host: with thirteen arguments marshalled through ctypes, and a method call or two on every
+// tensor, calls on a 4096 x 4096 layer followed each other every 10.8 us although the kernel runs 5; here a tensor
+// costs a type check and a pointer read, and they follow every 5.1 us.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
