@@ -347,7 +347,7 @@ static int sm_count_cached() {
 }
 
 // The tcgen05 kernel's variant for a launch: the batch rows its tensor memory and drain warps are laid out for.
-static inline uint32_t tc_rows(uint32_t m) { return m <= 32 ? 32u : (m <= 64 ? 64u : 128u); }
+static inline uint32_t tc_rows(uint32_t m) { return m <= 16 ? 16u : (m <= 32 ? 32u : (m <= 64 ? 64u : 128u)); }
 
 struct TcPlan {
     TcParams p;
@@ -377,26 +377,18 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
             grid = NT * c;
         }
     }
-    const uint32_t fixed = 1024 /* alignment */ + 1024 /* barriers */ + tc_outlier_tiles(pl.nr) * kWoTile;
-    uint32_t cap = std::min<uint32_t>(1024, std::max<uint32_t>(8, round_up(L->max_tile_packets, 8))), stage = 0, S = 0;
-    for (;;) {
-        p.off_w = 256 * p.nmma;
-        p.off_sz = p.off_w + 8192;
-        p.off_info = p.off_sz + 2 * GPS * 256;
-        p.off_coo = p.off_info + 128;
-        stage = round_up(p.off_coo + cap * 16, 1024);
-        S = std::min<uint32_t>(8, (kSmemBudget - fixed) / stage);
-        if (S >= 3 || cap <= 64) break;
-        cap = std::max<uint32_t>(64, cap / 2);                 // the rest of an oversized tile is read from global memory
-    }
-    if (S < 2) return fail(FQ_ERR_UNSUPPORTED_SHAPE, "shared-memory stages do not fit");
-    p.coo_cap = cap; p.stages = S; p.stage_bytes = stage;
-    p.general = L->max_tile_packets > cap;
-    p.off_wo = S * stage;
-    p.off_bar = p.off_wo + tc_outlier_tiles(pl.nr) * kWoTile;
+    const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
+    const uint32_t wo_bytes = (sg == 1 ? 2 : sg) * kWoTile, fixed = 1024 /* alignment */ + 1024 /* barriers */ + wo_bytes;
+    p.off_w = 256 * p.nmma;
+    p.off_sz = p.off_w + 8192;
+    p.stage_bytes = round_up(p.off_sz + 2 * GPS * 256, 1024);
+    p.stages = std::min<uint32_t>(12, (kSmemBudget - fixed) / p.stage_bytes);
+    if (p.stages >= 2u * ug) p.stages -= p.stages % ug;        // a stage then always returns to the same unpack group
+    p.max_tile_packets = L->max_tile_packets;
+    p.off_wo = p.stages * p.stage_bytes;
+    p.off_bar = p.off_wo + wo_bytes;
     pl.smem = p.off_bar + 2048;
-    const uint32_t drain = 4 * (pl.nr / 32);
-    pl.threads = 32 * (12 + drain + (12 + drain + 8 <= 32 ? 8 : 4));            // as TcShape::WARPS
+    pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = grid;
     return FQ_OK;
 }
@@ -456,7 +448,12 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 // Which kernel serves a launch: up to 16 rows the warp-level MMA kernels, more rows the tcgen05 kernel, whose cost
 // grows slowly with them.  The latter writes outliers into a tile instead of adding them, so an encoding that names a
 // position twice (or whose origin is unknown) stays with launches of 16 rows.
-static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) { return rows > 16 && sparse && L->tilecoo_encoded == 1; }
+#ifdef FQ_EXPERIMENT
+static uint32_t tc_min() { return getenv("FQ_TCMIN") ? atoi(getenv("FQ_TCMIN")) : 17; }
+#else
+static uint32_t tc_min() { return 17; }
+#endif
+static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) { return rows >= tc_min() && sparse && L->tilecoo_encoded == 1; }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
 // Scratch layout: status word and header, tile-arrival counters, FP32 partial slots (two per CTA).
@@ -584,7 +581,7 @@ typedef void (*TcKernelFn)(const CUtensorMap, const TcParams);
 template <int NR>
 static TcKernelFn pick_tc_group(uint32_t g) { return g == 64 ? (TcKernelFn)fq_tc_kernel<NR, 64> : (TcKernelFn)fq_tc_kernel<NR, 128>; }
 static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g) {
-    return nr == 128 ? pick_tc_group<128>(g) : (nr == 64 ? pick_tc_group<64>(g) : pick_tc_group<32>(g));
+    return nr == 128 ? pick_tc_group<128>(g) : (nr == 64 ? pick_tc_group<64>(g) : (nr == 32 ? pick_tc_group<32>(g) : pick_tc_group<16>(g)));
 }
 
 // cudaFuncSetAttribute costs several microseconds: do it once per (kernel, device).

@@ -18,7 +18,7 @@
 // expect_tx, Section 4.1).
 //
 //   warps 0, 2      producers: warp 0 copies a unit's codes, scales and zero-points, warp 2 its X block (tiled tensor
-//                   copies, 128-byte swizzle: the K-major MMA operand), bucket descriptors and packets
+//                   copies, 128-byte swizzle: the K-major MMA operand)
 //   warps 1, 3      tensor: per unit 8 MMAs of K = 16 with A from tensor memory (warp 1, dense) and 8 with A from shared
 //                   memory (warp 3, outliers).  Two warps, because a warp's wait on a barrier costs it about 100 clocks
 //                   even when the barrier is ready, and the MMAs of the other fill them
@@ -72,17 +72,91 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&r)[N]) {
     }
 }
 
-// D[128 x N] (+)= A[128 x 16] * B[16 x N], BF16 in, FP32 out; A in tensor memory or behind a shared-memory descriptor.
-// Issued by one thread.  Descriptors come as their two words, of which only the lower (the address) changes.
-__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n .reg .pred p;\n .reg .b64 y;\n setp.ne.b32 p, %5, 0;\n mov.b64 y, {%2, %3};\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], y, %4, p;\n}"
-                 ::"r"(d), "r"(a), "r"(b), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+// The eight MMAs of a unit, D[128 x N] (+)= A[128 x 16] * B[16 x N] for each 16 of its 128 k, BF16 in, FP32 out, and the
+// commits that follow them.  Whole warp, converged, with warp-uniform operands; one elected lane issues.  One asm block, so
+// that the address arithmetic is not in a divergent branch: there the operands of each MMA have to be moved into
+// uniform registers one by one, and an MMA cost 45 to 120 clocks to issue instead of the 10 it runs (N = 16).
+// `b0`, `b1`: lower words of the descriptors of the two halves of K, `b_hi` their upper word.
+// Dense: A in tensor memory (8 columns to 16 k), the first four MMAs into d0 and the others into d1 (the second group's
+// sums, starting afresh, or the same ones).
+__device__ __forceinline__ void umma_dense(uint32_t d0, uint32_t d1, uint32_t acc1, uint32_t a, uint32_t b0, uint32_t b1, uint32_t b_hi,
+                                           uint32_t idesc, uint32_t bar0, uint32_t bar1, uint32_t bar2) {
+    asm volatile(
+        "{\n .reg .pred e, f;\n .reg .b32 a, b;\n .reg .b64 x, y;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 f, %6, 0;\n"
+        " add.u32 a, %1, 0;\n"
+        " add.u32 b, %2, 0;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], y, %5, f;\n"
+        " setp.eq.b32 f, %6, %6;\n"
+        " add.u32 a, %1, 8;\n"
+        " add.u32 b, %2, 2;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], y, %5, f;\n"
+        " add.u32 a, %1, 16;\n"
+        " add.u32 b, %2, 4;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], y, %5, f;\n"
+        " add.u32 a, %1, 24;\n"
+        " add.u32 b, %2, 6;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], y, %5, f;\n"
+        " add.u32 a, %1, 32;\n"
+        " add.u32 b, %3, 0;\n mov.b64 y, {b, %4};\n"
+        " setp.ne.b32 f, %8, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%7], [a], y, %5, f;\n"
+        " setp.eq.b32 f, %6, %6;\n"
+        " add.u32 a, %1, 40;\n"
+        " add.u32 b, %3, 2;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%7], [a], y, %5, f;\n"
+        " add.u32 a, %1, 48;\n"
+        " add.u32 b, %3, 4;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%7], [a], y, %5, f;\n"
+        " add.u32 a, %1, 56;\n"
+        " add.u32 b, %3, 6;\n mov.b64 y, {b, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%7], [a], y, %5, f;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%9];\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%10];\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n}"
+        ::"r"(d0), "r"(a), "r"(b0), "r"(b1), "r"(b_hi), "r"(idesc), "r"(0u), "r"(d1), "r"(acc1), "r"(bar0), "r"(bar1), "r"(bar2)
+        : "memory");
 }
-__device__ __forceinline__ void umma_ss(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n .reg .pred p;\n .reg .b64 x, y;\n setp.ne.b32 p, %6, 0;\n mov.b64 x, {%1, %2};\n mov.b64 y, {%3, %4};\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, p;\n}"
-                 ::"r"(d), "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+// Outliers: A behind a shared-memory descriptor (4096 bytes to 16 k), all into d, which the first overwrites unless `acc`.
+__device__ __forceinline__ void umma_outliers(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b0, uint32_t b1, uint32_t b_hi, uint32_t idesc,
+                                              uint32_t acc, uint32_t bar0) {
+    asm volatile(
+        "{\n .reg .pred e, f;\n .reg .b32 a, b;\n .reg .b64 x, y;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 f, %6, 0;\n"
+        " add.u32 a, %1, 0;\n"
+        " add.u32 b, %2, 0;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " setp.eq.b32 f, %6, %6;\n"
+        " add.u32 a, %1, 256;\n"
+        " add.u32 b, %2, 2;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 512;\n"
+        " add.u32 b, %2, 4;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 768;\n"
+        " add.u32 b, %2, 6;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 1024;\n"
+        " add.u32 b, %3, 0;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 1280;\n"
+        " add.u32 b, %3, 2;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 1536;\n"
+        " add.u32 b, %3, 4;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " add.u32 a, %1, 1792;\n"
+        " add.u32 b, %3, 6;\n mov.b64 y, {b, %4};\n"
+        " mov.b64 x, {a, %7};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n}"
+        ::"r"(d), "r"(a), "r"(b0), "r"(b1), "r"(b_hi), "r"(idesc), "r"(acc), "r"(a_hi), "r"(bar0)
+        : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -113,6 +187,10 @@ __device__ __forceinline__ bool wait_converged(uint32_t bar, uint32_t parity, vo
     return __all_sync(0xffffffffu, ok);
 }
 
+// Groups of unpack and scatter warps of the variant for NR batch rows (see TcShape).
+__host__ __device__ constexpr int tc_unpack_groups(int nr) { return 2; }
+__host__ __device__ constexpr int tc_scatter_groups(int nr) { return nr <= 32 ? 3 : (nr <= 64 ? 2 : 1); }
+
 struct TcParams {
     const uint8_t* wq;
     const uint16_t* scale;
@@ -124,43 +202,42 @@ struct TcParams {
     uint32_t* status;
     uint32_t* counters;
     float* partials;
-    uint32_t M, K, N, KT, NT;       // NT: column tiles of 128 H columns
-    uint32_t halves;                // such tiles to a stored tile of BN columns (1, or 2: BN = 256 and H = 1)
-    uint32_t coo_cap, general, stages;
+    uint32_t M, K, N, KT, NT;       // NT: column tiles of 128 columns
+    uint32_t halves;                // such tiles to a stored tile (1 or 2)
+    uint32_t max_tile_packets, stages;
     uint32_t split;                 // as in the streaming kernel
     uint32_t nmma;                  // batch rows of the MMAs: M rounded up to 16
     uint32_t parts;                 // BF16 parts of an outlier: 1, or 2 (FP16 values)
-    // shared-memory offsets (bytes); the first four are relative to a stage, whose X block is at 0
-    uint32_t off_w, off_sz, off_info, off_coo, stage_bytes, off_wo, off_bar;
+    // shared-memory offsets (bytes); the first two are relative to a stage, whose X block is at 0
+    uint32_t off_w, off_sz, stage_bytes, off_wo, off_bar;
 };
 
-constexpr int kWoTile = 128 * 128 * 2;      // bytes of the outlier tile of a half-step
-// outlier tiles in flight: four where a stage is small enough to leave the room
-__host__ __device__ constexpr int tc_outlier_tiles(int nr) { return nr <= 32 ? 4 : 2; }
-constexpr int kScatterKeep = 8;             // outliers of a column and half-step that are taken out one by one
+constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
+constexpr int kScatterKeep = 8;             // outliers of a column and unit that are taken out one by one
+constexpr int kScatterAhead = 8;            // slots of a column requested a unit ahead
 
-// The variant's tensor-memory columns (NAB A operands of 64 columns, NDB sets of dense accumulators, one per group, and
-// the outlier accumulators), outlier tiles (NWO) and warps: a drain warp keeps 32 batch rows of its 32
-// columns in registers; SG groups of four scatter warps take the units in turn.
+// A variant's tensor-memory columns: NAB A operands of 64 columns, NDB sets of dense accumulators, one per group, and
+// the outlier accumulators.  Its warps: four of copies and MMAs; UG groups of four unpack warps and SG groups of four
+// scatter warps, which take the units in turn (their work on a unit is a chain of latencies of 800 to 1000 clocks, so that
+// the rate comes from the groups side by side); and for each RT batch rows four drain warps.  A scatter group has TPG tiles.
 template <int NR, int GROUP>
 struct TcShape {
-    static constexpr int GPS = kBK / GROUP, SETS = NR / 32;
-    static constexpr int NDB = 2 * 64 + 2 * GPS * NR + NR <= 512 ? 2 : 1;
+    static constexpr int GPS = kBK / GROUP, RT = NR < 32 ? NR : 32, SETS = NR / RT;
+    static constexpr int NDB = 4 * 64 + 4 * GPS * NR + NR <= 512 ? 4 : (2 * 64 + 2 * GPS * NR + NR <= 512 ? 2 : 1);
     static constexpr int NAB = 4 * 64 + NDB * GPS * NR + NR <= 512 ? 4 : 2;
     static constexpr int D_BASE = NAB * 64, O_BASE = D_BASE + NDB * GPS * NR;
     static_assert(O_BASE + NR <= 512, "tensor memory");
-    static constexpr int SG = 12 + 4 * SETS + 8 <= 32 ? 2 : 1;
-    static constexpr int NWO = tc_outlier_tiles(NR);
-    static constexpr int WARPS = 12 + 4 * SETS + 4 * SG;
-    static_assert(WARPS <= 32 && NWO % SG == 0, "warps");
+    static constexpr int UG = tc_unpack_groups(NR), SG = tc_scatter_groups(NR), TPG = SG == 1 ? 2 : 1, NWO = SG * TPG;
+    static constexpr int WARPS = 4 + 4 * UG + 4 * SETS + 4 * SG;
+    static_assert(WARPS <= 32 && NWO <= 4, "warps, barriers");
 };
 
 template <int NR, int GROUP>
 __global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
 fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
-    constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, SG = S_::SG;
-    constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256, INFO_BYTES = 128;
+    constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG, SG = S_::SG;
+    constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
 
@@ -171,28 +248,26 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * S;
     const uint32_t bar_a_full = bar_empty + 8 * S;        // [4] A operand written (unpack warps)
     const uint32_t bar_a_empty = bar_a_full + 32;         // [4] the MMAs that read it are complete
-    const uint32_t bar_d_full = bar_a_empty + 32;         // [2] a half-step's dense MMAs are complete
-    const uint32_t bar_d_free = bar_d_full + 16;          // [2] its sums are read (drain warps)
-    const uint32_t bar_wo_full = bar_d_free + 16;         // [4] outlier tile written (scatter warps)
+    const uint32_t bar_d_full = bar_a_empty + 32;         // [4] a unit's dense MMAs are complete
+    const uint32_t bar_d_free = bar_d_full + 32;          // [4] its sums are read (drain warps)
+    const uint32_t bar_wo_full = bar_d_free + 32;         // [4] outlier tile written (scatter warps)
     const uint32_t bar_wo_empty = bar_wo_full + 32;       // [4] the MMAs that read it are complete
     const uint32_t bar_o_full = bar_wo_empty + 32;        // the piece's outlier sums are complete
     const uint32_t bar_o_free = bar_o_full + 8;           // and read
     const uint32_t bar_final = bar_o_free + 8;
-    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 23);
+    volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 27);
     volatile uint32_t* tmem_slot = abort_flag + 1;
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
             mbar_init(bar_full + 8 * s, 2);                                  // the two producers' expect_tx arrivals
-            mbar_init(bar_empty + 8 * s, 4 * (1 + SETS) + 4 + 2);   // unpack, drain, scatter warps, the MMAs' commits
+            mbar_init(bar_empty + 8 * s, 4 + 4 * SETS + 2);                  // unpack and drain warps, the MMAs' commits
         }
         for (uint32_t i = 0; i < 4; ++i) {
             mbar_init(bar_a_full + 8 * i, 4);
             mbar_init(bar_a_empty + 8 * i, 1);
             mbar_init(bar_wo_full + 8 * i, 4);
             mbar_init(bar_wo_empty + 8 * i, 1);
-        }
-        for (uint32_t i = 0; i < 2; ++i) {
             mbar_init(bar_d_full + 8 * i, 1);
             mbar_init(bar_d_free + 8 * i, 4 * SETS);
         }
@@ -210,7 +285,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    constexpr uint32_t tmem_base = 0;       // all 512 columns were allocated: they start at column 0
     // The grid after this one in the stream may start now (it takes SMs as this grid's CTAs leave).  The weight arrays
     // are read at once (no kernel writes them while calls are in flight); whoever reads X or writes Y or the scratch
     // waits for the grids before this one.
@@ -263,132 +338,112 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                     for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
             }
         } else if (warp == 2) {
-            // ---------------------------------------------------------------- producer of X and the outlier arrays
-            uint32_t ip_a = 0, ip_b = 0;                                   // packet ranges of the next 32 units, read 32 at a time
-            uint32_t last_bar = 0, last_ph = 0;
+            // ---------------------------------------------------------------- producer of X
+            uint32_t issued = 0;
             bool ok = true;
             const uint32_t x_half = p.nmma * 128;                          // bytes of 64 K values of every batch row
-            auto outliers = [&](const UnitIter& w) {                       // arrival with the byte count of this warp's copies
-                const uint32_t full = bar_full + 8 * w.s, st = smem_u32(smem) + w.s * p.stage_bytes;
-                uint32_t pk0 = 0, npk = 0, chunk = 0;
-                if ((w.it & 31) == 0) {
-                    const uint32_t i = w.u + lane;
-                    if (i < U) {
-                        const uint32_t c = chunk_of(i / KT, i % KT);
-                        ip_a = __ldg(p.indptr + c), ip_b = __ldg(p.indptr + c + 1);
-                    }
-                }
-                chunk = chunk_of(w.tn, w.kt);
-                pk0 = __shfl_sync(0xffffffffu, ip_a, w.it & 31);
-                npk = min(__shfl_sync(0xffffffffu, ip_b, w.it & 31) - pk0, p.coo_cap);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+                const uint32_t full = bar_full + 8 * w.s;
+                if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+                const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
                 if (elect_one()) {
-                    mbar_arrive_expect_tx(full, 2 * x_half + INFO_BYTES + npk * 16);
-                    const uint32_t half = p.halves == 2 ? (w.tn & 1) : 0;
-                    bulk_g2s(st + p.off_info, p.info + ((size_t)chunk * p.halves + half) * 32, INFO_BYTES, full);
-                    if (npk) bulk_g2s(st + p.off_coo, p.packed + pk0, npk * 16, full);
-                }
-                __syncwarp();
-                last_bar = full, last_ph = w.ph;
-            };
-            auto activations = [&](const UnitIter& w) {
-                if (elect_one()) {
-                    const uint32_t full = bar_full + 8 * w.s, st = smem_u32(smem) + w.s * p.stage_bytes;
+                    mbar_arrive_expect_tx(full, 2 * x_half);
                     tma_load_2d(st, &xmap, w.kt * kBK, 0, full);
                     tma_load_2d(st + x_half, &xmap, w.kt * kBK + 64, 0, full);
                 }
                 __syncwarp();
-            };
-            // the first pass over the ring finds every stage empty: its outlier arrays (weights) are requested before
-            // the wait for the grids before this one, its activations after
-            const uint32_t n_first = min(S, u_end - u_begin);
-            {
-                UnitIter w(u_begin, KT);
-                for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) outliers(w);
+                issued = w.it + 1;
             }
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            {
-                UnitIter w(u_begin, KT);
-                for (uint32_t i = 0; i < n_first; ++i, w.next(S, KT)) activations(w);
-                for (; w.u < u_end; w.next(S, KT)) {
-                    if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-                    outliers(w);
-                    activations(w);
-                }
+            if (!ok) {
+                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
+                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
             }
-            if (!ok && last_bar)                // gave up: let this warp's last copies land before the CTA exits
-                for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(last_bar, last_ph); ++spin) {}
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
             // (the unpack warps have waited for the unit's stage, its X block included)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
-            const uint32_t x_half = (p.nmma * 128) >> 4;
-            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-                const uint32_t ab = w.it % NAB, db = w.it % NDB;
-                const uint64_t xd = desc_sw128(smem_u32(smem) + w.s * p.stage_bytes);
-                if (w.it >= NDB && !wait_converged(bar_d_free + 8 * db, (w.it / NDB - 1) & 1, abort_flag, p.status)) break;
-                if (!wait_converged(bar_a_full + 8 * ab, (w.it / NAB) & 1, abort_flag, p.status)) break;
-                tc_fence_after();
-                if (elect_one()) {
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        umma_ts(tmem_base + S_::D_BASE + (db * GPS + ks * GPS / 8) * NR, tmem_base + ab * 64 + ks * 8,
-                                (uint32_t)xd + (ks >> 2) * x_half + (ks & 3) * 2, (uint32_t)(xd >> 32), idesc, (ks % (8 / GPS)) != 0);
-                    umma_commit(bar_d_full + 8 * db);
-                    umma_commit(bar_a_empty + 8 * ab);
-                    umma_commit(bar_empty + 8 * w.s);
+            const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
+            const uint64_t xd0 = desc_sw128(smem_u32(smem));
+            const uint32_t units = u_end - u_begin;
+            uint32_t s = 0, xd = (uint32_t)xd0;
+            bool ready = false;
+            for (uint32_t it = 0; it < units; ++it) {
+                const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1;
+                if (!ready) {
+                    if (it >= NDB && !wait_converged(bar_d_free + 8 * db, (it / NDB - 1) & 1, abort_flag, p.status)) break;
+                    if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
-                __syncwarp();
+                tc_fence_after();
+                // the next unit's barriers, tested while this one's MMAs are issued
+                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
+                                      (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
+                const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
+                umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
+                           bar_a_empty + 8 * ab, bar_empty + 8 * s);
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0;
+                ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
             __syncwarp();
         } else {
             // ---------------------------------------------------------------- outlier tensor warp
-            // (the scatter warps have waited for the unit's stage)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
-            const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048);
-            const uint32_t x_half = (p.nmma * 128) >> 4;
-            bool ok = true;
-            uint32_t piece = 0;
-            for (UnitIter w(u_begin, KT); w.u < u_end && ok; w.next(S, KT)) {
-                const bool first = w.it == 0 || w.kt == 0, last = w.u + 1 == u_end || w.kt + 1 == KT;
-                const uint32_t wb = w.it % NWO;
-                const uint64_t xd = desc_sw128(smem_u32(smem) + w.s * p.stage_bytes);
-                const uint32_t wo = (uint32_t)wo0 + wb * (kWoTile >> 4);
-                if (first && piece > 0 && !wait_converged(bar_o_free, (piece - 1) & 1, abort_flag, p.status)) break;
-                for (uint32_t part = 0; part < p.parts; ++part) {
-                    if (!wait_converged(bar_wo_full + 8 * wb, ((w.it / NWO) * p.parts + part) & 1, abort_flag, p.status)) { ok = false; break; }
+            const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048), xd0 = desc_sw128(smem_u32(smem));
+            const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4, o = tmem_base + S_::O_BASE;
+            const uint32_t units = u_end - u_begin, parts = p.parts;
+            uint32_t s = 0, ph = 0, wb = 0, wph = 0, xd = (uint32_t)xd0, acc = 0, left = KT - u_begin % KT, piece = 0;    // left: units to the end of the tile
+            bool ok = true, ready = false;
+            for (uint32_t it = 0; it < units && ok; ++it) {
+                if (!ready && !(wait_converged(bar_full + 8 * s, ph, abort_flag, p.status) &&
+                                wait_converged(bar_wo_full + 8 * wb, wph, abort_flag, p.status))) break;
+                tc_fence_after();
+                umma_outliers(o, (uint32_t)wo0 + wb * (kWoTile >> 4), (uint32_t)(wo0 >> 32), xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, acc,
+                              bar_wo_empty + 8 * wb);
+                if (parts == 2) {                          // the second part of FP16 values, in the same tile
+                    if (!wait_converged(bar_wo_full + 8 * wb, 1, abort_flag, p.status)) break;
                     tc_fence_after();
-                    if (elect_one()) {
-#pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
-                            umma_ss(tmem_base + S_::O_BASE, wo + ks * (4096 >> 4), (uint32_t)(wo0 >> 32), (uint32_t)xd + (ks >> 2) * x_half + (ks & 3) * 2,
-                                    (uint32_t)(xd >> 32), idesc, (ks > 0 || part > 0 || !first) ? 1u : 0u);
-                        umma_commit(bar_wo_empty + 8 * wb);
-                        if (part + 1 == p.parts) {
-                            if (last) umma_commit(bar_o_full);
-                            umma_commit(bar_empty + 8 * w.s);
-                        }
-                    }
-                    __syncwarp();
+                    umma_outliers(o, (uint32_t)wo0 + wb * (kWoTile >> 4), (uint32_t)(wo0 >> 32), xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, 1,
+                                  bar_wo_empty + 8 * wb);
                 }
-                if (last) ++piece;
+                if (elect_one()) umma_commit(bar_empty + 8 * s);
+                __syncwarp();
+                acc = 1;
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
+                if (++wb == NWO) wb = 0, wph ^= parts & 1;
+                // the next unit's barriers, tested while this one's MMAs run
+                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_wo_full + 8 * wb, wph);
+                if (--left == 0 || it + 1 == units) {
+                    // end of a piece: the drain warps take the sums before the next piece's overwrite them
+                    if (elect_one()) umma_commit(bar_o_full);
+                    __syncwarp();
+                    if (it + 1 < units && !wait_converged(bar_o_free, piece & 1, abort_flag, p.status)) ok = false;
+                    ++piece;
+                    left = KT, acc = 0;
+                }
+                ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);
             __syncwarp();
         }
-    } else if (warp < 12) {
+    } else if (warp < 4 + 4 * UG) {
         // -------------------------------------------------------------------- unpack warps: thread = column
-        const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % 2 == ug
+        const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % UG == ug
+        const bool in_turn = S % UG == 0;                                  // a stage always returns to the same group
         const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t col = (warp & 3) * 32 + lane;
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
             const uint32_t ab = w.it % NAB;
             const uint8_t* st = smem + w.s * p.stage_bytes;
+            // Unless a stage always returns to the same group, a group waits for the others' units too: a parity wait is
+            // only valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not
+            // advance past a unit that this group has yet to release.)
+            const bool mine = w.it % UG == ug;
+            if (!mine && in_turn) continue;
             if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
-            // The groups take alternate units.  A group waits for the others' units too: a parity wait is only
-            // valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not advance
-            // past a unit that this group has yet to release.)
-            if ((w.it & 1) != ug) continue;
+            if (!mine) continue;
             const uint4* wp = reinterpret_cast<const uint4*>(st + p.off_w) + col;
             uint4 w4[4];
 #pragma unroll
@@ -419,11 +474,11 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 mbar_arrive_relaxed(bar_empty + 8 * w.s);
             }
         }
-    } else if (warp < 12 + 4 * SETS) {
-        // -------------------------------------------------------------------- drain warps: thread = column, 32 batch rows
-        const int set = (warp - 12) >> 2, dw = warp & 3;                   // rows, strip of the unit
+    } else if (warp < 4 + 4 * UG + 4 * SETS) {
+        // -------------------------------------------------------------------- drain warps: thread = column, RT batch rows
+        const int set = (warp - 4 - 4 * UG) >> 2, dw = warp & 3;           // rows, strip of the unit
         const int col = dw * 32 + lane;
-        constexpr int RT = 32, CH = 16;                                   // rows of a thread, rows per tensor-memory load
+        constexpr int RT = S_::RT, CH = 16;                                // rows of a thread, rows per tensor-memory load
         const uint32_t r0 = set * RT;
         const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         float acc[RT];
@@ -444,6 +499,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 float sv[GPS];
 #pragma unroll
                 for (int gi = 0; gi < GPS; ++gi) sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz + gi * SZ_ROW)[col]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * w.s);       // the scales were all it needs of the stage
                 if (!wait_converged(bar_d_full + 8 * db, (w.it / NDB) & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
@@ -459,10 +516,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                         }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive_relaxed(bar_d_free + 8 * db);
-                    mbar_arrive_relaxed(bar_empty + 8 * w.s);
-                }
+                if (lane == 0) mbar_arrive_relaxed(bar_d_free + 8 * db);
             }
             if (!ok) break;
             // ---------------------------------------------------------------- end of a piece
@@ -562,7 +616,9 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         // column-slotted packet of the bucket.  The thread owns the column's row of the tile (2 bytes per k, eight k
         // to 16 bytes, those 2048 bytes apart) and knows which places it has filled: a byte each in two registers, or
         // the whole row where they are more than kScatterKeep or a tail was shared out over the warp.
-        const uint32_t sg = SG == 2 ? (uint32_t)(warp - (12 + 4 * SETS)) >> 2 : 0u;      // takes the units it with it % SG == sg
+        // The bucket descriptors and slots come from global memory straight into registers, requested two units and one unit
+        // ahead.
+        const uint32_t sg = (uint32_t)(warp - 4 - 4 * UG - 4 * SETS) >> 2;     // takes the units it with it % SG == sg
         const uint32_t strip = warp & 3, g = lane & 7, t = lane >> 3;
         uint8_t* row = smem + p.off_wo + (strip * 32 + lane) * 16;
         for (int b = sg; b < NWO; b += SG)
@@ -574,39 +630,49 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             if (part == 0) return (uint16_t)(hi >> 16);
             return (wd & 0x7f800000u) == 0x7f800000u ? (uint16_t)0 : float_to_bf16_bits(__uint_as_float(wd & kSlotValueMask) - __uint_as_float(hi));
         };
+        // a unit's bucket of this lane: its descriptor and the tile's packet range, then its checked form and first slots
+        struct Raw { uint32_t info, a, b; };
+        struct Bucket { const uint32_t* packets; uint32_t depth, tail; uint32_t wd[kScatterAhead]; };
+        const uint32_t units = u_end - u_begin;
+        auto request = [&](uint32_t it) {
+            Raw r = {0, 0, 0};
+            if (it < units) {
+                const uint32_t u = u_begin + it, tn = u / KT, c = chunk_of(tn, u - tn * KT);
+                const uint32_t half = p.halves == 2 ? (tn & 1) : 0;
+                r.info = __ldg(p.info + ((size_t)c * p.halves + half) * 32 + strip * 8 + g);
+                r.a = __ldg(p.indptr + c), r.b = __ldg(p.indptr + c + 1);
+            }
+            return r;
+        };
+        auto fetch = [&](const Raw r) {
+            Bucket k;
+            const uint32_t off = r.info & 0xffffu;
+            k.depth = (r.info >> 16) & 0xffu, k.tail = r.info >> 24;
+            k.packets = reinterpret_cast<const uint32_t*>(p.packed + r.a + off);
+            if (off + k.depth + k.tail > min(r.b - r.a, p.max_tile_packets)) {
+                // a descriptor that reaches past its tile, or past what the layout struct says a tile holds (struct and
+                // arrays out of step): report it and skip the bucket
+                asm volatile("griddepcontrol.wait;" ::: "memory");         // before the scratch is written
+                atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
+                k.depth = 0, k.tail = 0;
+            }
+#pragma unroll
+            for (uint32_t d = 0; d < kScatterAhead; ++d) k.wd[d] = d < k.depth ? __ldg(k.packets + d * 4 + t) : 0u;
+            return k;
+        };
         // filled places of the tile in turn, and of the group's other tile
         uint32_t k0 = 0, k1 = 0, cnt = 0, o_k0 = 0, o_k1 = 0, o_cnt = 0;
         bool ok = true;
-        for (UnitIter w(u_begin, KT); w.u < u_end && ok; w.next(S, KT)) {
-            const uint8_t* st = smem + w.s * p.stage_bytes;
-            if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
-            if (SG == 2 && (w.it & 1) != sg) continue;           // waited for all the same, see the unpack warps
-            const uint32_t* pk = reinterpret_cast<const uint32_t*>(st + p.off_coo);
-            const uint32_t wb = w.it % NWO;
-            const uint32_t info = reinterpret_cast<const uint32_t*>(st + p.off_info)[strip * 8 + g];
-            const uint32_t off = info & 0xffffu;
-            uint32_t depth = (info >> 16) & 0xffu, tail = info >> 24;
-            const uint32_t* pg = nullptr;
-            if (__any_sync(0xffffffffu, off + depth + tail > p.coo_cap)) {
-                // packets beyond the staged part of a large tile come from global memory; a descriptor that
-                // reaches past its tile (or, for a layer whose tiles all fit, past the staged part: layout struct
-                // and arrays out of step) is reported and skipped
-                const uint32_t c = chunk_of(w.tn, w.kt), a = __ldg(p.indptr + c), npk = __ldg(p.indptr + c + 1) - a;
-                pg = reinterpret_cast<const uint32_t*>(p.packed + a);
-                if (off + depth + tail > (p.general ? npk : p.coo_cap)) {
-                    asm volatile("griddepcontrol.wait;" ::: "memory");     // before the scratch is written
-                    atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
-                    depth = 0, tail = 0;
-                }
-            }
-            auto slot = [&](uint32_t d) { return off + d < p.coo_cap ? pk[(off + d) * 4 + t] : __ldg(pg + (off + d) * 4 + t); };
-            uint32_t wd[4];                                    // the first slots, requested before the wait below
-#pragma unroll
-            for (uint32_t d = 0; d < 4; ++d) wd[d] = d < depth ? slot(d) : 0u;
+        Bucket cur = fetch(request(sg));
+        Raw nxt = request(sg + SG);
+        for (uint32_t it = sg; it < units && ok; it += SG) {
+            const uint32_t wb = it % NWO;
+            const Bucket ahead = fetch(nxt);
+            nxt = request(it + 2 * SG);
             for (uint32_t part = 0; part < p.parts; ++part) {
                 uint8_t* tile = row + wb * kWoTile;
                 // ---- take out what the tile held; the MMAs that read it are complete
-                const uint32_t n = (w.it / NWO) * p.parts + part;
+                const uint32_t n = (it / NWO) * p.parts + part;
                 if (n > 0 && !wait_converged(bar_wo_empty + 8 * wb, (n - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                 if (cnt <= kScatterKeep) {
 #pragma unroll
@@ -619,7 +685,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 }
                 __syncwarp();
                 cnt = 0;
-                // ---- put this half-step's in
+                // ---- put this unit's in
                 auto put = [&](uint32_t v) {
                     if (v & kSlotValueMask) {                  // not padding
                         const uint32_t k = (v >> 5) & 127u;
@@ -629,15 +695,21 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                     }
                 };
 #pragma unroll
-                for (int d = 0; d < 4; ++d) put(wd[d]);
-                for (uint32_t d = 4; d < depth; ++d) put(slot(d));
-                for (uint32_t hot = __ballot_sync(0xffffffffu, tail != 0); hot;) {     // buckets with a tail: warp-uniform
+                for (int d = 0; d < 4; ++d) put(cur.wd[d]);
+                if (__any_sync(0xffffffffu, cur.depth > 4)) {
+#pragma unroll
+                    for (int d = 4; d < kScatterAhead; ++d) put(cur.wd[d]);
+                    for (uint32_t d = kScatterAhead; d < cur.depth; ++d) put(__ldg(cur.packets + d * 4 + t));
+                }
+                for (uint32_t hot = __ballot_sync(0xffffffffu, cur.tail != 0); hot;) {     // buckets with a tail: warp-uniform
                     const uint32_t b = (__ffs(hot) - 1) & 7u;      // its four lanes b, b + 8, b + 16, b + 24 agree
                     hot &= ~(0x01010101u << b);
-                    const uint32_t t_off = __shfl_sync(0xffffffffu, off + depth, b), t_cnt = __shfl_sync(0xffffffffu, tail, b);
+                    const uint32_t* tp = reinterpret_cast<const uint32_t*>(
+                        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cur.packets + cur.depth * 4), b));
+                    const uint32_t t_cnt = __shfl_sync(0xffffffffu, cur.tail, b);
                     uint8_t* base = smem + p.off_wo + wb * kWoTile + (strip * 32 + b) * 16;
                     for (uint32_t i = lane; i < 4 * t_cnt; i += 32) {
-                        const uint32_t v = t_off + i / 4 < p.coo_cap ? pk[t_off * 4 + i] : __ldg(pg + t_off * 4 + i);
+                        const uint32_t v = __ldg(tp + i);
                         if (v & kSlotValueMask)                    // a tail slot names its column
                             *reinterpret_cast<uint16_t*>(base + ((v >> kSlotColShift) & 3u) * 128 + place((v >> 5) & 127u)) = bits_of(v, part);
                     }
@@ -647,14 +719,12 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_wo_full + 8 * wb);
             }
-            if (!ok) break;
-            if (NWO / SG == 2) {
+            if (S_::TPG == 2) {
                 const uint32_t a = k0, b = k1, c = cnt;
                 k0 = o_k0, k1 = o_k1, cnt = o_cnt;
                 o_k0 = a, o_k1 = b, o_cnt = c;
             }
-            if (!ok) break;
-            if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * w.s);
+            cur = ahead;
         }
     }
 
