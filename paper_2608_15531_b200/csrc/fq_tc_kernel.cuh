@@ -213,8 +213,7 @@ struct TcParams {
 };
 
 constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
-constexpr int kScatterKeep = 8;             // outliers of a column and unit that are taken out one by one
-constexpr int kScatterAhead = 8;            // slots of a column requested a unit ahead
+constexpr int kScatterAhead = 8;            // slots of a column requested a unit ahead, and taken out one by one
 
 // A variant's tensor-memory columns: NAB A operands of 64 columns, NDB sets of dense accumulators, one per group, and
 // the outlier accumulators.  Its warps: four of copies and MMAs; UG groups of four unpack warps and SG groups of four
@@ -232,11 +231,143 @@ struct TcShape {
     static_assert(WARPS <= 32 && NWO <= 4, "warps, barriers");
 };
 
+// 16 bits to shared-memory address `addr`, unless that is 0 (predicated: no branch).
+__device__ __forceinline__ void put_u16(uint32_t addr, uint32_t v) {
+    asm volatile("{\n .reg .pred p;\n .reg .b16 h;\n setp.ne.u32 p, %0, 0;\n cvt.u16.u32 h, %1;\n @p st.shared.u16 [%0], h;\n}" ::"r"(addr), "r"(v) : "memory");
+}
+// Byte offset inside a column's row of the place of a slot's k (slot bits 5-11).
+__device__ __forceinline__ uint32_t slot_place(uint32_t v) { return ((v & 0xf00u) << 3) | ((v >> 4) & 0xeu); }
+// What a part of an outlier is: its BF16 bits, or (second part) the fraction bits that BF16 cuts off.
+__device__ __forceinline__ uint32_t slot_bits(uint32_t v, uint32_t part) {
+    if (part == 0) return v >> 16;
+    return (v & 0x7f800000u) == 0x7f800000u ? 0u : float_to_bf16_bits(__uint_as_float(v & kSlotValueMask) - __uint_as_float(v & 0xffff0000u));
+}
+
+// The scatter warps' loop (see the kernel): group sg's units of [u_begin, u_end).
+template <int NR, int GROUP, int PARTS>
+__device__ __forceinline__ void tc_scatter(const TcParams& p, uint8_t* smem, uint32_t sg, uint32_t u_begin, uint32_t u_end, uint32_t bar_wo_full,
+                                           uint32_t bar_wo_empty, volatile uint32_t* abort_flag) {
+    using S_ = TcShape<NR, GROUP>;
+    constexpr uint32_t SG = S_::SG, NWO = S_::NWO, TPG = S_::TPG;
+    const uint32_t lane = threadIdx.x & 31, strip = (threadIdx.x >> 5) & 3, g = lane & 7, t = lane >> 3, KT = p.KT;
+    const uint32_t row0 = smem_u32(smem) + p.off_wo + (strip * 32 + lane) * 16;
+    auto clear_row = [&](uint32_t row) {
+#pragma unroll 4
+        for (int i = 0; i < 16; ++i) asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(row + i * 2048), "r"(0u) : "memory");
+    };
+    for (uint32_t b = sg; b < NWO; b += SG) clear_row(row0 + b * kWoTile);
+    // a unit's bucket of this lane: its descriptor and the tile's packet range, then its checked form and first slots
+    struct Raw { uint32_t info, a, b; };
+    struct Bucket { const uint32_t* packets; uint32_t depth, tail, wd[kScatterAhead]; };
+    uint32_t u = u_begin + sg, tn = u / KT, kt = u - tn * KT;              // the next unit to request
+    auto request = [&]() {
+        Raw r = {0, 0, 0};
+        if (u < u_end) {
+            const uint32_t two = p.halves == 2, c = (tn >> two) * KT + kt;
+            r.info = __ldg(p.info + (((size_t)c << two) + (tn & two)) * 32 + strip * 8 + g);
+            r.a = __ldg(p.indptr + c), r.b = __ldg(p.indptr + c + 1);
+        }
+        u += SG;
+        for (kt += SG; kt >= KT; kt -= KT) ++tn;
+        return r;
+    };
+    auto fetch = [&](const Raw r) {
+        Bucket k;
+        const uint32_t off = r.info & 0xffffu;
+        k.depth = (r.info >> 16) & 0xffu, k.tail = r.info >> 24;
+        k.packets = reinterpret_cast<const uint32_t*>(p.packed + r.a + off) + t;
+        if (off + k.depth + k.tail > min(r.b - r.a, p.max_tile_packets)) {
+            // a descriptor that reaches past its tile, or past what the layout struct says a tile holds (struct and
+            // arrays out of step): report it and skip the bucket
+            asm volatile("griddepcontrol.wait;" ::: "memory");             // before the scratch is written
+            atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
+            k.depth = 0, k.tail = 0;
+        }
+#pragma unroll
+        for (uint32_t d = 0; d < kScatterAhead; ++d) k.wd[d] = d < k.depth ? __ldg(k.packets + d * 4) : 0u;
+        return k;
+    };
+    // filled addresses of the group's tile in turn (0: none), how many of them to look at, and of its other tile
+    uint32_t filled[TPG][kScatterAhead] = {}, deep[TPG] = {};              // deep: 0 = up to four, 1 = all, 2 = clear the row
+    Bucket cur = fetch(request());
+    Raw nxt = request();
+    uint32_t wb = sg, use = 0;                                             // tile, how often it was handed over
+    for (uint32_t it = sg; it < u_end - u_begin; it += SG) {
+        const Bucket ahead = fetch(nxt);
+        nxt = request();
+        const uint32_t row = row0 + wb * kWoTile;
+        const bool hot = __any_sync(0xffffffffu, cur.tail != 0 || cur.depth > kScatterAhead), more = __any_sync(0xffffffffu, cur.depth > 4);
+#pragma unroll
+        for (int part = 0; part < PARTS; ++part) {
+            // ---- take out what the tile held; the MMAs that read it are complete
+            const uint32_t n = use * PARTS + part;
+            if (n > 0 && !wait_converged(bar_wo_empty + 8 * wb, (n - 1) & 1, abort_flag, p.status)) return;
+            if (deep[0] < 2) {
+#pragma unroll
+                for (int d = 0; d < 4; ++d) put_u16(filled[0][d], 0);
+                if (deep[0] == 1) {
+#pragma unroll
+                    for (int d = 4; d < kScatterAhead; ++d) put_u16(filled[0][d], 0);
+                }
+            } else {
+                clear_row(row);
+            }
+            __syncwarp();
+            // ---- put this unit's in (a padding slot has value 0)
+            auto put = [&](uint32_t v) {
+                const uint32_t at = (v & kSlotValueMask) ? row + slot_place(v) : 0u;
+                put_u16(at, slot_bits(v, part));
+                return at;
+            };
+#pragma unroll
+            for (int d = 0; d < 4; ++d) filled[0][d] = put(cur.wd[d]);
+            if (more) {
+#pragma unroll
+                for (int d = 4; d < kScatterAhead; ++d) filled[0][d] = put(cur.wd[d]);
+            }
+            deep[0] = more ? 1u : 0u;
+            if (hot) {
+                deep[0] = 2;
+                for (uint32_t d = kScatterAhead; d < cur.depth; ++d) put(__ldg(cur.packets + d * 4));
+                for (uint32_t left = __ballot_sync(0xffffffffu, cur.tail != 0); left;) {     // buckets with a tail: warp-uniform
+                    const uint32_t b = (__ffs(left) - 1) & 7u;             // its four lanes b, b + 8, b + 16, b + 24 agree; t = 0 in lane b
+                    left &= ~(0x01010101u << b);
+                    const uint32_t* tp = reinterpret_cast<const uint32_t*>(
+                        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cur.packets + cur.depth * 4), b));
+                    const uint32_t words = 4 * __shfl_sync(0xffffffffu, cur.tail, b);
+                    const uint32_t base = row + ((int)b - (int)lane) * 16;
+                    for (uint32_t i = lane; i < words; i += 32) {
+                        const uint32_t v = __ldg(tp + i);                  // a tail slot names its column
+                        put_u16((v & kSlotValueMask) ? base + ((v >> kSlotColShift) & 3u) * 128 + slot_place(v) : 0u, slot_bits(v, part));
+                    }
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_wo_full + 8 * wb);
+        }
+        if (TPG == 2) {
+            wb ^= 1;                                                       // SG == 1: tiles 0 and 1 in turn
+            use += wb == 0;
+#pragma unroll
+            for (int d = 0; d < kScatterAhead; ++d) {
+                const uint32_t x = filled[0][d];
+                filled[0][d] = filled[TPG - 1][d], filled[TPG - 1][d] = x;
+            }
+            const uint32_t x = deep[0];
+            deep[0] = deep[TPG - 1], deep[TPG - 1] = x;
+        } else {
+            ++use;
+        }
+        cur = ahead;
+    }
+}
+
 template <int NR, int GROUP>
 __global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
 fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
-    constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG, SG = S_::SG;
+    constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG;
     constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -614,118 +745,13 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         // -------------------------------------------------------------------- scatter warps: thread = column
         // Column 32 strip + l of a half is column number t = l / 8 of bucket g = l % 8 of the strip: slot t of every
         // column-slotted packet of the bucket.  The thread owns the column's row of the tile (2 bytes per k, eight k
-        // to 16 bytes, those 2048 bytes apart) and knows which places it has filled: a byte each in two registers, or
-        // the whole row where they are more than kScatterKeep or a tail was shared out over the warp.
+        // to 16 bytes, those 2048 bytes apart) and keeps the addresses that it has filled, to clear them for the next unit;
+        // where they are more than kScatterAhead, or a tail was shared out over the warp, it clears the whole row.
         // The bucket descriptors and slots come from global memory straight into registers, requested two units and one unit
         // ahead.
         const uint32_t sg = (uint32_t)(warp - 4 - 4 * UG - 4 * SETS) >> 2;     // takes the units it with it % SG == sg
-        const uint32_t strip = warp & 3, g = lane & 7, t = lane >> 3;
-        uint8_t* row = smem + p.off_wo + (strip * 32 + lane) * 16;
-        for (int b = sg; b < NWO; b += SG)
-            for (int i = 0; i < 16; ++i) *reinterpret_cast<uint4*>(row + b * kWoTile + i * 2048) = make_uint4(0, 0, 0, 0);
-        auto place = [&](uint32_t k) { return (k >> 3) * 2048 + (k & 7) * 2; };
-        // what a part of an outlier is: its BF16 bits, or (second part) the fraction bits that BF16 cuts off
-        auto bits_of = [&](uint32_t wd, uint32_t part) -> uint16_t {
-            const uint32_t hi = wd & 0xffff0000u;
-            if (part == 0) return (uint16_t)(hi >> 16);
-            return (wd & 0x7f800000u) == 0x7f800000u ? (uint16_t)0 : float_to_bf16_bits(__uint_as_float(wd & kSlotValueMask) - __uint_as_float(hi));
-        };
-        // a unit's bucket of this lane: its descriptor and the tile's packet range, then its checked form and first slots
-        struct Raw { uint32_t info, a, b; };
-        struct Bucket { const uint32_t* packets; uint32_t depth, tail; uint32_t wd[kScatterAhead]; };
-        const uint32_t units = u_end - u_begin;
-        auto request = [&](uint32_t it) {
-            Raw r = {0, 0, 0};
-            if (it < units) {
-                const uint32_t u = u_begin + it, tn = u / KT, c = chunk_of(tn, u - tn * KT);
-                const uint32_t half = p.halves == 2 ? (tn & 1) : 0;
-                r.info = __ldg(p.info + ((size_t)c * p.halves + half) * 32 + strip * 8 + g);
-                r.a = __ldg(p.indptr + c), r.b = __ldg(p.indptr + c + 1);
-            }
-            return r;
-        };
-        auto fetch = [&](const Raw r) {
-            Bucket k;
-            const uint32_t off = r.info & 0xffffu;
-            k.depth = (r.info >> 16) & 0xffu, k.tail = r.info >> 24;
-            k.packets = reinterpret_cast<const uint32_t*>(p.packed + r.a + off);
-            if (off + k.depth + k.tail > min(r.b - r.a, p.max_tile_packets)) {
-                // a descriptor that reaches past its tile, or past what the layout struct says a tile holds (struct and
-                // arrays out of step): report it and skip the bucket
-                asm volatile("griddepcontrol.wait;" ::: "memory");         // before the scratch is written
-                atomicExch(p.status, (uint32_t)FQ_ERR_FORMAT);
-                k.depth = 0, k.tail = 0;
-            }
-#pragma unroll
-            for (uint32_t d = 0; d < kScatterAhead; ++d) k.wd[d] = d < k.depth ? __ldg(k.packets + d * 4 + t) : 0u;
-            return k;
-        };
-        // filled places of the tile in turn, and of the group's other tile
-        uint32_t k0 = 0, k1 = 0, cnt = 0, o_k0 = 0, o_k1 = 0, o_cnt = 0;
-        bool ok = true;
-        Bucket cur = fetch(request(sg));
-        Raw nxt = request(sg + SG);
-        for (uint32_t it = sg; it < units && ok; it += SG) {
-            const uint32_t wb = it % NWO;
-            const Bucket ahead = fetch(nxt);
-            nxt = request(it + 2 * SG);
-            for (uint32_t part = 0; part < p.parts; ++part) {
-                uint8_t* tile = row + wb * kWoTile;
-                // ---- take out what the tile held; the MMAs that read it are complete
-                const uint32_t n = (it / NWO) * p.parts + part;
-                if (n > 0 && !wait_converged(bar_wo_empty + 8 * wb, (n - 1) & 1, abort_flag, p.status)) { ok = false; break; }
-                if (cnt <= kScatterKeep) {
-#pragma unroll
-                    for (uint32_t i = 0; i < 4; ++i)
-                        if (i < cnt) *reinterpret_cast<uint16_t*>(tile + place((k0 >> (8 * i)) & 127u)) = 0;
-                    for (uint32_t i = 4; i < cnt; ++i) *reinterpret_cast<uint16_t*>(tile + place((k1 >> (8 * (i - 4))) & 127u)) = 0;
-                } else {
-#pragma unroll 4
-                    for (int i = 0; i < 16; ++i) *reinterpret_cast<uint4*>(tile + i * 2048) = make_uint4(0, 0, 0, 0);
-                }
-                __syncwarp();
-                cnt = 0;
-                // ---- put this unit's in
-                auto put = [&](uint32_t v) {
-                    if (v & kSlotValueMask) {                  // not padding
-                        const uint32_t k = (v >> 5) & 127u;
-                        *reinterpret_cast<uint16_t*>(tile + place(k)) = bits_of(v, part);
-                        k1 = (k1 << 8) | (k0 >> 24), k0 = (k0 << 8) | k;
-                        ++cnt;
-                    }
-                };
-#pragma unroll
-                for (int d = 0; d < 4; ++d) put(cur.wd[d]);
-                if (__any_sync(0xffffffffu, cur.depth > 4)) {
-#pragma unroll
-                    for (int d = 4; d < kScatterAhead; ++d) put(cur.wd[d]);
-                    for (uint32_t d = kScatterAhead; d < cur.depth; ++d) put(__ldg(cur.packets + d * 4 + t));
-                }
-                for (uint32_t hot = __ballot_sync(0xffffffffu, cur.tail != 0); hot;) {     // buckets with a tail: warp-uniform
-                    const uint32_t b = (__ffs(hot) - 1) & 7u;      // its four lanes b, b + 8, b + 16, b + 24 agree
-                    hot &= ~(0x01010101u << b);
-                    const uint32_t* tp = reinterpret_cast<const uint32_t*>(
-                        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cur.packets + cur.depth * 4), b));
-                    const uint32_t t_cnt = __shfl_sync(0xffffffffu, cur.tail, b);
-                    uint8_t* base = smem + p.off_wo + wb * kWoTile + (strip * 32 + b) * 16;
-                    for (uint32_t i = lane; i < 4 * t_cnt; i += 32) {
-                        const uint32_t v = __ldg(tp + i);
-                        if (v & kSlotValueMask)                    // a tail slot names its column
-                            *reinterpret_cast<uint16_t*>(base + ((v >> kSlotColShift) & 3u) * 128 + place((v >> 5) & 127u)) = bits_of(v, part);
-                    }
-                    if (g == b) cnt = kScatterKeep + 1;
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_wo_full + 8 * wb);
-            }
-            if (S_::TPG == 2) {
-                const uint32_t a = k0, b = k1, c = cnt;
-                k0 = o_k0, k1 = o_k1, cnt = o_cnt;
-                o_k0 = a, o_k1 = b, o_cnt = c;
-            }
-            cur = ahead;
-        }
+        if (p.parts == 1) tc_scatter<NR, GROUP, 1>(p, smem, sg, u_begin, u_end, bar_wo_full, bar_wo_empty, abort_flag);
+        else tc_scatter<NR, GROUP, 2>(p, smem, sg, u_begin, u_end, bar_wo_full, bar_wo_empty, abort_flag);
     }
 
     // ---------------------------------------------------------------------- common exit
