@@ -380,8 +380,11 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
     const uint32_t sets = std::max<uint32_t>(1, pl.nr / 32), wo_bytes = (sg == 1 ? 2 : sg) * kWoTile, sv_bytes = 4 * sets * 8 * GPS * 64;
     const uint32_t fixed = 1024 /* alignment */ + 1024 /* barriers */ + wo_bytes + sv_bytes;
-    p.stage_bytes = 256 * p.nmma;
+    p.off_w = 256 * p.nmma;
+    p.off_z = p.off_w + 8192;
+    p.stage_bytes = round_up(p.off_z + GPS * 256, 1024);
     p.stages = std::min<uint32_t>(12, (kSmemBudget - fixed) / p.stage_bytes);
+    if (p.stages >= 2u * ug) p.stages -= p.stages % ug;        // a stage then always returns to the same unpack group
     p.max_tile_packets = L->max_tile_packets;
     p.off_wo = p.stages * p.stage_bytes;
     p.off_sv = p.off_wo + wo_bytes;

@@ -178,12 +178,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
 }
-// 16 bytes of weights, read once
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
 __device__ __forceinline__ void cp_async_4(uint32_t dst_smem, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
 }
@@ -221,7 +215,8 @@ struct TcParams {
     uint32_t split;                 // as in the streaming kernel
     uint32_t nmma;                  // batch rows of the MMAs: M rounded up to 16
     uint32_t parts;                 // BF16 parts of an outlier: 1, or 2 (FP16 values)
-    uint32_t stage_bytes, off_wo, off_sv, off_bar;         // shared memory (bytes): a stage of X; outlier tiles, scales, barriers
+    // shared memory (bytes): a stage with its X block at 0, codes and zero-points; then outlier tiles, scales, barriers
+    uint32_t off_w, off_z, stage_bytes, off_wo, off_sv, off_bar;
 };
 
 constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
@@ -402,8 +397,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
-            mbar_init(bar_full + 8 * s, 1);                    // the producer's expect_tx arrival
-            mbar_init(bar_empty + 8 * s, 2);                   // the commits of the two tensor warps
+            mbar_init(bar_full + 8 * s, 2);                    // the two producers' expect_tx arrivals
+            mbar_init(bar_empty + 8 * s, 4 + 2);               // unpack warps, the commits of the two tensor warps
         }
         for (uint32_t i = 0; i < 4; ++i) {
             mbar_init(bar_a_full + 8 * i, 4);
@@ -538,41 +533,68 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             }
             if (elect_one()) umma_commit(bar_final);
             __syncwarp();
+        } else {
+            // ---------------------------------------------------------------- producer of the dense arrays
+            uint32_t issued = 0;
+            bool ok = true;
+            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+                const uint32_t full = bar_full + 8 * w.s;
+                if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+                const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, 8192 + GPS * 256);
+                    if (p.halves == 2) {
+                        const uint8_t* src = p.wq + (size_t)((w.tn >> 1) * KT + w.kt) * 16384 + (w.tn & 1) * 2048;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) bulk_g2s(st + p.off_w + j * 2048, src + j * 4096, 2048, full);
+                    } else {
+                        bulk_g2s(st + p.off_w, p.wq + (size_t)w.u * 8192, 8192, full);
+                    }
+#pragma unroll
+                    for (int gi = 0; gi < GPS; ++gi)
+                        bulk_g2s(st + p.off_z + gi * 256, p.zero + (size_t)(w.kt * GPS + gi) * p.N + (size_t)w.tn * 128, 256, full);
+                }
+                __syncwarp();
+                issued = w.it + 1;
+            }
+            if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
+                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
+                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
+            }
         }
     } else if (warp < 4 + 4 * UG) {
         // -------------------------------------------------------------------- unpack warps: thread = column
         const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % UG == ug
+        const bool in_turn = S % UG == 0;                                  // a stage always returns to the same group
         const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t col = (warp & 3) * 32 + lane, two = p.halves == 2;
-        // The codes and zero-points of the group's next unit come from global memory straight into registers, requested
-        // before the work on this one.
-        struct Codes { uint4 w[4]; uint32_t z[GPS]; };
-        uint32_t u = u_begin + ug, tn = u / KT, kt = u - tn * KT;          // the next unit to request
-        auto request = [&]() {
-            Codes c = {};
-            if (u < u_end) {
-                const uint4* src = reinterpret_cast<const uint4*>(p.wq) + (((size_t)((tn >> two) * KT + kt) << two) * 512) + (tn & two) * 128 + col;
+        const uint32_t col = (warp & 3) * 32 + lane;
+        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+            // Unless a stage always returns to the same group, a group waits for the others' units too: a parity wait is
+            // only valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not
+            // advance past a unit that this group has yet to release.)
+            const bool mine = w.it % UG == ug;
+            if (!mine && in_turn) continue;
+            const uint32_t ab = w.it % NAB;
+            const uint8_t* st = smem + w.s * p.stage_bytes;
+            if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
+            if (!mine) continue;
+            // (the A operand's barrier is tested while the codes are on their way)
+            const uint32_t seen = w.it < NAB ? 1u : mbar_test_wait(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1);
+            const uint4* wp = reinterpret_cast<const uint4*>(st + p.off_w) + col;
+            uint4 w4[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) c.w[j] = ld_stream(src + ((j * 128) << two));
-#pragma unroll
-                for (int gi = 0; gi < GPS; ++gi) c.z[gi] = __ldg(p.zero + (size_t)(kt * GPS + gi) * p.N + (size_t)tn * 128 + col);
-            }
-            u += UG;
-            for (kt += UG; kt >= KT; kt -= KT) ++tn;
-            return c;
-        };
-        Codes cur = request();
-        for (uint32_t it = ug; it < u_end - u_begin; it += UG) {
-            const Codes nxt = request();
-            const uint32_t ab = it % NAB;
+            for (int j = 0; j < 4; ++j) w4[j] = wp[j * 128];
             uint32_t nz[GPS];                                              // -(128 + z) twice
 #pragma unroll
-            for (int gi = 0; gi < GPS; ++gi) nz[gi] = 0x80008000u ^ add_bf16x2(cur.z[gi] | (cur.z[gi] << 16), 0x43004300u);
-            if (it >= NAB && !wait_converged(bar_a_empty + 8 * ab, (it / NAB - 1) & 1, abort_flag, p.status)) break;
+            for (int gi = 0; gi < GPS; ++gi) {
+                const uint32_t z = reinterpret_cast<const uint16_t*>(st + p.off_z + gi * 256)[col];
+                nz[gi] = 0x80008000u ^ add_bf16x2(z | (z << 16), 0x43004300u);
+            }
+            if (!__all_sync(0xffffffffu, seen) && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const uint32_t ww[4] = {cur.w[j].x, cur.w[j].y, cur.w[j].z, cur.w[j].w};
+                const uint32_t ww[4] = {w4[j].x, w4[j].y, w4[j].z, w4[j].w};
                 uint32_t a[16];
 #pragma unroll
                 for (int x = 0; x < 4; ++x)
@@ -583,8 +605,10 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar_a_full + 8 * ab);
-            cur = nxt;
+            if (lane == 0) {
+                mbar_arrive_relaxed(bar_a_full + 8 * ab);
+                mbar_arrive_relaxed(bar_empty + 8 * w.s);
+            }
         }
     } else if (warp < 4 + 4 * UG + 4 * SETS) {
         // -------------------------------------------------------------------- drain warps: thread = column, RT batch rows
