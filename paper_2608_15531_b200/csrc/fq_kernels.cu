@@ -378,19 +378,17 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
         }
     }
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
-    const uint32_t sets = std::max<uint32_t>(1, pl.nr / 32), wo_bytes = (sg == 1 ? 2 : sg) * kWoTile, sv_bytes = 4 * sets * 8 * GPS * 64;
-    const uint32_t fixed = 1024 /* alignment */ + 1024 /* barriers */ + wo_bytes + sv_bytes;
+    const uint32_t wo_bytes = (sg == 1 ? 2 : sg) * kWoTile, fixed = 1024 /* alignment */ + 1024 /* barriers */ + wo_bytes;
     p.off_w = 256 * p.nmma;
-    p.off_z = p.off_w + 8192;
-    p.stage_bytes = round_up(p.off_z + GPS * 256, 1024);
+    p.off_sz = p.off_w + 8192;
+    p.stage_bytes = round_up(p.off_sz + 2 * GPS * 256, 1024);
     p.stages = std::min<uint32_t>(12, (kSmemBudget - fixed) / p.stage_bytes);
     if (p.stages >= 2u * ug) p.stages -= p.stages % ug;        // a stage then always returns to the same unpack group
     p.max_tile_packets = L->max_tile_packets;
     p.off_wo = p.stages * p.stage_bytes;
-    p.off_sv = p.off_wo + wo_bytes;
-    p.off_bar = p.off_sv + sv_bytes;
+    p.off_bar = p.off_wo + wo_bytes;
     pl.smem = p.off_bar + 2048;
-    pl.threads = 32 * (4 + 4 * ug + 4 * sets + 4 * sg);        // as TcShape::WARPS
+    pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = grid;
     return FQ_OK;
 }
@@ -447,15 +445,19 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
     return warps == 32 ? pick_direct_rows<32>(rows, g, sparse) : pick_direct_rows<16>(rows, g, sparse);
 }
 
-// Which kernel serves a launch: up to 16 rows the warp-level MMA kernels, more rows the tcgen05 kernel, whose cost
-// grows slowly with them.  The latter writes outliers into a tile instead of adding them, so an encoding that names a
-// position twice (or whose origin is unknown) stays with launches of 16 rows.
+// Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 29.3 us
+// at 8 to 16 rows, 31.6 at 32), the warp-level MMA kernels' grows (26.9 us at 8 rows, 36.7 at 16), and its
+// start-up costs about 4 us more than theirs.  So it takes every launch of more than 16 rows, and launches of 9 to 16 rows
+// on layers of at least 512 units of 128 x 128 weights (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
+// 2048).  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
+// origin is unknown) stays with launches of 16 rows on the other kernels, and so does the dense half of the unfused pair.
+static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) {
+    if (!sparse || L->tilecoo_encoded != 1) return false;
 #ifdef FQ_EXPERIMENT
-static uint32_t tc_min() { return getenv("FQ_TCMIN") ? atoi(getenv("FQ_TCMIN")) : 17; }
-#else
-static uint32_t tc_min() { return 17; }
+    if (getenv("FQ_TCMIN")) return rows >= (uint32_t)atoi(getenv("FQ_TCMIN"));
 #endif
-static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) { return rows >= tc_min() && sparse && L->tilecoo_encoded == 1; }
+    return rows > 16 || (rows >= 9 && (uint64_t)(L->K / kBK) * (L->N / 128) >= 512);
+}
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
 // Scratch layout: status word and header, tile-arrival counters, FP32 partial slots (two per CTA).

@@ -117,10 +117,8 @@ __device__ __forceinline__ void umma_dense(uint32_t d0, uint32_t d1, uint32_t ac
         : "memory");
 }
 // Outliers: A behind a shared-memory descriptor (4096 bytes to 16 k), all into d, which the first overwrites unless `acc`.
-// LAST: the stage is released too.
-template <bool LAST>
 __device__ __forceinline__ void umma_outliers(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b0, uint32_t b1, uint32_t b_hi, uint32_t idesc,
-                                              uint32_t acc, uint32_t bar0, uint32_t bar1) {
+                                              uint32_t acc, uint32_t bar0) {
     asm volatile(
         "{\n .reg .pred e, f;\n .reg .b32 a, b;\n .reg .b64 x, y;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 f, %6, 0;\n"
         " add.u32 a, %1, 0;\n"
@@ -156,10 +154,8 @@ __device__ __forceinline__ void umma_outliers(uint32_t d, uint32_t a, uint32_t a
         " add.u32 b, %3, 6;\n mov.b64 y, {b, %4};\n"
         " mov.b64 x, {a, %7};\n"
         " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %5, f;\n"
-        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n"
-        " setp.ne.and.b32 e, %10, 0, e;\n"
-        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%9];\n}"
-        ::"r"(d), "r"(a), "r"(b0), "r"(b1), "r"(b_hi), "r"(idesc), "r"(acc), "r"(a_hi), "r"(bar0), "r"(bar1), "n"(LAST ? 1 : 0)
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n}"
+        ::"r"(d), "r"(a), "r"(b0), "r"(b1), "r"(b_hi), "r"(idesc), "r"(acc), "r"(a_hi), "r"(bar0)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -178,9 +174,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void cp_async_4(uint32_t dst_smem, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
-}
 __device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
     uint32_t r;
     asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
@@ -195,7 +188,7 @@ __device__ __forceinline__ bool wait_converged(uint32_t bar, uint32_t parity, vo
 }
 
 // Groups of unpack and scatter warps of the variant for NR batch rows (see TcShape).
-__host__ __device__ constexpr int tc_unpack_groups(int nr) { return nr <= 32 ? 3 : 2; }
+__host__ __device__ constexpr int tc_unpack_groups(int nr) { return nr == 16 ? 3 : 2; }
 __host__ __device__ constexpr int tc_scatter_groups(int nr) { return nr <= 32 ? 3 : (nr <= 64 ? 2 : 1); }
 
 struct TcParams {
@@ -215,8 +208,8 @@ struct TcParams {
     uint32_t split;                 // as in the streaming kernel
     uint32_t nmma;                  // batch rows of the MMAs: M rounded up to 16
     uint32_t parts;                 // BF16 parts of an outlier: 1, or 2 (FP16 values)
-    // shared memory (bytes): a stage with its X block at 0, codes and zero-points; then outlier tiles, scales, barriers
-    uint32_t off_w, off_z, stage_bytes, off_wo, off_sv, off_bar;
+    // shared-memory offsets (bytes); the first two are relative to a stage, whose X block is at 0
+    uint32_t off_w, off_sz, stage_bytes, off_wo, off_bar;
 };
 
 constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
@@ -375,6 +368,7 @@ __global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
 fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
     constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG;
+    constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
 
@@ -397,8 +391,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
-            mbar_init(bar_full + 8 * s, 2);                    // the two producers' expect_tx arrivals
-            mbar_init(bar_empty + 8 * s, 4 + 2);               // unpack warps, the commits of the two tensor warps
+            mbar_init(bar_full + 8 * s, 2);                                  // the two producers' expect_tx arrivals
+            mbar_init(bar_empty + 8 * s, 4 + 4 * SETS + 2);                  // unpack and drain warps, the MMAs' commits
         }
         for (uint32_t i = 0; i < 4; ++i) {
             mbar_init(bar_a_full + 8 * i, 4);
@@ -444,6 +438,37 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 
     if (warp < 4) {
         if (warp == 0) {
+            // ---------------------------------------------------------------- producer of the dense arrays
+            uint32_t issued = 0;
+            bool ok = true;
+            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+                const uint32_t full = bar_full + 8 * w.s;
+                if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
+                const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(full, W_BYTES + 2 * GPS * SZ_ROW);
+                    if (p.halves == 2) {
+                        const uint8_t* src = p.wq + (size_t)chunk_of(w.tn, w.kt) * 16384 + (w.tn & 1) * 2048;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) bulk_g2s(st + p.off_w + j * 2048, src + j * 4096, 2048, full);
+                    } else {
+                        bulk_g2s(st + p.off_w, p.wq + (size_t)w.u * W_BYTES, W_BYTES, full);
+                    }
+#pragma unroll
+                    for (int gi = 0; gi < GPS; ++gi) {
+                        const size_t row = (size_t)(w.kt * GPS + gi) * p.N + (size_t)w.tn * 128;
+                        bulk_g2s(st + p.off_sz + gi * SZ_ROW, p.scale + row, SZ_ROW, full);
+                        bulk_g2s(st + p.off_sz + (GPS + gi) * SZ_ROW, p.zero + row, SZ_ROW, full);
+                    }
+                }
+                __syncwarp();
+                issued = w.it + 1;
+            }
+            if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
+                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
+                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
+            }
+        } else if (warp == 2) {
             // ---------------------------------------------------------------- producer of X
             uint32_t issued = 0;
             bool ok = true;
@@ -467,33 +492,33 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             }
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
+            // (the unpack warps have waited for the unit's stage, its X block included)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
             const uint64_t xd0 = desc_sw128(smem_u32(smem));
             const uint32_t units = u_end - u_begin;
-            uint32_t s = 0, ph = 0, xd = (uint32_t)xd0;
+            uint32_t s = 0, xd = (uint32_t)xd0;
             bool ready = false;
             for (uint32_t it = 0; it < units; ++it) {
-                const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1, ns = s + 1 == S ? 0 : s + 1, nph = ns ? ph : ph ^ 1;
+                const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1;
                 if (!ready) {
-                    if (!wait_converged(bar_full + 8 * s, ph, abort_flag, p.status)) break;
                     if (it >= NDB && !wait_converged(bar_d_free + 8 * db, (it / NDB - 1) & 1, abort_flag, p.status)) break;
                     if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
                 tc_fence_after();
                 // the next unit's barriers, tested while this one's MMAs are issued
-                const uint32_t seen = mbar_test_wait(bar_full + 8 * ns, nph) & mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
+                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
                                       (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
                 const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
                 umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
                            bar_a_empty + 8 * ab, bar_empty + 8 * s);
-                xd = ns ? xd + stage : (uint32_t)xd0;
-                s = ns, ph = nph;
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0;
                 ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
             __syncwarp();
-        } else if (warp == 2) {
+        } else {
             // ---------------------------------------------------------------- outlier tensor warp
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
             const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048), xd0 = desc_sw128(smem_u32(smem));
@@ -505,22 +530,22 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 if (!ready && !(wait_converged(bar_full + 8 * s, ph, abort_flag, p.status) &&
                                 wait_converged(bar_wo_full + 8 * wb, wph, abort_flag, p.status))) break;
                 tc_fence_after();
-                const uint32_t a = (uint32_t)wo0 + wb * (kWoTile >> 4), b_empty = bar_empty + 8 * s, b_wo = bar_wo_empty + 8 * wb, b0 = xd, b1 = xd + x_half;
-                xd += stage;
-                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
-                // the next unit's barriers, tested while this one's MMAs run
-                const uint32_t nw = wb + 1 == NWO ? 0 : wb + 1, nwph = nw ? wph : wph ^ (parts & 1);
-                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_wo_full + 8 * nw, nwph);
-                if (parts == 1) {
-                    umma_outliers<true>(o, a, (uint32_t)(wo0 >> 32), b0, b1, (uint32_t)(xd0 >> 32), idesc, acc, b_wo, b_empty);
-                } else {                                   // FP16 values: a second part, in the same tile
-                    umma_outliers<false>(o, a, (uint32_t)(wo0 >> 32), b0, b1, (uint32_t)(xd0 >> 32), idesc, acc, b_wo, b_empty);
+                umma_outliers(o, (uint32_t)wo0 + wb * (kWoTile >> 4), (uint32_t)(wo0 >> 32), xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, acc,
+                              bar_wo_empty + 8 * wb);
+                if (parts == 2) {                          // the second part of FP16 values, in the same tile
                     if (!wait_converged(bar_wo_full + 8 * wb, 1, abort_flag, p.status)) break;
                     tc_fence_after();
-                    umma_outliers<true>(o, a, (uint32_t)(wo0 >> 32), b0, b1, (uint32_t)(xd0 >> 32), idesc, 1, b_wo, b_empty);
+                    umma_outliers(o, (uint32_t)wo0 + wb * (kWoTile >> 4), (uint32_t)(wo0 >> 32), xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, 1,
+                                  bar_wo_empty + 8 * wb);
                 }
+                if (elect_one()) umma_commit(bar_empty + 8 * s);
+                __syncwarp();
                 acc = 1;
-                wb = nw, wph = nwph;
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
+                if (++wb == NWO) wb = 0, wph ^= parts & 1;
+                // the next unit's barriers, tested while this one's MMAs run
+                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_wo_full + 8 * wb, wph);
                 if (--left == 0 || it + 1 == units) {
                     // end of a piece: the drain warps take the sums before the next piece's overwrite them
                     if (elect_one()) umma_commit(bar_o_full);
@@ -533,34 +558,6 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             }
             if (elect_one()) umma_commit(bar_final);
             __syncwarp();
-        } else {
-            // ---------------------------------------------------------------- producer of the dense arrays
-            uint32_t issued = 0;
-            bool ok = true;
-            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-                const uint32_t full = bar_full + 8 * w.s;
-                if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
-                const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
-                if (elect_one()) {
-                    mbar_arrive_expect_tx(full, 8192 + GPS * 256);
-                    if (p.halves == 2) {
-                        const uint8_t* src = p.wq + (size_t)((w.tn >> 1) * KT + w.kt) * 16384 + (w.tn & 1) * 2048;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) bulk_g2s(st + p.off_w + j * 2048, src + j * 4096, 2048, full);
-                    } else {
-                        bulk_g2s(st + p.off_w, p.wq + (size_t)w.u * 8192, 8192, full);
-                    }
-#pragma unroll
-                    for (int gi = 0; gi < GPS; ++gi)
-                        bulk_g2s(st + p.off_z + gi * 256, p.zero + (size_t)(w.kt * GPS + gi) * p.N + (size_t)w.tn * 128, 256, full);
-                }
-                __syncwarp();
-                issued = w.it + 1;
-            }
-            if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
-                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
-                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
-            }
         }
     } else if (warp < 4 + 4 * UG) {
         // -------------------------------------------------------------------- unpack warps: thread = column
@@ -569,17 +566,18 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t col = (warp & 3) * 32 + lane;
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+            const uint32_t ab = w.it % NAB;
+            const uint8_t* st = smem + w.s * p.stage_bytes;
             // Unless a stage always returns to the same group, a group waits for the others' units too: a parity wait is
             // only valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not
             // advance past a unit that this group has yet to release.)
             const bool mine = w.it % UG == ug;
             if (!mine && in_turn) continue;
-            const uint32_t ab = w.it % NAB;
-            const uint8_t* st = smem + w.s * p.stage_bytes;
             if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
             if (!mine) continue;
-            // (the A operand's barrier is tested while the codes are on their way)
-            const uint32_t seen = w.it < NAB ? 1u : mbar_test_wait(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1);
+            // (with 16 rows the A operand's barrier is tested while the codes load: 3 % faster there, 2 % slower at 32)
+            uint32_t seen = 0;
+            if constexpr (NR == 16) seen = w.it < NAB ? 1u : mbar_test_wait(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1);
             const uint4* wp = reinterpret_cast<const uint4*>(st + p.off_w) + col;
             uint4 w4[4];
 #pragma unroll
@@ -587,10 +585,11 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             uint32_t nz[GPS];                                              // -(128 + z) twice
 #pragma unroll
             for (int gi = 0; gi < GPS; ++gi) {
-                const uint32_t z = reinterpret_cast<const uint16_t*>(st + p.off_z + gi * 256)[col];
+                const uint32_t z = reinterpret_cast<const uint16_t*>(st + p.off_sz + (GPS + gi) * SZ_ROW)[col];
                 nz[gi] = 0x80008000u ^ add_bf16x2(z | (z << 16), 0x43004300u);
             }
-            if (!__all_sync(0xffffffffu, seen) && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
+            if (NR == 16 && __all_sync(0xffffffffu, seen)) {}
+            else if (w.it >= NAB && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
             tc_fence_after();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -621,33 +620,23 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 #pragma unroll
         for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
         bool ok = true;
-        uint32_t it = 0, tn = u_begin / KT, piece = 0;
-        // The scales of the warp's columns: a ring of its own in shared memory, filled by cp.async seven units ahead.
-        uint8_t* sv_ring = smem + p.off_sv + (warp - 4 - 4 * UG) * (8 * GPS * 64);
-        uint32_t s_u = u_begin, s_tn = tn, s_kt = u_begin - tn * KT;       // the next unit whose scales are requested
-        auto request = [&]() {
-            if (s_u < u_end && lane < 16 * GPS)
-                cp_async_4(smem_u32(sv_ring + ((s_u - u_begin) & 7) * (GPS * 64) + lane * 4),
-                           p.scale + (size_t)(s_kt * GPS + (lane >> 4)) * p.N + (size_t)s_tn * 128 + dw * 32 + 2 * (lane & 15));
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            ++s_u;
-            if (++s_kt == KT) s_kt = 0, ++s_tn;
-        };
-        for (int i = 0; i < 7; ++i) request();
+        UnitIter w(u_begin, KT);
+        uint32_t tn = u_begin / KT, piece = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // outer loop: the pieces of this CTA's range (a piece = its units of one column tile)
         for (uint32_t piece_first = u_begin; piece_first < u_end && ok; ++tn, ++piece) {
             const uint32_t piece_stop = min(u_end, (tn + 1) * KT);        // one past the piece's last unit
             piece_first = piece_stop;
-            for (; u_begin + it < piece_stop; ++it) {
-                const uint32_t db = it % NDB;
-                asm volatile("cp.async.wait_group 6;" ::: "memory");
-                __syncwarp();
+            for (; w.u < piece_stop; w.next(S, KT)) {
+                const uint32_t db = w.it % NDB;
+                const uint8_t* st = smem + w.s * p.stage_bytes;
+                if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) { ok = false; break; }
                 float sv[GPS];
 #pragma unroll
-                for (int gi = 0; gi < GPS; ++gi) sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(sv_ring + ((it & 7) * GPS + gi) * 64)[lane]);
-                request();                                 // into the slot of the unit before this one
-                if (!wait_converged(bar_d_full + 8 * db, (it / NDB) & 1, abort_flag, p.status)) { ok = false; break; }
+                for (int gi = 0; gi < GPS; ++gi) sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz + gi * SZ_ROW)[col]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * w.s);       // the scales were all it needs of the stage
+                if (!wait_converged(bar_d_full + 8 * db, (w.it / NDB) & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
                 for (int gi = 0; gi < GPS; ++gi)
@@ -756,7 +745,6 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 #pragma unroll
             for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");                   // (a giving-up warp's requests)
     } else {
         // -------------------------------------------------------------------- scatter warps: thread = column
         // Column 32 strip + l of a half is column number t = l / 8 of bucket g = l % 8 of the strip: slot t of every
