@@ -108,11 +108,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_test_wait(bar, parity)) return true;   // already complete
     return mbar_wait_slow(bar, parity, abort_flag, status);
 }
-// Warp-uniform form: every lane waits, and the warp gives up together.
+// Warp-uniform form: every lane waits, and the warp gives up together.  Every lane polls and the outcome is a vote, which
+// the compiler knows to be the same in every lane; with one lane polling and a shuffle the loops around the waits were
+// compiled as divergent (streaming kernel 5 to 7 % slower: 4096 x 28672 at one row 23.5 us, so 22.3).
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t* status) {
-    uint32_t ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag, status) ? 1u : 0u;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    const bool ok = mbar_wait(bar, parity, abort_flag, status);
+    return __all_sync(0xffffffffu, ok);
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
