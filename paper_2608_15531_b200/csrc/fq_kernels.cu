@@ -450,14 +450,15 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 // at 8 to 16 rows, 31.6 at 32), the warp-level MMA kernels' grows (26.9 us at 8 rows, 36.7 at 16), and its
 // start-up costs about 4 us more than theirs.  So it takes every launch of more than 16 rows, and launches of 9 to 16 rows
 // on layers of at least 512 units of 128 x 128 weights (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
-// 2048).  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
+// 2048).  On layers with tiles of 128 columns, where the streaming kernel has half the dense warps, it is faster from two rows
+// up (2944 x 11136: 13.2 against 14.3 us at two to five rows, 8192 x 28800 52.4 against 61.6) unless they are short
+// jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
 // origin is unknown) stays with launches of 16 rows on the other kernels, and so does the dense half of the unfused pair.
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) {
     if (!sparse || L->tilecoo_encoded != 1) return false;
-#ifdef FQ_EXPERIMENT
-    if (getenv("FQ_TCMIN")) return rows >= (uint32_t)atoi(getenv("FQ_TCMIN"));
-#endif
-    return rows > 16 || (rows >= 9 && (uint64_t)(L->K / kBK) * (L->N / 128) >= 512);
+    const uint64_t units = (uint64_t)(L->K / kBK) * (L->N / 128);
+    if (rows > 16 || (rows >= 9 && units >= 512)) return true;
+    return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows) == 0;
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
@@ -628,6 +629,9 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
                                void* workspace, size_t workspace_bytes, void* stream, bool sparse) {
     fq_status_t st = check_gemm_args(L, X, M, wq, scale, zero, indptr, info, packed, Y, workspace, sparse);
     if (st != FQ_OK) return st;
+    // a layer without outliers: up to 16 rows the kernels that have no outlier step (4096 x 14336 at 8 rows 14.5 us, without
+    // it 11.5); beyond, the tcgen05 kernel, which is still the faster one
+    const bool empty = sparse && L->tilecoo_encoded && L->max_tile_packets == 0, outliers = sparse && !empty;
     const Scratch sc = scratch_layout(L->BN, M);
     if (workspace_bytes < sc.total) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, sc.total);
     cudaLaunchAttribute attr[1];
@@ -648,7 +652,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaError_t e;
-        if (tc_serves(L, mb, sparse)) {
+        if (tc_serves(L, mb, sparse) && !(empty && mb <= 16)) {
             TcPlan pl;
             st = make_plan_tc(L, mb, pl);
             if (st != FQ_OK) return st;
@@ -683,13 +687,13 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             // per warp: rows of activations, their k-major copy, scale and zero rows, staged packets; the warps'
             // sums reuse those bytes
             cfg.dynamicSmemBytes = warps * kDirectWarpBytes;
-            DirectFn dfn = pick_direct(mb, warps, L->group, sparse);
+            DirectFn dfn = pick_direct(mb, warps, L->group, outliers);
             e = ensure_smem_attr((const void*)dfn, 32 * kDirectWarpBytes);
             if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
             e = cudaLaunchKernelEx(&cfg, dfn, p);
         } else {
             MmaPlan pl;
-            st = make_plan_mma(L, mb, sparse, pl);
+            st = make_plan_mma(L, mb, outliers, pl);
             if (st != FQ_OK) return st;
             MmaParams& p = pl.p;
             p.X = Xm; p.Y = Ym;
@@ -698,7 +702,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             p.status = (uint32_t*)workspace;
             p.counters = (uint32_t*)((uint8_t*)workspace + kWsHeaderBytes);
             p.partials = (float*)((uint8_t*)workspace + sc.off_partials);
-            MmaKernelFn fn = pick_mma_kernel(L->BN, mb, L->group, sparse, pl.ngrp, pl.general);
+            MmaKernelFn fn = pick_mma_kernel(L->BN, mb, L->group, outliers, pl.ngrp, pl.general);
             e = ensure_smem_attr((const void*)fn, (int)kSmemBudget);
             if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
             cfg.gridDim = dim3(pl.grid);

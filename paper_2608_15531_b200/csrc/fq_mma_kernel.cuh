@@ -101,7 +101,10 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
     constexpr int LDC = 8 * MO;
     extern __shared__ __align__(128) uint8_t smem[];
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // The warp number through a shuffle: the compiler then knows that it is the same in every lane, and the branches on a
+    // warp's role are not compiled as divergent (8192 x 57344 without outliers at one row 53.7 us, so 48.8; with them 67.6
+    // and 65.2).  The kernels for short jobs, with one group, were 1 to 2 % slower with it.
+    const int tid = threadIdx.x, lane = tid & 31, warp = NGRP == 2 ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5;
     const uint32_t S = p.stages;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
     const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * S;

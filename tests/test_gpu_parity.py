@@ -597,3 +597,18 @@ def test_more_than_16_rows_of_a_layer_that_names_a_position_twice():
     X = _x(3, M, K)
     Yref, Yabs = H.oracle_result(P, X)
     H.check_tolerances(H.run_fused(P, X), Yref, Yabs, K)
+
+
+@pytest.mark.parametrize("K,N,BN,density", [(4096, 2048, 256, 0.01), (4096, 4224, 128, 0.01), (8192, 2176, 128, 0.01), (2048, 6144, 256, 0.0)])
+@pytest.mark.parametrize("M", [1, 2, 8, 9, 16, 17])
+def test_layers_where_the_kernel_changes_with_the_rows(K, N, BN, density, M):
+    """Either side of the rules that choose a launch's kernel: 8/9 and 16/17 rows at 512 units of 128 x 128 weights, 1/2 rows
+    on tiles of 128 columns, and a layer without outliers."""
+    lay = synth.layer(synth.tensor_seed(12, 50 + N // 128), K, N, density=density, layout="uniform")
+    P = H.pack_layer(lay, 128, BN)
+    X = _x(lay.seed + M, M, K)
+    cols = np.unique(np.concatenate([np.arange(0, N, 61), [N - 1]])).astype(np.uint32)
+    Y = H.run_fused(P, X)
+    Yref, Yabs = H.oracle_result(P, X, cols=cols)
+    H.check_tolerances(Y[:, cols], Yref, Yabs, K)
+    assert np.array_equal(H.run_fused(P, X), Y)
