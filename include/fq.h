@@ -225,16 +225,17 @@ fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes);
  * integers, scale and zero-point applied per group in FP32), adds the tile's
  * outliers into the accumulators of their columns, and writes Y once.  Which
  * kernel serves a launch is decided from its rows and the layer's shape alone:
- *   - up to 16 rows: warp-level MMAs (128 + q as BF16).  Layers with so few
- *     32-column strips and k-steps that every CTA's job would be short get one
- *     CTA per strip, whose warps split K among themselves and read the weights
- *     straight into registers; every other layer streams (tile, k-step) units
- *     through a bulk-copy/mbarrier ring on persistent CTAs;
- *   - 17 to 128 rows: one launch of a kernel built on tcgen05.mma with BF16
- *     operands (the exact integers q - z, and the outliers as a second matrix
- *     that is zero elsewhere).  If the encoding names a position twice, or was
- *     not made by fq_encode_tilecoo (L->tilecoo_encoded), M is cut into
- *     launches of 16 rows instead.
+ *   - few rows: warp-level MMAs (128 + q as BF16), up to 16 rows per launch.
+ *     Layers with so few 32-column strips and k-steps that every CTA's job would
+ *     be short get one CTA per strip, whose warps split K among themselves and
+ *     read the weights straight into registers; every other layer streams
+ *     (tile, k-step) units through a bulk-copy/mbarrier ring on persistent CTAs;
+ *   - more than 16 rows, 9 to 16 rows on all but small layers, 2 to 8 on large
+ *     layers with 128-column tiles: one launch of a kernel built on tcgen05.mma
+ *     with BF16 operands (the exact integers q - z, and the outliers as a second
+ *     matrix that is zero elsewhere).  If the encoding names a position twice, or
+ *     was not made by fq_encode_tilecoo (L->tilecoo_encoded), M is cut into
+ *     launches of 16 rows of the kernels above instead.
  * L->kernel_hint = 1 keeps the one-CTA-per-strip kernel out (for tests).
  * X: device, M x K BF16.  M in [1, FQ_MAX_M].  Y: device, M x N BF16,
  * overwritten.  All other arrays: device copies of the host packer/encoder

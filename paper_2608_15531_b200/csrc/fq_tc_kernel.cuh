@@ -22,20 +22,23 @@
 //   warps 1, 3      tensor: per unit 8 MMAs of K = 16 with A from tensor memory (warp 1, dense) and 8 with A from shared
 //                   memory (warp 3, outliers).  Two warps, because a warp's wait on a barrier costs it about 100 clocks
 //                   even when the barrier is ready, and the MMAs of the other fill them
-//   8 unpack warps  per 32 rows one 128-bit load of a column's 32 codes, seven logic operations and four BF16 pair
+//   unpack warps    (8 or 12) per 32 rows one 128-bit load of a column's 32 codes, seven logic operations and four BF16 pair
 //                   subtractions per eight codes, tcgen05.st into a ring of A operands
 //   drain warps     thread = column, 32 batch rows (4 warps for each 32 rows): tcgen05.ld of the group's sums, one FMA per
 //                   batch row; at the end of a piece the outlier accumulator, the split-tile settlement and the BF16
 //                   store of Y
-//   4-8 scatter w.  thread = column: take the previous outliers out of the tile and put the unit's in
+//   scatter warps   (4 to 12) thread = column: take the previous outliers out of the tile and put the unit's in
 //
-// What bounds it, per unit in SM clocks (MMAs issued back to back from one warp, two commits each): 8 dense + 8
-// outlier MMAs take 430 clocks at N = 16, 490 at 32, 650 at 64, 1030 at 128 (an outlier MMA is bound by reading its 4 KB
-// of A from shared memory up to N = 64); HBM at the measured copy rate would need 425.  The kernel takes 1560 at 32 rows and
-// 2480 at 128 (8192 x 28672, 1 % of outliers: 77.2 and 122.5 us): the chain copy - unpack - MMA - drain of a stage through its
-// barriers times the stages that fit, and the scatter (68.6 us without outliers, 116 at 3 %).  It replaces a
-// kernel on the 8-bit integer tensor path whose activations took three limbs and which applied the outliers row by row,
-// 32 rows to a launch (8192 x 10240 at 32 rows 65.1 us, now 34.6; 4096 x 28672 at 128 rows 305, now 68.4).
+// What bounds it, per unit in SM clocks: HBM at the measured copy rate would need 425; 8 dense + 8 outlier MMAs issued back
+// to back with their commits take 430 at N = 16, 490 at 32, 650 at 64, 1030 at 128 (an outlier MMA is bound by reading its 4 KB
+// of A from shared memory up to N = 64).  The kernel takes 1110 at 32 rows and 2000 at 128 (8192 x 28672, 1 % of outliers: 55
+// and 98 us).  That is instruction issue and latency: 2500 warp instructions a unit fill 63 % of the issue slots (some 1000 of
+// them the unpacking, seven logic operations and four BF16 pair additions for eight codes), and every role's work on a
+// unit is a chain of barriers and memory latencies of 800 clocks and more, which the groups of warps taking units in turn
+// hide only in part.  At 128 rows the tensor pipe is half busy and the drain's FMAs come on top.  Outliers cost little:
+// 55.2 us without any at 32 rows, 58.9 at 3 %.
+// Before, launches of 17 to 32 rows ran on the 8-bit integer tensor path, activations as three limbs and outliers applied row
+// by row (8192 x 28672 at 32 rows 124.5 us; 4096 x 28672 at 128 rows, in four launches, 305, now 55).
 
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
