@@ -419,10 +419,12 @@ static fq_status_t encode_x_map(const fq_layout_t* L, const uint16_t* X, uint32_
 // direct kernel, 0 = not a short job.  The bounds are where it measured faster than the streaming kernel
 // on B200: every strip a CTA of its own on its own SM and at most two k-steps to a warp (32 warps up to 8 rows,
 // 16 warps with twice the accumulators for 9-16 rows); for a single row also up to two CTAs of 16 warps to an SM.
+// Not layers with tails, which its lanes read packet by packet from global memory (4096 x 4096 clustered at one, four, eight
+// rows 14.5, 20.7, 24.5 us, on the streaming kernel 12.5, 13.5, 15.1; 2048 x 2048 at 16 rows 69 us, 8.1 on the tcgen05 kernel).
 typedef void (*DirectFn)(const DirectParams);
-static inline uint32_t direct_warps(const fq_layout_t* L, uint32_t rows) {
+static inline uint32_t direct_warps(const fq_layout_t* L, uint32_t rows, bool outliers) {
     const int sms = sm_count_cached();
-    if (sms <= 0 || rows > 16 || L->kernel_hint == 1) return 0;
+    if (sms <= 0 || rows > 16 || L->kernel_hint == 1 || (outliers && L->max_tail_packets > 0)) return 0;
     const uint32_t strips = L->N / 32, KT = L->K / kBK;
     if (strips <= (uint32_t)sms) {
         if (rows <= 8) return KT <= 64 ? 32u : 0u;
@@ -449,7 +451,7 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 // Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 29.3 us
 // at 8 to 16 rows, 31.6 at 32), the warp-level MMA kernels' grows (26.9 us at 8 rows, 36.7 at 16), and its
 // start-up costs about 4 us more than theirs.  So it takes every launch of more than 16 rows, and launches of 9 to 16 rows
-// on layers of at least 512 units of 128 x 128 weights (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
+// on layers of at least 512 units of 128 x 128 weights, or with tails (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
 // 2048).  On layers with tiles of 128 columns, where the streaming kernel has half the dense warps, it is faster from two rows
 // up (2944 x 11136: 13.2 against 14.3 us at two to five rows, 8192 x 28800 52.4 against 61.6) unless they are short
 // jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
@@ -457,8 +459,8 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) {
     if (!sparse || L->tilecoo_encoded != 1) return false;
     const uint64_t units = (uint64_t)(L->K / kBK) * (L->N / 128);
-    if (rows > 16 || (rows >= 9 && units >= 512)) return true;
-    return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows) == 0;
+    if (rows > 16 || (rows >= 9 && (units >= 512 || L->max_tail_packets > 0))) return true;
+    return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows, true) == 0;
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
@@ -673,7 +675,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             cfg.blockDim = dim3(pl.threads);
             cfg.dynamicSmemBytes = pl.smem;
             e = cudaLaunchKernelEx(&cfg, fn, xmap, p);
-        } else if (direct_warps(L, mb)) {
+        } else if (direct_warps(L, mb, outliers)) {
             DirectParams p;
             std::memset(&p, 0, sizeof(p));
             p.X = Xm; p.Y = Ym;
@@ -681,7 +683,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             p.indptr = (const uint32_t*)indptr; p.info = (const uint32_t*)info; p.packed = (const uint4*)packed;
             p.status = (uint32_t*)workspace;
             p.M = mb; p.K = L->K; p.N = L->N; p.KT = L->K / kBK; p.BN = L->BN; p.NB = L->buckets_per_tile;
-            const uint32_t warps = direct_warps(L, mb);
+            const uint32_t warps = direct_warps(L, mb, outliers);
             cfg.gridDim = dim3(L->N / 32);
             cfg.blockDim = dim3(32 * warps);
             // per warp: rows of activations, their k-major copy, scale and zero rows, staged packets; the warps'

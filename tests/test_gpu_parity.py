@@ -612,3 +612,15 @@ def test_layers_where_the_kernel_changes_with_the_rows(K, N, BN, density, M):
     Yref, Yabs = H.oracle_result(P, X, cols=cols)
     H.check_tolerances(Y[:, cols], Yref, Yabs, K)
     assert np.array_equal(H.run_fused(P, X), Y)
+
+
+@pytest.mark.parametrize("M", [1, 4, 8, 9, 16])
+def test_small_layers_with_tails(M):
+    """A small layer whose buckets have tails (a hot column) is no short job, whatever its size."""
+    K, N = 1024, 1024
+    lay = synth.layer(synth.tensor_seed(12, 60), K, N, density=0.02, layout="clustered")
+    P = H.pack_layer(lay, 128)
+    assert P.L.max_tail_packets > 0
+    X = _x(lay.seed + M, M, K)
+    Yref, Yabs = H.oracle_result(P, X)
+    H.check_tolerances(H.run_fused(P, X), Yref, Yabs, K)
