@@ -379,15 +379,13 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
         }
     }
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
-    const uint32_t wo_bytes = (sg == 1 ? 2 : sg) * kWoTile, fixed = 1024 /* alignment */ + 1024 /* barriers */ + wo_bytes;
     p.off_w = 256 * p.nmma;
     p.off_sz = p.off_w + 8192;
-    p.stage_bytes = round_up(p.off_sz + 2 * GPS * 256, 1024);
-    p.stages = std::min<uint32_t>(12, (kSmemBudget - fixed) / p.stage_bytes);
-    if (p.stages >= 2u * ug) p.stages -= p.stages % ug;        // a stage then always returns to the same unpack group
+    p.stage_bytes = tc_stage_bytes(p.nmma, GPS);
+    p.stages = tc_stages(pl.nr, p.nmma, GPS);
     p.max_tile_packets = L->max_tile_packets;
     p.off_wo = p.stages * p.stage_bytes;
-    p.off_bar = p.off_wo + wo_bytes;
+    p.off_bar = p.off_wo + tc_wo_bytes(pl.nr);
     pl.smem = p.off_bar + 2048;
     pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = grid;

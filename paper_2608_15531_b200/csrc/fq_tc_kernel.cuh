@@ -194,6 +194,18 @@ __device__ __forceinline__ bool wait_converged(uint32_t bar, uint32_t parity, vo
 __host__ __device__ constexpr int tc_unpack_groups(int nr) { return nr == 16 ? 3 : 2; }
 __host__ __device__ constexpr int tc_scatter_groups(int nr) { return nr <= 32 ? 3 : (nr <= 64 ? 2 : 1); }
 
+// Shared memory of a launch of the variant for nr rows: its outlier tiles, and as many stages as fit beside them.  A stage holds X
+// (nmma rows of 128 BF16 values), the codes, and the scales and zero-points of gps groups.
+constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
+__host__ __device__ constexpr uint32_t tc_wo_bytes(int nr) { return (tc_scatter_groups(nr) == 1 ? 2 : tc_scatter_groups(nr)) * kWoTile; }
+__host__ __device__ constexpr uint32_t tc_stage_bytes(uint32_t nmma, int gps) { return (256 * nmma + 8192 + 2 * gps * 256 + 1023) / 1024 * 1024; }
+__host__ __device__ constexpr uint32_t tc_stages(int nr, uint32_t nmma, int gps) {
+    const uint32_t fixed = 1024 /* alignment */ + 1024 /* barriers */ + tc_wo_bytes(nr), ug = tc_unpack_groups(nr);
+    uint32_t s = (kSmemBudget - fixed) / tc_stage_bytes(nmma, gps);
+    if (s > 12) s = 12;
+    return s >= 2 * ug ? s - s % ug : s;                   // a stage then always returns to the same unpack group
+}
+
 struct TcParams {
     const uint8_t* wq;
     const uint16_t* scale;
@@ -215,7 +227,6 @@ struct TcParams {
     uint32_t off_w, off_sz, stage_bytes, off_wo, off_bar;
 };
 
-constexpr int kWoTile = 128 * 128 * 2;      // bytes of a unit's outlier tile
 constexpr int kScatterAhead = 8;            // slots of a column requested a unit ahead, and taken out one by one
 
 // A variant's tensor-memory columns: NAB A operands of 64 columns, NDB sets of dense accumulators, one per group, and
@@ -232,6 +243,17 @@ struct TcShape {
     static constexpr int UG = tc_unpack_groups(NR), SG = tc_scatter_groups(NR), TPG = SG == 1 ? 2 : 1, NWO = SG * TPG;
     static constexpr int WARPS = 4 + 4 * UG + 4 * SETS + 4 * SG;
     static_assert(WARPS <= 32 && NWO <= 4, "warps, barriers");
+    // Stages of the shortest ring that a launch of this variant gets (its MMAs have more than NR / 2 and at most NR rows).
+    static constexpr uint32_t min_stages() {
+        uint32_t least = tc_stages(NR, NR, GPS);
+        for (uint32_t n = NR / 2 + 16; n < NR; n += 16)
+            if (tc_stages(NR, n, GPS) < least) least = tc_stages(NR, n, GPS);
+        return least;
+    }
+    // With this many stages an unpack group waits for a unit's stage before its A operand, so that the codes are on the way
+    // while it waits for the operand; with fewer the other way round, which takes NAB (see the unpack warps).
+    static constexpr uint32_t kStageFirst = UG + NAB;
+    static_assert(min_stages() >= NAB && (NR == 128 || min_stages() >= kStageFirst), "stages");
 };
 
 // 16 bits to shared-memory address `addr`, unless that is 0 (predicated: no branch).
@@ -565,19 +587,21 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     } else if (warp < 4 + 4 * UG) {
         // -------------------------------------------------------------------- unpack warps: thread = column
         const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % UG == ug
-        const bool in_turn = S % UG == 0;                                  // a stage always returns to the same group
         const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t col = (warp & 3) * 32 + lane;
+        const bool stage_first = NR < 128 || S >= S_::kStageFirst;
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+            if (w.it % UG != ug) continue;
             const uint32_t ab = w.it % NAB;
             const uint8_t* st = smem + w.s * p.stage_bytes;
-            // Unless a stage always returns to the same group, a group waits for the others' units too: a parity wait is
-            // only valid for a waiter that meets every phase of the barrier.  (It cannot miss one: the ring does not
-            // advance past a unit that this group has yet to release.)
-            const bool mine = w.it % UG == ug;
-            if (!mine && in_turn) continue;
+            // A parity wait is only valid for a waiter that knows the phase before to be complete, and a group does not meet
+            // the phases of the other groups' units.  What it knows: once the A operand of unit i is read, the stages of
+            // all units up to i have been filled, since their MMAs were issued in order behind their unpacking.  So the stage's
+            // phase before, that of unit it - S, is complete if the group has waited for the operand of unit it - NAB
+            // (S >= NAB), or, with the stage's wait in front, of unit it - UG - NAB (S >= UG + NAB, see kStageFirst).  And the phase
+            // cannot be over before the group has met it: the stage is not filled again until the group has released it.
+            if (!stage_first && w.it >= NAB && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
             if (!wait_converged(bar_full + 8 * w.s, w.ph, abort_flag, p.status)) break;
-            if (!mine) continue;
             // (with 16 rows the A operand's barrier is tested while the codes load: 3 % faster there, 2 % slower at 32)
             uint32_t seen = 0;
             if constexpr (NR == 16) seen = w.it < NAB ? 1u : mbar_test_wait(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1);
@@ -591,7 +615,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 const uint32_t z = reinterpret_cast<const uint16_t*>(st + p.off_sz + (GPS + gi) * SZ_ROW)[col];
                 nz[gi] = 0x80008000u ^ add_bf16x2(z | (z << 16), 0x43004300u);
             }
-            if (NR == 16 && __all_sync(0xffffffffu, seen)) {}
+            if (!stage_first || (NR == 16 && __all_sync(0xffffffffu, seen))) {}
             else if (w.it >= NAB && !wait_converged(bar_a_empty + 8 * ab, (w.it / NAB - 1) & 1, abort_flag, p.status)) break;
             tc_fence_after();
 #pragma unroll
