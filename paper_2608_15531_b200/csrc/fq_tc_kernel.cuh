@@ -517,28 +517,32 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             }
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
-            // (the unpack warps have waited for the unit's stage, its X block included)
+            // It waits for the unit's stage itself, although the unpack warps have done so: their arrival on the A operand's
+            // barrier is relaxed and hands on the order of tensor-memory operations only, not the bytes of the X block.
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
             const uint64_t xd0 = desc_sw128(smem_u32(smem));
             const uint32_t units = u_end - u_begin;
-            uint32_t s = 0, xd = (uint32_t)xd0;
+            uint32_t s = 0, ph = 0, xd = (uint32_t)xd0;
             bool ready = false;
             for (uint32_t it = 0; it < units; ++it) {
                 const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1;
                 if (!ready) {
                     if (it >= NDB && !wait_converged(bar_d_free + 8 * db, (it / NDB - 1) & 1, abort_flag, p.status)) break;
+                    if (!wait_converged(bar_full + 8 * s, ph, abort_flag, p.status)) break;
                     if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
                 tc_fence_after();
+                const uint32_t stage_s = s;
+                const uint32_t xd_s = xd;
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
                 // the next unit's barriers, tested while this one's MMAs are issued
-                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
+                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
                                       (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
                 const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
-                umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
-                           bar_a_empty + 8 * ab, bar_empty + 8 * s);
-                xd += stage;
-                if (++s == S) s = 0, xd = (uint32_t)xd0;
+                umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd_s, xd_s + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
+                           bar_a_empty + 8 * ab, bar_empty + 8 * stage_s);
                 ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired

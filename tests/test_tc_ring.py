@@ -88,6 +88,8 @@ def run(S, UG, NAB, NDB, units, order, rng):
                 yield
             while not a_full[it % NAB].passes(it // NAB):
                 yield
+            while not full[it % S].passes(it // S):
+                yield
             mmas.append(it)
             yield
 
