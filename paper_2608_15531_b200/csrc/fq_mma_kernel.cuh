@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * s);
+            if (lane == 0) mbar_arrive(bar_empty + 8 * s);
             }
 
           }

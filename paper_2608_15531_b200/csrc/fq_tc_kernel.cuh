@@ -517,32 +517,28 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             }
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
-            // It waits for the unit's stage itself, although the unpack warps have done so: their arrival on the A operand's
-            // barrier is relaxed and hands on the order of tensor-memory operations only, not the bytes of the X block.
+            // (the unpack warps have waited for the unit's stage, X block included, and their arrival hands that on: it is a release)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
             const uint64_t xd0 = desc_sw128(smem_u32(smem));
             const uint32_t units = u_end - u_begin;
-            uint32_t s = 0, ph = 0, xd = (uint32_t)xd0;
+            uint32_t s = 0, xd = (uint32_t)xd0;
             bool ready = false;
             for (uint32_t it = 0; it < units; ++it) {
                 const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1;
                 if (!ready) {
                     if (it >= NDB && !wait_converged(bar_d_free + 8 * db, (it / NDB - 1) & 1, abort_flag, p.status)) break;
-                    if (!wait_converged(bar_full + 8 * s, ph, abort_flag, p.status)) break;
                     if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
                 tc_fence_after();
-                const uint32_t stage_s = s;
-                const uint32_t xd_s = xd;
-                xd += stage;
-                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
                 // the next unit's barriers, tested while this one's MMAs are issued
-                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
+                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
                                       (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
                 const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
-                umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd_s, xd_s + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
-                           bar_a_empty + 8 * ab, bar_empty + 8 * stage_s);
+                umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
+                           bar_a_empty + 8 * ab, bar_empty + 8 * s);
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0;
                 ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
@@ -636,8 +632,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive_relaxed(bar_a_full + 8 * ab);
-                mbar_arrive_relaxed(bar_empty + 8 * w.s);
+                mbar_arrive(bar_a_full + 8 * ab);
+                mbar_arrive(bar_empty + 8 * w.s);
             }
         }
     } else if (warp < 4 + 4 * UG + 4 * SETS) {
@@ -666,7 +662,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 #pragma unroll
                 for (int gi = 0; gi < GPS; ++gi) sv[gi] = bf16_bits_to_float(reinterpret_cast<const uint16_t*>(st + p.off_sz + gi * SZ_ROW)[col]);
                 __syncwarp();
-                if (lane == 0) mbar_arrive_relaxed(bar_empty + 8 * w.s);       // the scales were all it needs of the stage
+                if (lane == 0) mbar_arrive(bar_empty + 8 * w.s);       // the scales were all it needs of the stage
                 if (!wait_converged(bar_d_full + 8 * db, (w.it / NDB) & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
@@ -682,7 +678,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                         }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_relaxed(bar_d_free + 8 * db);
+                if (lane == 0) mbar_arrive(bar_d_free + 8 * db);
             }
             if (!ok) break;
             // ---------------------------------------------------------------- end of a piece
@@ -699,7 +695,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar_o_free);
+            if (lane == 0) mbar_arrive(bar_o_free);
             const uint32_t kt = piece_stop - 1 - tn * KT;                 // k-step of the piece's last unit
             const uint32_t u_tile0 = tn * KT;
             const uint32_t piece_k0 = max(u_tile0, u_begin) - u_tile0;

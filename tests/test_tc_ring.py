@@ -88,8 +88,7 @@ def run(S, UG, NAB, NDB, units, order, rng):
                 yield
             while not a_full[it % NAB].passes(it // NAB):
                 yield
-            while not full[it % S].passes(it // S):
-                yield
+            assert full[it % S].phase > it // S            # (waited for by the unpack group)
             mmas.append(it)
             yield
 
