@@ -212,9 +212,9 @@ __device__ __forceinline__ void spmm_add(float (&acc)[RR], uint32_t w, const uin
 }
 
 template <int RR>
-__global__ void __launch_bounds__(kSpmmThreads, 2) fq_spmm_kernel(const uint16_t* __restrict__ X, const uint32_t* __restrict__ indptr,
+__global__ void __launch_bounds__(kSpmmThreads, 2) fq_spmm_kernel(const uint16_t* X, const uint32_t* __restrict__ indptr,
                                                     const uint32_t* __restrict__ info, const uint4* __restrict__ packed,
-                                                    uint16_t* __restrict__ Y, uint32_t M, uint32_t K, uint32_t N,
+                                                    uint16_t* Y, uint32_t M, uint32_t K, uint32_t N,
                                                     uint32_t BN, uint32_t slabs) {
     extern __shared__ __align__(16) uint8_t spmm_smem[];
     const uint32_t NB = BN / 4, NS = BN / 32, KW = kSpmmThreads / 32 / NS, KT = K / kBK;
@@ -252,7 +252,8 @@ __global__ void __launch_bounds__(kSpmmThreads, 2) fq_spmm_kernel(const uint16_t
 #pragma unroll
             for (int d = 0; d < 4; ++d) w[j][d] = (uint32_t)d < depth ? __ldg(pk[j] + d * 4 + t) : 0u;
         }
-        // descriptors and packets are weights; X and Y may come from the grid before this one in the stream
+        // descriptors and packets are weights; X and Y may come from the grid before this one in the stream, so that they
+        // are not read through the read-only path
         if (c0 == kt0) asm volatile("griddepcontrol.wait;" ::: "memory");
         // the chunk's activations: a thread takes eight consecutive k of one batch row at a time
         constexpr int XU = RR == 1 ? 1 : RR * 16 * kSpmmChunk / kSpmmThreads;
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kSpmmThreads, 2) fq_spmm_kernel(const uint16_t
         for (int j = 0; j < XU; ++j) {
             const uint32_t e = tid + j * kSpmmThreads, m = e % RR, o = e / RR;
             xr[j] = make_uint4(0, 0, 0, 0);
-            if (o < 16 * nk && m < M) xr[j] = __ldg(reinterpret_cast<const uint4*>(X + (size_t)m * K + (size_t)c0 * kBK) + o);
+            if (o < 16 * nk && m < M) xr[j] = __ldcg(reinterpret_cast<const uint4*>(X + (size_t)m * K + (size_t)c0 * kBK) + o);
         }
 #pragma unroll
         for (int j = 0; j < XU; ++j) {
@@ -844,14 +845,20 @@ fq_status_t fq_unfused_spmm(const fq_layout_t* L, const void* X, uint32_t M, con
 // 118 us.  So short copies of pinned memory are copied by a kernel, and the engine keeps pageable memory, which
 // only it can read, and long copies, where its transfer rate is what counts.
 constexpr size_t kKernelCopyMax = 4u << 20;
-__global__ void __launch_bounds__(256) fq_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, uint32_t n) {
+// (the loads are coherent ones, in program order behind the wait: the kernel before may still be writing `src` when this grid starts)
+__device__ __forceinline__ uint4 load_coherent(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.relaxed.sys.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__global__ void __launch_bounds__(256) fq_copy_kernel(const uint4* src, uint4* dst, uint32_t n) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t i0 = blockIdx.x * 1024 + threadIdx.x;
     uint4 v[4];                                            // four loads in flight: a read of host memory takes over a microsecond
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-        if (i0 + 256 * j < n) v[j] = src[i0 + 256 * j];
+        if (i0 + 256 * j < n) v[j] = load_coherent(src + i0 + 256 * j);
 #pragma unroll
     for (int j = 0; j < 4; ++j)
         if (i0 + 256 * j < n) dst[i0 + 256 * j] = v[j];

@@ -181,11 +181,11 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
         const bool real = (uint32_t)m < p.M;
         const uint8_t* xrow = reinterpret_cast<const uint8_t*>(p.X) + ((size_t)m * p.K) * 2 + part * CPL * 16;
         uint4 nxt[CPL];
-        auto load = [&](uint32_t kt) {
+        auto load = [&](uint32_t kt) {                       // (X is not constant for this grid's lifetime: no read-only loads)
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 nxt[c] = make_uint4(0, 0, 0, 0);
-                if (real) nxt[c] = __ldg(reinterpret_cast<const uint4*>(xrow + (size_t)kt * 256 + c * 16));
+                if (real) nxt[c] = __ldcg(reinterpret_cast<const uint4*>(xrow + (size_t)kt * 256 + c * 16));
             }
         };
         // the unit's range of outlier packets (lane 0), read one unit ahead like the activations
