@@ -441,7 +441,13 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    constexpr uint32_t tmem_base = 0;       // all 512 columns were allocated: they start at column 0
+    // Where the allocation starts; the shuffle tells the compiler that every lane has the same.  Each role reads it for itself: kept
+    // from here on it costs the drain warps of the larger variants a register that they do not have (4096 x 28672 at
+    // 128 rows 55.0 us, so 53.9; groups of 64 63.7 and 61.0).  With 32 rows it is the other way round (8192 x 28672 with groups of 64
+    // 61.4 us kept, 66.7 read again; groups of 128 54.4 and 55.1).
+    auto tmem_base_read = [&]() { return __shfl_sync(0xffffffffu, *tmem_slot, 0); };
+    const uint32_t tmem_base_kept = NR == 32 ? tmem_base_read() : 0u;
+    auto tmem_base_of = [&]() { return NR == 32 ? tmem_base_kept : tmem_base_read(); };
     // The grid after this one in the stream may start now (it takes SMs as this grid's CTAs leave).  The weight arrays
     // are read at once (no kernel writes them while calls are in flight); whoever reads X or writes Y or the scratch
     // waits for the grids before this one.
@@ -518,7 +524,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
             // (the unpack warps have waited for the unit's stage, X block included, and their arrival hands that on: it is a release)
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24), tmem_base = tmem_base_of();
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
             const uint64_t xd0 = desc_sw128(smem_u32(smem));
             const uint32_t units = u_end - u_begin;
@@ -545,7 +551,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             __syncwarp();
         } else {
             // ---------------------------------------------------------------- outlier tensor warp
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24);
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24), tmem_base = tmem_base_of();
             const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048), xd0 = desc_sw128(smem_u32(smem));
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4, o = tmem_base + S_::O_BASE;
             const uint32_t units = u_end - u_begin, parts = p.parts;
@@ -587,7 +593,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     } else if (warp < 4 + 4 * UG) {
         // -------------------------------------------------------------------- unpack warps: thread = column
         const uint32_t ug = (warp - 4) >> 2;                               // takes the units it with it % UG == ug
-        const uint32_t t_a = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t t_a = tmem_base_of() + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t col = (warp & 3) * 32 + lane;
         const bool stage_first = NR < 128 || S >= S_::kStageFirst;
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
@@ -642,7 +648,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         const int col = dw * 32 + lane;
         constexpr int RT = S_::RT, CH = 16;                                // rows of a thread, rows per tensor-memory load
         const uint32_t r0 = set * RT;
-        const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t t_lane = tmem_base_of() + ((uint32_t)((warp & 3) * 32) << 16);
         float acc[RT];
 #pragma unroll
         for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
@@ -793,6 +799,6 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         for (uint32_t spin = 0; spin < (1u << 24) && !mbar_try_wait(bar_final, 0); ++spin) {}
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(tmem_base_of(), kTmemCols);
     }
 }
