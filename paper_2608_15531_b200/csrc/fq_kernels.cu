@@ -863,11 +863,34 @@ __global__ void __launch_bounds__(256) fq_copy_kernel(const uint4* src, uint4* d
     for (int j = 0; j < 4; ++j)
         if (i0 + 256 * j < n) dst[i0 + 256 * j] = v[j];
 }
+// Device address of `bytes` of pinned host memory, or null: not pinned, or not all of it (a kernel, unlike a copy engine's copy, would
+// read on past the end of what is pinned, and fault).
+static void* pinned_view(const void* host, size_t bytes) {
+    typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const AttributesFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult qr;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &qr) != cudaSuccess || qr != cudaDriverEntryPointSuccess) f = nullptr;
+        return (AttributesFn)f;
+    }();
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+        cudaGetLastError();                                // not an error here
+        return nullptr;
+    }
+    if (!fn || at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[2] = {&start, &size};
+    if (fn(2, what, out, (CUdeviceptr)host) != CUDA_SUCCESS) return nullptr;
+    const size_t before = (size_t)((CUdeviceptr)host - start);
+    return before <= size && bytes <= size - before ? at.devicePointer : nullptr;
+}
 // `host`: the one of the two that is host memory.
 static cudaError_t enqueue_copy(void* dst, const void* src, const void* host, size_t bytes, cudaMemcpyKind kind, cudaStream_t s) {
     if (bytes <= kKernelCopyMax && bytes % 16 == 0 && aligned(src, 16) && aligned(dst, 16)) {
-        cudaPointerAttributes at;
-        if (cudaPointerGetAttributes(&at, host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer) {
+        if (void* view = pinned_view(host, bytes)) {
             const uint32_t n = (uint32_t)(bytes / 16);
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((n + 1023) / 1024);
@@ -878,10 +901,9 @@ static cudaError_t enqueue_copy(void* dst, const void* src, const void* host, si
             pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             pdl[0].val.programmaticStreamSerializationAllowed = 1;
             cfg.attrs = pdl, cfg.numAttrs = 1;
-            return cudaLaunchKernelEx(&cfg, fq_copy_kernel, (const uint4*)(src == host ? at.devicePointer : src),
-                                      (uint4*)(dst == host ? at.devicePointer : dst), n);
+            return cudaLaunchKernelEx(&cfg, fq_copy_kernel, (const uint4*)(src == host ? view : src),
+                                      (uint4*)(dst == host ? view : dst), n);
         }
-        cudaGetLastError();                                // an unregistered pointer is not an error here
     }
     return cudaMemcpyAsync(dst, src, bytes, kind, s);
 }

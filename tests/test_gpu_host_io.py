@@ -59,3 +59,34 @@ def test_every_kind_of_host_memory(K, N, M):
         fq.fq_fused_host_io(P.L, Xh, M, x, *_weights(P), y, Yh, P.ws)
         assert np.array_equal(np.asarray(Yh).view(np.uint16), Y)
         x.zero_(), y.zero_()
+
+
+@pytest.mark.parametrize("side", ["X", "Y"])
+def test_host_memory_that_is_pinned_in_part(side):
+    """Only the first 4 KB of a buffer are registered: no kernel may copy it.  The copy engine's copy refuses it or copies it, and
+    a result that is returned is right."""
+    K, N, M = 1024, 1024, 8
+    P = H.pack_layer(synth.layer(synth.tensor_seed(13, 7), K, N, density=0.01, layout="uniform"), 128)
+    Xb = synth.activations(6, M, K)
+    Y = H.run_fused(P, Xb)
+    Xh, Yh = torch.from_numpy(Xb.view(np.int16).copy()).pin_memory(), torch.zeros((M, N), dtype=torch.int16).pin_memory()
+    pages = np.frombuffer(mmap.mmap(-1, 1 << 16), dtype=np.int16)
+    part = torch.from_numpy(pages[: M * K]).view(M, K)
+    if side == "X":
+        part.copy_(Xh)
+        Xh = part
+    else:
+        Yh = part
+    cudart = torch.cuda.cudart()
+    assert int(cudart.cudaHostRegister(part.data_ptr(), 4096, 0)) == 0
+    try:
+        x, y = torch.empty((M, K), dtype=torch.int16, device="cuda"), torch.empty((M, N), dtype=torch.int16, device="cuda")
+        try:
+            fq.fq_fused_host_io(P.L, Xh, M, x, *_weights(P), y, Yh, P.ws)
+            assert np.array_equal(Yh.numpy().view(np.uint16), Y)
+        except fq.FqError as e:
+            assert e.code == fq.FQ_ERR_CUDA and "copy of " + side in str(e)
+        torch.cuda.synchronize()
+    finally:
+        assert int(cudart.cudaHostUnregister(part.data_ptr())) == 0
+    assert np.array_equal(H.run_fused(P, Xb), Y)
