@@ -14,8 +14,24 @@
 
 namespace {
 
-// Device pointer of a contiguous CUDA tensor; None is the null pointer.
-bool device_pointer(PyObject* o, void** out) {
+// What a call of the tensor library threw (a tensor without storage, or of a kind that has no strides) as a Python error: nothing
+// may leave a C entry.
+template <class F>
+bool guarded(F&& f) {
+    try {
+        return f();
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    }
+    return false;
+}
+
+// Device pointer of a contiguous CUDA tensor; None is the null pointer.  `written`: the call writes to it, so that a
+// tensor that shares its storage until it is written gets one of its own.  `bytes` (if given): its size.
+bool device_pointer(PyObject* o, void** out, bool written = false, size_t* bytes = nullptr) {
+    if (bytes) *bytes = 0;
     if (o == Py_None) {
         *out = nullptr;
         return true;
@@ -24,26 +40,25 @@ bool device_pointer(PyObject* o, void** out) {
         PyErr_SetString(PyExc_TypeError, "expected a torch tensor");
         return false;
     }
-    const at::Tensor& t = THPVariable_Unpack(o);
-    if (!t.is_cuda() || !t.is_contiguous()) {
-        PyErr_SetString(PyExc_ValueError, "expected a contiguous CUDA tensor");
-        return false;
-    }
-    *out = const_cast<void*>(t.const_data_ptr());
-    return true;
+    return guarded([&] {
+        const at::Tensor& t = THPVariable_Unpack(o);
+        if (!t.is_cuda() || !t.is_contiguous()) {
+            PyErr_SetString(PyExc_ValueError, "expected a contiguous CUDA tensor");
+            return false;
+        }
+        *out = written ? t.mutable_data_ptr() : const_cast<void*>(t.const_data_ptr());
+        if (bytes) *bytes = t.nbytes();
+        return true;
+    });
 }
 
 // The stream's handle: the given stream object's, or the current stream of the current device.
 bool stream_handle(PyObject* o, void** out) {
-    if (o == Py_None) {
-        try {
+    if (o == Py_None)                                      // (throws where there is no usable device)
+        return guarded([&] {
             *out = c10::cuda::getCurrentCUDAStream().stream();
-        } catch (const c10::Error& e) {                    // no usable device
-            PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
-            return false;
-        }
-        return true;
-    }
+            return true;
+        });
     PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
     if (!h) return false;
     *out = PyLong_AsVoidPtr(h);
@@ -71,8 +86,6 @@ struct LayoutView {
     }
 };
 
-size_t nbytes_of(PyObject* o) { return o == Py_None ? 0 : THPVariable_Unpack(o).nbytes(); }
-
 bool take(PyObject* const* args, Py_ssize_t n, Py_ssize_t want) {
     if (n != want) PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
     return n == want;
@@ -90,8 +103,8 @@ PyObject* fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!device_pointer(a[1], &X)) return nullptr;
     for (int i = 0; i < 6; ++i)
         if (!device_pointer(a[3 + i], &w[i])) return nullptr;
-    if (!device_pointer(a[9], &Y) || !device_pointer(a[10], &ws) || !stream_handle(a[11], &stream)) return nullptr;
-    const size_t ws_bytes = nbytes_of(a[10]);
+    size_t ws_bytes;
+    if (!device_pointer(a[9], &Y, true) || !device_pointer(a[10], &ws, true, &ws_bytes) || !stream_handle(a[11], &stream)) return nullptr;
     fq_status_t st;
     Py_BEGIN_ALLOW_THREADS
     st = fq_fused_w4a16_outlier_gemm(L, X, (uint32_t)M, w[0], w[1], w[2], w[3], w[4], w[5], Y, ws, ws_bytes, stream);
@@ -108,11 +121,11 @@ PyObject* host_io(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const unsigned long M = PyLong_AsUnsignedLongMask(a[2]);
     if (PyErr_Occurred()) return nullptr;
     void *xh, *yh, *x, *w[6], *y, *ws, *stream;
-    if (!host_pointer(a[1], &xh) || !host_pointer(a[11], &yh) || !device_pointer(a[3], &x)) return nullptr;
+    if (!host_pointer(a[1], &xh) || !host_pointer(a[11], &yh) || !device_pointer(a[3], &x, true)) return nullptr;
     for (int i = 0; i < 6; ++i)
         if (!device_pointer(a[4 + i], &w[i])) return nullptr;
-    if (!device_pointer(a[10], &y) || !device_pointer(a[12], &ws) || !stream_handle(a[13], &stream)) return nullptr;
-    const size_t ws_bytes = nbytes_of(a[12]);
+    size_t ws_bytes;
+    if (!device_pointer(a[10], &y, true) || !device_pointer(a[12], &ws, true, &ws_bytes) || !stream_handle(a[13], &stream)) return nullptr;
     const auto call = a[14] == Py_True ? fq_fused_host_io : fq_fused_host_io_async;
     fq_status_t st;
     Py_BEGIN_ALLOW_THREADS

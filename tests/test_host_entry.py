@@ -1,0 +1,29 @@
+"""The entries from the host: what they do with arguments that are no good, and with values at the edge of a type.  CPU only."""
+import os
+import subprocess
+import sys
+
+from paper_2608_15531_b200 import binding as fq
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_BATCHED_TENSOR = """
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+from paper_2608_15531_b200 import binding as fq
+L = fq.fq_get_layout(128, 128, 128)
+with FakeTensorMode():
+    t = torch.empty(2, 128, dtype=torch.int16, device="cuda")
+for call in (lambda x: fq.fq_fused_w4a16_outlier_gemm(L, x, 1, t, t, t, t, t, t, t, t),
+             lambda x: fq.fq_fused_host_io_async(L, torch.empty(1), 1, x, t, t, t, t, t, t, t, torch.empty(1), t)):
+    try:
+        torch.func.vmap(lambda x: (call(x), x)[1])(t)
+    except RuntimeError as e:
+        print("refused:", "storage" in str(e))
+"""
+
+
+def test_a_tensor_without_storage_is_a_python_error():
+    """What the tensor library throws must not leave the CPython entry (the process would end)."""
+    p = subprocess.run([sys.executable, "-c", _BATCHED_TENSOR], cwd=ROOT, capture_output=True, text=True)
+    assert p.returncode == 0 and p.stdout.split("\n")[:2] == ["refused: True"] * 2, (p.returncode, p.stdout, p.stderr[-500:])
