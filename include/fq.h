@@ -95,7 +95,8 @@ typedef int32_t fq_status_t;
 #define FQ_ERR_TIMEOUT (-5)           /* a bounded device-side wait expired */
 #define FQ_ERR_FORMAT (-6)            /* Tile-COO validator: bad indptr / offset / index */
 
-#define FQ_ABI_VERSION 2u
+#define FQ_ABI_VERSION 2u             /* as fq_get_layout writes it */
+#define FQ_ABI_ENCODED 3u             /* as fq_encode_tilecoo leaves it: tilecoo_encoded tells repeated positions apart */
 #define FQ_VALUE_BF16 0u
 #define FQ_VALUE_FP16 1u
 #define FQ_MAX_M 128u
@@ -103,10 +104,10 @@ typedef int32_t fq_status_t;
 
 /* Plain data, caller-owned.  Filled by fq_get_layout(); fq_encode_tilecoo()
  * writes max_tile_packets, max_bucket_packets and max_tail_packets (the kernels
- * size their staging by the first and choose their outlier path by the third).  Pass the same
+ * size their staging by the first and choose their outlier path by the third), tilecoo_encoded and abi.  Pass the same
  * struct to every later call. */
 typedef struct fq_layout {
-    uint32_t abi;
+    uint32_t abi;              /* FQ_ABI_VERSION or FQ_ABI_ENCODED */
     uint32_t K, N;
     uint32_t group;            /* 64 or 128, along K */
     uint32_t BK;               /* 128 */
@@ -119,7 +120,10 @@ typedef struct fq_layout {
     uint32_t max_tail_packets; /* longest tail; 0 = every packet is column-slotted */
     uint32_t tilecoo_encoded;  /* 1 = the three maxima above describe the arrays in use (set by
                                   fq_encode_tilecoo); 2 = likewise, and some position holds more than one outlier (their
-                                  sum counts); 0 = unknown: the kernels assume the worst */
+                                  sum counts); 0 = unknown: the kernels assume the worst.  With 1 and abi FQ_ABI_ENCODED
+                                  every position holds one outlier at most; a layout of an earlier encoder, or one filled in
+                                  by hand, has abi FQ_ABI_VERSION and says nothing about that: such a layer is served by
+                                  the kernels that add outliers one by one */
     uint32_t kernel_hint;      /* 0 = the library chooses the kernel of a launch from its rows and the layer's
                                   shape; 1 = never the short-job kernel (one CTA per strip of 32 columns), so
                                   that tests reach the streaming kernels on small layers too */
@@ -188,7 +192,7 @@ fq_status_t fq_unpack_int4(const fq_layout_t* L, const void* wq, uint8_t* q_cano
  * fq_encode_tilecoo_sizes: element counts of the three arrays (tile_indptr in
  * uint32, bucket_info in uint32, packets in 16-byte units) and the largest
  * tile.  fq_encode_tilecoo: writes them and stores max_tile_packets,
- * max_bucket_packets and max_tail_packets in *L.
+ * max_bucket_packets, max_tail_packets, tilecoo_encoded and abi in *L.
  */
 fq_status_t fq_encode_tilecoo_sizes(const fq_layout_t* L, const uint32_t* k, const uint32_t* n,
                                     const uint16_t* val_bf16, size_t nnz, size_t* n_indptr,
@@ -234,8 +238,8 @@ fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes);
  *     layers with 128-column tiles: one launch of a kernel built on tcgen05.mma
  *     with BF16 operands (the exact integers q - z, and the outliers as a second
  *     matrix that is zero elsewhere).  If the encoding names a position twice, or
- *     was not made by fq_encode_tilecoo (L->tilecoo_encoded), M is cut into
- *     launches of 16 rows of the kernels above instead.
+ *     that is not known (L->tilecoo_encoded, L->abi), M is cut into launches of
+ *     16 rows of the kernels above instead.
  * L->kernel_hint = 1 keeps the one-CTA-per-strip kernel out (for tests).
  * X: device, M x K BF16.  M in [1, FQ_MAX_M].  Y: device, M x N BF16,
  * overwritten.  All other arrays: device copies of the host packer/encoder

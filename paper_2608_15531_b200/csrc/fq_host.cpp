@@ -645,6 +645,7 @@ fq_status_t fq_encode_tilecoo(fq_layout_t* L, const uint32_t* k, const uint32_t*
     L->max_bucket_packets = E.max_bucket_packets;
     L->max_tail_packets = E.max_tail_packets;
     L->tilecoo_encoded = E.repeated ? 2 : 1;
+    L->abi = FQ_ABI_ENCODED;
     return FQ_OK;
 }
 

@@ -19,7 +19,7 @@ inline fq_status_t fail(fq_status_t code, const char* fmt, ...) {
 }
 
 inline bool layout_ok(const fq_layout_t* L) {
-    if (!L || L->abi != FQ_ABI_VERSION) return false;
+    if (!L || (L->abi != FQ_ABI_VERSION && L->abi != FQ_ABI_ENCODED)) return false;
     if (L->BK != FQ_BK || (L->BN != 128 && L->BN != 256)) return false;
     if (L->group != 64 && L->group != 128) return false;
     if (L->K == 0 || L->N == 0 || L->K % FQ_BK != 0 || L->N % L->BN != 0) return false;

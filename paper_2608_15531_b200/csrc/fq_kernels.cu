@@ -453,7 +453,7 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 // jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
 // origin is unknown) stays with launches of 16 rows on the other kernels, and so does the dense half of the unfused pair.
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) {
-    if (!sparse || L->tilecoo_encoded != 1) return false;
+    if (!sparse || L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
     const uint64_t units = (uint64_t)(L->K / kBK) * (L->N / 128);
     if (rows > 16 || (rows >= 9 && (units >= 512 || L->max_tail_packets > 0))) return true;
     return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows, true) == 0;

@@ -1,0 +1,31 @@
+"""Layouts that say little of their arrays, or what is not so: through every kernel that serves them.  Needs a B200."""
+import numpy as np
+import pytest
+
+from paper_2608_15531_b200 import binding as fq
+from paper_2608_15531_b200 import synth
+
+import harness as H
+
+pytestmark = pytest.mark.gpu
+
+
+def _repeated_layer(seed, K, N, g, density=0.01):
+    lay = synth.layer(synth.tensor_seed(14, seed), K, N, density=density, layout="uniform")
+    lay.coo_k, lay.coo_n, lay.coo_v = (np.concatenate([a, a[:50]]) for a in (lay.coo_k, lay.coo_n, lay.coo_v))
+    return H.pack_layer(lay, g)
+
+
+@pytest.mark.parametrize("M", [9, 16, 24, 40, 128])
+def test_a_saved_layout_that_says_nothing_of_repeats(M):
+    """A layout struct as encoders wrote it before repeated positions were told apart (the three maxima and tilecoo_encoded = 1,
+    whether positions repeat or not), saved and loaded again: the sum of the outliers of a position counts."""
+    K, N = 4096, 2048
+    P = _repeated_layer(1, K, N, 128)
+    assert P.L.tilecoo_encoded == 2
+    P.L.abi, P.L.tilecoo_encoded = 2, 1
+    P.L = fq.Layout.from_buffer_copy(bytes(P.L))
+    X = synth.activations(3, M, K)
+    cols = np.unique(P.layer.coo_n[-50:])
+    Yref, Yabs = H.oracle_result(P, X, cols=cols)
+    H.check_tolerances(H.run_fused(P, X)[:, cols], Yref, Yabs, K)
