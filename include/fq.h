@@ -220,7 +220,8 @@ fq_status_t fq_validate_tilecoo(const fq_layout_t* L, const uint32_t* tile_indpt
 /* Bytes of caller-allocated device scratch for calls with this layout and M.
  * The scratch must be zeroed once before its first use; every completed call
  * leaves it ready for the next one on the same stream.  Calls that may overlap
- * on the GPU need distinct scratch. */
+ * on the GPU need distinct scratch.  A call accepts less, down to the bytes for
+ * M = 32 (groups of 64: M = 16), and then takes several launches. */
 fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes);
 
 /*
@@ -275,7 +276,8 @@ fq_status_t fq_fused_w4a16_outlier_gemm(const fq_layout_t* L, const void* X, uin
  * Instead of a caller-provided workspace, the kernel uses an array that is part
  * of the library image: FQ_STATIC_SCRATCH_BYTES of device memory on every GPU
  * that loads the library, held until the process exits.  That fixes the limit:
- * calls whose fq_workspace_bytes() exceeds it (M > FQ_STATIC_SCRATCH_MAX_M) are
+ * calls whose fq_workspace_bytes() exceeds it (M > FQ_STATIC_SCRATCH_MAX_M) are,
+ * with groups of 128 (with groups of 64 every M fits, in several launches),
  * refused with FQ_ERR_BUFFER_TOO_SMALL and nothing is launched.  The function calls no cudaMalloc / cudaFree and no allocating
  * library routine; per call it enqueues one small memset (status word and tile
  * counters, which must start at zero) and the kernel.

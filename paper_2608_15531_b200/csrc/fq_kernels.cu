@@ -474,6 +474,17 @@ static Scratch scratch_layout(uint32_t BN, uint32_t rows) {
     return sc;
 }
 
+// The rows of the largest launch that `bytes` of scratch are enough for; 0: too few for this M.  fq_workspace_bytes states what one
+// launch of all rows needs; with less, a larger M takes launches of 64, 32 or 16 rows.  The least that is accepted
+// is the scratch of 32 rows (groups of 128) or 16 (groups of 64), or of M if that is fewer.
+static uint32_t rows_for_scratch(const fq_layout_t* L, uint32_t M, size_t bytes) {
+    const uint32_t least = std::min<uint32_t>(M, L->group == 64 ? 16 : 32);
+    if (bytes < scratch_layout(L->BN, least).total) return 0;
+    for (uint32_t rows : {M, 64u, 32u})
+        if (rows <= M && bytes >= scratch_layout(L->BN, rows).total) return rows;
+    return least;
+}
+
 struct MmaPlan {
     MmaParams p;
     uint32_t threads, smem, grid;
@@ -631,7 +642,8 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
     // it 11.5); beyond, the tcgen05 kernel, which is still the faster one
     const bool empty = sparse && L->tilecoo_encoded && L->max_tile_packets == 0, outliers = sparse && !empty;
     const Scratch sc = scratch_layout(L->BN, M);
-    if (workspace_bytes < sc.total) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, sc.total);
+    const uint32_t most_rows = rows_for_scratch(L, M, workspace_bytes);
+    if (!most_rows) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, sc.total);
     cudaLaunchAttribute attr[1];
     std::memset(attr, 0, sizeof(attr));
     // Programmatic dependent launch: a grid may become resident while the kernel before it in the stream
@@ -641,7 +653,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     for (uint32_t m0 = 0; m0 < M;) {
-        const uint32_t mb = rows_per_launch(L, M - m0, sparse);
+        const uint32_t mb = rows_per_launch(L, std::min(M - m0, most_rows), sparse);
         const uint16_t* Xm = (const uint16_t*)X + (size_t)m0 * L->K;
         uint16_t* Ym = (uint16_t*)Y + (size_t)m0 * L->N;
         cudaLaunchConfig_t cfg;
@@ -791,7 +803,7 @@ fq_status_t fq_fused_w4a16_outlier_gemm_noalloc(const fq_layout_t* L, const void
     fq_status_t st = check_gemm_args(L, X, M, wq, scale, zero, tile_indptr, bucket_info, packed_outliers, Y, (void*)256, true);
     if (st != FQ_OK) return st;
     const size_t need = scratch_layout(L->BN, M).total;
-    if (need > (size_t)FQ_STATIC_SCRATCH_BYTES)
+    if (need > (size_t)FQ_STATIC_SCRATCH_BYTES && (L->group != 64 || !rows_for_scratch(L, M, FQ_STATIC_SCRATCH_BYTES)))
         return fail(FQ_ERR_BUFFER_TOO_SMALL,
                     "this call needs %zu bytes of scratch but the built-in scratch holds %zu (M <= %u always fits); "
                     "use fq_fused_w4a16_outlier_gemm with caller-allocated scratch",
