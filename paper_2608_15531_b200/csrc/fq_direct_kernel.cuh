@@ -319,4 +319,5 @@ __global__ void __launch_bounds__(32 * WARPS, (MO == 1 && WARPS == 16) ? 2 : 1) 
         }
         if (m < p.M) p.Y[(size_t)m * p.N + (size_t)strip * 32 + g + 16 * cg + 8 * h] = float_to_bf16_bits(sum);
     }
+    if (!SPARSE && blockIdx.x == 0 && warp == 0) report_packets(p.indptr, p.N / BN * KT, p.status);
 }

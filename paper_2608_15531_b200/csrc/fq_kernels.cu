@@ -171,6 +171,14 @@ struct UnitIter {
     }
 };
 
+// A layer whose layout struct knows of no outliers is served without an outlier step.  If its arrays hold some all the same
+// (struct and arrays out of step), a warp of the first CTA reports it.  `indptr` is null where there is no sparse part at all.
+__device__ __forceinline__ void report_packets(const uint32_t* indptr, uint32_t tiles, uint32_t* status) {
+    if (!indptr || __ldg(indptr + tiles) == 0) return;
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // before the scratch is written
+    if ((threadIdx.x & 31) == 0) atomicExch(status, (uint32_t)FQ_ERR_FORMAT);
+}
+
 #include "fq_tc_kernel.cuh"
 #include "fq_mma_kernel.cuh"
 #include "fq_direct_kernel.cuh"

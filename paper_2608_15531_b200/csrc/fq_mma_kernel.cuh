@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
                 for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
         }
+        if (!SPARSE && blockIdx.x == 0) report_packets(p.indptr, p.NT * KT, p.status);
     } else if (warp < DW0) {
         // ------------------------------------------------------------------ activation warps
         const uint32_t aw = warp - 1;

@@ -29,3 +29,24 @@ def test_a_saved_layout_that_says_nothing_of_repeats(M):
     cols = np.unique(P.layer.coo_n[-50:])
     Yref, Yabs = H.oracle_result(P, X, cols=cols)
     H.check_tolerances(H.run_fused(P, X)[:, cols], Yref, Yabs, K)
+
+
+@pytest.mark.parametrize("K,N", [(1024, 768), (2048, 6144)])
+@pytest.mark.parametrize("M", [1, 8, 16, 17])
+@pytest.mark.parametrize("streaming_only", [False, True])
+def test_a_layout_without_outliers_on_arrays_that_have_some(K, N, M, streaming_only):
+    """The struct of a layer without outliers with the arrays of one that has some: reported, by every kernel, as the
+    descriptors that reach past their tile are; the same struct with its own (empty) arrays is not."""
+    P = H.pack_layer(synth.layer(synth.tensor_seed(14, 5), K, N, density=0.03, layout="uniform"), 128)
+    E = H.pack_layer(synth.layer(synth.tensor_seed(14, 6), K, N, density=0.0), 128)
+    assert E.L.max_tile_packets == 0 and E.L.tilecoo_encoded == 1
+    X = synth.activations(4, M, K)
+    H.run_fused(E, X, streaming_only=streaming_only)
+    mine, E.d = E.d, P.d
+    with pytest.raises(fq.FqError) as e:
+        H.run_fused(E, X, streaming_only=streaming_only)
+    assert e.value.code == fq.FQ_ERR_FORMAT
+    E.d = mine
+    cols = np.arange(0, N, 37, dtype=np.uint32)
+    Yref, Yabs = H.oracle_result(E, X, cols=cols)
+    H.check_tolerances(H.run_fused(E, X, streaming_only=streaming_only)[:, cols], Yref, Yabs, K)
