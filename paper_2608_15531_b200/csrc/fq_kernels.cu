@@ -458,15 +458,18 @@ static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool spar
 // on layers of at least 512 units of 128 x 128 weights, or with tails (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
 // 2048).  On layers with tiles of 128 columns, where the streaming kernel has half the dense warps, it is faster from two rows
 // up (2944 x 11136: 13.2 against 14.3 us at two to five rows, 8192 x 28800 52.4 against 61.6) unless they are short
-// jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or whose
-// origin is unknown) stays with launches of 16 rows on the other kernels, and so does the dense half of the unfused pair.
-static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool sparse) {
-    if (!sparse || L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
+// jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or may do so) stays
+// with launches of 16 rows on the other kernels.  Without outliers (the layer has none, or the call is the dense half of the
+// unfused pair) it takes launches of more than 16 rows, and the others, which have variants without the outlier step,
+// those of up to 16 (4096 x 14336 at 8 rows 14.5 us with the step, 11.5 without).
+static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers) {
+    if (!outliers) return rows > 16;
+    if (L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
     const uint64_t units = (uint64_t)(L->K / kBK) * (L->N / 128);
     if (rows > 16 || (rows >= 9 && (units >= 512 || L->max_tail_packets > 0))) return true;
     return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows, true) == 0;
 }
-static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool sparse) { return tc_serves(L, rows_left, sparse) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
+static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool outliers) { return tc_serves(L, rows_left, outliers) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
 // Scratch layout: status word and header, tile-arrival counters, FP32 partial slots (two per CTA).
 struct Scratch {
@@ -646,9 +649,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
                                void* workspace, size_t workspace_bytes, void* stream, bool sparse) {
     fq_status_t st = check_gemm_args(L, X, M, wq, scale, zero, indptr, info, packed, Y, workspace, sparse);
     if (st != FQ_OK) return st;
-    // a layer without outliers: up to 16 rows the kernels that have no outlier step (4096 x 14336 at 8 rows 14.5 us, without
-    // it 11.5); beyond, the tcgen05 kernel, which is still the faster one
-    const bool empty = sparse && L->tilecoo_encoded && L->max_tile_packets == 0, outliers = sparse && !empty;
+    const bool outliers = sparse && !(L->tilecoo_encoded && L->max_tile_packets == 0);
     const Scratch sc = scratch_layout(L->BN, M);
     const uint32_t most_rows = rows_for_scratch(L, M, workspace_bytes);
     if (!most_rows) return fail(FQ_ERR_BUFFER_TOO_SMALL, "workspace holds %zu bytes, %zu needed", workspace_bytes, sc.total);
@@ -661,7 +662,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     for (uint32_t m0 = 0; m0 < M;) {
-        const uint32_t mb = rows_per_launch(L, std::min(M - m0, most_rows), sparse);
+        const uint32_t mb = rows_per_launch(L, std::min(M - m0, most_rows), outliers);
         const uint16_t* Xm = (const uint16_t*)X + (size_t)m0 * L->K;
         uint16_t* Ym = (uint16_t*)Y + (size_t)m0 * L->N;
         cudaLaunchConfig_t cfg;
@@ -670,7 +671,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaError_t e;
-        if (tc_serves(L, mb, sparse) && !(empty && mb <= 16)) {
+        if (tc_serves(L, mb, outliers)) {
             TcPlan pl;
             st = make_plan_tc(L, mb, pl);
             if (st != FQ_OK) return st;

@@ -287,7 +287,7 @@ __device__ __forceinline__ void tc_scatter(const TcParams& p, uint8_t* smem, uin
     uint32_t u = u_begin + sg, tn = u / KT, kt = u - tn * KT;              // the next unit to request
     auto request = [&]() {
         Raw r = {0, 0, 0};
-        if (u < u_end) {
+        if (p.info && u < u_end) {                         // (no descriptors: the dense half of the unfused pair)
             const uint32_t two = p.halves == 2, c = (tn >> two) * KT + kt;
             r.info = __ldg(p.info + (((size_t)c << two) + (tn & two)) * 32 + strip * 8 + g);
             r.a = __ldg(p.indptr + c), r.b = __ldg(p.indptr + c + 1);

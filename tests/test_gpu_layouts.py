@@ -10,6 +10,21 @@ import harness as H
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("K,N,g,BN", [(2944, 1408, 128, 128), (1024, 1024, 64, 256)])
+@pytest.mark.parametrize("M", [16, 17, 48, 128])
+def test_the_dense_half_is_the_fused_kernel_without_outliers(K, N, g, BN, M):
+    """fq_unfused_gemm on a layer with outliers (no sparse array is given), against the oracle's dense half; and bit for bit the fused
+    call on the same codes without outliers."""
+    P = H.pack_layer(synth.layer(synth.tensor_seed(14, 9), K, N, density=0.01, layout="mixed"), g, BN)
+    X = synth.activations(2, M, K)
+    Y = H.run_unfused(P, X, with_spmm=False)
+    Yref, Yabs = H.oracle_result(P, X, dense_only=True)
+    H.check_tolerances(Y, Yref, Yabs, K)
+    E = H.pack_layer(synth.layer(synth.tensor_seed(14, 9), K, N, density=0.0), g, BN)
+    E.d |= {k: P.d[k] for k in ("wq", "scale", "zero")}
+    assert np.array_equal(H.run_fused(E, X), Y)
+
+
 def _repeated_layer(seed, K, N, g, density=0.01):
     lay = synth.layer(synth.tensor_seed(14, seed), K, N, density=density, layout="uniform")
     lay.coo_k, lay.coo_n, lay.coo_v = (np.concatenate([a, a[:50]]) for a in (lay.coo_k, lay.coo_n, lay.coo_v))
