@@ -176,7 +176,8 @@ def fq_encode_tilecoo_sizes(L: Layout, k, n, val):
 def fq_encode_tilecoo(L: Layout, k, n, val):
     """Returns (tile_indptr uint32, bucket_info uint32, packed uint8[n_packets, 16]); sets L.max_tile_packets."""
     k, n, val = _np(k, np.uint32), _np(n, np.uint32), _np(val, np.uint16)
-    tiles = (L.K // max(L.BK, 1)) * (L.N // max(L.BN, 1))
+    fq_pack_int4_sizes(L)                        # refuses a bad layout before arrays are made by it
+    tiles = (L.K // L.BK) * (L.N // L.BN)
     indptr = np.empty(tiles + 1, dtype=np.uint32)
     info = np.empty(tiles * L.buckets_per_tile, dtype=np.uint32)
     # every packet holds at least one outlier, so there are at most as many; pages that stay unwritten cost nothing

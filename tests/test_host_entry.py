@@ -3,6 +3,8 @@ import os
 import subprocess
 import sys
 
+import pytest
+
 from paper_2608_15531_b200 import binding as fq
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -27,3 +29,12 @@ def test_a_tensor_without_storage_is_a_python_error():
     """What the tensor library throws must not leave the CPython entry (the process would end)."""
     p = subprocess.run([sys.executable, "-c", _BATCHED_TENSOR], cwd=ROOT, capture_output=True, text=True)
     assert p.returncode == 0 and p.stdout.split("\n")[:2] == ["refused: True"] * 2, (p.returncode, p.stdout, p.stderr[-500:])
+
+
+@pytest.mark.parametrize("field,value", [("abi", 7), ("BK", 0), ("BK", 1), ("BN", 0), ("buckets_per_tile", 2 ** 31), ("K", 0)])
+def test_the_encoder_refuses_a_bad_layout_before_it_makes_arrays(field, value):
+    L = fq.fq_get_layout(1 << 20, 1 << 18, 128)
+    setattr(L, field, value)
+    with pytest.raises(fq.FqError) as e:
+        fq.fq_encode_tilecoo(L, [], [], [])
+    assert e.value.code == fq.FQ_ERR_INVALID_ARG
