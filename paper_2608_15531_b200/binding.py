@@ -73,8 +73,11 @@ def _pycall():
     global _call
     if _call is None:
         lib()
-        import torch  # noqa: F401  (its libraries have to be there first)
+        import torch                             # (its libraries have to be there first)
         from . import _fqcall
+        if _fqcall.built_for != f"torch {torch.__version__}":
+            raise ImportError(f"_fqcall.so was built for {_fqcall.built_for}, not torch {torch.__version__}: "
+                              "build it with `python -m paper_2608_15531_b200.build`")
         _call = _fqcall
     return _call
 

@@ -40,15 +40,22 @@ def build_lib(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def _built_for(lib: str, tag: str) -> bool:
+    """Whether `lib` was compiled with this tag (a string constant of its source)."""
+    with open(lib, "rb") as f:
+        return tag.encode() + b"\0" in f.read()
+
+
 def build_pycall(force: bool = False) -> str:
     """The CPython entry to the fused calls: links libfq.so (beside it) and the libraries of the torch that will be
-    imported with it."""
-    if force or stale(PYCALL, (PYCALL_SOURCE, HEADERS[-1])):
+    imported with it, whose C++ interface it uses: it is built anew for another torch."""
+    import torch
+    tag = f"torch {torch.__version__}"
+    if force or stale(PYCALL, (PYCALL_SOURCE, HEADERS[-1])) or not _built_for(PYCALL, tag):
         import sysconfig
-        import torch
         t = os.path.join(os.path.dirname(torch.__file__))
         cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DFQ_TORCH_TAG="{tag}"',
                "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(t, "include"),
                "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
                "-o", PYCALL, PYCALL_SOURCE, "-L", HERE, "-l:libfq.so", "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda",

@@ -142,4 +142,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fqcall", nullptr, -1, methods};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__fqcall(void) { return PyModule_Create(&module); }
+// `built_for`: the torch whose C++ interface this file was compiled against.
+PyMODINIT_FUNC PyInit__fqcall(void) {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", FQ_TORCH_TAG) != 0) Py_CLEAR(m);
+    return m;
+}

@@ -38,3 +38,20 @@ def test_the_encoder_refuses_a_bad_layout_before_it_makes_arrays(field, value):
     with pytest.raises(fq.FqError) as e:
         fq.fq_encode_tilecoo(L, [], [], [])
     assert e.value.code == fq.FQ_ERR_INVALID_ARG
+
+
+def test_the_entry_belongs_to_the_torch_it_was_built_for(monkeypatch):
+    """Another torch version: the binding refuses the old build, and the build step sees that it is stale."""
+    import torch
+    from paper_2608_15531_b200 import build
+    assert fq._pycall().built_for == f"torch {torch.__version__}"
+    calls = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: calls.append(cmd))
+    build.build_pycall()
+    assert not calls
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    build.build_pycall()
+    assert len(calls) == 1
+    monkeypatch.setattr(fq, "_call", None)
+    with pytest.raises(ImportError, match="built for"):
+        fq._pycall()
