@@ -119,8 +119,9 @@ FQ_SIMD_CLONES void group_range(const float* W, size_t w_step, const uint8_t* ma
     }
 }
 
-// Scales and zero-points of a group's columns; live = 0 marks a degenerate group (scale 1, zero-point 0, all codes 0).
-FQ_SIMD_CLONES void group_scale(const float* wmin, const float* wmax, uint32_t BN, float* sf, int32_t* zz, int32_t* live, uint16_t* scale, uint16_t* zero) {
+// Scales and zero-points of a group's columns.  A degenerate group (scale 1, zero-point 0, all codes 0) is divided by
+// infinity.
+FQ_SIMD_CLONES void group_scale(const float* wmin, const float* wmax, uint32_t BN, float* sf, float* zf, uint16_t* scale, uint16_t* zero) {
     for (uint32_t c = 0; c < BN; ++c) {
         const float s32 = (wmax[c] - wmin[c]) / 15.0f;
         uint32_t u;
@@ -129,21 +130,21 @@ FQ_SIMD_CLONES void group_scale(const float* wmin, const float* wmax, uint32_t B
         float s;
         std::memcpy(&s, &u, 4);
         const int32_t m = all_ones(s > 0.0f);
-        int32_t z = (int32_t)nearbyintf(-wmin[c] / s);
-        z = z < 0 ? 0 : z;
-        z = z > 15 ? 15 : z;
-        z &= m;
-        const float zf = (float)z;                             // 0 to 15: exact in BF16
+        float zq = nearbyintf(-wmin[c] / s);
+        zq = zq > 0.0f ? zq : 0.0f;
+        zq = zq < 15.0f ? zq : 15.0f;
+        zf[c] = select_or_zero(m, zq);                         // 0 to 15: exact in BF16
         uint32_t zu;
-        std::memcpy(&zu, &zf, 4);
-        sf[c] = s, zz[c] = z, live[c] = m;
+        std::memcpy(&zu, &zf[c], 4);
+        u = (u & (uint32_t)m) | (0x7f800000u & ~(uint32_t)m);
+        std::memcpy(&sf[c], &u, 4);
         scale[c] = (uint16_t)(((u >> 16) & (uint32_t)m) | (0x3f80u & ~(uint32_t)m));
         zero[c] = (uint16_t)(zu >> 16);
     }
 }
 
 // The words of eight rows (one word a column): nibble i + 4h is row 2i + h.  An outlier's place holds the zero-point.
-FQ_SIMD_CLONES void eight_rows(const float* W, size_t w_step, const uint8_t* mask, size_t m_step, uint32_t BN, const float* sf, const int32_t* zz, const int32_t* live,
+FQ_SIMD_CLONES void eight_rows(const float* W, size_t w_step, const uint8_t* mask, size_t m_step, uint32_t BN, const float* sf, const float* zf,
                                uint32_t* words) {
     for (uint32_t c = 0; c < BN; ++c) words[c] = 0;
     for (uint32_t r = 0; r < 8; ++r) {
@@ -151,12 +152,11 @@ FQ_SIMD_CLONES void eight_rows(const float* W, size_t w_step, const uint8_t* mas
         const uint8_t* mr = mask + r * m_step;
         const uint32_t shift = 4 * ((r >> 1) + 4 * (r & 1));
         for (uint32_t c = 0; c < BN; ++c) {
-            int32_t q = (int32_t)nearbyintf(wr[c] / sf[c]) + zz[c];
-            q = q < 0 ? 0 : q;
-            q = q > 15 ? 15 : q;
-            const int32_t m = all_ones(mr[c] != 0);
-            q = ((q & ~m) | (zz[c] & m)) & live[c];
-            words[c] |= (uint32_t)q << shift;
+            // clamped before the conversion (not a number gives 0); an outlier counts as 0, whose code is the zero-point
+            float v = nearbyintf(select_or_zero(all_ones(mr[c] == 0), wr[c]) / sf[c]) + zf[c];
+            v = v > 0.0f ? v : 0.0f;
+            v = v < 15.0f ? v : 15.0f;
+            words[c] |= (uint32_t)(int32_t)v << shift;
         }
     }
 }
@@ -181,8 +181,7 @@ fq_status_t fq_pack_int4(const fq_layout_t* L, const float* W, const uint8_t* ma
         const uint32_t kt = (uint32_t)(ch / NT), tn = (uint32_t)(ch % NT);
         uint32_t* chunk = wq + ((size_t)tn * KT + kt) * chunk_words;
         const size_t n0 = (size_t)tn * BN;
-        float wmin[kMaxBN], wmax[kMaxBN], sf[kMaxBN];
-        int32_t zz[kMaxBN], live[kMaxBN];
+        float wmin[kMaxBN], wmax[kMaxBN], sf[kMaxBN], zf[kMaxBN];
         uint32_t words[4][kMaxBN];
         for (uint32_t gi = 0; gi < gpc; ++gi) {
             const uint32_t k0 = kt * FQ_BK + gi * g;
@@ -190,10 +189,10 @@ fq_status_t fq_pack_int4(const fq_layout_t* L, const float* W, const uint8_t* ma
             const float* Wg = W + (size_t)k0 * N + n0;
             const uint8_t* mg = mask ? mask + (size_t)k0 * N + n0 : no_mask.data();
             group_range(Wg, N, mg, mask_step, g, BN, wmin, wmax);
-            group_scale(wmin, wmax, BN, sf, zz, live, scale + grow * N + n0, zero + grow * N + n0);
+            group_scale(wmin, wmax, BN, sf, zf, scale + grow * N + n0, zero + grow * N + n0);
             for (uint32_t j = 0; j < g / 32; ++j) {
                 for (uint32_t w = 0; w < 4; ++w)
-                    eight_rows(Wg + (size_t)(32 * j + 8 * w) * N, N, mg + (32 * j + 8 * w) * mask_step, mask_step, BN, sf, zz, live, words[w]);
+                    eight_rows(Wg + (size_t)(32 * j + 8 * w) * N, N, mg + (32 * j + 8 * w) * mask_step, mask_step, BN, sf, zf, words[w]);
                 uint32_t* out = chunk + (size_t)(gi * (g / 32) + j) * BN * 4;
                 for (uint32_t c = 0; c < BN; ++c)
                     for (uint32_t w = 0; w < 4; ++w) out[4 * c + w] = words[w][c];

@@ -55,3 +55,32 @@ def test_the_entry_belongs_to_the_torch_it_was_built_for(monkeypatch):
     monkeypatch.setattr(fq, "_call", None)
     with pytest.raises(ImportError, match="built for"):
         fq._pycall()
+
+
+_PACK = """
+import sys, numpy as np
+from paper_2608_15531_b200 import binding as fq
+fq.LIB_PATH = sys.argv[1]
+fq.EXPORTS = [n for n in fq.EXPORTS if n in ("fq_get_layout", "fq_pack_int4", "fq_pack_int4_sizes", "fq_last_error")]
+K, N = 128, 256
+W = (0.02 * np.random.default_rng(0).standard_normal((K, N))).astype(np.float32)
+mask = np.zeros((K, N), dtype=np.uint8)
+W[:, 0] = 0.0                                       # degenerate: 0 / 0
+W[:, 1] *= 1e-38; W[5, 1] = 3e38; mask[5, 1] = 1    # an outlier over a tiny scale: beyond any integer
+W[:, 2] = 0.0; W[9, 2] = 7.0; mask[9, 2] = 1        # nothing but an outlier: 7 / 0
+W[3, 3] = np.inf; W[4, 4] = -np.inf; W[6, 5] = np.nan
+out = fq.fq_pack_int4(fq.fq_get_layout(K, N, 128), W, mask)
+sys.stdout.write("".join(a.tobytes().hex() for a in out))
+"""
+
+
+def test_packing_converts_only_what_an_integer_holds(tmp_path):
+    """The packer under -fsanitize=float-cast-overflow: quotients that are no numbers, infinite, or too large for an integer are settled
+    before they are converted.  The arrays are those of the library."""
+    lib = str(tmp_path / "libfq_ubsan.so")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-fopenmp", "-ffp-contract=off", "-fsanitize=float-cast-overflow",
+                    "-fno-sanitize-recover=all", "-I", os.path.join(ROOT, "include"), os.path.join(ROOT, "paper_2608_15531_b200", "csrc", "fq_host.cpp"),
+                    "-o", lib], check=True)
+    runs = [subprocess.run([sys.executable, "-c", _PACK, path], cwd=ROOT, capture_output=True, text=True) for path in (lib, fq.LIB_PATH)]
+    assert runs[0].returncode == 0, runs[0].stderr
+    assert runs[1].returncode == 0 and runs[0].stdout and runs[0].stdout == runs[1].stdout
