@@ -112,6 +112,15 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     const bool ok = mbar_wait(bar, parity, abort_flag, status);
     return __all_sync(0xffffffffu, ok);
 }
+// A wait of a CTA that is leaving: no status, no abort flag, at most 100 ms.
+__device__ __forceinline__ void mbar_wait_leaving(uint32_t bar, uint32_t parity) {
+    const unsigned long long t0 = globaltimer_ns();
+    while (!mbar_try_wait(bar, parity) && globaltimer_ns() - t0 < 100000000ull) {}
+}
+// What a producer does that gives up: it lets the copies already issued land before the CTA's shared memory goes away.
+__device__ __forceinline__ void let_copies_land(uint32_t bar_full, uint32_t issued, uint32_t S) {
+    for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j) mbar_wait_leaving(bar_full + 8 * (j % S), (j / S) & 1);
+}
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)

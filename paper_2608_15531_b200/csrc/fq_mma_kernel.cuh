@@ -166,10 +166,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             }
             issued = it + 1;
         }
-        if (!ok) {
-            for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
-                for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
-        }
+        if (!ok) let_copies_land(bar_full, issued, S);
         if (!SPARSE && blockIdx.x == 0) report_packets(p.indptr, p.NT * KT, p.status);
     } else if (warp < DW0) {
         // ------------------------------------------------------------------ activation warps
@@ -289,7 +286,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             if (lane == 0) mbar_arrive(bar_full + 8 * s);
         }
         if (!ok && last_bar)                // gave up: let this warp's last copies land before the CTA exits
-            for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(last_bar, last_ph); ++spin) {}
+            mbar_wait_leaving(last_bar, last_ph);
     } else if (warp >= DW0 && warp < DW0 + NGRP * NDW) {
         // ------------------------------------------------------------------ dense warps (all alike)
         // Two groups of NDW warps take alternate units, each with accumulators of its own: twice the

@@ -495,10 +495,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 __syncwarp();
                 issued = w.it + 1;
             }
-            if (!ok) {   // giving up: let the copies already issued land before the CTA's shared memory goes away
-                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
-                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
-            }
+            if (!ok) let_copies_land(bar_full, issued, S);
         } else if (warp == 2) {
             // ---------------------------------------------------------------- producer of X
             uint32_t issued = 0;
@@ -517,10 +514,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 __syncwarp();
                 issued = w.it + 1;
             }
-            if (!ok) {
-                for (uint32_t j = (issued > S ? issued - S : 0); j < issued; ++j)
-                    for (uint32_t spin = 0; spin < (1u << 20) && !mbar_try_wait(bar_full + 8 * (j % S), (j / S) & 1); ++spin) {}
-            }
+            if (!ok) let_copies_land(bar_full, issued, S);
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
             // (the unpack warps have waited for the unit's stage, X block included, and their arrival hands that on: it is a release)
@@ -796,7 +790,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     __syncthreads();
     if (warp == 1) {
         // every tcgen05 operation of this CTA must have retired before its tensor memory is released
-        for (uint32_t spin = 0; spin < (1u << 24) && !mbar_try_wait(bar_final, 0); ++spin) {}
+        mbar_wait_leaving(bar_final, 0);
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base_of(), kTmemCols);
