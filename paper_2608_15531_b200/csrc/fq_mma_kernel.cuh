@@ -90,10 +90,10 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
     constexpr int DW0 = 1 + NA;                             // first dense warp
     // NGRP dense warp groups: group r takes the units it with it mod NGRP == r
     constexpr int CG = 2;                                   // 16-column MMA strips per warp
-    // two groups of 16-row warps share the register file, and 32-row warps fill it alone: one packet
+    // two groups of 16-row warps share the register file: one packet
     // requested ahead instead of two and its activation rows, two contributors in flight when a split
     // tile is settled
-    constexpr bool kTight = (MO == 2 && NGRP == 2) || MO == 4;
+    constexpr bool kTight = MO == 2 && NGRP == 2;
     constexpr int GPS = kBK / GROUP;
     constexpr int W_BYTES = 16 * BN * 4;
     constexpr int SZ_ROW = BN * 2;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
         const uint32_t aw = warp - 1;
         // lane -> (row m, part): 16-byte chunks of that row; rows beyond M are zero
         constexpr int ROWS = 8 * MO;
-        constexpr int LPR = 32 / ROWS;                       // lanes per row: 4 (8 rows), 2 (16 rows) or 1 (32 rows)
+        constexpr int LPR = 32 / ROWS;                       // lanes per row: 4 (8 rows) or 2 (16 rows)
         constexpr int CPL = 16 / LPR;                        // chunks per lane
         const int m = lane % ROWS, part = lane / ROWS;
         const bool real = (uint32_t)m < p.M;
@@ -235,12 +235,11 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             if (lane == 0 && w.it >= S) request(w.u, w.tn, w.kt, smem_u32(st), bar_full + 8 * s, ip, npk);
             uint8_t* dst = st + p.off_xcan + m * kXPitch;
             const int swz = (m & 1) << 2;
-            float sum = 0.0f, sum_lo = 0.0f;          // sum_lo: chunks 0-7 where a lane holds a whole row
+            float sum = 0.0f;
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 const uint4 v = xv[c];
                 *reinterpret_cast<uint4*>(dst + ((part * CPL + c) ^ swz) * 16) = v;
-                if (LPR == 1 && c == 8) sum_lo = sum, sum = 0.0f;
                 sum += (bf16lo(v.x) + bf16hi(v.x)) + (bf16lo(v.y) + bf16hi(v.y)) + (bf16lo(v.z) + bf16hi(v.z)) +
                        (bf16lo(v.w) + bf16hi(v.w));
             }
@@ -251,13 +250,10 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
                 const float s2 = s1 + __shfl_xor_sync(0xffffffffu, s1, 16);
                 if (GPS == 2) { if ((part & 1) == 0) xsum[(part >> 1) * ROWS + m] = s1; }
                 else if (part == 0) xsum[m] = s2;
-            } else if (LPR == 2) {
+            } else {
                 const float s1 = sum + __shfl_xor_sync(0xffffffffu, sum, 16);
                 if (GPS == 2) xsum[part * ROWS + m] = sum;
                 else if (part == 0) xsum[m] = s1;
-            } else {
-                if (GPS == 2) xsum[m] = sum_lo, xsum[ROWS + m] = sum;
-                else xsum[m] = sum_lo + sum;
             }
             __syncwarp();
             if (SPARSE && MS == 1) {
