@@ -112,10 +112,12 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     const bool ok = mbar_wait(bar, parity, abort_flag, status);
     return __all_sync(0xffffffffu, ok);
 }
-// A wait of a CTA that is leaving: no status, no abort flag, at most 100 ms.
+// A wait of a CTA that is leaving: no status, no abort flag, at most 100 ms (and no fewer than 4096 polls: the clock also runs while
+// the context is switched out).
 __device__ __forceinline__ void mbar_wait_leaving(uint32_t bar, uint32_t parity) {
     const unsigned long long t0 = globaltimer_ns();
-    while (!mbar_try_wait(bar, parity) && globaltimer_ns() - t0 < 100000000ull) {}
+    for (uint32_t polls = 0; !mbar_try_wait(bar, parity); ++polls)
+        if (polls >= 4096 && globaltimer_ns() - t0 > 100000000ull) return;
 }
 // What a producer does that gives up: it lets the copies already issued land before the CTA's shared memory goes away.
 __device__ __forceinline__ void let_copies_land(uint32_t bar_full, uint32_t issued, uint32_t S) {
