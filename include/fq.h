@@ -39,9 +39,8 @@
  *   consecutive columns follow each other: a thread that owns a column fetches
  *   them with one 128-bit load, a warp without bank conflicts.  One
  *   shift-and-mask turns nibbles i and i+4 of a word into a BF16 pair of
- *   consecutive rows, the operand order of the warp-level MMA; one mask each
- *   turns the even and the odd nibbles into four bytes, the operand of the
- *   integer MMA.)
+ *   consecutive rows, the operand order of the warp-level MMA and of a row of
+ *   the tcgen05 MMA's A operand in tensor memory.)
  *
  *   Scale, zero.  (K/group) x N row-major BF16.  zero holds the integer 0..15.
  *
@@ -133,8 +132,9 @@ typedef struct fq_layout {
                                   Every kernel accepts either; the arrays decode to the same set */
     uint32_t value_type;       /* type of the outlier values handed to fq_encode_tilecoo and returned by
                                   fq_decode_tilecoo, 16 bits each: FQ_VALUE_BF16 (default) or FQ_VALUE_FP16 (IEEE
-                                  binary16; Table 1's value field).  The packed slots hold either exactly, and the
-                                  kernels read them the same way */
+                                  binary16; Table 1's value field).  The packed slots hold either exactly.  It has to
+                                  be the type that the arrays were encoded with: the tcgen05 kernel multiplies binary16
+                                  values in two BF16 parts and BF16 values in one */
 } fq_layout_t;
 
 /* Choose tile sizes for a K x N layer.  bn_hint: 0 = library default (256 when
@@ -235,8 +235,8 @@ fq_status_t fq_workspace_bytes(const fq_layout_t* L, uint32_t M, size_t* bytes);
  *     be short get one CTA per strip, whose warps split K among themselves and
  *     read the weights straight into registers; every other layer streams
  *     (tile, k-step) units through a bulk-copy/mbarrier ring on persistent CTAs;
- *   - more than 16 rows, 9 to 16 rows on all but small layers, 2 to 8 on large
- *     layers with 128-column tiles: one launch of a kernel built on tcgen05.mma
+ *   - more than 16 rows, 9 to 16 rows on all but small layers and on layers with
+ *     tails, 2 to 8 on large ones with 128-column tiles: one launch of a kernel built on tcgen05.mma
  *     with BF16 operands (the exact integers q - z, and the outliers as a second
  *     matrix that is zero elsewhere).  If the encoding names a position twice, or
  *     that is not known (L->tilecoo_encoded, L->abi), M is cut into launches of
@@ -299,8 +299,10 @@ fq_status_t fq_fused_w4a16_outlier_gemm_noalloc(const fq_layout_t* L, const void
                                                 const void* packed_outliers, void* Y,
                                                 void* cuda_stream);
 
-/* Unfused baseline, dense half: Y = X * dequant(W_Q) (same kernel, sparse path
- * compiled out). */
+/* Unfused baseline, dense half: Y = X * dequant(W_Q), on the kernels that serve
+ * the fused call of a layer without outliers: up to 16 rows the warp-level MMA
+ * kernels with the sparse path compiled out, beyond the tcgen05 kernel with an
+ * empty outlier tile. */
 fq_status_t fq_unfused_gemm(const fq_layout_t* L, const void* X, uint32_t M, const void* wq,
                             const void* scale, const void* zero, void* Y, void* workspace,
                             size_t workspace_bytes, void* cuda_stream);
