@@ -90,3 +90,22 @@ def test_host_memory_that_is_pinned_in_part(side):
     finally:
         assert int(cudart.cudaHostUnregister(part.data_ptr())) == 0
     assert np.array_equal(H.run_fused(P, Xb), Y)
+
+
+@pytest.mark.parametrize("M", [1, 8, 40])
+def test_a_captured_call_reads_its_buffers_anew(M):
+    """A call from pinned to pinned memory in a CUDA graph, replayed with other values in the same buffers."""
+    K, N = 2048, 2304
+    P = H.pack_layer(synth.layer(synth.tensor_seed(13, 1), K, N, density=0.01, layout="mixed"), 128)
+    Xh, Yh = torch.zeros((M, K), dtype=torch.int16).pin_memory(), torch.zeros((M, N), dtype=torch.int16).pin_memory()
+    x, y = torch.empty((M, K), dtype=torch.int16, device="cuda"), torch.empty((M, N), dtype=torch.int16, device="cuda")
+    fq.fq_fused_host_io(P.L, Xh, M, x, *_weights(P), y, Yh, P.ws)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fq.fq_fused_host_io_async(P.L, Xh, M, x, *_weights(P), y, Yh, P.ws)
+    for i in range(3):
+        Xb = synth.activations(200 + i, M, K)
+        Xh.copy_(torch.from_numpy(Xb.view(np.int16)))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(Yh.numpy().view(np.uint16), H.run_fused(P, Xb))
