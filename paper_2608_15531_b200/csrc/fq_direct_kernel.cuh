@@ -45,7 +45,7 @@ constexpr int kDirectSlots = 8;     // packets of a bucket that are requested wi
 // bytes of shared memory a warp of the direct kernel owns: rows of X, k-major copy, scale and zero rows, packets
 constexpr int kDirectWarpBytes = 16 * 256 + 256 + 8 * kDirectSlots * 16;
 
-template <int MO, int MS, int GROUP, bool SPARSE, int WARPS>
+template <int MO, int MS, int GROUP, bool SPARSE, int WARPS, bool UNI>
 __global__ void __launch_bounds__(32 * WARPS, (MO == 1 && WARPS == 16) ? 2 : 1) fq_direct_kernel(const DirectParams p) {
     constexpr int CG = 2, GPS = kBK / GROUP, NV = MO * CG * 4;
     // Shared memory, per warp: its block of activations, 8 MO rows of 256 B (16-byte chunk c of an odd row at
@@ -55,9 +55,8 @@ __global__ void __launch_bounds__(32 * WARPS, (MO == 1 && WARPS == 16) ? 2 : 1) 
     // read different banks).  After the last k-step the same bytes hold the warps' sums, [WARPS][NV + R][32] FP32.
     extern __shared__ __align__(16) float red[];
     constexpr bool kMajor = SPARSE && (MS == 4 || MS == 8);
-    // The warp number through a shuffle tells the compiler that it is the same in every lane (4096 x 4096 without outliers at
-    // one row 4.81 us, so 4.48; with two CTAs of 16 warps to an SM 6.54 and 6.70).
-    const int tid = threadIdx.x, lane = tid & 31, warp = WARPS == 32 ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5, g = lane >> 2, t = lane & 3;
+    // (the warp number through a shuffle tells the compiler that it is the same in every lane; where, see direct_uniform)
+    const int tid = threadIdx.x, lane = tid & 31, warp = UNI ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5, g = lane >> 2, t = lane & 3;
     uint8_t* xrow_s = reinterpret_cast<uint8_t*>(red) + warp * kDirectWarpBytes;
     uint8_t* xk8 = xrow_s + 8 * 256;                                // MO == 1 only (two octets of rows fill these bytes)
     uint8_t* szs = xrow_s + 16 * 256;

@@ -1,9 +1,9 @@
 // CUDA side of the library (sm_100a): the fused W4A16 + Tile-COO outlier decode matmul
 // (Eq. 1; Sections 3.1, 4.1, 4.2), its two unfused baselines and the launchers behind the C ABI.
 //
-// Three kernels serve the fused operator, chosen per launch from its rows and the layer's shape (launch_gemm): a
+// Three kernels serve the fused operator, chosen per launch from its rows and the layer's shape (tc_serves, direct_warps): a
 // streaming kernel and a short-job kernel with warp-level MMAs for up to 16 rows (fq_mma_kernel.cuh,
-// fq_direct_kernel.cuh) and a tcgen05 kernel for 17 to 128 (fq_tc_kernel.cuh).  The streaming kernels are
+// fq_direct_kernel.cuh) and a tcgen05 kernel for up to 128 (fq_tc_kernel.cuh).  The streaming kernels are
 // persistent and warp-specialised: (tile, k-step) units of 128 rows stream through a ring of shared-memory stages
 // (bulk copies + mbarrier expect_tx).  All feed the tensor cores exact integers and apply the scale once per group in FP32:
 //     acc[m] += s * sum_k x (q - z)                                     (Eq. 3 inside Eq. 1)
@@ -364,6 +364,20 @@ static int sm_count_cached() {
     return cached[dev];
 }
 
+// How the NT x KT units of a launch are shared out over persistent CTAs: split = 0, one contiguous range each; else a tile-aligned
+// split, every column tile to `split` CTAs, when that costs at most one more unit per CTA: then no CTA has to settle two
+// split tiles in a row.
+struct Split {
+    uint32_t grid, split, units_per_cta;
+};
+static Split split_units(uint32_t NT, uint32_t KT, int sms) {
+    const uint32_t grid = std::min<uint32_t>({(uint32_t)sms, kMaxCtas, NT * KT}), units_per_cta = (NT * KT + grid - 1) / grid;
+    const uint32_t c = std::min<uint32_t>(grid / NT, KT);
+    if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) return {NT * c, c, (KT + c - 1) / c};
+    return {grid, 0, units_per_cta};
+}
+constexpr uint32_t kTwoGroups = 8;      // units per CTA from which the streaming kernel runs two groups of dense warps
+
 // The tcgen05 kernel's variant for a launch: the batch rows its tensor memory and drain warps are laid out for.
 static inline uint32_t tc_rows(uint32_t m) { return m <= 16 ? 16u : (m <= 32 ? 32u : (m <= 64 ? 64u : 128u)); }
 
@@ -383,19 +397,8 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     p.halves = L->BN / 128;
     p.nmma = round_up(M, 16);
     p.parts = L->value_type == FQ_VALUE_FP16 ? 2 : 1;
-    const uint32_t NT = p.NT, KT = p.KT;
-    uint32_t grid = std::min<uint32_t>({(uint32_t)sms, kMaxCtas, NT * KT});
-    const uint32_t units_per_cta = (NT * KT + grid - 1) / grid;
-    // Tile-aligned split instead of one contiguous range per CTA when it costs at most one more unit
-    // per CTA: then no CTA has to settle two split tiles in a row.
-    if (NT <= grid) {
-        const uint32_t c = std::min<uint32_t>(grid / NT, KT);
-        if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) {
-            p.split = c;
-            grid = NT * c;
-        }
-    }
-    const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
+    const Split sp = split_units(p.NT, p.KT, sms);
+    p.split = sp.split;
     p.off_w = 256 * p.nmma;
     p.off_sz = p.off_w + 8192;
     p.stage_bytes = tc_stage_bytes(p.nmma, GPS);
@@ -404,8 +407,9 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     p.off_wo = p.stages * p.stage_bytes;
     p.off_bar = p.off_wo + tc_wo_bytes(pl.nr);
     pl.smem = p.off_bar + 2048;
+    const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
     pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
-    pl.grid = grid;
+    pl.grid = sp.grid;
     return FQ_OK;
 }
 
@@ -447,38 +451,66 @@ static inline uint32_t direct_warps(const fq_layout_t* L, uint32_t rows, bool ou
     }
     return (rows == 1 && strips <= 2u * (uint32_t)sms && KT <= 32) ? 16u : 0u;
 }
-template <int MO, int MS, int W>
-static DirectFn pick_direct_group(uint32_t g, bool sparse) {
-    if (!sparse) return g == 64 ? (DirectFn)fq_direct_kernel<MO, 8 * MO, 64, false, W> : (DirectFn)fq_direct_kernel<MO, 8 * MO, 128, false, W>;
-    return g == 64 ? (DirectFn)fq_direct_kernel<MO, MS, 64, true, W> : (DirectFn)fq_direct_kernel<MO, MS, 128, true, W>;
+// UNI: whether the kernel tells the compiler that a warp's number is the same in all its lanes.  Without outliers that is
+// always faster (4096 x 4096 at one row 4.8 us, so 4.1).  With outliers it goes both ways with the size of the job (us, without /
+// with): at one to four rows, 8192 x 1024 at four 9.9 / 10.4, 4096 x 2176 at two 5.8 / 6.1, 2048 x 2048 4.2 / 4.2, 2048 x 4608 4.4 / 4.3, 8192 x 4736
+// 11.0 / 10.8; at five to eight, 1024 x 1024 4.1 / 3.9, 2048 x 4608 5.3 / 5.0, 4096 x 4096 7.3 / 7.5, 8192 x 1024 11.5 / 12.0, 8192 x 4736 at five
+// 12.5 / 12.0, and with groups of 64 1024 x 1024 4.1 / 4.05, 2048 x 2048 5.0 / 5.1, 8192 x 1024 11.8 / 12.5, 6016 x 4096 10.3 / 10.6.
+static inline bool direct_uniform(const fq_layout_t* L, uint32_t rows) {
+    const uint32_t strips = L->N / 32, KT = L->K / kBK;
+    if (rows <= 4) return strips > 96;
+    return L->group == 64 ? KT <= 8 : (KT <= 16 || strips * KT >= 5500);
 }
-template <int W>
-static DirectFn pick_direct_rows(uint32_t rows, uint32_t g, bool sparse) {
-    if (rows == 1) return pick_direct_group<1, 1, W>(g, sparse);
-    if (rows <= 4) return pick_direct_group<1, 4, W>(g, sparse);
-    return pick_direct_group<1, 8, W>(g, sparse);
+template <int MO, int MS, int W, bool UNI>
+static DirectFn pick_direct_group(uint32_t g) {
+    return g == 64 ? (DirectFn)fq_direct_kernel<MO, MS, 64, true, W, UNI> : (DirectFn)fq_direct_kernel<MO, MS, 128, true, W, UNI>;
 }
-static DirectFn pick_direct(uint32_t rows, uint32_t warps, uint32_t g, bool sparse) {
-    if (rows > 8) return pick_direct_group<2, 16, 16>(g, sparse);
-    return warps == 32 ? pick_direct_rows<32>(rows, g, sparse) : pick_direct_rows<16>(rows, g, sparse);
+template <int W, bool UNI>
+static DirectFn pick_direct_rows(uint32_t rows, uint32_t g) {
+    if (rows == 1) return pick_direct_group<1, 1, W, UNI>(g);
+    if (rows <= 4) return pick_direct_group<1, 4, W, UNI>(g);
+    return pick_direct_group<1, 8, W, UNI>(g);
+}
+template <int MO, int W, bool UNI>
+static DirectFn pick_direct_dense(uint32_t g) {
+    return g == 64 ? (DirectFn)fq_direct_kernel<MO, 8 * MO, 64, false, W, UNI> : (DirectFn)fq_direct_kernel<MO, 8 * MO, 128, false, W, UNI>;
+}
+static DirectFn pick_direct(const fq_layout_t* L, uint32_t rows, uint32_t warps, bool sparse) {
+    const uint32_t g = L->group;
+    if (!sparse) return rows > 8 ? pick_direct_dense<2, 16, false>(g) : (warps == 32 ? pick_direct_dense<1, 32, true>(g) : pick_direct_dense<1, 16, false>(g));
+    if (rows > 8) return pick_direct_group<2, 16, 16, false>(g);
+    if (warps == 16) return pick_direct_group<1, 1, 16, false>(g);      // (two CTAs to an SM: a single row only)
+    return direct_uniform(L, rows) ? pick_direct_rows<32, true>(rows, g) : pick_direct_rows<32, false>(rows, g);
 }
 
-// Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 29.3 us
-// at 8 to 16 rows, 31.6 at 32), the warp-level MMA kernels' grows (26.9 us at 8 rows, 36.7 at 16), and its
-// start-up costs about 4 us more than theirs.  So it takes every launch of more than 16 rows, and launches of 9 to 16 rows
-// on layers of at least 512 units of 128 x 128 weights, or with tails (9.3 against 10.9 us on 4096 x 4096, but 7.5 against 6.7 on 2048 x
-// 2048).  On layers with tiles of 128 columns, where the streaming kernel has half the dense warps, it is faster from two rows
-// up (2944 x 11136: 13.2 against 14.3 us at two to five rows, 8192 x 28800 52.4 against 61.6) unless they are short
-// jobs.  It writes outliers into a tile instead of adding them, so an encoding that names a position twice (or may do so) stays
-// with launches of 16 rows on the other kernels.  Without outliers (the layer has none, or the call is the dense half of the
-// unfused pair) it takes launches of more than 16 rows, and the others, which have variants without the outlier step,
-// those of up to 16 (4096 x 14336 at 8 rows 14.5 us with the step, 11.5 without).
+// Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 28.7 us
+// at 9 to 16 rows, 32.3 at 32), the warp-level MMA kernels' grows (24.7 us at 8 rows, 34.6 at 16), and its start-up costs about
+// 4 us more than theirs.  It writes outliers into a tile instead of adding them, so an encoding that names a position
+// twice (or may do so) stays with launches of 16 rows on the other kernels.  Times below: us, theirs / its, 1 % unless stated.
+//   more than 16 rows   always
+//   9 to 16 rows        with tails (2048 x 2048 9.2 / 7.5), or from 512 units of 128 x 128 weights up (4096 x 4096 10.7 / 8.8, 1024 x 8192
+//                       7.8 / 6.8; 2048 x 2048 6.0 / 7.5 before it stayed out).  But not jobs of one k-step to a warp of the short-job
+//                       kernel (2048 x 4096 6.2 / 7.0, at 0.5 % 5.7 / 7.0), unless their buckets are deep (5 %: 12.4 / 7.9).
+//   2 to 8 rows         tiles of 128 columns, where the streaming kernel has half the dense warps, at least 1024 units, no short job; and
+//     with tails        always (4096 x 6272 at 2 % 14.6 / 13.1, 8 rows 17.2 / 13.1; 8192 x 16512 58.3 / 56.5, 72.4 / 56.4)
+//     else              where the streaming kernel would run one group of dense warps (1024 x 16512 10.2 / 9.5); from 4096 units at
+//                       up to four rows (8192 x 16512 32.9 / 32.1, 2048 x 28800 17.3 / 17.6) if buckets are not deep (8192 x 16512 at 2 %
+//                       34.1 / 33.1, at 5 % 38.2 / 46.9); from 3072 at five and more (2048 x 28800 at 8 rows 18.7 / 17.6, 4096 x 11136 15.6 /
+//                       15.9; at 5 % 25.1 / 23.9)
+// Without outliers (the layer has none, or the call is the dense half of the unfused pair) it takes launches of more than 16
+// rows, and the others, which have variants without the outlier step, those of up to 16 (4096 x 14336 at 8 rows 14.5 us with the
+// step, 11.5 without).
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers) {
     if (!outliers) return rows > 16;
     if (L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
-    const uint64_t units = (uint64_t)(L->K / kBK) * (L->N / 128);
-    if (rows > 16 || (rows >= 9 && (units >= 512 || L->max_tail_packets > 0))) return true;
-    return L->BN == 128 && rows >= 2 && units >= 1024 && direct_warps(L, rows, true) == 0;
+    if (rows > 16) return true;
+    const uint32_t KT = L->K / kBK, depth = L->max_bucket_packets;
+    const uint64_t units = (uint64_t)KT * (L->N / 128);
+    const bool tails = L->max_tail_packets > 0;
+    if (rows >= 9) return tails || (units >= 512 && !(KT <= 16 && depth <= 10 && direct_warps(L, rows, true)));
+    if (L->BN != 128 || rows < 2 || units < 1024 || direct_warps(L, rows, true)) return false;
+    if (tails || split_units(L->N / 128, KT, sm_count_cached()).units_per_cta < kTwoGroups) return true;
+    return rows <= 4 ? units >= 4096 && depth <= 13 : units >= 3072;
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool outliers) { return tc_serves(L, rows_left, outliers) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 
@@ -530,22 +562,9 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     // the outlier step of that variant prefetches less (96 registers per thread).
     const int sms = sm_count_cached();
     if (sms <= 0) return fail(FQ_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
-    const uint32_t NT = L->N / BN, KT = L->K / kBK;
-    uint32_t grid = std::min<uint32_t>({(uint32_t)sms, kMaxCtas, NT * KT});
-    uint32_t units_per_cta = (NT * KT + grid - 1) / grid;
-    // Tile-aligned split instead of one contiguous range per CTA when it costs at most one more unit
-    // per CTA: then no CTA has to settle two split tiles in a row.
-    uint32_t split = 0;
-    if (NT <= grid) {
-        const uint32_t c = std::min<uint32_t>(grid / NT, KT);
-        if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) {
-            split = c;
-            grid = NT * c;
-            units_per_cta = (KT + c - 1) / c;
-        }
-    }
-    p.split = split;
-    pl.ngrp = units_per_cta >= 8 ? 2 : 1;
+    const Split sp = split_units(p.NT, p.KT, sms);
+    p.split = sp.split;
+    pl.ngrp = sp.units_per_cta >= kTwoGroups ? 2 : 1;
     const uint32_t xch_bytes = pl.ngrp > 1 ? BN * ROWS * 4 : 0;   // hand-over of a group's partial sums
     const uint32_t fixed = 1024 + xch_bytes;
     const uint32_t budget = kSmemBudget;
@@ -578,7 +597,7 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     p.off_bar = p.off_shc + xch_bytes;
     pl.smem = p.off_bar + 1024;
     pl.threads = 32 * (1 + kActWarps + pl.ngrp * NDW);
-    pl.grid = grid;
+    pl.grid = sp.grid;
     return FQ_OK;
 }
 
@@ -717,7 +736,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             // per warp: rows of activations, their k-major copy, scale and zero rows, staged packets; the warps'
             // sums reuse those bytes
             cfg.dynamicSmemBytes = warps * kDirectWarpBytes;
-            DirectFn dfn = pick_direct(mb, warps, L->group, outliers);
+            DirectFn dfn = pick_direct(L, mb, warps, outliers);
             e = ensure_smem_attr((const void*)dfn, 32 * kDirectWarpBytes);
             if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
             e = cudaLaunchKernelEx(&cfg, dfn, p);

@@ -1,0 +1,38 @@
+"""Either side of the rules that choose a launch's kernel, on sampled columns against the oracle.  Needs a B200."""
+import numpy as np
+import pytest
+
+from paper_2608_15531_b200 import synth
+
+import harness as H
+
+pytestmark = pytest.mark.gpu
+
+_SHAPES = [
+    (2048, 4096, 0.01, (9, 16)),           # 16 k-steps, shallow buckets: a short job; deep ones: tcgen05
+    (2048, 4096, 0.05, (9, 16)),
+    (2176, 4096, 0.01, (9, 16)),           # 17 k-steps: tcgen05
+    (1024, 16512, 0.01, (2, 8)),           # tiles of 128 columns, one group of dense warps: tcgen05
+    (8192, 6272, 0.01, (4, 5)),            # 3136 units: tcgen05 from five rows up
+    (8192, 8320, 0.01, (1, 2, 4)),         # 4160 units: from two rows up, unless buckets are deep
+    (8192, 8320, 0.05, (2, 5)),
+    (2048, 3072, 0.01, (1, 4)),            # both builds of the short-job kernel: 96 strips, 97 and more
+    (2048, 3200, 0.01, (1, 4)),
+    (2048, 2048, 0.01, (5, 8)),            # and 16 k-steps, 17 and more
+    (2176, 2048, 0.01, (5, 8)),
+    (6016, 4096, 0.01, (5, 8)),
+]
+
+
+@pytest.mark.parametrize("K,N,density,rows", _SHAPES)
+@pytest.mark.parametrize("g", [64, 128])
+def test_either_side_of_a_rule(K, N, density, rows, g):
+    lay = synth.layer(synth.tensor_seed(17, K // 128 + N // 128), K, N, density=density, layout="uniform")
+    P = H.pack_layer(lay, g)
+    cols = np.unique(np.concatenate([np.arange(0, N, 97), [N - 1]])).astype(np.uint32)
+    for M in rows:
+        X = synth.activations(lay.seed + M, M, K)
+        Y = H.run_fused(P, X)
+        Yref, Yabs = H.oracle_result(P, X, cols=cols)
+        H.check_tolerances(Y[:, cols], Yref, Yabs, K)
+        assert np.array_equal(H.run_fused(P, X), Y)
