@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(32 * WARPS, (MO == 1 && WARPS == 16) ? 2 : 1) 
         }
         if (!waited) {
             // everything above is weights; the activations may come from the grid before this one
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (SPARSE) asm volatile("griddepcontrol.wait;" ::: "memory");
+            else grid_wait_dense(strip == 0 && warp == 0, p.indptr, p.N / BN * KT, p.status);
             waited = true;
         }
         // ---- this k-step's block of X into the warp's rows (rows beyond M are zero)
@@ -318,5 +319,4 @@ __global__ void __launch_bounds__(32 * WARPS, (MO == 1 && WARPS == 16) ? 2 : 1) 
         }
         if (m < p.M) p.Y[(size_t)m * p.N + (size_t)strip * 32 + g + 16 * cg + 8 * h] = float_to_bf16_bits(sum);
     }
-    if (!SPARSE && blockIdx.x == 0 && warp == 0) report_packets(p.indptr, p.N / BN * KT, p.status);
 }

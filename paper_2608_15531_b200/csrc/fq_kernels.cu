@@ -182,12 +182,15 @@ struct UnitIter {
     }
 };
 
-// A layer whose layout struct knows of no outliers is served without an outlier step.  If its arrays hold some all the same
-// (struct and arrays out of step), a warp of the first CTA reports it.  `indptr` is null where there is no sparse part at all.
-__device__ __forceinline__ void report_packets(const uint32_t* indptr, uint32_t tiles, uint32_t* status) {
-    if (!indptr || __ldg(indptr + tiles) == 0) return;
-    asm volatile("griddepcontrol.wait;" ::: "memory");     // before the scratch is written
-    if ((threadIdx.x & 31) == 0) atomicExch(status, (uint32_t)FQ_ERR_FORMAT);
+// Waits for the grid before this one, in a kernel without an outlier step.  That serves layers whose layout struct knows of no
+// outliers; if the arrays hold some all the same (struct and arrays out of step), the warp that is told to `look` reports it.
+// The load is on its way during the wait (at the end of the kernel it cost 2432 x 1152 at two rows 0.3 of 3.1 us).  `indptr` is
+// null where there is no sparse part at all.
+__device__ __forceinline__ void grid_wait_dense(bool look, const uint32_t* indptr, uint32_t tiles, uint32_t* status) {
+    uint32_t packets = 0;
+    if (look && indptr) packets = __ldg(indptr + tiles);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (packets) atomicExch(status, (uint32_t)FQ_ERR_FORMAT);
 }
 
 #include "fq_tc_kernel.cuh"
@@ -459,7 +462,7 @@ static inline uint32_t direct_warps(const fq_layout_t* L, uint32_t rows, bool ou
 static inline bool direct_uniform(const fq_layout_t* L, uint32_t rows) {
     const uint32_t strips = L->N / 32, KT = L->K / kBK;
     if (rows <= 4) return strips > 96;
-    return L->group == 64 ? KT <= 8 : (KT <= 16 || strips * KT >= 5500);
+    return L->group == 64 ? KT <= 8 : (KT <= 16 || strips * KT >= 4500);
 }
 template <int MO, int MS, int W, bool UNI>
 static DirectFn pick_direct_group(uint32_t g) {
@@ -489,28 +492,29 @@ static DirectFn pick_direct(const fq_layout_t* L, uint32_t rows, uint32_t warps,
 // twice (or may do so) stays with launches of 16 rows on the other kernels.  Times below: us, theirs / its, 1 % unless stated.
 //   more than 16 rows   always
 //   9 to 16 rows        with tails (2048 x 2048 9.2 / 7.5), or from 512 units of 128 x 128 weights up (4096 x 4096 10.7 / 8.8, 1024 x 8192
-//                       7.8 / 6.8; 2048 x 2048 6.0 / 7.5 before it stayed out).  But not jobs of one k-step to a warp of the short-job
-//                       kernel (2048 x 4096 6.2 / 7.0, at 0.5 % 5.7 / 7.0), unless their buckets are deep (5 %: 12.4 / 7.9).
+//                       7.8 / 6.8).  But not jobs of one k-step to a warp of the short-job kernel (2048 x 4096 6.2 / 6.9, at 0.5 % 5.7 /
+//                       6.9, 2048 x 4608 6.2 / 7.2), unless their buckets are deep (2 %: 7.6 / 7.1, 5 %: 12.4 / 7.9).
 //   2 to 8 rows         tiles of 128 columns, where the streaming kernel has half the dense warps, at least 1024 units, no short job; and
 //     with tails        always (4096 x 6272 at 2 % 14.6 / 13.1, 8 rows 17.2 / 13.1; 8192 x 16512 58.3 / 56.5, 72.4 / 56.4)
 //     else              where the streaming kernel would run one group of dense warps (1024 x 16512 10.2 / 9.5); from 4096 units at
 //                       up to four rows (8192 x 16512 32.9 / 32.1, 2048 x 28800 17.3 / 17.6) if buckets are not deep (8192 x 16512 at 2 %
 //                       34.1 / 33.1, at 5 % 38.2 / 46.9); from 3072 at five and more (2048 x 28800 at 8 rows 18.7 / 17.6, 4096 x 11136 15.6 /
-//                       15.9; at 5 % 25.1 / 23.9)
+//                       15.9), or from 2048 with buckets of middling depth (4096 x 9344 at 2 % 14.9 / 13.9, at 5 % 17.1 / 18.0 at five)
 // Without outliers (the layer has none, or the call is the dense half of the unfused pair) it takes launches of more than 16
 // rows, and the others, which have variants without the outlier step, those of up to 16 (4096 x 14336 at 8 rows 14.5 us with the
-// step, 11.5 without).
+// step, 11.5 without); two or three launches of the short-job kernel are faster than one of it on small layers (1024 x 1024 at 32
+// rows 5.0 / 9.3, at 48 7.4 / 9.2, at 64 9.8 / 9.6; 4096 x 4096 at 32 11.9 / 11.0).
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers) {
-    if (!outliers) return rows > 16;
-    if (L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
-    if (rows > 16) return true;
     const uint32_t KT = L->K / kBK, depth = L->max_bucket_packets;
     const uint64_t units = (uint64_t)KT * (L->N / 128);
+    if (!outliers) return rows > 16 && !(rows <= (units <= 128 ? 48u : 32u) && units <= 512 && direct_warps(L, 16, false));
+    if (L->tilecoo_encoded != 1 || L->abi != FQ_ABI_ENCODED) return false;
+    if (rows > 16) return true;
     const bool tails = L->max_tail_packets > 0;
-    if (rows >= 9) return tails || (units >= 512 && !(KT <= 16 && depth <= 10 && direct_warps(L, rows, true)));
+    if (rows >= 9) return tails || (units >= 512 && !(KT <= 16 && depth <= 9 && direct_warps(L, rows, true)));
     if (L->BN != 128 || rows < 2 || units < 1024 || direct_warps(L, rows, true)) return false;
     if (tails || split_units(L->N / 128, KT, sm_count_cached()).units_per_cta < kTwoGroups) return true;
-    return rows <= 4 ? units >= 4096 && depth <= 13 : units >= 3072;
+    return rows <= 4 ? units >= 4096 && depth <= 13 : units >= 3072 || (units >= 2048 && depth > 10 && depth <= 18);
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool outliers) { return tc_serves(L, rows_left, outliers) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
 

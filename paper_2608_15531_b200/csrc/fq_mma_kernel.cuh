@@ -167,7 +167,6 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             issued = it + 1;
         }
         if (!ok) let_copies_land(bar_full, issued, S);
-        if (!SPARSE && blockIdx.x == 0) report_packets(p.indptr, p.NT * KT, p.status);
     } else if (warp < DW0) {
         // ------------------------------------------------------------------ activation warps
         const uint32_t aw = warp - 1;
@@ -218,7 +217,8 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
                 request(u, tn, u - tn * KT, smem_u32(smem) + it0 * p.stage_bytes, bar_full + 8 * it0, a, npk);
             }
             __syncwarp();
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (SPARSE) asm volatile("griddepcontrol.wait;" ::: "memory");
+            else grid_wait_dense(blockIdx.x == 0 && aw == 0, p.indptr, U, p.status);
         }
         if (u_begin + aw < u_end) { load((u_begin + aw) % KT); load_ip(u_begin + aw); }
         for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
