@@ -34,10 +34,10 @@ CONFIG_ID = 2                      # the LLaMA-3-8B layer set
 REPEATS = 5                        # repetitions of the timed region (K steps each); the median is the value
 L2_COVER_BYTES = 400 << 20         # rotating copies per layer cover at least this (L2 is 126 MB)
 METRIC = "effective_hbm_gbs_fused_w4a16_outlier_gemm_m1_8_16"
-# dram__bytes_read + dram__bytes_write of a fused launch over its algorithmic bytes, per layer, from the ncu captures
-# summarised in profiles/fq_kernels_llama3_8b_decode_set.md (the padding of the column-slotted packets; the ratio
-# does not depend on M).  Not measured by a bench run: `roofline.traffic` applies them to the step's launches.
-NCU_TRAFFIC_RATIO = {"gate_up": 1.072, "down": 1.053, "qkv": 1.049, "o_proj": 1.048}
+# dram__bytes_read + dram__bytes_write of a fused launch over its algorithmic bytes, per layer: the mean over M = 1, 8, 16 (which
+# differ by 1 % at most) of the ncu captures summarised in profiles/fq_tc_kernel_counters.md (the padding of the column-slotted
+# packets).  Not measured by a bench run: `roofline.traffic` applies them to the step's launches.
+NCU_TRAFFIC_RATIO = {"gate_up": 1.064, "down": 1.053, "qkv": 1.050, "o_proj": 1.050}
 
 
 def algorithmic_bytes(K, N, g, nnz, n_tile, n_bucket, M):
