@@ -387,7 +387,12 @@ static inline uint32_t tc_rows(uint32_t m) { return m <= 16 ? 16u : (m <= 32 ? 3
 struct TcPlan {
     TcParams p;
     uint32_t threads, smem, grid, nr;
+    bool coop;      // the CTA, not its drain warps, finishes a split tile at the end of its range
 };
+
+// (See the kernel.  With more than 32 rows from about eight contributors to a tile: 11008 x 2048 at 90 rows 26.6 us, so 20.4; 8192 x 1024 at 128 29.0
+// and 19.7; but 14336 x 4096 at 128, with five, 37.5 and 39.8, at 64 25.0 and 25.5.)
+static inline bool tc_coop(uint32_t nr, uint32_t KT, uint32_t units_per_cta) { return nr <= 32 || KT >= 8 * units_per_cta; }
 
 static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     TcParams& p = pl.p;
@@ -413,6 +418,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
     pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = sp.grid;
+    pl.coop = tc_coop(pl.nr, p.KT, sp.units_per_cta);
     return FQ_OK;
 }
 
@@ -638,10 +644,12 @@ static MmaKernelFn pick_mma_kernel(uint32_t bn, uint32_t M, uint32_t g, bool spa
 }
 
 typedef void (*TcKernelFn)(const CUtensorMap, const TcParams);
-template <int NR>
-static TcKernelFn pick_tc_group(uint32_t g) { return g == 64 ? (TcKernelFn)fq_tc_kernel<NR, 64> : (TcKernelFn)fq_tc_kernel<NR, 128>; }
-static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g) {
-    return nr == 128 ? pick_tc_group<128>(g) : (nr == 64 ? pick_tc_group<64>(g) : (nr == 32 ? pick_tc_group<32>(g) : pick_tc_group<16>(g)));
+template <int NR, bool COOP>
+static TcKernelFn pick_tc_group(uint32_t g) { return g == 64 ? (TcKernelFn)fq_tc_kernel<NR, 64, COOP> : (TcKernelFn)fq_tc_kernel<NR, 128, COOP>; }
+static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g, bool coop) {
+    if (nr == 128) return coop ? pick_tc_group<128, true>(g) : pick_tc_group<128, false>(g);
+    if (nr == 64) return coop ? pick_tc_group<64, true>(g) : pick_tc_group<64, false>(g);
+    return nr == 32 ? pick_tc_group<32, true>(g) : pick_tc_group<16, true>(g);
 }
 
 // cudaFuncSetAttribute costs several microseconds: do it once per (kernel, device).
@@ -719,7 +727,7 @@ static fq_status_t launch_gemm(const fq_layout_t* L, const void* X, uint32_t M, 
             CUtensorMap xmap;
             st = encode_x_map(L, Xm, mb, p.nmma, &xmap);
             if (st != FQ_OK) return st;
-            TcKernelFn fn = pick_tc_kernel(pl.nr, L->group);
+            TcKernelFn fn = pick_tc_kernel(pl.nr, L->group, pl.coop);
             e = ensure_smem_attr((const void*)fn, (int)kSmemBudget);
             if (e != cudaSuccess) return fail(FQ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
             cfg.gridDim = dim3(pl.grid);

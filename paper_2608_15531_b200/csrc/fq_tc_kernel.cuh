@@ -389,7 +389,12 @@ __device__ __forceinline__ void tc_scatter(const TcParams& p, uint8_t* smem, uin
     }
 }
 
-template <int NR, int GROUP>
+// COOP: who finishes a split tile that is the last of a CTA's range and to which the CTA was the last to add.  The drain warps that
+// hold it, one to a scheduler, take 0.6 us for each contributor and 1 us to write 32 rows of Y, a chain of latencies; all warps of
+// the CTA together, when their own work is done, about 1 us for everything.  us, by the drain warps / by the CTA: 8192 x 1024 at 24
+// rows 14.7 / 9.0, 14336 x 4096 at 32 22.3 / 20.3, 4096 x 4096 at 32 11.0 / 10.0.  With 64 and 128 rows the code of it costs the rest
+// of the kernel something (4096 x 28672 at 64 rows 36.6 / 39.0, at 128 54.7 / 57.2): tc_coop.
+template <int NR, int GROUP, bool COOP>
 __global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
 fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
@@ -414,6 +419,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     const uint32_t bar_final = bar_o_free + 8;
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 27);
     volatile uint32_t* tmem_slot = abort_flag + 1;
+    uint32_t* settle = const_cast<uint32_t*>(abort_flag) + 2;    // COOP: strips and sets (bit strip + 4 set) that the CTA finishes on its way out
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
@@ -432,6 +438,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         mbar_init(bar_o_free, 4 * SETS);
         mbar_init(bar_final, 2);
         *abort_flag = 0;
+        if (COOP) *settle = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -705,8 +712,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             if (!full_piece) {
                 // Split tile.  Every warp settles its own 32 columns and rows, without CTA-wide barriers: FP32 partial, four
                 // rows of a column to 16 bytes, then one arrival per (tile, strip, set of rows: a byte of the strip's
-                // counter each); the last warp to arrive adds the partials in CTA order (the same order in every run)
-                // and writes Y.
+                // counter each); the last to arrive adds the partials in CTA order (the same order in every run) and writes Y:
+                // this warp, or the whole CTA if the range ends here (COOP).
                 constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;      // float4 per slot
                 const uint32_t which = (p.split || u_begin / KT == tn) ? 0u : 1u;
                 float4* slots = reinterpret_cast<float4*>(p.partials) + (size_t)(r0 / 4) * COLS + col;
@@ -729,10 +736,14 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 }
                 last = __shfl_sync(0xffffffffu, last, 0);
                 __syncwarp();
-                if (last) {
+                if (COOP && last && lane == 0) {
+                    atomicSub(counter, (c_last - c_first + 1) << (8 * set));                     // ready for the next call
+                    if (piece_stop == u_end) atomicOr(settle, 1u << (set * 4 + dw));
+                }
+                if (last && !(COOP && piece_stop == u_end)) {
                     write_y = true;
                     // 16 rows at a time, ND contributors' loads in flight; the additions keep CTA order
-                    constexpr int ND = 2;
+                    constexpr int ND = NR >= 64 || !COOP ? 2 : 1;
 #pragma unroll
                     for (int i0 = 0; i0 < RT / 4; i0 += 4)
                         if (r0 + 4 * i0 < p.M) {
@@ -761,7 +772,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                                     }
                             }
                         }
-                    if (lane == 0) atomicSub(counter, (c_last - c_first + 1) << (8 * set));      // ready for the next call
+                    if (!COOP && lane == 0) atomicSub(counter, (c_last - c_first + 1) << (8 * set));      // ready for the next call
                 }
             }
             if (write_y) {
@@ -795,5 +806,44 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base_of(), kTmemCols);
+    }
+    if constexpr (COOP) {
+        if (const uint32_t mine = *settle) {
+            // The sums of the range's last tile (the drain warps' acquire is handed on by the barrier above): a thread takes four
+            // rows of a column, with ND contributors' loads in flight.
+            constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;
+            constexpr int ND = 6;
+            uint32_t cta = blockIdx.x, ctas = P;
+            if (NR >= 64) {                                   // the range anew, so that nothing of it is kept in registers until here
+                asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+                asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(ctas));
+            }
+            const uint32_t q2 = U / ctas, r2 = U % ctas;
+            const uint32_t tn = NR < 64 ? (u_end - 1) / KT : (p.split ? cta / p.split : (unit_begin_of(cta + 1, q2, r2) - 1) / KT), u_tile0 = tn * KT;
+            const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q2, r2);
+            const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q2, r2);
+            const float4* slots = reinterpret_cast<const float4*>(p.partials);
+            for (uint32_t e = threadIdx.x; e < (p.M + 3) / 4 * COLS; e += blockDim.x) {
+                const uint32_t i = e / COLS, col = e % COLS;
+                if (!((mine >> (4 * i / S_::RT * 4 + col / 32)) & 1u)) continue;
+                float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                for (uint32_t c = c_first; c <= c_last; c += ND) {
+                    float4 v[ND];
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) {
+                        const uint32_t wch = (p.split || unit_begin_of(c + d, q2, r2) / KT == tn) ? 0u : 1u;
+                        if (c + d <= c_last) v[d] = __ldcg(slots + ((size_t)(c + d) * 2 + wch) * SLOT + e);
+                    }
+#pragma unroll
+                    for (int d = 0; d < ND; ++d)
+                        if (c + d <= c_last) sum.x += v[d].x, sum.y += v[d].y, sum.z += v[d].z, sum.w += v[d].w;
+                }
+                uint16_t* y = p.Y + (size_t)(4 * i) * p.N + (size_t)tn * COLS + col;
+                const float rows[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    if (4 * i + m < p.M) y[(size_t)m * p.N] = float_to_bf16_bits(rows[m]);
+            }
+        }
     }
 }

@@ -36,3 +36,20 @@ def test_either_side_of_a_rule(K, N, density, rows, g):
         Yref, Yabs = H.oracle_result(P, X, cols=cols)
         H.check_tolerances(Y[:, cols], Yref, Yabs, K)
         assert np.array_equal(H.run_fused(P, X), Y)
+
+
+# Layers whose column tiles are shared by many CTAs of the tcgen05 kernel (8192 x 1024: 18 of them to a tile, 2944 x 1152: 16, ranges over
+# two tiles; 4096 x 4096: a split along the tiles): the sums at the end of a range are the whole CTA's work up to 32 rows, and beyond
+# from eight contributors up.  Rows at the edges of the sets of 32 rows and of the quads of rows that a thread takes.
+@pytest.mark.parametrize("K,N", [(8192, 1024), (2944, 1152), (4096, 4096)])
+@pytest.mark.parametrize("g", [64, 128])
+def test_tiles_with_many_contributors(K, N, g):
+    lay = synth.layer(synth.tensor_seed(18, K // 128 + N // 128), K, N, density=0.01, layout="mixed")
+    P = H.pack_layer(lay, g)
+    cols = np.unique(np.concatenate([np.arange(0, N, 61), [N - 1]])).astype(np.uint32)
+    X = synth.activations(lay.seed, 128, K)
+    Yref, Yabs = H.oracle_result(P, X, cols=cols)
+    for M in (9, 16, 17, 31, 33, 63, 65, 128):
+        Y = H.run_fused(P, X[:M])
+        H.check_tolerances(Y[:, cols], Yref[:M], Yabs[:M], K)
+        assert np.array_equal(H.run_fused(P, X[:M]), Y)
