@@ -407,7 +407,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const uint32_t S = p.stages;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
-    const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * S;
+    const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * S;      // [S] a unit's codes, scales, zero-points are here; the stage is free
     const uint32_t bar_a_full = bar_empty + 8 * S;        // [4] A operand written (unpack warps)
     const uint32_t bar_a_empty = bar_a_full + 32;         // [4] the MMAs that read it are complete
     const uint32_t bar_d_full = bar_a_empty + 32;         // [4] a unit's dense MMAs are complete
@@ -417,13 +417,19 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     const uint32_t bar_o_full = bar_wo_empty + 32;        // the piece's outlier sums are complete
     const uint32_t bar_o_free = bar_o_full + 8;           // and read
     const uint32_t bar_final = bar_o_free + 8;
+    // The activations' arrival, [S], has barriers of its own up to 32 rows, so that the first units are unpacked while the wait for the grid
+    // before is still on (us, with / without: 4096 x 4096 at 32 rows 9.7 / 10.0, 8192 x 1024 at 24 8.7 / 9.0; with 64 rows no gain, with groups of 64
+    // spills: 8192 x 28672 73.5 / 68.9).
+    constexpr bool XB = NR <= 32;
+    const uint32_t bar_x_full = XB ? bar_final + 32 : bar_full;
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 27);
     volatile uint32_t* tmem_slot = abort_flag + 1;
     uint32_t* settle = const_cast<uint32_t*>(abort_flag) + 2;    // COOP: strips and sets (bit strip + 4 set) that the CTA finishes on its way out
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
-            mbar_init(bar_full + 8 * s, 2);                                  // the two producers' expect_tx arrivals
+            mbar_init(bar_full + 8 * s, XB ? 1 : 2);                         // the producers' expect_tx arrivals
+            if (XB) mbar_init(bar_x_full + 8 * s, 1);
             mbar_init(bar_empty + 8 * s, 4 + 4 * SETS + 2);                  // unpack and drain warps, the MMAs' commits
         }
         for (uint32_t i = 0; i < 4; ++i) {
@@ -509,9 +515,10 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             uint32_t issued = 0;
             bool ok = true;
             const uint32_t x_half = p.nmma * 128;                          // bytes of 64 K values of every batch row
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&xmap) : "memory");
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
-                const uint32_t full = bar_full + 8 * w.s;
+                const uint32_t full = bar_x_full + 8 * w.s;
                 if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
                 const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
                 if (elect_one()) {
@@ -522,31 +529,33 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 __syncwarp();
                 issued = w.it + 1;
             }
-            if (!ok) let_copies_land(bar_full, issued, S);
+            if (!ok) let_copies_land(bar_x_full, issued, S);
         } else if (warp == 1) {
             // ---------------------------------------------------------------- dense tensor warp
-            // (the unpack warps have waited for the unit's stage, X block included, and their arrival hands that on: it is a release)
+            // (without XB the unpack warps have waited for the whole stage, X block included, and their arrival hands that on: it is a release)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((p.nmma >> 3) << 17) | (8u << 24), tmem_base = tmem_base_of();
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4;
             const uint64_t xd0 = desc_sw128(smem_u32(smem));
             const uint32_t units = u_end - u_begin;
-            uint32_t s = 0, xd = (uint32_t)xd0;
+            uint32_t s = 0, ph = 0, xd = (uint32_t)xd0;
             bool ready = false;
             for (uint32_t it = 0; it < units; ++it) {
                 const uint32_t ab = it % NAB, db = it % NDB, nx = it + 1;
                 if (!ready) {
                     if (it >= NDB && !wait_converged(bar_d_free + 8 * db, (it / NDB - 1) & 1, abort_flag, p.status)) break;
+                    if (XB && !wait_converged(bar_x_full + 8 * s, ph, abort_flag, p.status)) break;
                     if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
                 tc_fence_after();
+                const uint32_t sn = s + 1 == S ? 0 : s + 1, phn = sn ? ph : ph ^ 1;
                 // the next unit's barriers, tested while this one's MMAs are issued
-                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
+                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) & (XB ? mbar_test_wait(bar_x_full + 8 * sn, phn) : 1u) &
                                       (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
                 const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
                 umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
                            bar_a_empty + 8 * ab, bar_empty + 8 * s);
-                xd += stage;
-                if (++s == S) s = 0, xd = (uint32_t)xd0;
+                xd = sn ? xd + stage : (uint32_t)xd0;
+                s = sn, ph = phn;
                 ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
@@ -560,7 +569,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             uint32_t s = 0, ph = 0, wb = 0, wph = 0, xd = (uint32_t)xd0, acc = 0, left = KT - u_begin % KT, piece = 0;    // left: units to the end of the tile
             bool ok = true, ready = false;
             for (uint32_t it = 0; it < units && ok; ++it) {
-                if (!ready && !(wait_converged(bar_full + 8 * s, ph, abort_flag, p.status) &&
+                if (!ready && !(wait_converged(bar_x_full + 8 * s, ph, abort_flag, p.status) &&
                                 wait_converged(bar_wo_full + 8 * wb, wph, abort_flag, p.status))) break;
                 tc_fence_after();
                 umma_outliers(o, (uint32_t)wo0 + wb * (kWoTile >> 4), (uint32_t)(wo0 >> 32), xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, acc,
@@ -578,7 +587,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= 1;
                 if (++wb == NWO) wb = 0, wph ^= parts & 1;
                 // the next unit's barriers, tested while this one's MMAs run
-                const uint32_t seen = mbar_test_wait(bar_full + 8 * s, ph) & mbar_test_wait(bar_wo_full + 8 * wb, wph);
+                const uint32_t seen = mbar_test_wait(bar_x_full + 8 * s, ph) & mbar_test_wait(bar_wo_full + 8 * wb, wph);
                 if (--left == 0 || it + 1 == units) {
                     // end of a piece: the drain warps take the sums before the next piece's overwrite them
                     if (elect_one()) umma_commit(bar_o_full);
