@@ -160,18 +160,58 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Which CTA owns unit u when U units are dealt out as contiguous ranges, the first r CTAs one longer.
-__device__ __forceinline__ uint32_t cta_of_unit(uint32_t u, uint32_t q, uint32_t r) {
-    const uint32_t big = r * (q + 1);
-    return u < big ? u / (q + 1) : r + (u - big) / q;
-}
-__device__ __forceinline__ uint32_t unit_begin_of(uint32_t c, uint32_t q, uint32_t r) { return c * q + min(c, r); }
+// Division by a number that the host knows: n / d = upper half of n * (floor(2^64 / d) + 1), exact for every 32-bit n; d = 1 has
+// no such factor (0).  The compiler's division is a chain of some forty instructions, and up to ten of them stood between a CTA's last
+// unit and its last sum: 14336 x 4096 at 16 rows 17.8 us, so 17.1; 4096 x 4096 at 16 8.6 and 8.3; 4096 x 28672 at 8 24.7 and 24.3.
+struct Divisor {
+    uint32_t lo, hi;
+    __host__ __device__ static Divisor of(uint32_t d) {
+        const uint64_t m = d > 1 ? ~0ull / d + 1 : 0;         // (a power of two: ~0 / d + 1 = 2^64 / d exactly)
+        return {(uint32_t)m, (uint32_t)(m >> 32)};
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t n) const {
+        const uint32_t quotient = (uint32_t)(((uint64_t)hi * n + (((uint64_t)lo * n) >> 32)) >> 32);
+        return (lo | hi) ? quotient : n;
+    }
+};
+// How NT x KT units are shared out (see split_units): q units and one more for the first r CTAs, or `split` CTAs to a tile.
+struct Shares {
+    uint32_t q, r;
+    uint32_t split;   // 0 = units dealt out as one contiguous range per CTA (stream-K);
+                      // c > 0 = every column tile belongs to c CTAs, CTA b takes part b mod c of tile b / c
+    Divisor by_q, by_q1, by_split, by_kt;
+    // which CTA owns unit u, and the first unit of CTA c, of contiguous ranges
+    __device__ __forceinline__ uint32_t cta_of_unit(uint32_t u) const {
+        const uint32_t big = r * (q + 1);
+        return u < big ? by_q1(u) : r + by_q(u - big);
+    }
+    __device__ __forceinline__ uint32_t unit_begin_of(uint32_t c) const { return c * q + min(c, r); }
+    // the units [begin, end) of CTA c
+    __device__ __forceinline__ void range(uint32_t c, uint32_t KT, uint32_t& begin, uint32_t& end) const {
+        if (split) {
+            // tile-aligned: no CTA works on two tiles, so none settles two split tiles one after the other
+            const uint32_t tile = by_split(c), part = c - tile * split;
+            begin = tile * KT + by_split(part * KT);
+            end = tile * KT + by_split((part + 1) * KT);
+        } else {
+            begin = unit_begin_of(c);
+            end = begin + q + (c < r ? 1u : 0u);
+        }
+    }
+    // the first and the last CTA that have units of tile tn
+    __device__ __forceinline__ void owners(uint32_t tn, uint32_t KT, uint32_t& first, uint32_t& last) const {
+        first = split ? tn * split : cta_of_unit(tn * KT);
+        last = split ? first + split - 1 : cta_of_unit(tn * KT + KT - 1);
+    }
+    // which of its two partial slots CTA c uses for its part of tile tn: the second if its range begins before the tile
+    __device__ __forceinline__ uint32_t slot_of(uint32_t c, uint32_t tn, uint32_t KT) const { return split || unit_begin_of(c) >= tn * KT ? 0u : 1u; }
+};
 
 // Walks a CTA's units without integer division: ring slot s with its parity, tile tn, k-step kt.
 struct UnitIter {
     uint32_t u, it, s, ph, tn, kt;
-    __device__ __forceinline__ UnitIter(uint32_t u_begin, uint32_t KT) : u(u_begin), it(0), s(0), ph(0) {
-        tn = u_begin / KT;
+    __device__ __forceinline__ UnitIter(uint32_t u_begin, uint32_t KT, const Divisor& by_kt) : u(u_begin), it(0), s(0), ph(0) {
+        tn = by_kt(u_begin);
         kt = u_begin - tn * KT;
     }
     __device__ __forceinline__ void next(uint32_t S, uint32_t KT) {
@@ -379,6 +419,10 @@ static Split split_units(uint32_t NT, uint32_t KT, int sms) {
     if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) return {NT * c, c, (KT + c - 1) / c};
     return {grid, 0, units_per_cta};
 }
+static Shares shares_of(const Split& sp, uint32_t NT, uint32_t KT) {
+    const uint32_t q = NT * KT / sp.grid, r = NT * KT % sp.grid;
+    return {q, r, sp.split, Divisor::of(q ? q : 1), Divisor::of(q + 1), Divisor::of(sp.split ? sp.split : 1), Divisor::of(KT)};
+}
 constexpr uint32_t kTwoGroups = 8;      // units per CTA from which the streaming kernel runs two groups of dense warps
 
 // The tcgen05 kernel's variant for a launch: the batch rows its tensor memory and drain warps are laid out for.
@@ -390,9 +434,12 @@ struct TcPlan {
     bool coop;      // the CTA, not its drain warps, finishes a split tile at the end of its range
 };
 
-// (See the kernel.  With more than 32 rows from about eight contributors to a tile: 11008 x 2048 at 90 rows 26.6 us, so 20.4; 8192 x 1024 at 128 29.0
-// and 19.7; but 14336 x 4096 at 128, with five, 37.5 and 39.8, at 64 25.0 and 25.5.)
-static inline bool tc_coop(uint32_t nr, uint32_t KT, uint32_t units_per_cta) { return nr <= 32 || KT >= 8 * units_per_cta; }
+// (See the kernel.  us, by the drain warps / by the CTA.  33 to 64 rows, at 64: groups of 64 2944 x 11136 at 48 rows 17.4 / 16.7, 8192 x 28672 69.4 / 69.0; groups
+// of 128 4096 x 4096 11.9 / 12.3, 4096 x 28672 36.4 / 37.4, 14336 x 4096, with five CTAs to a tile, 24.1 / 23.9.  Beyond, at 128: 14336 x
+// 4096 35.7 / 34.3, 4096 x 4096 17.7 / 17.4, but 4096 x 28672, where a CTA has a tile and a half, 53.6 / 55.1.)
+static inline bool tc_coop(uint32_t nr, uint32_t group, uint32_t KT, uint32_t units_per_cta) {
+    return nr <= 32 || (nr == 64 ? group == 64 || KT >= 8 * units_per_cta : KT >= 2 * units_per_cta);
+}
 
 static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     TcParams& p = pl.p;
@@ -406,7 +453,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     p.nmma = round_up(M, 16);
     p.parts = L->value_type == FQ_VALUE_FP16 ? 2 : 1;
     const Split sp = split_units(p.NT, p.KT, sms);
-    p.split = sp.split;
+    p.shares = shares_of(sp, p.NT, p.KT);
     p.off_w = 256 * p.nmma;
     p.off_sz = p.off_w + 8192;
     p.stage_bytes = tc_stage_bytes(p.nmma, GPS);
@@ -418,7 +465,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
     pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = sp.grid;
-    pl.coop = tc_coop(pl.nr, p.KT, sp.units_per_cta);
+    pl.coop = tc_coop(pl.nr, L->group, p.KT, sp.units_per_cta);
     return FQ_OK;
 }
 
@@ -573,7 +620,7 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     const int sms = sm_count_cached();
     if (sms <= 0) return fail(FQ_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
     const Split sp = split_units(p.NT, p.KT, sms);
-    p.split = sp.split;
+    p.shares = shares_of(sp, p.NT, p.KT);
     pl.ngrp = sp.units_per_cta >= kTwoGroups ? 2 : 1;
     const uint32_t xch_bytes = pl.ngrp > 1 ? BN * ROWS * 4 : 0;   // hand-over of a group's partial sums
     const uint32_t fixed = 1024 + xch_bytes;

@@ -20,8 +20,7 @@ struct MmaParams {
     float* partials;
     uint32_t M, K, N, KT, NT;
     uint32_t NB, coo_cap, stages;
-    uint32_t split;   // 0 = units dealt out as one contiguous range per CTA (stream-K);
-                      // c > 0 = every column tile belongs to c CTAs, CTA b takes part b mod c of tile b / c
+    Shares shares;
     // shared-memory offsets (bytes); the first five are relative to a stage
     uint32_t stage_bytes, off_sz, off_xcan, off_xsum, off_info, off_coo;
     uint32_t off_shc, off_xt, off_bar;
@@ -128,17 +127,8 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
     if (warp >= DW0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const uint32_t KT = p.KT;
-    const uint32_t U = p.NT * KT, P = gridDim.x, q = U / P, r = U % P;
     uint32_t u_begin, u_end;
-    if (p.split) {
-        // tile-aligned split: no CTA works on two tiles, so none settles two split tiles one after the other
-        const uint32_t tile = blockIdx.x / p.split, part = blockIdx.x - tile * p.split;
-        u_begin = tile * KT + part * KT / p.split;
-        u_end = tile * KT + (part + 1) * KT / p.split;
-    } else {
-        u_begin = unit_begin_of(blockIdx.x, q, r);
-        u_end = u_begin + q + (blockIdx.x < r ? 1u : 0u);
-    }
+    p.shares.range(blockIdx.x, KT, u_begin, u_end);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
@@ -149,7 +139,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
         // kernels with one octet of rows, and this split measured best.
         uint32_t issued = 0;
         bool ok = true;
-        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+        for (UnitIter w(u_begin, KT, p.shares.by_kt); w.u < u_end; w.next(S, KT)) {
             const uint32_t u = w.u, it = w.it, s = w.s, ph = w.ph;
             if (!warp_wait(bar_empty + 8 * s, ph ^ 1, abort_flag, p.status)) { ok = false; break; }
             const uint32_t full = bar_full + 8 * s;
@@ -211,17 +201,17 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             // lane l requests those of this warp's l-th unit before the wait for the previous grid.
             const uint32_t it0 = aw + NA * lane;
             if (it0 < min(S, u_end - u_begin)) {
-                const uint32_t u = u_begin + it0, tn = u / KT;
+                const uint32_t u = u_begin + it0, tn = p.shares.by_kt(u);
                 uint32_t a = 0, npk = 0;
                 if (SPARSE) { a = __ldg(p.indptr + u); npk = min(__ldg(p.indptr + u + 1) - a, p.coo_cap); }
                 request(u, tn, u - tn * KT, smem_u32(smem) + it0 * p.stage_bytes, bar_full + 8 * it0, a, npk);
             }
             __syncwarp();
             if (SPARSE) asm volatile("griddepcontrol.wait;" ::: "memory");
-            else grid_wait_dense(blockIdx.x == 0 && aw == 0, p.indptr, U, p.status);
+            else grid_wait_dense(blockIdx.x == 0 && aw == 0, p.indptr, p.NT * KT, p.status);
         }
-        if (u_begin + aw < u_end) { load((u_begin + aw) % KT); load_ip(u_begin + aw); }
-        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+        if (u_begin + aw < u_end) { load(u_begin + aw - p.shares.by_kt(u_begin + aw) * KT); load_ip(u_begin + aw); }
+        for (UnitIter w(u_begin, KT, p.shares.by_kt); w.u < u_end; w.next(S, KT)) {
             if (w.it % NA != aw) continue;
             const uint32_t s = w.s, ph = w.ph;
             uint8_t* st = smem + s * p.stage_bytes;
@@ -229,7 +219,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
 #pragma unroll
             for (int c = 0; c < CPL; ++c) xv[c] = nxt[c];
             const uint32_t ip = ip_nxt, npk = min(ip_nxt_end - ip_nxt, p.coo_cap);
-            if (w.u + NA < u_end) { uint32_t kn = w.kt + NA; load(kn >= KT ? kn % KT : kn); load_ip(w.u + NA); }   // this warp's next unit
+            if (w.u + NA < u_end) { uint32_t kn = w.kt + NA; while (kn >= KT) kn -= KT; load(kn); load_ip(w.u + NA); }   // this warp's next unit
             if (!warp_wait(bar_empty + 8 * s, ph ^ 1, abort_flag, p.status)) { ok = false; break; }
             last_bar = bar_full + 8 * s, last_ph = ph;
             if (lane == 0 && w.it >= S) request(w.u, w.tn, w.kt, smem_u32(st), bar_full + 8 * s, ip, npk);
@@ -312,7 +302,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
         // this group's units of the piece (every NGRP-th unit of the range; the ring length is a multiple
         // of NGRP).  The end-of-piece code stays out of the inner loop's body.
         uint32_t u = u_begin + grp, s = grp, ph = 0;                    // this group's next unit, its stage and parity
-        uint32_t tn = u_begin / KT;
+        uint32_t tn = p.shares.by_kt(u_begin);
         for (uint32_t piece_first = u_begin; piece_first < u_end && ok; ++tn) {
           const uint32_t piece_stop = min(u_end, (tn + 1) * KT);        // one past the piece's last unit
           piece_first = piece_stop;
@@ -640,7 +630,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
                     // barriers: FP32 partial in fragment order, then one arrival per (tile, strip);
                     // the last warp to arrive adds the partials in CTA order (the same order in
                     // every run) and writes Y.
-                    const uint32_t which = (p.split || u_begin / KT == tn) ? 0u : 1u;
+                    const uint32_t which = p.shares.slot_of(blockIdx.x, tn, KT);
                     float* slot = p.partials + ((size_t)blockIdx.x * 2 + which) * (size_t)(BN * LDC) + dw * (32 * LDC) + lane;
 #pragma unroll
                     for (int o = 0; o < MO; ++o)
@@ -649,8 +639,8 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
 #pragma unroll
                             for (int i = 0; i < 4; ++i) __stcg(slot + ((o * CG + cg) * 4 + i) * 32, accf[o][cg][i]);
                     __syncwarp();
-                    const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q, r);
-                    const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q, r);
+                    uint32_t c_first, c_last;
+                    p.shares.owners(tn, KT, c_first, c_last);
                     uint32_t last = 0;
                     if (lane == 0) {
                         // one arrival, release and acquire at GPU scope: the warp's stores (ordered before
@@ -678,7 +668,7 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
 #pragma unroll
                             for (int d = 0; d < ND; ++d) {
                                 const uint32_t cc = min(c + d, c_last);
-                                const uint32_t wch = (p.split || unit_begin_of(cc, q, r) / KT == tn) ? 0u : 1u;
+                                const uint32_t wch = p.shares.slot_of(cc, tn, KT);
                                 const float* sl = p.partials + ((size_t)cc * 2 + wch) * (size_t)(BN * LDC) + dw * (32 * LDC) + lane;
 #pragma unroll
                                 for (int e = 0; e < MO * CG * 4; ++e) v[d][e] = __ldcg(sl + e * 32);

@@ -221,7 +221,7 @@ struct TcParams {
     uint32_t M, K, N, KT, NT;       // NT: column tiles of 128 columns
     uint32_t halves;                // such tiles to a stored tile (1 or 2)
     uint32_t max_tile_packets, stages;
-    uint32_t split;                 // as in the streaming kernel
+    Shares shares;                  // as in the streaming kernel
     uint32_t nmma;                  // batch rows of the MMAs: M rounded up to 16
     uint32_t parts;                 // BF16 parts of an outlier: 1, or 2 (FP16 values)
     // shared-memory offsets (bytes); the first two are relative to a stage, whose X block is at 0
@@ -285,7 +285,7 @@ __device__ __forceinline__ void tc_scatter(const TcParams& p, uint8_t* smem, uin
     // a unit's bucket of this lane: its descriptor and the tile's packet range, then its checked form and first slots
     struct Raw { uint32_t info, a, b; };
     struct Bucket { const uint32_t* packets; uint32_t depth, tail, wd[kScatterAhead]; };
-    uint32_t u = u_begin + sg, tn = u / KT, kt = u - tn * KT;              // the next unit to request
+    uint32_t u = u_begin + sg, tn = p.shares.by_kt(u), kt = u - tn * KT;              // the next unit to request
     auto request = [&]() {
         Raw r = {0, 0, 0};
         if (p.info && u < u_end) {                         // (no descriptors: the dense half of the unfused pair)
@@ -392,14 +392,14 @@ __device__ __forceinline__ void tc_scatter(const TcParams& p, uint8_t* smem, uin
 // COOP: who finishes a split tile that is the last of a CTA's range and to which the CTA was the last to add.  The drain warps that
 // hold it, one to a scheduler, take 0.6 us for each contributor and 1 us to write 32 rows of Y, a chain of latencies; all warps of
 // the CTA together, when their own work is done, about 1 us for everything.  us, by the drain warps / by the CTA: 8192 x 1024 at 24
-// rows 14.7 / 9.0, 14336 x 4096 at 32 22.3 / 20.3, 4096 x 4096 at 32 11.0 / 10.0.  With 64 and 128 rows the code of it costs the rest
-// of the kernel something (4096 x 28672 at 64 rows 36.6 / 39.0, at 128 54.7 / 57.2): tc_coop.
+// rows 14.7 / 9.0, 14336 x 4096 at 32 22.3 / 20.3, 4096 x 4096 at 32 11.0 / 10.0; with more rows see tc_coop.
 template <int NR, int GROUP, bool COOP>
 __global__ void __launch_bounds__(32 * TcShape<NR, GROUP>::WARPS, 1)
 fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
     constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG;
     constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
+    constexpr bool DEFER = COOP && NR == 32;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
 
@@ -424,7 +424,10 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     const uint32_t bar_x_full = XB ? bar_final + 32 : bar_full;
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * S + 27);
     volatile uint32_t* tmem_slot = abort_flag + 1;
-    uint32_t* settle = const_cast<uint32_t*>(abort_flag) + 2;    // COOP: strips and sets (bit strip + 4 set) that the CTA finishes on its way out
+    // COOP: strips and sets (bit strip + 4 set) that the CTA finishes on its way out, of its range's last tile and (DEFER) of its first, of
+    // which it seldom is the last contributor.  With 32 rows the sums in the drain warps' loop cost it registers (4096 x 28672 32.3 us, so 31.1;
+    // 8192 x 28672 55.9 and 53.8); with 16 the sums of the first tile are better done at once (4096 x 28672 28.3 and 29.0).
+    uint32_t* settle = const_cast<uint32_t*>(abort_flag) + 2;
 
     if (tid == 0) {
         for (uint32_t s = 0; s < S; ++s) {
@@ -444,7 +447,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         mbar_init(bar_o_free, 4 * SETS);
         mbar_init(bar_final, 2);
         *abort_flag = 0;
-        if (COOP) *settle = 0;
+        if (COOP) settle[0] = settle[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -468,16 +471,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const uint32_t KT = p.KT;
-    const uint32_t U = p.NT * KT, P = gridDim.x, q = U / P, r = U % P;
     uint32_t u_begin, u_end;
-    if (p.split) {
-        const uint32_t tile = blockIdx.x / p.split, part = blockIdx.x - tile * p.split;
-        u_begin = tile * KT + part * KT / p.split;
-        u_end = tile * KT + (part + 1) * KT / p.split;
-    } else {
-        u_begin = unit_begin_of(blockIdx.x, q, r);
-        u_end = u_begin + q + (blockIdx.x < r ? 1u : 0u);
-    }
+    p.shares.range(blockIdx.x, KT, u_begin, u_end);
     // stored tile of a unit (Tile-COO and codes) and the unit's half of it
     auto chunk_of = [&](uint32_t tn, uint32_t kt) { return (p.halves == 2 ? tn >> 1 : tn) * KT + kt; };
 
@@ -486,7 +481,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             // ---------------------------------------------------------------- producer of the dense arrays
             uint32_t issued = 0;
             bool ok = true;
-            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+            for (UnitIter w(u_begin, KT, p.shares.by_kt); w.u < u_end; w.next(S, KT)) {
                 const uint32_t full = bar_full + 8 * w.s;
                 if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
                 const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
@@ -517,7 +512,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             const uint32_t x_half = p.nmma * 128;                          // bytes of 64 K values of every batch row
             asm volatile("prefetch.tensormap [%0];" ::"l"(&xmap) : "memory");
             asm volatile("griddepcontrol.wait;" ::: "memory");
-            for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+            for (UnitIter w(u_begin, KT, p.shares.by_kt); w.u < u_end; w.next(S, KT)) {
                 const uint32_t full = bar_x_full + 8 * w.s;
                 if (!wait_converged(bar_empty + 8 * w.s, w.ph ^ 1, abort_flag, p.status)) { ok = false; break; }
                 const uint32_t st = smem_u32(smem) + w.s * p.stage_bytes;
@@ -547,15 +542,15 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                     if (!wait_converged(bar_a_full + 8 * ab, (it / NAB) & 1, abort_flag, p.status)) break;
                 }
                 tc_fence_after();
-                const uint32_t sn = s + 1 == S ? 0 : s + 1, phn = sn ? ph : ph ^ 1;
                 // the next unit's barriers, tested while this one's MMAs are issued
-                const uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) & (XB ? mbar_test_wait(bar_x_full + 8 * sn, phn) : 1u) &
+                uint32_t seen = mbar_test_wait(bar_a_full + 8 * (nx % NAB), (nx / NAB) & 1) &
                                       (nx < NDB ? 1u : mbar_test_wait(bar_d_free + 8 * (nx % NDB), (nx / NDB - 1) & 1));
                 const uint32_t d = tmem_base + S_::D_BASE + db * (GPS * NR);
                 umma_dense(d, d + (GPS - 1) * NR, GPS == 1, tmem_base + ab * 64, xd, xd + x_half, (uint32_t)(xd0 >> 32), idesc, bar_d_full + 8 * db,
                            bar_a_empty + 8 * ab, bar_empty + 8 * s);
-                xd = sn ? xd + stage : (uint32_t)xd0;
-                s = sn, ph = phn;
+                xd += stage;
+                if (++s == S) s = 0, xd = (uint32_t)xd0, ph ^= XB;
+                if (XB) seen &= mbar_test_wait(bar_x_full + 8 * s, ph);
                 ready = __all_sync(0xffffffffu, seen);
             }
             if (elect_one()) umma_commit(bar_final);     // fires when every MMA this warp issued has retired
@@ -566,7 +561,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
             const uint64_t wo0 = desc_plain(smem_u32(smem) + p.off_wo, 2048), xd0 = desc_sw128(smem_u32(smem));
             const uint32_t x_half = (p.nmma * 128) >> 4, stage = p.stage_bytes >> 4, o = tmem_base + S_::O_BASE;
             const uint32_t units = u_end - u_begin, parts = p.parts;
-            uint32_t s = 0, ph = 0, wb = 0, wph = 0, xd = (uint32_t)xd0, acc = 0, left = KT - u_begin % KT, piece = 0;    // left: units to the end of the tile
+            uint32_t s = 0, ph = 0, wb = 0, wph = 0, xd = (uint32_t)xd0, acc = 0, left = KT - (u_begin - p.shares.by_kt(u_begin) * KT), piece = 0;    // left: units to the end of the tile
             bool ok = true, ready = false;
             for (uint32_t it = 0; it < units && ok; ++it) {
                 if (!ready && !(wait_converged(bar_x_full + 8 * s, ph, abort_flag, p.status) &&
@@ -607,7 +602,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         const uint32_t t_a = tmem_base_of() + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t col = (warp & 3) * 32 + lane;
         const bool stage_first = NR < 128 || S >= S_::kStageFirst;
-        for (UnitIter w(u_begin, KT); w.u < u_end; w.next(S, KT)) {
+        for (UnitIter w(u_begin, KT, p.shares.by_kt); w.u < u_end; w.next(S, KT)) {
             if (w.it % UG != ug) continue;
             const uint32_t ab = w.it % NAB;
             const uint8_t* st = smem + w.s * p.stage_bytes;
@@ -664,8 +659,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 #pragma unroll
         for (int i = 0; i < RT; ++i) acc[i] = 0.0f;
         bool ok = true;
-        UnitIter w(u_begin, KT);
-        uint32_t tn = u_begin / KT, piece = 0;
+        UnitIter w(u_begin, KT, p.shares.by_kt);
+        uint32_t tn = p.shares.by_kt(u_begin), piece = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // outer loop: the pieces of this CTA's range (a piece = its units of one column tile)
         for (uint32_t piece_first = u_begin; piece_first < u_end && ok; ++tn, ++piece) {
@@ -724,15 +719,15 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 // counter each); the last to arrive adds the partials in CTA order (the same order in every run) and writes Y:
                 // this warp, or the whole CTA if the range ends here (COOP).
                 constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;      // float4 per slot
-                const uint32_t which = (p.split || u_begin / KT == tn) ? 0u : 1u;
+                const uint32_t which = p.shares.slot_of(blockIdx.x, tn, KT);
                 float4* slots = reinterpret_cast<float4*>(p.partials) + (size_t)(r0 / 4) * COLS + col;
                 float4* slot = slots + ((size_t)blockIdx.x * 2 + which) * SLOT;
 #pragma unroll
                 for (int i = 0; i < RT / 4; ++i)
                     if (r0 + 4 * i < p.M) __stcg(slot + i * COLS, make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]));
                 __syncwarp();
-                const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q, r);
-                const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q, r);
+                uint32_t c_first, c_last;
+                p.shares.owners(tn, KT, c_first, c_last);
                 uint32_t* counter = p.counters + tn * 4 + dw;
                 uint32_t last = 0;
                 if (lane == 0) {
@@ -747,9 +742,9 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 __syncwarp();
                 if (COOP && last && lane == 0) {
                     atomicSub(counter, (c_last - c_first + 1) << (8 * set));                     // ready for the next call
-                    if (piece_stop == u_end) atomicOr(settle, 1u << (set * 4 + dw));
+                    if (DEFER || piece_stop == u_end) atomicOr(settle + (piece_stop == u_end ? 0 : 1), 1u << (set * 4 + dw));
                 }
-                if (last && !(COOP && piece_stop == u_end)) {
+                if (!DEFER && last && !(COOP && piece_stop == u_end)) {
                     write_y = true;
                     // 16 rows at a time, ND contributors' loads in flight; the additions keep CTA order
                     constexpr int ND = NR >= 64 || !COOP ? 2 : 1;
@@ -763,7 +758,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
 #pragma unroll
                                 for (int dd = 0; dd < ND; ++dd) {
                                     const uint32_t cc = min(c + dd, c_last);
-                                    const uint32_t wch = (p.split || unit_begin_of(cc, q, r) / KT == tn) ? 0u : 1u;
+                                    const uint32_t wch = p.shares.slot_of(cc, tn, KT);
                                     const float4* sl = slots + ((size_t)cc * 2 + wch) * SLOT;
 #pragma unroll
                                     for (int i = 0; i < 4; ++i) v[dd][i] = __ldcg(sl + (i0 + i) * COLS);
@@ -817,20 +812,21 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         tmem_dealloc(tmem_base_of(), kTmemCols);
     }
     if constexpr (COOP) {
-        if (const uint32_t mine = *settle) {
+        for (uint32_t side = 0; side < (DEFER ? 2u : 1u); ++side) {
+            const uint32_t mine = settle[side];
+            if (!mine) continue;
             // The sums of the range's last tile (the drain warps' acquire is handed on by the barrier above): a thread takes four
             // rows of a column, with ND contributors' loads in flight.
             constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;
             constexpr int ND = 6;
-            uint32_t cta = blockIdx.x, ctas = P;
-            if (NR >= 64) {                                   // the range anew, so that nothing of it is kept in registers until here
+            uint32_t begin = u_begin, end = u_end, c_first, c_last;
+            if (NR >= 32) {                                   // the range anew, so that nothing of it is kept in registers until here
+                uint32_t cta;
                 asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
-                asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(ctas));
+                p.shares.range(cta, p.KT, begin, end);
             }
-            const uint32_t q2 = U / ctas, r2 = U % ctas;
-            const uint32_t tn = NR < 64 ? (u_end - 1) / KT : (p.split ? cta / p.split : (unit_begin_of(cta + 1, q2, r2) - 1) / KT), u_tile0 = tn * KT;
-            const uint32_t c_first = p.split ? tn * p.split : cta_of_unit(u_tile0, q2, r2);
-            const uint32_t c_last = p.split ? c_first + p.split - 1 : cta_of_unit(u_tile0 + KT - 1, q2, r2);
+            const uint32_t tn = p.shares.by_kt(side ? begin : end - 1);
+            p.shares.owners(tn, p.KT, c_first, c_last);
             const float4* slots = reinterpret_cast<const float4*>(p.partials);
             for (uint32_t e = threadIdx.x; e < (p.M + 3) / 4 * COLS; e += blockDim.x) {
                 const uint32_t i = e / COLS, col = e % COLS;
@@ -840,7 +836,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                     float4 v[ND];
 #pragma unroll
                     for (int d = 0; d < ND; ++d) {
-                        const uint32_t wch = (p.split || unit_begin_of(c + d, q2, r2) / KT == tn) ? 0u : 1u;
+                        const uint32_t wch = p.shares.slot_of(c + d, tn, p.KT);
                         if (c + d <= c_last) v[d] = __ldcg(slots + ((size_t)(c + d) * 2 + wch) * SLOT + e);
                     }
 #pragma unroll
