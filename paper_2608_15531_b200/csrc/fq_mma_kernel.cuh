@@ -55,6 +55,17 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// the same with an accumulator that starts at zero
+__device__ __forceinline__ void mma_bf16_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.0f));
+}
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+
 constexpr int kActWarps = 2;   // activation warps of the streaming kernel
 // Activation row in shared memory: 256 B, its sixteen 16-byte chunks stored at chunk ^ 4 in odd rows.
 // The fragment loads of a quarter warp (rows g and g + 1, four consecutive chunks each) then touch
@@ -310,13 +321,17 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             const uint8_t* st = smem + s * p.stage_bytes;
             {
             if (!warp_wait(bar_full + 8 * s, ph, abort_flag, p.status)) { ok = false; break; }
-            const uint32_t* wp = reinterpret_cast<const uint32_t*>(st) + (dw * 32 + g) * 4 + t;   // word t of column c0; the others 8 columns on
+            // Codes by ldmatrix: the 16 bytes of a column in a 32-row block are one row of a matrix, so that lane (g, t) gets
+            // word t of columns c0, c0 + 8, c0 + 16, c0 + 24 with one instruction.
+            const uint32_t wa = smem_u32(st) + (dw * 32 + lane) * 16;
             // chunk 4j + t of row g (+ 8 per octet): at (4j + t) ^ 4 in odd rows, i.e. 64 B further for
             // even j and 64 B back for odd j
             const uint8_t* xrow = st + p.off_xcan + g * kXPitch + t * 16;
             const uint8_t* xrow_e = xrow + ((g & 1) << 6);
             const uint8_t* xrow_o = xrow - ((g & 1) << 6);
-            const uint16_t* sc = reinterpret_cast<const uint16_t*>(st + p.off_sz);
+            // Scales and zero-points likewise: eight times the same 16 bytes (eight columns) as the rows of a matrix, and its
+            // transpose gives every lane of group g column c0's value, twice.
+            const uint32_t sza = smem_u32(st) + p.off_sz + (dw * 32 + (lane & 24)) * 2;
             const float* xsum = reinterpret_cast<const float*>(st + p.off_xsum);
             // outliers: the bucket descriptor and the first two (MS != 8: four) packets are requested now and used
             // after the dense math of the unit.  A bucket's packets are column-slotted: slot j of a packet
@@ -379,32 +394,32 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
             for (int gi = 0; gi < GPS; ++gi) {
                 float accg[MO][CG][4];
 #pragma unroll
-                for (int o = 0; o < MO; ++o)
-#pragma unroll
-                    for (int cg = 0; cg < CG; ++cg)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) accg[o][cg][i] = 0.0f;
-#pragma unroll
                 for (int j = gi * (4 / GPS); j < (gi + 1) * (4 / GPS); ++j) {
                     uint4 xb[MO];
 #pragma unroll
                     for (int o = 0; o < MO; ++o) xb[o] = *reinterpret_cast<const uint4*>(((j & 1) ? xrow_o : xrow_e) + o * 8 * kXPitch + j * 64);
-                    const uint4 w4 = make_uint4(wp[j * BN * 4], wp[j * BN * 4 + 32], wp[j * BN * 4 + 64], wp[j * BN * 4 + 96]);   // columns +0, +8, +16, +24
+                    uint32_t w4[4];                           // columns +0, +8, +16, +24
+                    ldmatrix_x4(wa + j * BN * 16, w4);
 #pragma unroll
                     for (int cg = 0; cg < CG; ++cg) {
-                        const uint32_t wa = cg ? w4.z : w4.x, wb = cg ? w4.w : w4.y;
-                        const uint32_t a0 = codes_to_bf16x2(wa), a1 = codes_to_bf16x2(wa >> 4);
-                        const uint32_t a2 = codes_to_bf16x2(wa >> 8), a3 = codes_to_bf16x2(wa >> 12);
-                        const uint32_t b0 = codes_to_bf16x2(wb), b1 = codes_to_bf16x2(wb >> 4);
-                        const uint32_t b2 = codes_to_bf16x2(wb >> 8), b3 = codes_to_bf16x2(wb >> 12);
+                        const uint32_t w0 = w4[2 * cg], w1 = w4[2 * cg + 1];
+                        const uint32_t a0 = codes_to_bf16x2(w0), a1 = codes_to_bf16x2(w0 >> 4);
+                        const uint32_t a2 = codes_to_bf16x2(w0 >> 8), a3 = codes_to_bf16x2(w0 >> 12);
+                        const uint32_t b0 = codes_to_bf16x2(w1), b1 = codes_to_bf16x2(w1 >> 4);
+                        const uint32_t b2 = codes_to_bf16x2(w1 >> 8), b3 = codes_to_bf16x2(w1 >> 12);
 #pragma unroll
                         for (int o = 0; o < MO; ++o) {
-                            mma_bf16(accg[o][cg], a0, b0, a1, b1, xb[o].x, xb[o].y);   // rows 8t+0..3 of the block
-                            mma_bf16(accg[o][cg], a2, b2, a3, b3, xb[o].z, xb[o].w);   // rows 8t+4..7
+                            // rows 8t+0..3 of the block, then 8t+4..7
+                            if (j == gi * (4 / GPS)) mma_bf16_first(accg[o][cg], a0, b0, a1, b1, xb[o].x, xb[o].y);
+                            else mma_bf16(accg[o][cg], a0, b0, a1, b1, xb[o].x, xb[o].y);
+                            mma_bf16(accg[o][cg], a2, b2, a3, b3, xb[o].z, xb[o].w);
                         }
                     }
                 }
                 // once per group: acc += s * (sum x (128+q) - (128+z) sum x)     (Eq. 3 inside Eq. 1)
+                uint32_t s4[4], z4[4];
+                ldmatrix_x4_trans(sza + gi * SZ_ROW, s4[0], s4[1], s4[2], s4[3]);
+                ldmatrix_x4_trans(sza + (GPS + gi) * SZ_ROW, z4[0], z4[1], z4[2], z4[3]);
                 float2 xs[MO];
 #pragma unroll
                 for (int o = 0; o < MO; ++o) xs[o] = *reinterpret_cast<const float2*>(xsum + gi * LDC + o * 8 + 2 * t);
@@ -412,9 +427,8 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
                 for (int cg = 0; cg < CG; ++cg)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const int col = c0 + 16 * cg + 8 * h;
-                        const float sv = bf16_bits_to_float(sc[gi * BN + col]);
-                        const float zc = -(128.0f + bf16_bits_to_float(sc[(GPS + gi) * BN + col]));
+                        const float sv = bf16hi(s4[2 * cg + h]);
+                        const float zc = -(128.0f + bf16hi(z4[2 * cg + h]));
 #pragma unroll
                         for (int o = 0; o < MO; ++o) {
                             accf[o][cg][2 * h + 0] = fmaf(sv, fmaf(zc, xs[o].x, accg[o][cg][2 * h + 0]), accf[o][cg][2 * h + 0]);
