@@ -135,6 +135,14 @@ __global__ void __launch_bounds__(32 * (1 + kActWarps + NGRP * (BN / 32)), 1) fq
     // only weights, which no kernel writes while calls are in flight.  (The activation warps first
     // request the other weight arrays of their first units, see there.)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    {
+        // The activations into the L2, by all CTAs together, before the wait: they may have been written long ago, and a step's weights
+        // stream through the L2 meanwhile.  Only a hint: if the grid before writes them it writes to the same L2, and they are
+        // read after the wait.  (4096 x 28672 at one row 20.3 us, so 20.1; 14336 x 4096 at eight 15.3 and 15.2.  In the tcgen05 kernel 4096 x
+        // 28672 at 16 rows 28.1 and 28.7, in the short-job kernel 8192 x 1024 at one 7.6 and 8.0: not there.)
+        const size_t at = (size_t)(blockIdx.x * blockDim.x + threadIdx.x) * 64;
+        if (at < (size_t)p.M * p.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.X + at));
+    }
     if (warp >= DW0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const uint32_t KT = p.KT;
