@@ -408,15 +408,18 @@ static int sm_count_cached() {
 }
 
 // How the NT x KT units of a launch are shared out over persistent CTAs: split = 0, one contiguous range each; else a tile-aligned
-// split, every column tile to `split` CTAs, when that costs at most one more unit per CTA: then no CTA has to settle two
-// split tiles in a row.
+// split, every column tile to `split` CTAs, when that costs at most `slack` more units per CTA: then no CTA has to settle two
+// split tiles in a row.  us, ranges / tiles: two units more in the streaming kernel 8192 x 8192 at one row 14.7 / 13.6, at eight 16.5 / 16.1,
+// but seven more 28672 x 8192 33.9 / 36.0; in the tcgen05 kernel three or four more at 64 rows and groups of 128 5120 x 5120 16.2 / 14.8, 11008 x 4096 20.7 /
+// 19.4, 14336 x 4096 23.6 / 22.7, 8192 x 8192 24.3 / 23.9, six more 13824 x 5120 25.9 / 26.7; otherwise one, at 32 rows three more 14336 x
+// 4096 18.6 / 19.0, at 128 33.6 / 34.1, with groups of 64 at 24 19.2 / 20.3.
 struct Split {
     uint32_t grid, split, units_per_cta;
 };
-static Split split_units(uint32_t NT, uint32_t KT, int sms) {
+static Split split_units(uint32_t NT, uint32_t KT, int sms, uint32_t slack) {
     const uint32_t grid = std::min<uint32_t>({(uint32_t)sms, kMaxCtas, NT * KT}), units_per_cta = (NT * KT + grid - 1) / grid;
     const uint32_t c = std::min<uint32_t>(grid / NT, KT);
-    if (c >= 2 && (KT + c - 1) / c <= units_per_cta + 1) return {NT * c, c, (KT + c - 1) / c};
+    if (c >= 2 && (KT + c - 1) / c <= units_per_cta + slack) return {NT * c, c, (KT + c - 1) / c};
     return {grid, 0, units_per_cta};
 }
 static Shares shares_of(const Split& sp, uint32_t NT, uint32_t KT) {
@@ -438,7 +441,7 @@ struct TcPlan {
 // of 128 4096 x 4096 11.9 / 12.3, 4096 x 28672 36.4 / 37.4, 14336 x 4096, with five CTAs to a tile, 24.1 / 23.9.  Beyond, at 128: 14336 x
 // 4096 35.7 / 34.3, 4096 x 4096 17.7 / 17.4, but 4096 x 28672, where a CTA has a tile and a half, 53.6 / 55.1.)
 static inline bool tc_coop(uint32_t nr, uint32_t group, uint32_t KT, uint32_t units_per_cta) {
-    return nr <= 32 || (nr == 64 ? group == 64 || KT >= 8 * units_per_cta : KT >= 2 * units_per_cta);
+    return nr <= 32 || (nr == 64 ? KT >= (group == 64 ? 1 : 8) * units_per_cta : KT >= 2 * units_per_cta);
 }
 
 static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
@@ -452,7 +455,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     p.halves = L->BN / 128;
     p.nmma = round_up(M, 16);
     p.parts = L->value_type == FQ_VALUE_FP16 ? 2 : 1;
-    const Split sp = split_units(p.NT, p.KT, sms);
+    const Split sp = split_units(p.NT, p.KT, sms, pl.nr == 64 && L->group == 128 ? 4 : 1);
     p.shares = shares_of(sp, p.NT, p.KT);
     p.off_w = 256 * p.nmma;
     p.off_sz = p.off_w + 8192;
@@ -566,7 +569,7 @@ static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers)
     const bool tails = L->max_tail_packets > 0;
     if (rows >= 9) return tails || (units >= 512 && !(KT <= 16 && depth <= 9 && direct_warps(L, rows, true)));
     if (L->BN != 128 || rows < 2 || units < 1024 || direct_warps(L, rows, true)) return false;
-    if (tails || split_units(L->N / 128, KT, sm_count_cached()).units_per_cta < kTwoGroups) return true;
+    if (tails || split_units(L->N / 128, KT, sm_count_cached(), 1).units_per_cta < kTwoGroups) return true;
     return rows <= 4 ? units >= 4096 && depth <= 13 : units >= 3072 || (units >= 2048 && depth > 10 && depth <= 18);
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool outliers) { return tc_serves(L, rows_left, outliers) ? rows_left : std::min<uint32_t>(rows_left, 16u); }
@@ -619,7 +622,7 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     // the outlier step of that variant prefetches less (96 registers per thread).
     const int sms = sm_count_cached();
     if (sms <= 0) return fail(FQ_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
-    const Split sp = split_units(p.NT, p.KT, sms);
+    const Split sp = split_units(p.NT, p.KT, sms, 2);
     p.shares = shares_of(sp, p.NT, p.KT);
     pl.ngrp = sp.units_per_cta >= kTwoGroups ? 2 : 1;
     const uint32_t xch_bytes = pl.ngrp > 1 ? BN * ROWS * 4 : 0;   // hand-over of a group's partial sums
