@@ -437,11 +437,13 @@ struct TcPlan {
     bool coop;      // the CTA, not its drain warps, finishes a split tile at the end of its range
 };
 
-// (See the kernel.  us, by the drain warps / by the CTA.  33 to 64 rows, at 64: groups of 64 2944 x 11136 at 48 rows 17.4 / 16.7, 8192 x 28672 69.4 / 69.0; groups
+// (See the kernel.  us, by the drain warps / by the CTA.  33 to 64 rows: groups of 64 2944 x 11136 at 48 17.4 / 16.7, 8192 x 28672, 97 units a CTA, at 40
+// 66.9 / 65.9 and at 64 69.5 / 69.1, but 4096 x 28672, 49 units, at 64 40.1 / 40.5; at 64, groups
 // of 128 4096 x 4096 11.9 / 12.3, 4096 x 28672 36.4 / 37.4, 14336 x 4096, with five CTAs to a tile, 24.1 / 23.9.  Beyond, at 128: 14336 x
 // 4096 35.7 / 34.3, 4096 x 4096 17.7 / 17.4, but 4096 x 28672, where a CTA has a tile and a half, 53.6 / 55.1.)
 static inline bool tc_coop(uint32_t nr, uint32_t group, uint32_t KT, uint32_t units_per_cta) {
-    return nr <= 32 || (nr == 64 ? KT >= (group == 64 ? 1 : 8) * units_per_cta : KT >= 2 * units_per_cta);
+    if (nr == 64) return group == 64 ? KT >= units_per_cta || units_per_cta >= 64 : KT >= 8 * units_per_cta;
+    return nr <= 32 || KT >= 2 * units_per_cta;
 }
 
 static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
