@@ -11,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfq.so")
 SOURCES = [os.path.join(CSRC, "fq_host.cpp"), os.path.join(CSRC, "fq_kernels.cu")]
-HEADERS = [os.path.join(CSRC, "fq_internal.h"), os.path.join(CSRC, "fq_tc_kernel.cuh"), os.path.join(CSRC, "fq_mma_kernel.cuh"),
+HEADERS = [os.path.join(CSRC, "fq_internal.h"), os.path.join(CSRC, "fq_shares.h"), os.path.join(CSRC, "fq_tc_kernel.cuh"), os.path.join(CSRC, "fq_mma_kernel.cuh"),
            os.path.join(CSRC, "fq_direct_kernel.cuh"), os.path.join(ROOT, "include", "fq.h")]
 
 NVCC_FLAGS = [

@@ -1,0 +1,94 @@
+"""How a launch's units are shared out over its CTAs, gone through on the CPU: the structs are compiled for the host.  CPU only."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_PROGRAM = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include <vector>
+#include "fq_shares.h"
+using namespace fq;
+#define CHECK(c, ...) do { if (!(c)) { std::printf("%s: ", #c); std::printf(__VA_ARGS__); std::printf("\n"); std::exit(1); } } while (0)
+
+static void divisors() {
+    std::mt19937 rng(1);
+    std::vector<uint32_t> ds;
+    for (uint32_t d = 1; d <= 4096; ++d) ds.push_back(d);
+    for (int b = 12; b < 32; ++b)
+        for (int e = -1; e <= 1; ++e) ds.push_back((1u << b) + e);
+    for (int i = 0; i < 20000; ++i) ds.push_back((rng() >> (rng() % 32)) | 1u);
+    ds.push_back(~0u), ds.push_back(~0u - 1);
+    for (uint32_t d : ds) {
+        const Divisor by = Divisor::of(d);
+        const auto at = [&](uint32_t n) { CHECK(by(n) == n / d, "%u / %u", n, d); };
+        const uint32_t top = ~0u / d * d;                      // the largest multiple
+        for (uint32_t n : {0u, 1u, d - 1, d, d + 1, top - 1, top, ~0u - 1, ~0u}) at(n);
+        for (int i = 0; i < 200; ++i) {
+            const uint32_t n = rng(), m = n / d * d;
+            at(n), at(m), at(m - 1);
+        }
+    }
+}
+
+static void plan(uint32_t NT, uint32_t KT, uint32_t sms, uint32_t slack) {
+    const Split sp = split_units(NT, KT, sms, slack);
+    const Shares sh = shares_of(sp, NT, KT);
+    const uint32_t even = (NT * KT + std::min(sms, kMaxCtas) - 1) / std::min(sms, kMaxCtas);
+    std::vector<uint32_t> first(NT, ~0u), last(NT, 0);
+    uint32_t at = 0, longest = 0;
+    CHECK(sp.grid >= 1 && sp.grid <= std::min(sms, kMaxCtas), "%u x %u: %u CTAs", NT, KT, sp.grid);
+    for (uint32_t c = 0; c < sp.grid; ++c) {
+        uint32_t begin, end;
+        sh.range(c, KT, begin, end);
+        CHECK(begin == at && end > begin, "%u x %u: CTA %u has [%u, %u) behind %u", NT, KT, c, begin, end, at);
+        at = end;
+        longest = std::max(longest, end - begin);
+        int slots[2] = {0, 0};
+        for (uint32_t tn = begin / KT; tn <= (end - 1) / KT; ++tn) {
+            first[tn] = std::min(first[tn], c), last[tn] = std::max(last[tn], c);
+            const bool whole = begin <= tn * KT && end >= (tn + 1) * KT;
+            if (!whole) {
+                const uint32_t s = sh.slot_of(c, tn, KT);
+                CHECK(s < 2 && ++slots[s] == 1, "%u x %u: CTA %u, tile %u, slot %u", NT, KT, c, tn, s);
+            }
+        }
+        CHECK(!sp.split || begin / KT == (end - 1) / KT, "%u x %u: CTA %u has parts of two tiles", NT, KT, c);
+    }
+    CHECK(at == NT * KT, "%u x %u: %u units dealt out", NT, KT, at);
+    CHECK(longest == sp.units_per_cta && longest <= even + (sp.split ? slack : 0u), "%u x %u: %u units", NT, KT, longest);
+    for (uint32_t tn = 0; tn < NT; ++tn) {
+        uint32_t a, b;
+        sh.owners(tn, KT, a, b);
+        CHECK(a == first[tn] && b == last[tn], "%u x %u: tile %u of CTAs %u to %u, said to be of %u to %u", NT, KT, tn, first[tn], last[tn], a, b);
+        CHECK(b - a < 255, "%u x %u: contributors of tile %u", NT, KT, tn);       // (arrivals are counted in bytes)
+    }
+}
+
+int main() {
+    divisors();
+    for (uint32_t sms : {148u, 132u, 1u, 7u, 192u, 300u})
+        for (uint32_t KT = 1; KT <= 224; KT += sms == 148 ? 1 : 13)
+            for (uint32_t NT = 1; NT <= 448; NT += sms == 148 ? 1 : 11)
+                for (uint32_t slack : {0u, 1u, 2u, 4u}) plan(NT, KT, sms, slack);
+    for (uint32_t NT : {1023u, 1024u, 2048u})
+        for (uint32_t KT : {1u, 2u, 73u, 1024u}) plan(NT, KT, 148, 1);
+    std::printf("ok\n");
+}
+"""
+
+
+@pytest.mark.skipif(subprocess.run(["which", "g++"], capture_output=True).returncode != 0, reason="no C++ compiler")
+def test_ranges_owners_slots_and_division(tmp_path):
+    """Every unit belongs to one CTA; the owners of a tile are those that have units of it; no CTA uses a slot twice; the
+    divisions by multiplication are exact."""
+    src, exe = tmp_path / "shares.cpp", tmp_path / "shares"
+    src.write_text(_PROGRAM)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "paper_2608_15531_b200", "csrc"), "-I", os.path.join(ROOT, "include"),
+                    "-o", str(exe), str(src)], check=True)
+    p = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert p.returncode == 0 and p.stdout == "ok\n", p.stdout
