@@ -35,30 +35,32 @@ def shape(nr, gps, nmma):
     ug, sg = 3 if nr == 16 else 2, 3 if nr <= 32 else 2 if nr <= 64 else 1
     stage = -(-(256 * nmma + 8192 + 512 * gps) // 1024) * 1024
     s = min(12, (232448 - 2048 - (2 if sg == 1 else sg) * 32768) // stage)
-    return dict(S=s - s % ug if s >= 2 * ug else s, UG=ug, NAB=nab, NDB=ndb)
+    return dict(S=s - s % ug if s >= 2 * ug else s, UG=ug, NAB=nab, NDB=ndb, XB=nr <= 32)
 
 
-def run(S, UG, NAB, NDB, units, order, rng):
-    full, empty = [Barrier(1) for _ in range(S)], [Barrier(4) for _ in range(S)]
+def run(S, UG, NAB, NDB, XB, units, order, rng, drop=None):
+    """XB: the activations' arrival in a stage has barriers of its own; else both producers arrive on the stage's one."""
+    full, empty = [Barrier(1 if XB else 2) for _ in range(S)], [Barrier(4) for _ in range(S)]
+    x_full = [Barrier(1) for _ in range(S)] if XB else full
     a_full, a_empty = [Barrier(1) for _ in range(NAB)], [Barrier(1) for _ in range(NAB)]
     d_full, d_free = [Barrier(1) for _ in range(NDB)], [Barrier(1) for _ in range(NDB)]
-    mmas, loads = [], []                                   # issued, not yet complete
+    mmas = []                                              # issued, not yet complete
+    codes_here, x_here = set(), set()                      # units whose copies have landed
 
-    def stage_free(it):
-        return it < S or empty[it % S].passes(it // S - 1)
-
-    def producer():
+    def producer(loads):
         for it in range(units):
-            while not stage_free(it):
+            while it >= S and not empty[it % S].passes(it // S - 1):
                 yield
             loads.append(it)
             yield
 
-    def landing():                                         # copies land in any order
+    def landing(loads, barriers, here):                    # copies land in any order, those of the two producers independently
         done = 0
         while done < units:
             if loads:
-                full[loads.pop(rng.randrange(len(loads))) % S].arrive()
+                it = loads.pop(rng.randrange(len(loads)))
+                here.add(it)
+                barriers[it % S].arrive()
                 done += 1
             yield
 
@@ -74,6 +76,7 @@ def run(S, UG, NAB, NDB, units, order, rng):
                 yield
             if not mine:
                 continue
+            assert it in codes_here, "codes are not here"
             yield
             if order != "operand first" and it >= NAB:
                 while not a_empty[ab].passes(it // NAB - 1):
@@ -83,13 +86,22 @@ def run(S, UG, NAB, NDB, units, order, rng):
             empty[it % S].arrive()
 
     def dense():
+        ready = False
         for it in range(units):
-            while it >= NDB and not d_free[it % NDB].passes(it // NDB - 1):
-                yield
-            while not a_full[it % NAB].passes(it // NAB):
-                yield
-            assert full[it % S].phase > it // S            # (waited for by the unpack group)
+            if not ready:
+                while it >= NDB and not d_free[it % NDB].passes(it // NDB - 1):
+                    yield
+                while XB and drop != "dense warp's wait for X" and not x_full[it % S].passes(it // S):
+                    yield
+                while not a_full[it % NAB].passes(it // NAB):
+                    yield
+            assert it in x_here, "the dense MMAs' activations are not here"     # (without XB the unpack group has waited for them)
+            nx = it + 1                                    # the next unit's barriers, looked at once
+            ready = nx < units and a_full[nx % NAB].passes(nx // NAB) and (nx < NDB or d_free[nx % NDB].passes(nx // NDB - 1))
+            yield
             mmas.append(it)
+            if XB and drop != "dense warp's wait for X" and nx < units:
+                ready = x_full[nx % S].passes(nx // S) and ready
             yield
 
     def tensor_pipe():                                     # MMAs retire in order
@@ -105,6 +117,7 @@ def run(S, UG, NAB, NDB, units, order, rng):
         for it in range(units):
             while not full[it % S].passes(it // S):
                 yield
+            assert it in codes_here, "scales are not here"
             empty[it % S].arrive()
             while not d_full[it % NDB].passes(it // NDB):
                 yield
@@ -112,12 +125,15 @@ def run(S, UG, NAB, NDB, units, order, rng):
 
     def outliers():
         for it in range(units):
-            while not full[it % S].passes(it // S):
+            while drop != "outlier warp's wait for X" and not x_full[it % S].passes(it // S):
                 yield
+            assert it in x_here, "the outlier MMAs' activations are not here"
             yield
             empty[it % S].arrive()
 
-    procs = [producer(), landing(), dense(), tensor_pipe(), drain(), outliers()] + [unpack(g) for g in range(UG)]
+    codes, xs = [], []                                     # copies under way
+    procs = [producer(codes), producer(xs), landing(codes, full, codes_here), landing(xs, x_full, x_here), dense(), tensor_pipe(), drain(),
+             outliers()] + [unpack(g) for g in range(UG)]
     weight = [10 ** rng.uniform(-2, 0) for _ in procs]     # some much slower than others
     live = list(range(len(procs)))
     for _ in range(4000 * units):
@@ -154,3 +170,13 @@ def test_the_ring_of_three_stages_needs_the_operand_first(order):
     with pytest.raises(AssertionError, match="phase"):
         for _ in range(400):
             run(**sh, units=30, order=order, rng=rng)
+
+
+@pytest.mark.parametrize("drop", ["dense warp's wait for X", "outlier warp's wait for X"])
+@pytest.mark.parametrize("nr", [16, 32])
+def test_neither_tensor_warp_may_drop_its_wait_for_the_activations(nr, drop):
+    """Up to 32 rows the unpack warps do not wait for X, so that nobody else's wait covers it."""
+    sh, rng = shape(nr, 1, nr), random.Random(2)
+    with pytest.raises(AssertionError, match=f"the {drop.split()[0]} MMAs' activations"):
+        for _ in range(400):
+            run(**sh, units=30, order="stage first", rng=rng, drop=drop)
