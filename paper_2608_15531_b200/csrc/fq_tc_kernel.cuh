@@ -399,7 +399,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
     constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG;
     constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
-    constexpr bool DEFER = COOP && NR == 32;
+    constexpr bool DEFER = COOP && (NR == 32 || (NR == 16 && GROUP == 64));
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
 
@@ -426,7 +426,9 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     volatile uint32_t* tmem_slot = abort_flag + 1;
     // COOP: strips and sets (bit strip + 4 set) that the CTA finishes on its way out, of its range's last tile and (DEFER) of its first, of
     // which it seldom is the last contributor.  With 32 rows the sums in the drain warps' loop cost it registers (4096 x 28672 32.3 us, so 31.1;
-    // 8192 x 28672 55.9 and 53.8); with 16 the sums of the first tile are better done at once (4096 x 28672 28.3 and 29.0).
+    // 8192 x 28672 55.9 and 53.8), with 16 and groups of 64 too, 20 bytes of spills (28672 x 8192 52.6, so 50.9; 4096 x 28672 29.5 and 28.9;
+    // but 8192 x 1024 at nine 7.6 and 7.8); with 16 and groups of 128 the sums of the first tile are better done at once (4096 x 28672
+    // 28.3 and 29.0).
     uint32_t* settle = const_cast<uint32_t*>(abort_flag) + 2;
 
     if (tid == 0) {
