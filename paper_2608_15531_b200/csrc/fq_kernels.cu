@@ -30,6 +30,7 @@ namespace fq {
 
 constexpr int kBK = 128;
 constexpr int kSmemBudget = 232448;    // 227 KB per CTA on sm_100
+constexpr uint32_t kSmemOneCta = 116736;   // of which no two CTAs fit on an SM: 228 KB, and 1 KB of a CTA is the system's
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 constexpr uint32_t kTmemCols = 512;
 
@@ -592,7 +593,11 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     pl.general = sparse && (L->max_tail_packets > 0 || L->max_tile_packets > cap || !L->tilecoo_encoded);
     p.off_shc = S * stage;
     p.off_bar = p.off_shc + xch_bytes;
-    pl.smem = p.off_bar + 1024;
+    // One CTA to an SM, also where two would fit: the next call's grid is there before this one ends (programmatic dependent launch), and if
+    // a grid has fewer CTAs than the GPU SMs, the free SMs take two of the next one's, which then last longest (us, two fit / one: without
+    // outliers on tiles of 128 columns 9472 x 1408, 143 CTAs, at one row 7.4 / 6.3, at 16 11.5 / 8.9, 6272 x 8832, 138 CTAs, 17.4 / 11.9; with them
+    // 8448 x 1152 at one 7.6 / 7.0; and of grids that fill the GPU 14336 x 4224 13.05 / 12.9, 1024 x 11136 6.3 / 6.2).
+    pl.smem = std::max<uint32_t>(p.off_bar + 1024, kSmemOneCta);
     pl.threads = 32 * (1 + kActWarps + pl.ngrp * NDW);
     pl.grid = sp.grid;
     return FQ_OK;
