@@ -362,8 +362,6 @@ static int sm_count_cached() {
     return cached[dev];
 }
 
-constexpr uint32_t kTwoGroups = 8;      // units per CTA from which the streaming kernel runs two groups of dense warps
-
 // The tcgen05 kernel's variant for a launch: the batch rows its tensor memory and drain warps are laid out for.
 static inline uint32_t tc_rows(uint32_t m) { return m <= 16 ? 16u : (m <= 32 ? 32u : (m <= 64 ? 64u : 128u)); }
 
@@ -393,7 +391,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     p.halves = L->BN / 128;
     p.nmma = round_up(M, 16);
     p.parts = L->value_type == FQ_VALUE_FP16 ? 2 : 1;
-    const Split sp = split_units(p.NT, p.KT, sms, pl.nr == 64 && L->group == 128 ? 4 : 1);
+    const Split sp = split_tc(p.NT, p.KT, sms, pl.nr, L->group);
     p.shares = shares_of(sp, p.NT, p.KT);
     p.off_w = 256 * p.nmma;
     p.off_sz = p.off_w + 8192;
@@ -560,7 +558,7 @@ static fq_status_t make_plan_mma(const fq_layout_t* L, uint32_t M, bool sparse, 
     // the outlier step of that variant prefetches less (96 registers per thread).
     const int sms = sm_count_cached();
     if (sms <= 0) return fail(FQ_ERR_CUDA, "no CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
-    const Split sp = split_units(p.NT, p.KT, sms, 2);
+    const Split sp = split_streaming(BN, p.NT, p.KT, sms, M, sparse);
     p.shares = shares_of(sp, p.NT, p.KT);
     pl.ngrp = sp.units_per_cta >= kTwoGroups ? 2 : 1;
     const uint32_t xch_bytes = pl.ngrp > 1 ? BN * ROWS * 4 : 0;   // hand-over of a group's partial sums

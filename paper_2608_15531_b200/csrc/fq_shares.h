@@ -63,10 +63,7 @@ struct Shares {
 
 // How the NT x KT units of a launch are shared out over persistent CTAs: split = 0, one contiguous range each; else a tile-aligned
 // split, every column tile to `split` CTAs, when that costs at most `slack` more units per CTA: then no CTA has to settle two
-// split tiles in a row.  us, ranges / tiles: two units more in the streaming kernel 8192 x 8192 at one row 14.7 / 13.6, at eight 16.5 / 16.1,
-// but seven more 28672 x 8192 33.9 / 36.0; in the tcgen05 kernel three or four more at 64 rows and groups of 128 5120 x 5120 16.2 / 14.8, 11008 x 4096 20.7 /
-// 19.4, 14336 x 4096 23.6 / 22.7, 8192 x 8192 24.3 / 23.9, six more 13824 x 5120 25.9 / 26.7; otherwise one, at 32 rows three more 14336 x
-// 4096 18.6 / 19.0, at 128 33.6 / 34.1, with groups of 64 at 24 19.2 / 20.3.
+// split tiles in a row.
 struct Split {
     uint32_t grid, split, units_per_cta;
 };
@@ -75,6 +72,33 @@ inline Split split_units(uint32_t NT, uint32_t KT, uint32_t sms, uint32_t slack)
     const uint32_t c = std::min<uint32_t>(grid / NT, KT);
     if (c >= 2 && (KT + c - 1) / c <= units_per_cta + slack) return {NT * c, c, (KT + c - 1) / c};
     return {grid, 0, units_per_cta};
+}
+constexpr uint32_t kTwoGroups = 8;      // units per CTA from which the streaming kernel runs two groups of dense warps
+
+// The streaming kernel's.  One unit more is always worth it, a second one where it costs less than the second split tile (about 1 us; with two CTAs to
+// a tile, and so the fewest CTAs, less).  us, ranges / tiles:
+//   the longer share brings the second group of dense warps: 2048 x 12800 at one row 9.7 / 8.5, at eight 11.0 / 9.9, 1920 x 7040 at eight
+//     9.4 / 7.6; without outliers also where both shares are short, 1664 x 14336 at eight 7.9 / 7.4, 2432 x 14080 8.9 / 8.4, with them not (1408 x 13312 9.2 / 9.4)
+//   up to four rows (one on tiles of 128 columns, whose units are worth half): three CTAs and more to a tile 8192 x 8192 at one 14.7 / 13.6, 8192 x 6400
+//     13.6 / 12.5, 18688 x 8960 26.5 / 26.0; two, up to 16 units, 3200 x 15616 12.5 / 12.0, 3840 x 15360 13.7 / 13.3, 2816 x 13824 10.2 / 10.6, beyond them
+//     5120 x 16384 16.0 / 16.1, 12288 x 17920 at four 34.8 / 35.6; without outliers up to 24, 6400 x 17152 15.8 / 15.4, 14976 x 18176 30.5 / 30.8
+//   five rows and more, and two to four on tiles of 128 columns: no (3328 x 14592 at eight 13.2 / 14.3, 24320 x 3840 20.5 / 21.5, 11520 x 4224 15.9 / 16.9,
+//     8192 x 6400 14.9 / 14.6; without outliers, where the CTAs of tiles read the same rows of X at a time, 15232 x 18432 at eight
+//     32.1 / 35.7, 10880 x 9088 at 16 23.5 / 25.9; 22656 x 2176 at four 15.9 / 16.2)
+// (Seven units more, 28672 x 8192 at one row: 33.9 / 36.0.)
+inline Split split_streaming(uint32_t BN, uint32_t NT, uint32_t KT, uint32_t sms, uint32_t rows, bool outliers) {
+    const Split one = split_units(NT, KT, sms, 1), two = split_units(NT, KT, sms, 2);
+    if (one.split || !two.split) return one;
+    const uint32_t units = one.units_per_cta;                 // of a range
+    if (units <= kTwoGroups && (two.units_per_cta >= kTwoGroups || !outliers)) return two;
+    if (rows <= (BN == 256 ? 4 : 1) && (two.split > 2 || units * BN < (outliers ? 16u : 24u) * 256)) return two;
+    return one;
+}
+// The tcgen05 kernel's.  us, ranges / tiles: three or four more at 33 to 64 rows and groups of 128, 5120 x 5120 16.2 / 14.8, 11008 x 4096 20.7 / 19.4, 2176 x
+// 6400 13.9 / 11.4, 25344 x 9088 63.2 / 61.9, 3456 x 6400 at 40 13.1 / 13.3, six more 13824 x 5120 25.9 / 26.7; otherwise one: at 32 rows
+// three more 14336 x 4096 18.6 / 19.0, at 128 33.6 / 34.1, with groups of 64 at 24 19.2 / 20.3.
+inline Split split_tc(uint32_t NT, uint32_t KT, uint32_t sms, uint32_t nr, uint32_t group) {
+    return split_units(NT, KT, sms, nr == 64 && group == 128 ? 4 : 1);
 }
 inline Shares shares_of(const Split& sp, uint32_t NT, uint32_t KT) {
     const uint32_t q = NT * KT / sp.grid, r = NT * KT % sp.grid;

@@ -21,6 +21,15 @@ _SHAPES = [
     (2048, 2048, 0.01, (5, 8)),            # and 16 k-steps, 17 and more
     (2176, 2048, 0.01, (5, 8)),
     (6016, 4096, 0.01, (5, 8)),
+    (2048, 12800, 0.01, (1, 8)),           # streaming kernel, tiles for two units more: they bring the second group
+    (1664, 14336, 0.01, (4, 8)),           # one group either way: ranges with outliers and five rows or more, else tiles
+    (1664, 14336, 0.0, (1, 16)),
+    (8192, 6400, 0.01, (4, 5)),            # five CTAs to a tile up to four rows, ranges beyond
+    (3840, 15360, 0.01, (1, 5)),           # two, 15 units
+    (5120, 16384, 0.01, (1,)),             # two, 20 units: ranges, without outliers tiles
+    (5120, 16384, 0.0, (1, 5)),
+    (6272, 8832, 0.0, (1, 8)),             # tiles of 128 columns and a grid of fewer CTAs than SMs, ranges
+    (6528, 5504, 0.01, (1, 2)),
 ]
 
 

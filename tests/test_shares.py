@@ -69,8 +69,36 @@ static void plan(uint32_t NT, uint32_t KT, uint32_t sms, uint32_t slack) {
     }
 }
 
+// Plans that tests of the kernels name, on 148 SMs: CTAs to a tile (0: ranges) and units to a CTA
+static void named() {
+    const auto is = [](const Split& sp, uint32_t split, uint32_t units, int line) {
+        CHECK(sp.split == split && sp.units_per_cta == units, "line %d: %u, %u", line, sp.split, sp.units_per_cta);
+    };
+    const auto st = [](uint32_t K, uint32_t N, uint32_t rows, bool outliers) {
+        const uint32_t BN = N % 256 ? 128 : 256;
+        return split_streaming(BN, N / BN, K / 128, 148, rows, outliers);
+    };
+    for (uint32_t rows : {1u, 8u, 16u}) is(st(2048, 12800, rows, true), 2, 8, __LINE__);
+    is(st(2304, 7296, 5, true), 2, 9, __LINE__);
+    is(st(1664, 14336, 4, true), 2, 7, __LINE__);
+    is(st(1664, 14336, 8, true), 0, 5, __LINE__);
+    is(st(1664, 14336, 16, false), 2, 7, __LINE__);
+    is(st(8192, 6400, 4, true), 5, 13, __LINE__);
+    is(st(8192, 6400, 5, true), 0, 11, __LINE__);
+    is(st(3840, 15360, 1, true), 2, 15, __LINE__);
+    is(st(3840, 15360, 5, true), 0, 13, __LINE__);
+    is(st(5120, 16384, 1, true), 0, 18, __LINE__);
+    is(st(5120, 16384, 1, false), 2, 20, __LINE__);
+    is(st(5120, 16384, 5, false), 0, 18, __LINE__);
+    is(st(6272, 8832, 1, false), 2, 25, __LINE__);
+    is(st(6272, 8832, 8, false), 0, 23, __LINE__);
+    is(st(6528, 5504, 1, true), 3, 17, __LINE__);
+    is(st(6528, 5504, 2, true), 0, 15, __LINE__);
+}
+
 int main() {
     divisors();
+    named();
     for (uint32_t sms : {148u, 132u, 1u, 7u, 192u, 300u})
         for (uint32_t KT = 1; KT <= 224; KT += sms == 148 ? 1 : 13)
             for (uint32_t NT = 1; NT <= 448; NT += sms == 148 ? 1 : 11)
