@@ -371,13 +371,23 @@ struct TcPlan {
     bool coop;      // the CTA, not its drain warps, finishes a split tile at the end of its range
 };
 
-// (See the kernel.  us, by the drain warps / by the CTA.  33 to 64 rows: groups of 64 2944 x 11136 at 48 17.4 / 16.7, 8192 x 28672, 97 units a CTA, at 40
-// 66.9 / 65.9 and at 64 69.5 / 69.1, but 4096 x 28672, 49 units, at 64 40.1 / 40.5; at 64, groups
-// of 128 4096 x 4096 11.9 / 12.3, 4096 x 28672 36.4 / 37.4, 14336 x 4096, with five CTAs to a tile, 24.1 / 23.9.  Beyond, at 128: 14336 x
-// 4096 35.7 / 34.3, 4096 x 4096 17.7 / 17.4, but 4096 x 28672, where a CTA has a tile and a half, 53.6 / 55.1.)
-static inline bool tc_coop(uint32_t nr, uint32_t group, uint32_t KT, uint32_t units_per_cta) {
-    if (nr == 64) return group == 64 ? KT >= units_per_cta || units_per_cta >= 64 : KT >= 8 * units_per_cta;
-    return nr <= 32 || KT >= 2 * units_per_cta;
+// (See the kernel.  The CTA's sums cost one pass of its threads for each `threads` quads of rows of a column, the drain warps' one round trip for
+// two contributors, and the drain warps of a tile's first CTAs are done while the last ones still run.  us, by the drain warps / by the CTA:
+//   two CTAs to a tile in a split along the tiles, whose ends all come at once: 1536 x 9472 at 33 10.0 / 10.3, at 64 10.8 / 11.8, at 128 15.5 / 16.8
+//   three and more, or ranges shorter than a tile, up to 56 rows (two passes): 3072 x 5120 at 33 11.0 / 10.5, at 56 11.7 / 11.3, 4096 x 4096 at 48 11.3 / 11.0,
+//     2048 x 14336 at 48 16.1 / 15.8, 16384 x 5120 at 56 29.9 / 28.4, 8192 x 1024 at 48 15.5 / 11.9; but 1024 x 14336, a tile of eight units to ranges of
+//     seven, at 33 11.4 / 11.7
+//   57 to 64 rows (three passes): 4096 x 4096 at 64 12.0 / 12.5, 1024 x 1024, eight CTAs to a tile, 9.6 / 10.4, 2048 x 2048, nine, 11.4 / 11.3, 8192 x 1024, 18,
+//     16.2 / 15.0; ranges 4096 x 8192, 2.3 to a tile, 18.45 / 18.55, 5120 x 5120 with groups of 64, 3.6 to a tile, 17.3 / 16.9
+//   beyond: 3072 x 5120 at 65 14.9 / 13.8, at 128 17.2 / 17.05; ranges 1024 x 12800 at 128 18.1 / 18.9, 4096 x 8192 at 65 23.1 / 22.2, at 128 27.2 / 27.2
+// With groups of 64 and 33 to 64 rows the loop of this variant is 1 % faster a unit besides, so that it is taken for long ranges too: 2048 x 57344,
+// 65 units, at 33 39.3 / 38.6, at 64 41.35 / 41.5, 8192 x 38400, 130, 86.1 / 84.7 and 92.5 / 90.9, but 4096 x 28672, 49, at 64 40.1 / 40.6.)
+static inline bool tc_coop(uint32_t nr, uint32_t group, uint32_t rows, uint32_t threads, uint32_t KT, const Split& sp) {
+    const uint32_t units = sp.units_per_cta;
+    if (nr == 128) return sp.split ? sp.split > 2 : KT >= 2 * units;
+    if (nr <= 32 || (!sp.split && group == 64 && units >= 64)) return true;
+    if ((rows + 3) / 4 * 128 <= 2 * threads) return sp.split ? sp.split > 2 : KT >= units + 2;
+    return sp.split ? sp.split > 8 : KT >= 3 * units;
 }
 
 static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
@@ -404,7 +414,7 @@ static fq_status_t make_plan_tc(const fq_layout_t* L, uint32_t M, TcPlan& pl) {
     const int ug = tc_unpack_groups(pl.nr), sg = tc_scatter_groups(pl.nr);
     pl.threads = 32 * (4 + 4 * ug + 4 * std::max<uint32_t>(1, pl.nr / 32) + 4 * sg);     // as TcShape::WARPS
     pl.grid = sp.grid;
-    pl.coop = tc_coop(pl.nr, L->group, p.KT, sp.units_per_cta);
+    pl.coop = tc_coop(pl.nr, L->group, M, pl.threads, p.KT, sp);
     return FQ_OK;
 }
 

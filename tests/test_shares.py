@@ -74,6 +74,19 @@ static void named() {
     const auto is = [](const Split& sp, uint32_t split, uint32_t units, int line) {
         CHECK(sp.split == split && sp.units_per_cta == units, "line %d: %u, %u", line, sp.split, sp.units_per_cta);
     };
+    for (uint32_t nr : {16u, 32u, 64u, 128u})
+        for (uint32_t g : {64u, 128u}) {
+            const bool wide = nr == 64 && g == 128;
+            const auto tc = [&](uint32_t K, uint32_t N) { return split_tc(N / 128, K / 128, 148, nr, g); };
+            is(tc(8192, 1024), 18, 4, __LINE__);
+            is(tc(2944, 1152), 16, 2, __LINE__);
+            is(tc(4096, 4096), 4, 8, __LINE__);
+            is(tc(3072, 5120), 3, 8, __LINE__);
+            is(tc(1536, 9472), 2, 6, __LINE__);
+            is(tc(5120, 5120), wide ? 3 : 0, wide ? 14 : 11, __LINE__);
+            is(tc(14336, 4096), wide ? 4 : 0, wide ? 28 : 25, __LINE__);
+            is(tc(2944, 11136), 0, 14, __LINE__);
+        }
     const auto st = [](uint32_t K, uint32_t N, uint32_t rows, bool outliers) {
         const uint32_t BN = N % 256 ? 128 : 256;
         return split_streaming(BN, N / BN, K / 128, 148, rows, outliers);
