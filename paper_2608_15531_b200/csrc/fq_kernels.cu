@@ -488,24 +488,27 @@ static DirectFn pick_direct(const fq_layout_t* L, uint32_t rows, uint32_t warps,
     return direct_uniform(L, rows) ? pick_direct_rows<32, true>(rows, g) : pick_direct_rows<32, false>(rows, g);
 }
 
-// Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 28.7 us
-// at 9 to 16 rows, 32.3 at 32), the warp-level MMA kernels' grows (24.7 us at 8 rows, 34.6 at 16), and its start-up costs about
-// 4 us more than theirs.  It writes outliers into a tile instead of adding them, so an encoding that names a position
-// twice (or may do so) stays with launches of 16 rows on the other kernels.  Times below: us, theirs / its, 1 % unless stated.
+// Which kernel serves a launch.  The tcgen05 kernel's time hardly depends on the rows (4096 x 28672, 1 % of outliers: 28.0 us
+// at nine rows, 28.2 at 16, 31.1 at 32), the warp-level MMA kernels' grows (20.4 us at one row, 24.0 at eight, 34.8 at 16), and its start
+// and end cost more than theirs (1024 x 4096 at nine 4.3 / 5.6).  It writes outliers into a tile instead of adding them, so an encoding that names a
+// position twice (or may do so) stays with launches of 16 rows on the other kernels.  Times below: us, theirs / its, 1 % unless stated.
 //   more than 16 rows   always
-//   9 to 16 rows        with tails (2048 x 2048 9.2 / 7.5), or from 512 units of 128 x 128 weights up (4096 x 4096 10.7 / 8.8, 1024 x 8192
-//                       7.8 / 6.8).  But not jobs of one k-step to a warp of the short-job kernel (2048 x 4096 6.2 / 6.9, at 0.5 % 5.7 /
-//                       6.9, 2048 x 4608 6.2 / 7.2), unless their buckets are deep (2 %: 7.6 / 7.1, 5 %: 12.4 / 7.9).
+//   9 to 16 rows        with tails (2048 x 2048 8.8 / 6.2), or from 512 units of 128 x 128 weights up (4096 x 4096 10.4 / 8.2, 1024 x 8192
+//                       7.5 / 6.5; 1024 x 6144, which is no short job either and stays with theirs, 8.1 / 6.2).  But not jobs of one k-step to a warp of
+//                       the short-job kernel (2048 x 4096 6.2 / 6.35, at 0.5 % 5.6 / 6.3, 2048 x 4608 6.2 / 6.65), unless their buckets are
+//                       deep (2 %: 8.5 / 6.5, 5 %: 12.5 / 7.5).
 //   2 to 8 rows         tiles of 128 columns, where the streaming kernel has half the dense warps, at least 1024 units, no short job; and
-//     with tails        always (4096 x 6272 at 2 % 14.6 / 13.1, 8 rows 17.2 / 13.1; 8192 x 16512 58.3 / 56.5, 72.4 / 56.4)
-//     else              where the streaming kernel would run one group of dense warps (1024 x 16512 10.2 / 9.5); from 4096 units at
-//                       up to four rows (8192 x 16512 32.9 / 32.1, 2048 x 28800 17.3 / 17.6) if buckets are not deep (8192 x 16512 at 2 %
-//                       34.1 / 33.1, at 5 % 38.2 / 46.9); from 3072 at five and more (2048 x 28800 at 8 rows 18.7 / 17.6, 4096 x 11136 15.6 /
-//                       15.9), or from 2048 with buckets of middling depth (4096 x 9344 at 2 % 14.9 / 13.9, at 5 % 17.1 / 18.0 at five)
+//     with tails        always (4096 x 6272 at 2 % 14.4 / 12.1, 8 rows 17.1 / 12.2; 8192 x 16512 57.3 / 56.5, 71.2 / 56.6)
+//     else              where the streaming kernel would run one group of dense warps (1024 x 16512 9.5 / 9.2, 8 rows 10.4 / 9.3), or two only by its split along
+//                       the tiles and buckets are deep (2304 x 7296 at five 8.2 / 8.75, at 3 % 9.6 / 9.2, at four 8.7 / 9.2); from 4096 units at
+//                       up to four rows (8192 x 16512 32.3 / 31.2, 2048 x 28800 16.7 / 16.8) if buckets are not deep (8192 x 16512 at 5 %
+//                       37.5 / 46.1; at 2 %, which stays with theirs, 33.7 / 32.4); from 3072 at five and more (2048 x 28800 at 8 rows 17.9 /
+//                       17.0, 8192 x 6272 at five 15.3 / 15.3), or from 2048 with buckets of middling depth (4096 x 9344 at 2 % at five 13.6 / 13.1,
+//                       but at 1 % 12.3 / 12.7; at 5 % 16.7 / 17.2)
 // Without outliers (the layer has none, or the call is the dense half of the unfused pair) it takes launches of more than 16
-// rows, and the others, which have variants without the outlier step, those of up to 16 (4096 x 14336 at 8 rows 14.5 us with the
-// step, 11.5 without); two or three launches of the short-job kernel are faster than one of it on small layers (1024 x 1024 at 32
-// rows 5.0 / 9.3, at 48 7.4 / 9.2, at 64 9.8 / 9.6; 4096 x 4096 at 32 11.9 / 11.0).
+// rows, and the others, which have variants without the outlier step, those of up to 16 (4096 x 14336 at 16 rows 14.8 / 14.9); two or
+// three launches of the short-job kernel are faster than one of it on small layers (1024 x 1024 at 32 rows 4.9 / 7.6, at 48 7.4 / 8.5, at 64
+// 9.8 / 9.7; 2048 x 2048 at 32 7.1 / 8.3, at 48 10.6 / 9.2; 4096 x 4096 at 32 11.9 / 9.7).
 static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers) {
     const uint32_t KT = L->K / kBK, depth = L->max_bucket_packets;
     const uint64_t units = (uint64_t)KT * (L->N / 128);
@@ -515,7 +518,9 @@ static inline bool tc_serves(const fq_layout_t* L, uint32_t rows, bool outliers)
     const bool tails = L->max_tail_packets > 0;
     if (rows >= 9) return tails || (units >= 512 && !(KT <= 16 && depth <= 9 && direct_warps(L, rows, true)));
     if (L->BN != 128 || rows < 2 || units < 1024 || direct_warps(L, rows, true)) return false;
-    if (tails || split_units(L->N / 128, KT, sm_count_cached(), 1).units_per_cta < kTwoGroups) return true;
+    const uint32_t sms = (uint32_t)sm_count_cached();
+    const Split theirs = rows <= 4 || depth <= 10 ? split_streaming(128, L->N / 128, KT, sms, rows, true) : split_units(L->N / 128, KT, sms, 1);
+    if (tails || theirs.units_per_cta < kTwoGroups) return true;
     return rows <= 4 ? units >= 4096 && depth <= 13 : units >= 3072 || (units >= 2048 && depth > 10 && depth <= 18);
 }
 static inline uint32_t rows_per_launch(const fq_layout_t* L, uint32_t rows_left, bool outliers) { return tc_serves(L, rows_left, outliers) ? rows_left : std::min<uint32_t>(rows_left, 16u); }

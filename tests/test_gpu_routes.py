@@ -21,6 +21,8 @@ _SHAPES = [
     (2048, 2048, 0.01, (5, 8)),            # and 16 k-steps, 17 and more
     (2176, 2048, 0.01, (5, 8)),
     (6016, 4096, 0.01, (5, 8)),
+    (2304, 7296, 0.01, (4, 5)),            # tiles of 128 columns, a second group of dense warps only by a split along the tiles: streaming;
+    (2304, 7296, 0.05, (4, 5)),            # from five rows up, if buckets are deep, tcgen05
     (2048, 12800, 0.01, (1, 8)),           # streaming kernel, tiles for two units more: they bring the second group
     (1664, 14336, 0.01, (4, 8)),           # one group either way: ranges with outliers and five rows or more, else tiles
     (1664, 14336, 0.0, (1, 16)),
