@@ -651,7 +651,7 @@ static MmaKernelFn pick_mma_kernel(uint32_t bn, uint32_t M, uint32_t g, bool spa
 typedef void (*TcKernelFn)(const CUtensorMap, const TcParams);
 template <int NR, bool COOP>
 static TcKernelFn pick_tc_group(uint32_t g) { return g == 64 ? (TcKernelFn)fq_tc_kernel<NR, 64, COOP> : (TcKernelFn)fq_tc_kernel<NR, 128, COOP>; }
-static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g, bool coop) {
+static TcKernelFn pick_tc_kernel(uint32_t nr, uint32_t g, bool coop) {             // (coop: always, up to 32 rows)
     if (nr == 128) return coop ? pick_tc_group<128, true>(g) : pick_tc_group<128, false>(g);
     if (nr == 64) return coop ? pick_tc_group<64, true>(g) : pick_tc_group<64, false>(g);
     return nr == 32 ? pick_tc_group<32, true>(g) : pick_tc_group<16, true>(g);

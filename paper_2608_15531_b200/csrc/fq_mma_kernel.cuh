@@ -84,9 +84,9 @@ constexpr int kXPitch = 256;
 //                     the unit's bucket descriptors and packets (or of its zero-points)
 //   then NGRP x BN/32 dense + outliers.  Lane (g, t) of warp w holds the accumulators of columns
 //                     32w + {g, g+8, g+16, g+24}, batch rows 2t, 2t+1 (+8 per octet).  Dense: the
-//                     lane loads, as one 16-byte word group, word t of its four columns of each
-//                     32-row block: 8 codes per column = its share of two k16 steps (the k order
-//                     inside a block follows the 16-byte activation loads of the lanes).  Outliers:
+//                     lane gets, by one ldmatrix, word t of its four columns of each 32-row
+//                     block: 8 codes per column = its share of two k16 steps (the k order inside a
+//                     block follows the 16-byte activation loads of the lanes).  Outliers:
 //                     those four columns are one Tile-COO bucket, so the four lanes of group g walk
 //                     that bucket's packets and add v * x[row][k] straight into their accumulators,
 //                     slot j into column number j (Section 4.2 without the shared-memory scatter:

@@ -15,8 +15,9 @@
 namespace fq {
 
 // Division by a number that the host knows: n / d = upper half of n * (floor(2^64 / d) + 1), exact for every 32-bit n; d = 1 has
-// no such factor (0).  The compiler's division is a chain of some forty instructions, and up to ten of them stood between a CTA's last
-// unit and its last sum: 14336 x 4096 at 16 rows 17.8 us, so 17.1; 4096 x 4096 at 16 8.6 and 8.3; 4096 x 28672 at 8 24.7 and 24.3.
+// no such factor (0).  (Granlund and Montgomery, Division by invariant integers using multiplication, 1994.)  Of the compiler's divisions,
+// each a chain of dependent instructions, up to ten stood between a CTA's last unit and its last sum: 14336 x 4096 at 16 rows 17.8 us,
+// so 17.1; 4096 x 4096 at 16 8.6 and 8.3; 4096 x 28672 at 8 24.7 and 24.3.
 struct Divisor {
     uint32_t lo, hi;
     FQ_HD static Divisor of(uint32_t d) {

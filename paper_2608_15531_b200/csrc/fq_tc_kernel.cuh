@@ -399,6 +399,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
     using S_ = TcShape<NR, GROUP>;
     constexpr int GPS = S_::GPS, NAB = S_::NAB, NDB = S_::NDB, SETS = S_::SETS, NWO = S_::NWO, UG = S_::UG;
     constexpr uint32_t W_BYTES = 8192, SZ_ROW = 256;
+    static_assert(COOP || NR >= 64, "see tc_coop");
     constexpr bool DEFER = COOP && (NR == 32 || (NR == 16 && GROUP == 64));
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -719,7 +720,7 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                 // Split tile.  Every warp settles its own 32 columns and rows, without CTA-wide barriers: FP32 partial, four
                 // rows of a column to 16 bytes, then one arrival per (tile, strip, set of rows: a byte of the strip's
                 // counter each); the last to arrive adds the partials in CTA order (the same order in every run) and writes Y:
-                // this warp, or the whole CTA if the range ends here (COOP).
+                // this warp, or the whole CTA if the range ends here (COOP), and wherever it is the last (DEFER).
                 constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;      // float4 per slot
                 const uint32_t which = p.shares.slot_of(blockIdx.x, tn, KT);
                 float4* slots = reinterpret_cast<float4*>(p.partials) + (size_t)(r0 / 4) * COLS + col;
@@ -746,10 +747,10 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
                     atomicSub(counter, (c_last - c_first + 1) << (8 * set));                     // ready for the next call
                     if (DEFER || piece_stop == u_end) atomicOr(settle + (piece_stop == u_end ? 0 : 1), 1u << (set * 4 + dw));
                 }
-                if (!DEFER && last && !(COOP && piece_stop == u_end)) {
+                if constexpr (!DEFER) if (last && !(COOP && piece_stop == u_end)) {
                     write_y = true;
                     // 16 rows at a time, ND contributors' loads in flight; the additions keep CTA order
-                    constexpr int ND = NR >= 64 || !COOP ? 2 : 1;
+                    constexpr int ND = NR >= 64 ? 2 : 1;
 #pragma unroll
                     for (int i0 = 0; i0 < RT / 4; i0 += 4)
                         if (r0 + 4 * i0 < p.M) {
@@ -817,8 +818,8 @@ fq_tc_kernel(const __grid_constant__ CUtensorMap xmap, const TcParams p) {
         for (uint32_t side = 0; side < (DEFER ? 2u : 1u); ++side) {
             const uint32_t mine = settle[side];
             if (!mine) continue;
-            // The sums of the range's last tile (the drain warps' acquire is handed on by the barrier above): a thread takes four
-            // rows of a column, with ND contributors' loads in flight.
+            // The sums of the range's last tile, or (side 1) of its first (the drain warps' acquire is handed on by the barrier above): a
+            // thread takes four rows of a column, with ND contributors' loads in flight.
             constexpr uint32_t COLS = 128, SLOT = COLS * NR / 4;
             constexpr int ND = 6;
             uint32_t begin = u_begin, end = u_end, c_first, c_last;
