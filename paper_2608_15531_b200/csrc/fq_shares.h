@@ -84,7 +84,7 @@ constexpr uint32_t kTwoGroups = 8;      // units per CTA from which the streamin
 //     13.6 / 12.5, 18688 x 8960 26.5 / 26.0; two, up to 16 units, 3200 x 15616 12.5 / 12.0, 3840 x 15360 13.7 / 13.3, 2816 x 13824 10.2 / 10.6, beyond them
 //     5120 x 16384 16.0 / 16.1, 12288 x 17920 at four 34.8 / 35.6; without outliers up to 24, 6400 x 17152 15.8 / 15.4, 14976 x 18176 30.5 / 30.8
 //   five rows and more, and two to four on tiles of 128 columns: no (3328 x 14592 at eight 13.2 / 14.3, 24320 x 3840 20.5 / 21.5, 11520 x 4224 15.9 / 16.9,
-//     8192 x 6400 14.9 / 14.6; without outliers, where the CTAs of tiles read the same rows of X at a time, 15232 x 18432 at eight
+//     8192 x 6400 14.9 / 14.6; without outliers, where the CTAs, all at the same k-steps, take 4 to 9 % longer for a unit, 15232 x 18432 at eight
 //     32.1 / 35.7, 10880 x 9088 at 16 23.5 / 25.9; 22656 x 2176 at four 15.9 / 16.2)
 // (Seven units more, 28672 x 8192 at one row: 33.9 / 36.0.)
 inline Split split_streaming(uint32_t BN, uint32_t NT, uint32_t KT, uint32_t sms, uint32_t rows, bool outliers) {

@@ -31,15 +31,15 @@
 //
 // What bounds it, per unit in SM clocks: HBM at the measured copy rate would need 425; 8 dense + 8 outlier MMAs issued back
 // to back with their commits take 430 at N = 16, 490 at 32, 650 at 64, 1030 at 128 (an outlier MMA is bound by reading its 4 KB
-// of A from shared memory up to N = 64).  The kernel takes 1100 at 32 rows and 1880 at 112 (8192 x 28672, 1 % of outliers: 54.4
-// and 92.7 us).  That is instruction issue and latency: 2670 warp instructions a unit at 32 rows and 4580 at 128 fill 65 % of the issue
-// slots (900 to 1170 of them on the half-rate integer pipe, half of those the unpacking, seven logic operations and four BF16 pair
+// of A from shared memory up to N = 64).  The kernel takes 1100 at 32 rows and 1880 at 112 (8192 x 28672, 1 % of outliers: 53.4
+// and 92.9 us).  That is instruction issue and latency: 2660 warp instructions a unit at 32 rows and 4530 at 128 fill 67 % of the issue
+// slots (980 to 1210 of them on the half-rate integer pipe, half of those the unpacking, seven logic operations and four BF16 pair
 // additions for eight codes), and every role's work on a unit is a chain of barriers and memory latencies of 800 clocks and
-// more, which the groups of warps taking units in turn hide only in part.  At 128 rows the tensor pipe is busy 59 % of the time,
-// the drain's FMAs come on top, and both variants spill.  Outliers cost little: 55.2 us without any at 32 rows, 58.9 at 3 %
-// (when 1 % took 55.4).
+// more, which the groups of warps taking units in turn hide only in part.  At 128 rows the tensor pipe is busy 61 % of the time,
+// the drain's FMAs come on top, and both variants spill.  Outliers cost little: 52.7 us without any at 32 rows, 57.0 at 3 %
+// (1 %: 53.6).
 // Before, launches of 17 to 32 rows ran on the 8-bit integer tensor path, activations as three limbs and outliers applied row
-// by row (8192 x 28672 at 32 rows 124.5 us; 4096 x 28672 at 128 rows, in four launches, 305, now 55).
+// by row (8192 x 28672 at 32 rows 124.5 us; 4096 x 28672 at 128 rows, in four launches, 305, now 53).
 
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
